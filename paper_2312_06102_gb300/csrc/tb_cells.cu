@@ -304,6 +304,8 @@ __global__ void __launch_bounds__(kScanThreads)
     info->max_depth = dmax;
     if (cell_cap > 0 && off > cell_cap) info->status |= kErrOverflow;
     info->misc_ctr[1] = 0;
+    // the moments' leaf queues, and the barrier count of their upward pass
+    for (int i : {2, 5, 7}) info->misc_ctr[i] = 0;
 }
 
 // Emission over the leaf starts only, one count tile (1024 particles) per

@@ -173,6 +173,12 @@ __device__ __forceinline__ uint64_t ld_relaxed_u64(const uint64_t *p) {
     return v;
 }
 
+__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 __device__ __forceinline__ void st_relaxed_u64(uint64_t *p, uint64_t v) {
     asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
@@ -244,6 +250,11 @@ __device__ __forceinline__ void bulk_load(void *dst_smem, const void *src, uint3
         : "memory");
 }
 
+// The same bytes into L2 only (same size and alignment rules), not awaited.
+__device__ __forceinline__ void bulk_prefetch(const void *src, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+}
+
 // Shared -> global bulk copy (same size and alignment rules), tracked by the
 // issuing thread's bulk group.
 __device__ __forceinline__ void bulk_store(void *dst, const void *src_smem, uint32_t bytes) {
@@ -274,6 +285,11 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // copies (the asynchronous proxy) that touch the same memory.
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+
+// The same for accesses to any memory, global writes among them.
+__device__ __forceinline__ void fence_proxy_async() {
+    asm volatile("fence.proxy.async;" ::: "memory");
 }
 
 }  // namespace tb

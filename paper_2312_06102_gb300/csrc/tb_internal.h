@@ -45,8 +45,9 @@ struct DevInfo {
     int64_t level_offset[kLevels + 1];
     uint32_t sort_tile_ctr[16];   // dynamic tile ids, one counter per sort pass
     uint32_t misc_ctr[8];         // [0] bbox blocks done, [1] level-scan blocks done,
-                                  // [2] big-leaf queue length, [3] big-leaf tickets,
-                                  // [4] key blocks done, [5] long sort runs, [6] their tickets
+                                  // [2] big-leaf queue length, [4] key blocks done,
+                                  // [5] long sort runs, later the long-leaf queue length,
+                                  // [6] long sort runs' tickets, [7] upward-pass barrier
 };
 
 // Sort tuning: a compiled variant.
@@ -185,6 +186,27 @@ inline bool first_on_device(std::atomic<uint64_t> &done) {
     if (done.load(std::memory_order_acquire) & bit) return false;
     done.fetch_or(bit, std::memory_order_acq_rel);
     return true;
+}
+
+// Blocks of a kernel that are resident at once on the current device, looked
+// up once per device and kept in `known` (zero-initialised, one per kernel).
+inline cudaError_t resident_blocks(std::atomic<int> (&known)[64], const void *kernel, int threads,
+                                   size_t smem, int64_t &blocks) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    int v = dev >= 0 && dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+    if (v == 0) {
+        int sms = 0, per_sm = 0;
+        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem)) !=
+                cudaSuccess)
+            return e;
+        v = sms * (per_sm > 0 ? per_sm : 1);
+        if (dev >= 0 && dev < 64) known[dev].store(v, std::memory_order_relaxed);
+    }
+    blocks = v;
+    return cudaSuccess;
 }
 
 }  // namespace tb

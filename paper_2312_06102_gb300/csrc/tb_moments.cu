@@ -7,14 +7,12 @@
 //                          into shared memory, its (x, y, z, m) records
 //                          gathered beside it (Sec. 2.3 step 3, the reorder),
 //                          one thread per leaf summing from there;
-//   long_leaf_kernel     : leaves the tile could not hold, members read
-//                          through the permutation;
-//   big_leaf_kernel      : depth-21 leaves of identical keys that are too long
-//                          for one thread, summed block-wide;
-//   level_moments_kernel : one launch per level, deepest first: the children
-//                          of the level, in tiles bulk-copied (TMA) into
-//                          shared memory, and every non-leaf cell of the
-//                          level combined from its tile.
+//   upward_kernel        : leaves the tiles could not hold, members read
+//                          through the permutation (a warp, or a block, per
+//                          leaf); then level by level, deepest first, the
+//                          children of the level, in tiles bulk-copied (TMA)
+//                          into shared memory, and every non-leaf cell of
+//                          the level combined from its tile.
 //
 // Moments of a cell: M = sum m; centre of mass c = sum m x / M; central
 // second moment Q = sum m (x - c)(x - c)^T (6 components xx xy xz yy yz zz);
@@ -121,7 +119,7 @@ __device__ __forceinline__ void warp_leaf_sum(const MomOut &o, Src src, int64_t 
 //   4. One thread per leaf sums its members from shared memory.  A leaf that
 //      runs past the staged span (only a depth-21 leaf of identical keys, or
 //      n_crit above the halo, can) and, in the compensated mode, a leaf of
-//      more than kSplitLeaf members go to the queue of long_leaf_kernel.
+//      more than kSplitLeaf members go to the queues of upward_kernel.
 constexpr int kLtThreads = 256;
 constexpr int kLtTile = 2048;                  // two cell-pass tiles of 1024
 constexpr int kLtHalo = 64;
@@ -151,8 +149,8 @@ __global__ void __launch_bounds__(kLtThreads, 4)
     leaf_tile_kernel(MomOut o, const int32_t *__restrict__ leaf_cell,
                      const int32_t *__restrict__ perm, const float4 *__restrict__ xm,
                      const uint16_t *__restrict__ ml, const uint32_t *__restrict__ leaf_off,
-                     int64_t n, float4 *__restrict__ xs, int32_t *long_queue, DevInfo *info,
-                     int64_t wait_limit) {
+                     const int32_t *__restrict__ pend, int64_t n, float4 *__restrict__ xs,
+                     int32_t *long_queue, int32_t *big_queue, DevInfo *info, int64_t wait_limit) {
     if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout)) return;
     extern __shared__ __align__(128) unsigned char lt_raw[];
     LeafTileSmem &S = *reinterpret_cast<LeafTileSmem *>(lt_raw);
@@ -285,7 +283,11 @@ __global__ void __launch_bounds__(kLtThreads, 4)
         const int64_t c = leaf_cell[jbase + r];
         const bool staged = xe >= 0;
         if (!staged) {
-            long_queue[atomicAdd(&info->misc_ctr[5], 1u)] = (int32_t)c;
+            // the end is past the span: leaves too long for one warp apart
+            if (pend[c] - (int32_t)(k0 + x) > kBigLeafThread)
+                big_queue[atomicAdd(&info->misc_ctr[2], 1u)] = (int32_t)c;
+            else
+                long_queue[atomicAdd(&info->misc_ctr[5], 1u)] = (int32_t)c;
             continue;
         }
         if (MODE == TB_MOM_FP32_COMP && xe - x > kSplitLeaf) {
@@ -309,30 +311,8 @@ __global__ void __launch_bounds__(kLtThreads, 4)
     if (xs && threadIdx.x == 0) bulk_store_wait_read();
 }
 
-// The queued leaves, one warp per leaf, members read through the
-// permutation (32 independent loads per round).  Leaves of more than
-// kBigLeafThread members -- only depth-21 leaves of identical keys -- are
-// queued again for big_leaf_kernel.
-template <int MODE>
-__global__ void __launch_bounds__(kMomThreads, 4)
-    long_leaf_kernel(TreeIn T, MomOut o, PermSrc src, const int32_t *long_queue, DevInfo *info) {
-    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t nq = *(volatile const uint32_t *)&info->misc_ctr[5];
-    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x / 32);
-    for (int64_t q = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32; q < nq; q += nwarps) {
-        const int64_t c = long_queue[q];
-        const int64_t pf = T.pfirst[c], pe = T.pend[c];
-        if (pe - pf > kBigLeafThread) {
-            if (lane == 0) T.big_leaf[atomicAdd(&info->misc_ctr[2], 1u)] = (int32_t)c;
-            continue;
-        }
-        warp_leaf_sum<MODE>(o, src, c, pf, pe);
-    }
-}
-
-// Non-leaf cells of level d from their children at level d + 1, which the
-// leaf launches or the launch for level d + 1 finished.  The children of
+// Non-leaf cells level by level, deepest first, each level d from its
+// children at level d + 1.  The children of
 // consecutive cells are consecutive cells, so level d + 1 is cut into tiles
 // of kLmTile children: a block bulk-copies (TMA) the FP32 moments and the
 // parent links of its tile -- plus the few children past it that belong to
@@ -343,8 +323,8 @@ __global__ void __launch_bounds__(kMomThreads, 4)
 // 16-byte boundary; the moment and parent arrays are allocated kMomentPad
 // cells past the capacity, which the rounding never passes.  The up to three
 // cells the rounding adds before a level's first tile belong to level d,
-// which this launch writes: they are copied but never read.  Blocks loop
-// over the tiles of the level (one persistent grid per launch).
+// which is being written: they are copied but never read.  Blocks loop
+// over the tiles of the level.
 constexpr int kLmThreads = 128;
 constexpr int kLmTile = 512;
 constexpr int kLmSpan = kLmTile + 16;   // 3 before the tile, 7 past it, rounding to 4
@@ -378,106 +358,158 @@ struct CellsStaged {
     }
 };
 
+// The parents of the children tile t of level d + 1, [off1, off2), staged and
+// combined by one block; false when a copy did not complete.
 template <int MODE>
-__global__ void __launch_bounds__(kLmThreads, 5)
-    level_moments_kernel(TreeIn T, MomOut o, DevInfo *info, int d, int64_t wait_limit) {
-    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout)) return;
-    extern __shared__ __align__(128) unsigned char lm_raw[];
-    LevelSmem &S = *reinterpret_cast<LevelSmem *>(lm_raw);
+__device__ __forceinline__ bool level_tile(const TreeIn &T, const MomOut &o, DevInfo *info, LevelSmem &S,
+                                           int64_t off1, int64_t off2, int tile, int64_t t,
+                                           uint32_t &phase, int64_t wait_limit) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t off1 = info->level_offset[d + 1], off2 = info->level_offset[d + 2];
-    const int64_t tiles = (off2 - off1 + kLmTile - 1) / kLmTile;
-    if ((int64_t)blockIdx.x >= tiles) return;
+    const int64_t c_lo = off1 + t * tile, c_hi = min64(c_lo + tile, off2);
+    const int64_t s_lo = c_lo & ~int64_t(3);
+    const int64_t s_hi = (min64(c_hi + 7, off2) + 3) & ~int64_t(3);
+    // parent links from one group of four before s_lo (the cell before
+    // c_lo), or from the level's start
+    const int64_t p_lo = s_lo >= off1 + 4 ? s_lo - 4 : (off1 & ~int64_t(3));
     if (threadIdx.x == 0) {
-        mbar_init(&S.bar, 1);
-        mbar_init_fence();
-    }
-    __syncthreads();
-    uint32_t phase = 0;
-    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-        const int64_t c_lo = off1 + t * kLmTile, c_hi = min64(c_lo + kLmTile, off2);
-        const int64_t s_lo = c_lo & ~int64_t(3);
-        const int64_t s_hi = (min64(c_hi + 7, off2) + 3) & ~int64_t(3);
-        // parent links from one group of four before s_lo (the cell before
-        // c_lo), or from the level's start
-        const int64_t p_lo = s_lo >= off1 + 4 ? s_lo - 4 : (off1 & ~int64_t(3));
-        if (threadIdx.x == 0) {
-            const uint32_t len = (uint32_t)(s_hi - s_lo);
-            const uint32_t plen = (uint32_t)(s_hi - p_lo);
-            mbar_arrive_expect_tx(&S.bar, len * 76u + plen * 4u);
+        const uint32_t len = (uint32_t)(s_hi - s_lo);
+        const uint32_t plen = (uint32_t)(s_hi - p_lo);
+        // the FP64 mode reads its sums from the tree, only the boxes from here
+        constexpr bool f32 = MODE != TB_MOM_FP64;
+        mbar_arrive_expect_tx(&S.bar, len * (f32 ? 76u : 24u) + plen * 4u);
+        if constexpr (f32) {
             bulk_load(S.mass, o.mass + s_lo, len * 4u, &S.bar);
             bulk_load(S.com, o.com + 3 * s_lo, len * 12u, &S.bar);
             bulk_load(S.com_lo, o.com_lo + 3 * s_lo, len * 12u, &S.bar);
             bulk_load(S.quad, o.quad + 6 * s_lo, len * 24u, &S.bar);
-            bulk_load(S.aabb, o.aabb + 6 * s_lo, len * 24u, &S.bar);
-            bulk_load(S.par, T.parent + p_lo, plen * 4u, &S.bar);
         }
-        const bool ok = mbar_wait_bounded(&S.bar, phase, wait_limit);
-        phase ^= 1u;
-        if (!__syncthreads_and(ok)) {
-            if (threadIdx.x == 0) {
-                flag_error(&info->status, kErrTimeout);
-                mbar_wait_bounded(&S.bar, phase ^ 1u, wait_limit);
-            }
-            return;
+        bulk_load(S.aabb, o.aabb + 6 * s_lo, len * 24u, &S.bar);
+        bulk_load(S.par, T.parent + p_lo, plen * 4u, &S.bar);
+    }
+    const bool ok = mbar_wait_bounded(&S.bar, phase, wait_limit);
+    phase ^= 1u;
+    if (!__syncthreads_and(ok)) {
+        if (threadIdx.x == 0) {
+            flag_error(&info->status, kErrTimeout);
+            mbar_wait_bounded(&S.bar, phase ^ 1u, wait_limit);
         }
-        // the parents whose first child is in the tile, in order: four
-        // children per thread, a warp prefix and one across the warps
-        const int nt = (int)(c_hi - c_lo);
-        uint32_t fl = 0;
+        return false;
+    }
+    // the block's next tile of the level on its way to L2 meanwhile
+    const int64_t n_lo = (off1 + (t + gridDim.x) * tile) & ~int64_t(3);
+    if (threadIdx.x == 0 && n_lo < off2) {
+        const uint32_t len = (uint32_t)(((min64(n_lo + tile, off2) + 3) & ~int64_t(3)) - n_lo);
+        if constexpr (MODE != TB_MOM_FP64) {
+            bulk_prefetch(o.mass + n_lo, len * 4u);
+            bulk_prefetch(o.com + 3 * n_lo, len * 12u);
+            bulk_prefetch(o.com_lo + 3 * n_lo, len * 12u);
+            bulk_prefetch(o.quad + 6 * n_lo, len * 24u);
+        }
+        bulk_prefetch(o.aabb + 6 * n_lo, len * 24u);
+        bulk_prefetch(T.parent + n_lo, len * 4u);
+    }
+    // the parents whose first child is in the tile, in order: four
+    // children per thread, a warp prefix and one across the warps
+    const int nt = (int)(c_hi - c_lo);
+    uint32_t fl = 0;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int x = 4 * (int)threadIdx.x + j;
-            if (x < nt) {
-                const int64_t c = c_lo + x;
-                if (c == off1 || S.par[c - p_lo] != S.par[c - 1 - p_lo]) fl |= 1u << j;
-            }
+    for (int j = 0; j < 4; ++j) {
+        const int x = 4 * (int)threadIdx.x + j;
+        if (x < nt) {
+            const int64_t c = c_lo + x;
+            if (c == off1 || S.par[c - p_lo] != S.par[c - 1 - p_lo]) fl |= 1u << j;
         }
-        const uint32_t cnt = __popc(fl);
-        uint32_t incl = cnt;
+    }
+    const uint32_t cnt = __popc(fl);
+    uint32_t incl = cnt;
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += y;
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+    }
+    if (lane == 31) S.wcount[warp] = incl;
+    __syncthreads();
+    uint32_t pos = incl - cnt, before = 0;
+#pragma unroll
+    for (int w = 0; w < kLmThreads / 32; ++w) {
+        const uint32_t v = S.wcount[w];
+        if (w < warp) pos += v;
+        before += v;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (fl & (1u << j)) S.own[pos++] = S.par[c_lo + 4 * (int)threadIdx.x + j - p_lo];
+    __syncthreads();
+    const CellsStaged src{&S, s_lo};
+    if constexpr (MODE == TB_MOM_FP64) {
+        for (uint32_t b = 0; b < before; b += kLmThreads / 4) {
+            const uint32_t i = b + threadIdx.x / 4;
+            combine_f64_quad(T, o, i < before ? S.own[i] : -1, src);
         }
-        if (lane == 31) S.wcount[warp] = incl;
-        __syncthreads();
-        uint32_t pos = incl - cnt, before = 0;
-#pragma unroll
-        for (int w = 0; w < kLmThreads / 32; ++w) {
-            const uint32_t v = S.wcount[w];
-            if (w < warp) pos += v;
-            before += v;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (fl & (1u << j)) S.own[pos++] = S.par[c_lo + 4 * (int)threadIdx.x + j - p_lo];
-        __syncthreads();
-        const CellsStaged src{&S, s_lo};
+    } else {
         for (uint32_t i = threadIdx.x; i < before; i += kLmThreads)
             combine_children<MODE>(T, o, S.own[i], src);
-        // the next tile's copies overwrite what this one read
-        fence_proxy_async_smem();
-        __syncthreads();
     }
+    return true;
 }
 
-// Block-wide sums of the long depth-21 leaves queued by the leaf launch.
+// Arrival of this block at the gen-th barrier of the grid (cooperative launch:
+// every block is resident), and with `wait` the wait for all others.  What
+// the blocks wrote before is then visible, to bulk copies too (the proxy
+// fences).  The wait is bounded; false when it ran out.
+__device__ __forceinline__ bool grid_meet(uint32_t *ctr, uint32_t gen, bool wait, int64_t limit,
+                                          DevInfo *info) {
+    bool ok = true;
+    fence_proxy_async();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(ctr, 1u);
+        if (wait) {
+            int64_t it = 0;
+            while (ld_acquire_u32(ctr) < gen * gridDim.x)
+                if (!poll_backoff(it, limit)) {
+                    flag_error(&info->status, kErrTimeout);
+                    ok = false;
+                    break;
+                }
+            __threadfence();
+            fence_proxy_async();
+        }
+    }
+    return wait ? __syncthreads_and(ok) != 0 : true;
+}
+
+constexpr int kBigThreads = kLmThreads;
+struct BigLeafSmem {
+    double d[kBigThreads][10];
+    float f[kBigThreads][20];
+    float bb[kBigThreads][6];
+};
+static_assert(sizeof(BigLeafSmem) <= sizeof(LevelSmem), "shares the level tiles' memory");
+
+// The leaves the leaf launch queued: the long ones one warp per leaf, members
+// read through the permutation (32 independent loads per round); those of
+// more than kBigLeafThread members -- only depth-21 leaves of identical keys --
+// summed by a whole block, one after another.
 template <int MODE>
-__global__ void __launch_bounds__(kBigThreads)
-    big_leaf_kernel(TreeIn T, MomOut o, PermSrc xs, DevInfo *info) {
-    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout)) return;
-    __shared__ uint32_t s_q;
-    __shared__ float s_bb[kBigThreads][6];
-    __shared__ double s_d[kBigThreads][10];
-    __shared__ float s_f[kBigThreads][20];
-    const uint32_t nq = *(volatile uint32_t *)&info->misc_ctr[2];
-    for (;;) {
-        if (threadIdx.x == 0) s_q = atomicAdd(&info->misc_ctr[3], 1u);
-        __syncthreads();
-        const uint32_t q = s_q;
-        __syncthreads();
-        if (q >= nq) return;
+__device__ __noinline__ void queued_leaves(TreeIn T, MomOut o, PermSrc xs,
+                                           const int32_t *long_queue, DevInfo *info,
+                                           unsigned char *raw) {
+    {
+        const int64_t nl = info->misc_ctr[5];
+        const int64_t nwarps = (int64_t)gridDim.x * (kLmThreads / 32);
+        for (int64_t q = (blockIdx.x * (int64_t)kLmThreads + threadIdx.x) / 32; q < nl; q += nwarps) {
+            const int64_t c = long_queue[q];
+            warp_leaf_sum<MODE>(o, xs, c, T.pfirst[c], T.pend[c]);
+        }
+    }
+    BigLeafSmem &S = *reinterpret_cast<BigLeafSmem *>(raw);
+    auto &s_d = S.d;
+    auto &s_f = S.f;
+    auto &s_bb = S.bb;
+    const uint32_t nq = info->misc_ctr[2];
+    for (uint32_t q = blockIdx.x; q < nq; q += gridDim.x) {
         const int64_t c = T.big_leaf[q];
         const int64_t pf = T.pfirst[c], pe = T.pend[c];
         const int64_t cnt = pe - pf;
@@ -581,6 +613,76 @@ __global__ void __launch_bounds__(kBigThreads)
     }
 }
 
+// Queued leaves, then the non-leaf cells of levels d_hi .. d_lo, deepest first.
+// One cooperative launch takes every level (d_hi = 20, d_lo = 0), with a grid
+// barrier between levels; levels that do not exist cost nothing.  From the
+// first level on whose children, and those of every level above, fill one
+// tile at most, block 0 goes on alone and the levels are separated by block
+// barriers.  At 65,536 uniform particles this takes 30 us; 21 launches of one
+// level each took 78 us (16 of them for levels without parents, 2.8 us each)
+// and two more for queued leaves 6 us.  At 2^27 clustered, where the big
+// levels' bytes bound it, 0.78 ms against 0.79.  In FP64, bound by latency and
+// the FP64 pipe, 0.45 ms against 0.52 at 6,000,000.  A device that
+// takes no cooperative launch gets one launch per level (d_hi = d_lo, no
+// barrier), queued leaves first (d_hi < 0).
+template <int MODE>
+__global__ void __launch_bounds__(kLmThreads, 5)
+    upward_kernel(TreeIn T, MomOut o, PermSrc src, const int32_t *long_queue, DevInfo *info, int d_hi,
+                  int d_lo, bool leaves, int64_t wait_limit) {
+    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout)) return;
+    extern __shared__ __align__(128) unsigned char lm_raw[];
+    LevelSmem &S = *reinterpret_cast<LevelSmem *>(lm_raw);
+    __shared__ int64_t s_off[kLevels + 1];
+    __shared__ uint32_t s_queued;
+    uint32_t *meet = &info->misc_ctr[7];
+    if (threadIdx.x <= kLevels) s_off[threadIdx.x] = info->level_offset[threadIdx.x];
+    if (threadIdx.x == 0) s_queued = leaves ? (info->misc_ctr[2] | info->misc_ctr[5]) : 0u;
+    __syncthreads();
+    uint32_t gen = 0, phase = 0;
+    if (s_queued) {
+        queued_leaves<MODE>(T, o, src, long_queue, info, lm_raw);
+        if (d_hi >= 0 && !grid_meet(meet, ++gen, true, wait_limit, info)) return;
+    }
+    if (d_hi < 0) return;
+    if (threadIdx.x == 0) {
+        mbar_init(&S.bar, 1);
+        mbar_init_fence();
+    }
+    __syncthreads();
+    // levels 0 .. solo: at most one tile of children each
+    int solo = -1;
+    while (solo < d_hi && s_off[solo + 3] - s_off[solo + 2] <= kLmTile) ++solo;
+    for (int d = d_hi; d >= d_lo; --d) {
+        const int64_t off1 = s_off[d + 1], off2 = s_off[d + 2];
+        if (off1 == off2) continue;
+        if (d <= solo && blockIdx.x != 0) return;
+        // smaller tiles where the level would leave blocks idle or give a few
+        // of them one tile more
+        int tile = kLmTile;
+        if (d > solo)
+            while (tile > kLmTile / 4 && off2 - off1 <= (int64_t)gridDim.x * tile * 2) tile /= 2;
+        const int64_t tiles = (off2 - off1 + tile - 1) / tile;
+        for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+            if (!level_tile<MODE>(T, o, info, S, off1, off2, tile, t, phase, wait_limit)) return;
+            // the next tile's copies overwrite what this one read
+            fence_proxy_async_smem();
+            __syncthreads();
+        }
+        if (d == d_lo) break;
+        if (d > solo) {
+            if (!grid_meet(meet, ++gen, d - 1 > solo || blockIdx.x == 0, wait_limit, info)) return;
+        } else {
+            // this block's own cells are the next level's children
+            __threadfence();
+            fence_proxy_async();
+            __syncthreads();
+        }
+    }
+    // block 0 leaves the counters clear for the next call on this build
+    if (blockIdx.x == 0 && threadIdx.x == 0 && d_lo == 0)
+        for (int i : {2, 5, 7}) info->misc_ctr[i] = 0;
+}
+
 __global__ void wait_selftest_kernel(int64_t limit, uint32_t *status, const uint32_t *flag) {
     int64_t iter = 0;
     while (*(volatile const uint32_t *)flag == 0u) {
@@ -596,18 +698,16 @@ cudaError_t moments_impl(tb_tree &t, Workspace &ws, cudaStream_t s) {
     TreeIn T{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
     MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
     const int64_t n = t.n_particles;
-    // misc_ctr[2..3]: big-leaf queue and tickets; [5]: long-leaf queue
-    cudaError_t e = cudaMemsetAsync(&ws.info->misc_ctr[2], 0, 4 * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     static std::atomic<uint64_t> attr_done{0};
     if (first_on_device(attr_done)) {
         cudaFuncSetAttribute(leaf_tile_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)leaf_tile_smem());
         cudaFuncSetAttribute(leaf_tile_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(level_moments_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(upward_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(LevelSmem));
-        cudaFuncSetAttribute(level_moments_kernel<MODE>,
+        cudaFuncSetAttribute(upward_kernel<MODE>,
                              cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
     }
@@ -619,29 +719,41 @@ cudaError_t moments_impl(tb_tree &t, Workspace &ws, cudaStream_t s) {
     const int64_t level_tiles = (n + level_tile_size() - 1) / level_tile_size();
     const uint32_t *leaf_off = ws.level_cnt + (int64_t)kLevels * level_tiles;
     leaf_tile_kernel<MODE><<<(unsigned)tiles, kLtThreads, leaf_tile_smem(), s>>>(
-        o, t.leaf_cell, t.perm, ws.xm, ws.ml, leaf_off, n,
-        t.pos_sorted ? reinterpret_cast<float4 *>(t.pos_sorted) : nullptr, longq, ws.info,
+        o, t.leaf_cell, t.perm, ws.xm, ws.ml, leaf_off, t.pend, n,
+        t.pos_sorted ? reinterpret_cast<float4 *>(t.pos_sorted) : nullptr, longq, ws.big_leaf, ws.info,
         g_wait_limit);
     ++g_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const PermSrc src{ws.xm, t.perm};
-    long_leaf_kernel<MODE><<<152 * 2, kMomThreads, 0, s>>>(T, o, src, longq, ws.info);
-    ++g_launches;
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    big_leaf_kernel<MODE><<<152, kBigThreads, 0, s>>>(T, o, src, ws.info);
-    ++g_launches;
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     mark(ws, "leaves", s);
-    // one persistent grid per launch: five blocks per SM, never more than
-    // the tiles a level of at most n cells can have
-    int64_t grid = (n + kLmTile - 1) / kLmTile;
-    if (grid > 152 * 5) grid = 152 * 5;
-    if (grid < 1) grid = 1;
-    for (int d = kDepthMax - 1; d >= 0; --d) {
-        level_moments_kernel<MODE><<<(unsigned)grid, kLmThreads, sizeof(LevelSmem), s>>>(
-            T, o, ws.info, d, g_wait_limit);
+    // every level in one cooperative launch of as many blocks as are resident
+    // at once, never more than the tiles a level of at most n cells can have
+    PermSrc src{ws.xm, t.perm};
+    int d_hi = kDepthMax - 1, d_lo = 0;
+    bool leaves = true;
+    static std::atomic<int> resident[64];
+    int64_t grid = 0;
+    if ((e = resident_blocks(resident, reinterpret_cast<const void *>(upward_kernel<MODE>), kLmThreads,
+                             sizeof(LevelSmem), grid)) != cudaSuccess)
+        return e;
+    const int64_t most = (n + kLmTile / 4 - 1) / (kLmTile / 4);
+    if (grid > most) grid = most;
+    const int32_t *lq = longq;
+    int64_t lim = g_wait_limit;
+    void *args[] = {&T, &o, &src, &lq, &ws.info, &d_hi, &d_lo, &leaves, &lim};
+    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(upward_kernel<MODE>),
+                                    dim3((unsigned)grid), dim3(kLmThreads), args, sizeof(LevelSmem), s);
+    if (e == cudaSuccess) {
         ++g_launches;
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    } else {
+        // no cooperative launch here: the queued leaves, then one launch per level
+        cudaGetLastError();
+        for (int d = kDepthMax; d >= 0; --d) {
+            upward_kernel<MODE><<<(unsigned)grid, kLmThreads, sizeof(LevelSmem), s>>>(
+                T, o, src, lq, ws.info, d == kDepthMax ? -1 : d, d == kDepthMax ? -1 : d,
+                d == kDepthMax, lim);
+            ++g_launches;
+            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        }
     }
     mark(ws, "moments", s);
     return cudaSuccess;

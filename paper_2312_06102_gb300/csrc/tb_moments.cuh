@@ -4,6 +4,7 @@
 // tb_moments.cu for the method.
 #pragma once
 
+#include <cfloat>
 #include <type_traits>
 
 #include "tb_device.cuh"
@@ -13,7 +14,6 @@ namespace {
 
 constexpr int kMomThreads = 256;
 constexpr int kBigLeafThread = 2048;   // longer leaves are summed by a block
-constexpr int kBigThreads = 256;
 
 struct MomOut {
     float *mass, *com, *com_lo, *quad, *aabb;
@@ -394,7 +394,7 @@ __device__ __forceinline__ void leaf_sum_split(const MomOut &o, Src xs, int64_t 
 // Sum the members [pf, pe) of one leaf from the key-ordered records; loads
 // are issued four at a time before any is used.  Leaves reaching this path
 // hold at most 2048 particles (longer ones, only possible at depth 21, go to
-// big_leaf_kernel), so the FP32 modes never need the FP64 route here.
+// queued_leaves), so the FP32 modes never need the FP64 route here.
 template <int MODE, class Src>
 __device__ void leaf_sum(const MomOut &o, Src xs, int64_t c, int64_t pf, int64_t pe) {
     constexpr int G = 4;
@@ -461,7 +461,7 @@ __device__ __forceinline__ void child_offset(const Src &o, int64_t c, int a, flo
 // than 2^20 particles in the FP32-plain mode).  Kept out of line so that its
 // registers do not weigh on the FP32 path.
 template <int MODE>
-__device__ __noinline__ void combine_f64(const MomOut &o, int64_t p, int32_t c0, int32_t c1,
+__device__ __noinline__ void combine_f64(MomOut o, int64_t p, int32_t c0, int32_t c1,
                                          const float bb[6]) {
         // FP64: relative to the first child's centre
         double ref[3];
@@ -499,6 +499,83 @@ __device__ __noinline__ void combine_f64(const MomOut &o, int64_t p, int32_t c0,
                 }
         }
         write_cell_f64(o, p, M, com, Q, bb, MODE == TB_MOM_FP64);
+}
+
+// FP64 mode: parent p (none when p < 0) from its children by four lanes,
+// lane j taking children j and j + 4; the lanes' sums meet in two shuffle
+// rounds.  The same two passes as combine_f64 -- mass and first moment about
+// the first child's centre, then second moments about the centre of mass --
+// with a quarter of its chain of dependent FP64 operations, whose latency is
+// what a level of few cells costs (20 us a level with one lane per parent).
+// All lanes of the warp call it.
+template <class Src>
+__device__ __forceinline__ void combine_f64_quad(const TreeIn &T, const MomOut &o, int64_t p,
+                                                 const Src &src) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int j = threadIdx.x & 3;
+    int32_t c0 = 0, c1 = 0;
+    if (p >= 0) {
+        c0 = T.child_first[p];
+        c1 = T.child_end[p];
+    }
+    double ref[3] = {0.0, 0.0, 0.0}, m[2] = {0.0, 0.0}, d[2][3];
+    if (p >= 0)
+        for (int a = 0; a < 3; ++a) ref[a] = o.com64[3 * (int64_t)c0 + a];
+    double M = 0.0, S[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int64_t c = c0 + j + 4 * k;
+        if (c < c1) {
+            m[k] = o.mass64[c];
+            M += m[k];
+            for (int a = 0; a < 3; ++a) {
+                d[k][a] = o.com64[3 * c + a] - ref[a];
+                S[a] += m[k] * d[k][a];
+            }
+        }
+    }
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+        M += __shfl_xor_sync(kAll, M, off);
+        for (int a = 0; a < 3; ++a) S[a] += __shfl_xor_sync(kAll, S[a], off);
+    }
+    // one division per lane: lane a takes axis a
+    const double sj = j == 0 ? S[0] : (j == 1 ? S[1] : S[2]);
+    const double rj = (M != 0.0) ? sj / M : 0.0;
+    double r[3], Q[6] = {0, 0, 0, 0, 0, 0};
+    float bb[6] = {FLT_MAX, FLT_MAX, FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX};
+    for (int a = 0; a < 3; ++a) r[a] = __shfl_sync(kAll, rj, a, 4);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int64_t c = c0 + j + 4 * k;
+        if (c < c1) {
+            double e[3];
+            for (int a = 0; a < 3; ++a) e[a] = d[k][a] - r[a];
+            int q = 0;
+            for (int a = 0; a < 3; ++a)
+                for (int b = a; b < 3; ++b, ++q) Q[q] += o.quad64[6 * c + q] + m[k] * e[a] * e[b];
+            const float2 lo = src.b2(c, 0), mid = src.b2(c, 1), hi = src.b2(c, 2);
+            bb[0] = fminf(bb[0], lo.x);
+            bb[1] = fminf(bb[1], lo.y);
+            bb[2] = fminf(bb[2], mid.x);
+            bb[3] = fmaxf(bb[3], mid.y);
+            bb[4] = fmaxf(bb[4], hi.x);
+            bb[5] = fmaxf(bb[5], hi.y);
+        }
+    }
+#pragma unroll
+    for (int off = 1; off < 4; off <<= 1) {
+        for (int q = 0; q < 6; ++q) Q[q] += __shfl_xor_sync(kAll, Q[q], off);
+        for (int a = 0; a < 3; ++a) {
+            bb[a] = fminf(bb[a], __shfl_xor_sync(kAll, bb[a], off));
+            bb[3 + a] = fmaxf(bb[3 + a], __shfl_xor_sync(kAll, bb[3 + a], off));
+        }
+    }
+    if (p >= 0 && j == 0) {
+        double com[3];
+        for (int a = 0; a < 3; ++a) com[a] = ref[a] + r[a];
+        write_cell_f64(o, p, M, com, Q, bb, true);
+    }
 }
 
 // Parent p from its children, whose FP32 moments come from `src` (the tree's
