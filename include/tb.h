@@ -95,7 +95,9 @@ typedef struct {
     int32_t reorder;         /* 1: tb_moments also writes pos_sorted (particles in key
                                 order, Sec. 2.3 step 3) */
     int32_t radix_bits;      /* 0 = tuned default; else 8..11 (sort digit width);
-                                tb_build only */
+                                tb_build only.  With all three sort fields 0 a
+                                set of up to 65,536 particles takes one launch for
+                                root, keys and sort (unless tb_profile is on) */
     int32_t sort_threads;    /* 0 = tuned default; else threads per sort tile; tb_build only */
     int32_t sort_items;      /* 0 = tuned default; else keys per thread of a sort tile
                                 (compiled variants: see tb_sort_variant); tb_build only */
@@ -298,7 +300,8 @@ int64_t tb_kernel_launches(void);
  * tb_stage_times synchronises the stream and writes up to `max` elapsed
  * times (ms) of the last build and moment call, returning the count; names
  * come from tb_stage_name.  Stage 0 is the root cell, 1 the keys, 2..1+P the
- * P sort passes, then level counts, cell emission and moments. */
+ * P sort passes, then level counts, cell emission and moments (a small set,
+ * otherwise sorted in one launch, takes these stages too while profiled). */
 tb_status tb_profile(tb_tree *tree, int32_t enable);
 int32_t tb_stage_times(tb_tree *tree, tb_stream stream, float *ms, int32_t max);
 const char *tb_stage_name(tb_tree *tree, int32_t i);

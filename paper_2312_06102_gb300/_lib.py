@@ -251,6 +251,9 @@ def _check(code, what):
 
 
 KEYS_MORTON, KEYS_HILBERT = 0, 1
+# sets up to this size are sorted in one launch when no variant is named: a
+# tuned variant of the radix passes would only slow them down
+ONE_LAUNCH_SORT_MAX = 65536
 
 
 def build(pos: torch.Tensor, mass: torch.Tensor | None = None, n_crit: int = 16,
@@ -264,7 +267,7 @@ def build(pos: torch.Tensor, mass: torch.Tensor | None = None, n_crit: int = 16,
     if pos.dtype != torch.float32 or pos.dim() != 2 or pos.shape[1] != 3:
         raise ValueError("pos must be a [n,3] float32 tensor")
     t = tree if tree is not None else Tree()
-    if sort_cfg is None and not radix_bits:
+    if sort_cfg is None and not radix_bits and pos.shape[0] > ONE_LAUNCH_SORT_MAX:
         from . import autotune
         sort_cfg = autotune.cached(pos.shape[0])
     p = _params(n_crit, mom_mode, cell_capacity, reorder, radix_bits, 0, sort_cfg)

@@ -46,6 +46,9 @@ void dev_free(T *&p) {
     p = nullptr;
 }
 
+int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
+int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
+
 struct TreeState {
     tb_tree pub;
     Workspace ws;
@@ -115,7 +118,10 @@ tb_status ensure_particles(TreeState &S, int64_t n, const SortCfg &cfg, bool reo
     Workspace &ws = S.ws;
     tb_tree &t = S.pub;
     const int64_t tiles = (n + cfg.tile() - 1) / cfg.tile();
-    const int64_t need_lb = tiles * (int64_t(1) << cfg.radix_bits);
+    // look-back words for this set and for any smaller one rebuilt in its
+    // place, which may take smaller tiles (2048 keys up to kSmallTileMax)
+    const int64_t small = (min64(n, kSmallTileMax) + 2047) / 2048 * 256;
+    const int64_t need_lb = max64(tiles * (int64_t(1) << cfg.radix_bits), small);
     const int64_t ltiles = (n + level_tile_size() - 1) / level_tile_size();
     if (n > ws.n_cap || need_lb > ws.tiles_cap || ltiles > ws.level_tiles_cap) {
         cudaDeviceSynchronize();
@@ -200,14 +206,15 @@ tb_status read_info(TreeState &S, cudaStream_t s) {
     return from_dev(S.ws.h_info->status);
 }
 
-SortCfg pick_cfg(const tb_params *p) {
-    SortCfg c = default_sort_cfg(p->radix_bits ? p->radix_bits : 8);
+SortCfg pick_cfg(const tb_params *p, int64_t n) {
+    const int bits = p->radix_bits ? p->radix_bits : 8;
+    SortCfg c = p->sort_threads || p->sort_items ? first_sort_cfg(bits) : default_sort_cfg(bits, n);
     if (p->sort_threads) c.threads = p->sort_threads;
     if (p->sort_items) c.items = p->sort_items;
     return c;
 }
 
-bool valid_params(const tb_params *p) {
+bool valid_params(const tb_params *p, int64_t n) {
     return p && p->n_crit >= 1 && p->n_crit <= kMaxNcrit && p->mom_mode >= 0 && p->mom_mode <= 2 &&
            p->cell_capacity >= 0 && p->cell_capacity <= kMaxCells &&
            (p->radix_bits == 0 || (p->radix_bits >= 8 && p->radix_bits <= 11)) &&
@@ -215,7 +222,7 @@ bool valid_params(const tb_params *p) {
            batch_threads_valid(p->batch_threads) &&
            (p->batch_one_launch == 0 || p->batch_one_launch == 1) &&
            (p->root_pow2 == 0 || p->root_pow2 == 1) &&
-           sort_cfg_valid(pick_cfg(p));
+           sort_cfg_valid(pick_cfg(p, n));
 }
 
 }  // namespace
@@ -273,7 +280,7 @@ int32_t tb_sort_variant(int32_t i, int32_t *radix_bits, int32_t *threads, int32_
 
 tb_status tb_build(const float *d_pos, const float *d_mass, int64_t n, const tb_params *params,
                    tb_stream stream, tb_tree **tree) {
-    if (!tree || !valid_params(params) || n < 0 || n > 2147483647LL) return TB_EINVAL;
+    if (!tree || !valid_params(params, n) || n < 0 || n > 2147483647LL) return TB_EINVAL;
     if (n > 0 && (!d_pos || (reinterpret_cast<uintptr_t>(d_pos) & 3u))) return TB_EINVAL;
     if (reinterpret_cast<uintptr_t>(d_mass) & 3u) return TB_EINVAL;
     if (*tree && (*tree)->n_sets != 0) return TB_EINVAL;   // a batched tree
@@ -291,7 +298,7 @@ tb_status tb_build(const float *d_pos, const float *d_mass, int64_t n, const tb_
     Workspace &ws = S->ws;
     tb_tree &t = S->pub;
     S->params = *params;
-    const SortCfg cfg = pick_cfg(params);
+    const SortCfg cfg = pick_cfg(params, n);
     S->radix_bits = cfg.radix_bits;
     ws.last_stream = s;
     ws.moments_ready = false;
@@ -317,27 +324,37 @@ tb_status tb_build(const float *d_pos, const float *d_mass, int64_t n, const tb_
         st = ensure_cells(*S, params->cell_capacity, params->mom_mode == TB_MOM_FP64);
         if (st != TB_OK) return st;
     }
-    const int passes = sort_plan(cfg).passes;
     mark(ws, "start", s);
     ws.root_pow2 = params->root_pow2 != 0;
-    cudaError_t e = launch_root(d_pos, n, ws, passes << cfg.radix_bits, s);
-    if (e != cudaSuccess) return from_cuda(e);
-    mark(ws, "root", s);
-    // the unsorted keys go where the last pass will read from the other buffer
-    uint64_t *ka = (passes & 1) ? ws.keys_alt : t.pkey;
-    uint64_t *kb = (passes & 1) ? t.pkey : ws.keys_alt;
-    int32_t *pa = (passes & 1) ? ws.perm_alt : t.perm;
-    int32_t *pb = (passes & 1) ? t.perm : ws.perm_alt;
-    e = launch_keys(d_pos, d_mass, n, ka, ws, cfg, params->key_order, s);
-    if (e != cudaSuccess) return from_cuda(e);
+    cudaError_t e;
+    // a small set's root, keys and sort in one launch, unless the caller names
+    // a sort variant or times the stages
+    const bool named = params->radix_bits || params->sort_threads || params->sort_items;
+    if (!named && !ws.profile && n <= small_sort_max()) {
+        e = launch_small_sort(d_pos, d_mass, n, t.pkey, t.perm, ws.keys_alt, ws.perm_alt, ws,
+                              params->key_order, s);
+        if (e != cudaSuccess) return from_cuda(e);
+    } else {
+        const int passes = sort_plan(cfg).passes;
+        e = launch_root(d_pos, n, ws, passes << cfg.radix_bits, s);
+        if (e != cudaSuccess) return from_cuda(e);
+        mark(ws, "root", s);
+        // the unsorted keys go where the last pass will read from the other buffer
+        uint64_t *ka = (passes & 1) ? ws.keys_alt : t.pkey;
+        uint64_t *kb = (passes & 1) ? t.pkey : ws.keys_alt;
+        int32_t *pa = (passes & 1) ? ws.perm_alt : t.perm;
+        int32_t *pb = (passes & 1) ? t.perm : ws.perm_alt;
+        e = launch_keys(d_pos, d_mass, n, ka, ws, cfg, params->key_order, s);
+        if (e != cudaSuccess) return from_cuda(e);
+        mark(ws, "keys", s);
+        uint64_t *kout = nullptr;
+        int32_t *pout = nullptr;
+        e = launch_sort(ka, kb, pa, pb, n, ws, cfg, kout, pout, s);
+        if (e != cudaSuccess) return from_cuda(e);
+        if (kout != t.pkey || pout != t.perm) return TB_ECUDA;
+    }
     ws.xm_pos = d_pos;
     ws.xm_mass = d_mass;
-    mark(ws, "keys", s);
-    uint64_t *kout = nullptr;
-    int32_t *pout = nullptr;
-    e = launch_sort(ka, kb, pa, pb, n, ws, cfg, kout, pout, s);
-    if (e != cudaSuccess) return from_cuda(e);
-    if (kout != t.pkey || pout != t.perm) return TB_ECUDA;
     e = launch_levels(t.pkey, n, params->n_crit, ws, s);
     if (e != cudaSuccess) return from_cuda(e);
     mark(ws, "levels", s);
@@ -423,7 +440,7 @@ tb_status tb_moments(tb_tree *tree, const float *d_pos, const float *d_mass, tb_
 tb_status tb_build_batched(const float *d_pos, const float *d_mass, const int64_t *d_set_offsets,
                            int32_t n_sets, int64_t n_total, const tb_params *params,
                            tb_stream stream, tb_tree **tree) {
-    if (!tree || !valid_params(params) || n_sets < 0 || n_total < 0 || n_total > 2147483647LL)
+    if (!tree || !valid_params(params, n_total) || n_sets < 0 || n_total < 0 || n_total > 2147483647LL)
         return TB_EINVAL;
     if (params->key_order != TB_KEYS_MORTON) return TB_EINVAL;   // batched: Morton keys only
     if (n_sets > 0 && !d_set_offsets) return TB_EINVAL;
@@ -449,7 +466,7 @@ tb_status tb_build_batched(const float *d_pos, const float *d_mass, const int64_
     t.n_particles = n_total;
     t.n_crit = params->n_crit;
     t.n_sets = n_sets;
-    st = ensure_particles(*S, n_total, default_sort_cfg(8), false, true);
+    st = ensure_particles(*S, n_total, default_sort_cfg(8, n_total), false, true);
     if (st != TB_OK) return st;
     if (n_sets > ws.set_cap || !t.set_cell_offset) {
         cudaDeviceSynchronize();

@@ -200,24 +200,17 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
         __syncthreads();
         set_root_cube(A.pos, o, ns, s_red, &s_bad);
         if (threadIdx.x == 0) {
-            double L = 0.0;
-            float amax = 0.f;
+            const RootCube r = root_cube(s_red, s_red + 3, A.root_pow2 != 0);
+            s_scale = r.scale;
+            s_shi = r.s_hi;
+            s_slo = r.s_lo;
+            s_exact = r.exact_only;
+            s_f32 = r.s_fp32;
             for (int a = 0; a < 3; ++a) {
-                s_lo[a] = s_red[a];
-                const double e = __dsub_rn((double)s_red[3 + a], (double)s_red[a]);
-                if (e > L) L = e;
-                amax = fmaxf(amax, fmaxf(fabsf(s_red[a]), fabsf(s_red[3 + a])));
+                s_lo[a] = r.lo[a];
+                A.set_root[4 * (int64_t)set + a] = (double)r.lo[a];
             }
-            if (!(L > 0.0)) L = 1.0;
-            if (A.root_pow2) L = pow2_ceil(L);
-            const double scale = __ddiv_rn(2097152.0, L);
-            s_scale = scale;
-            s_shi = (float)scale;
-            s_slo = (float)__dsub_rn(scale, (double)s_shi);
-            s_exact = !(scale < 1e30 && scale > 1e-30 && amax < 1e30f);
-            s_f32 = (double)s_shi == scale;
-            for (int a = 0; a < 3; ++a) A.set_root[4 * (int64_t)set + a] = (double)s_lo[a];
-            A.set_root[4 * (int64_t)set + 3] = L;
+            A.set_root[4 * (int64_t)set + 3] = r.side;
             if (s_bad) atomicOr(&A.info->status, kErrNonFinite);
         }
         for (int i = threadIdx.x; i < kBPasses * kBRadix; i += blockDim.x) (&sm.hist[0][0])[i] = 0;

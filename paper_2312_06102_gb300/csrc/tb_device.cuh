@@ -156,6 +156,63 @@ __device__ __forceinline__ uint32_t quantise(float x, float lo, float s_hi, floa
     return (uint32_t)f;
 }
 
+// ------------------------------------------------------------ root cube
+
+// Corner lo, side L = largest extent (1 if all are 0; with pow2 the smallest
+// power of two at least that), scale 2^21 / L and how to quantise.
+struct RootCube {
+    float lo[3];
+    double side, scale;
+    float s_hi, s_lo;
+    bool exact_only, s_fp32;
+};
+
+__device__ __forceinline__ RootCube root_cube(const float *mn, const float *mx, bool pow2) {
+    RootCube r;
+    double L = 0.0;
+    float amax = 0.f;
+    for (int a = 0; a < 3; ++a) {
+        r.lo[a] = mn[a];
+        const double e = __dsub_rn((double)mx[a], (double)mn[a]);
+        if (e > L) L = e;
+        amax = fmaxf(amax, fmaxf(fabsf(mn[a]), fabsf(mx[a])));
+    }
+    if (!(L > 0.0)) L = 1.0;
+    if (pow2) L = pow2_ceil(L);
+    const double scale = __ddiv_rn(2097152.0, L);
+    r.side = L;
+    r.scale = scale;
+    r.s_hi = (float)scale;
+    r.s_lo = (float)__dsub_rn(scale, (double)r.s_hi);
+    // the FP32 route needs x - lo and its products to stay far from overflow
+    // and underflow; otherwise every coordinate takes the FP64 route
+    r.exact_only = !(scale < 1e30 && scale > 1e-30 && amax < 1e30f);
+    r.s_fp32 = (double)r.s_hi == scale;
+    return r;
+}
+
+// The build record's start: root cube, status, look-back epoch, counters.
+__device__ __forceinline__ void begin_build(DevInfo *info, const RootCube &r, const float *mx,
+                                            bool bad) {
+    for (int a = 0; a < 3; ++a) {
+        info->lo[a] = r.lo[a];
+        info->hi[a] = mx[a];
+    }
+    info->side = r.side;
+    info->scale = r.scale;
+    info->s_hi = r.s_hi;
+    info->s_lo = r.s_lo;
+    info->exact_only = r.exact_only ? 1u : 0u;
+    info->s_fp32 = r.s_fp32 ? 1u : 0u;
+    info->status = bad ? kErrNonFinite : 0u;
+    info->epoch = (info->epoch + 16u) & 0x3fffffffu;
+    for (int p = 0; p < 16; ++p) info->sort_tile_ctr[p] = 0;
+    for (int p = 1; p < 8; ++p) info->misc_ctr[p] = 0;
+    info->n_cells = 0;
+    info->n_leaves = 0;
+    info->max_depth = 0;
+}
+
 // ------------------------------------------------------- bounded waits
 
 // Spin limit for every wait on another block.  A wait that runs out sets

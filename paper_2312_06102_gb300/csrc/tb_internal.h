@@ -147,7 +147,9 @@ cudaError_t launch_wait_selftest(int64_t limit, uint32_t *status, uint32_t *flag
 
 int level_tile_size();
 int64_t bbox_grid();
-SortCfg default_sort_cfg(int radix_bits);
+constexpr int64_t kSmallTileMax = int64_t(1) << 19;   // keys that take the small tiles by default
+SortCfg default_sort_cfg(int radix_bits, int64_t n);
+SortCfg first_sort_cfg(int radix_bits);
 const SortCfg *sort_variant(int i);
 bool sort_cfg_valid(const SortCfg &c);
 
@@ -168,6 +170,19 @@ cudaError_t launch_runs(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t 
                         int shift0, int32_t *long_runs, Workspace &ws, cudaStream_t s);
 int64_t long_run_capacity(int64_t n);
 
+// Loads onto the current device, now rather than at their first launch, the
+// kernels tb_keys_sorted_noalloc can reach.
+cudaError_t load_key_kernels();
+cudaError_t load_sort_kernels();
+cudaError_t load_run_kernels();
+cudaError_t load_small_kernels();
+
+// root, keys and sort of a small set in one launch
+int64_t small_sort_max();
+cudaError_t launch_small_sort(const float *pos, const float *mass, int64_t n, uint64_t *pkey, int32_t *perm,
+                              uint64_t *alt_k, int32_t *alt_v, Workspace &ws, int key_order,
+                              cudaStream_t s);
+
 // tree walk: int32 words of its scratch (counters, groups, per-warp stacks)
 int64_t walk_buffer_words(int64_t n_cells);
 cudaError_t launch_walk(const tb_tree &t, Workspace &ws, float theta, float eps, int n_group,
@@ -186,6 +201,12 @@ inline bool first_on_device(std::atomic<uint64_t> &done) {
     if (done.load(std::memory_order_acquire) & bit) return false;
     done.fetch_or(bit, std::memory_order_acq_rel);
     return true;
+}
+
+template <class K>
+cudaError_t load_kernel(K kernel) {
+    cudaFuncAttributes a;
+    return cudaFuncGetAttributes(&a, kernel);
 }
 
 // Blocks of a kernel that are resident at once on the current device, looked

@@ -136,36 +136,8 @@ __global__ void __launch_bounds__(kRootThreads) root_kernel(const float *__restr
     for (int i = threadIdx.x; i < hist_len; i += blockDim.x) hist[i] = 0;
     __syncthreads();
     if (threadIdx.x == 0) {
-        uint32_t bad = __float_as_uint(s_red[0][6]);
-        double L = 0.0;
-        float amax = 0.f;
-        for (int a = 0; a < 3; ++a) {
-            info->lo[a] = s_red[0][a];
-            info->hi[a] = s_red[0][3 + a];
-            double e = __dsub_rn((double)s_red[0][3 + a], (double)s_red[0][a]);
-            if (e > L) L = e;
-            amax = fmaxf(amax, fmaxf(fabsf(s_red[0][a]), fabsf(s_red[0][3 + a])));
-        }
-        if (!(L > 0.0)) L = 1.0;
-        if (pow2) L = pow2_ceil(L);
-        double scale = __ddiv_rn(2097152.0, L);
-        float s_hi = (float)scale;
-        float s_lo = (float)__dsub_rn(scale, (double)s_hi);
-        info->side = L;
-        info->scale = scale;
-        info->s_hi = s_hi;
-        info->s_lo = s_lo;
-        // the FP32 route needs x - lo and its products to stay far from overflow
-        // and underflow; otherwise every coordinate takes the FP64 route
-        info->exact_only = !(scale < 1e30 && scale > 1e-30 && amax < 1e30f) ? 1u : 0u;
-        info->s_fp32 = (double)s_hi == scale ? 1u : 0u;
-        info->status = bad ? kErrNonFinite : 0u;
-        info->epoch = (info->epoch + 16u) & 0x3fffffffu;
-        for (int p = 0; p < 16; ++p) info->sort_tile_ctr[p] = 0;
-        for (int p = 1; p < 8; ++p) info->misc_ctr[p] = 0;
-        info->n_cells = 0;
-        info->n_leaves = 0;
-        info->max_depth = 0;
+        begin_build(info, root_cube(&s_red[0][0], &s_red[0][3], pow2), &s_red[0][3],
+                    __float_as_uint(s_red[0][6]) != 0u);
         __threadfence();
         info->misc_ctr[0] = 0;
     }
@@ -252,29 +224,31 @@ __global__ void __launch_bounds__(kKeysThreads, 6) keys_kernel(const float *__re
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    // last block: counts -> exclusive offsets, one pass at a time
-    __shared__ uint32_t s_warp[kKeysThreads / 32];
-    for (int p = 0; p < passes; ++p) {
-        uint32_t carry = 0;
-        for (int base = 0; base < RADIX; base += kKeysThreads) {
-            int d = base + threadIdx.x;
-            uint32_t v = (d < RADIX) ? __ldcg(&hist[p * RADIX + d]) : 0u;
-            uint32_t x = v;
-            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-            for (int off = 1; off < 32; off <<= 1) {
-                uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
-                if (lane >= off) x += y;
-            }
-            if (lane == 31) s_warp[warp] = x;
-            __syncthreads();
-            uint32_t wpre = 0, tot = 0;
-            for (int w = 0; w < kKeysThreads / 32; ++w) {
-                if (w < warp) wpre += s_warp[w];
-                tot += s_warp[w];
-            }
-            if (d < RADIX) hist[p * RADIX + d] = carry + wpre + x - v;
-            carry += tot;
-            __syncthreads();
+    // last block: counts -> exclusive offsets, a warp per pass, each lane a
+    // run of digits (one pass after another, with block barriers, took 4 us
+    // more: most of the kernel for a small set)
+    const int lane = threadIdx.x & 31;
+    for (int p = threadIdx.x >> 5; p < passes; p += kKeysThreads / 32) {
+        constexpr int Q = RADIX / 128;   // uint4 per lane
+        uint4 *row = reinterpret_cast<uint4 *>(hist + p * RADIX) + lane * Q;
+        uint32_t sum = 0;
+#pragma unroll 2
+        for (int j = 0; j < Q; ++j) {
+            const uint4 v = __ldcg(row + j);
+            sum += v.x + v.y + v.z + v.w;
+        }
+        uint32_t x = sum;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        x -= sum;
+#pragma unroll 2
+        for (int j = 0; j < Q; ++j) {
+            const uint4 v = __ldcg(row + j);
+            row[j] = make_uint4(x, x + v.x, x + v.x + v.y, x + v.x + v.y + v.z);
+            x += v.x + v.y + v.z + v.w;
         }
     }
     if (threadIdx.x == 0) info->misc_ctr[4] = 0;
@@ -333,6 +307,11 @@ cudaError_t launch_keys(const float *pos, const float *mass, int64_t n, uint64_t
                           : keys_impl<11, false>(pos, mass, n, keys, ws, passes, shift0, s);
         default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t load_key_kernels() {
+    cudaError_t e = load_kernel(root_kernel);
+    return e == cudaSuccess ? load_kernel(keys_kernel<8, false>) : e;
 }
 
 // (x, y, z, m) of each particle in input order, for moment calls whose

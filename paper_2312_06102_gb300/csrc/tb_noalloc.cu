@@ -45,8 +45,8 @@ constexpr size_t kOffInfo = 0;
 constexpr size_t kOffHist = align256(kOffInfo + sizeof(DevInfo));
 constexpr size_t kOffPart = align256(kOffHist + sizeof(uint32_t) * 16 * 2048);
 constexpr size_t kOffLook = align256(kOffPart + sizeof(float) * 8 * 152 * 4);
-// look-back: one 64-bit word per tile and digit; the smallest compiled tile
-// of 8-bit digits holds 2048 keys
+// look-back: one 64-bit word per tile and digit; a tile holds 2048 keys
+static_assert(kNoAllocMaxN <= kSmallTileMax, "load_sort_kernels loads the small tiles only");
 constexpr size_t kLookWords = ((kNoAllocMaxN + 2047) / 2048) * (size_t(1) << kNoAllocRadixBits);
 constexpr size_t kOffKeys = align256(kOffLook + sizeof(uint64_t) * kLookWords);
 constexpr size_t kOffPerm = align256(kOffKeys + sizeof(uint64_t) * kNoAllocMaxN);
@@ -79,6 +79,18 @@ cudaError_t scratch_address(unsigned char **out) {
     }
     *out = g_scratch_addr[dev];
     return cudaSuccess;
+}
+
+// Every kernel a call can reach, loaded by the first call that sorts, whatever
+// its size: sets of up to 65,536 particles and larger ones take different
+// kernels, and a later call of the other kind must not load (allocate).
+cudaError_t load_kernels_once() {
+    static std::atomic<uint64_t> done{0};
+    if (!first_on_device(done)) return cudaSuccess;
+    cudaError_t e = load_key_kernels();
+    if (e == cudaSuccess) e = load_sort_kernels();
+    if (e == cudaSuccess) e = load_run_kernels();
+    return e == cudaSuccess ? load_small_kernels() : e;
 }
 
 tb_status status_of(cudaError_t e) {
@@ -120,7 +132,7 @@ extern "C" tb_status tb_keys_sorted_noalloc(const float *d_pos, int64_t n, uint6
     // call runs with the same look-back epoch and the words a larger earlier
     // call left would read as published; a tile only reads the words of
     // tiles before it, so clearing this call's tiles is enough.
-    const SortCfg cfg = default_sort_cfg(kNoAllocRadixBits);
+    const SortCfg cfg = default_sort_cfg(kNoAllocRadixBits, n);
     const int64_t look_words = ((n + cfg.tile() - 1) / cfg.tile()) << cfg.radix_bits;
     if (look_words > (int64_t)kLookWords) return TB_ECUDA;
     if ((e = cudaMemsetAsync(ws.info, 0, sizeof(DevInfo), s)) != cudaSuccess) return status_of(e);
@@ -134,20 +146,27 @@ extern "C" tb_status tb_keys_sorted_noalloc(const float *d_pos, int64_t n, uint6
         }
         return status_of(cudaStreamSynchronize(s));
     }
-    const int passes = sort_plan(cfg).passes;
-    if ((e = launch_root(d_pos, n, ws, passes << cfg.radix_bits, s)) != cudaSuccess)
-        return status_of(e);
-    uint64_t *ka = (passes & 1) ? ws.keys_alt : d_pkey;
-    uint64_t *kb = (passes & 1) ? d_pkey : ws.keys_alt;
-    int32_t *pa = (passes & 1) ? ws.perm_alt : d_perm;
-    int32_t *pb = (passes & 1) ? d_perm : ws.perm_alt;
-    if ((e = launch_keys(d_pos, nullptr, n, ka, ws, cfg, TB_KEYS_MORTON, s)) != cudaSuccess)
-        return status_of(e);
-    uint64_t *kout = nullptr;
-    int32_t *pout = nullptr;
-    if ((e = launch_sort(ka, kb, pa, pb, n, ws, cfg, kout, pout, s)) != cudaSuccess)
-        return status_of(e);
-    if (kout != d_pkey || pout != d_perm) return TB_ECUDA;
+    if (n >= 2 && (e = load_kernels_once()) != cudaSuccess) return status_of(e);
+    if (n <= small_sort_max()) {
+        if ((e = launch_small_sort(d_pos, nullptr, n, d_pkey, d_perm, ws.keys_alt, ws.perm_alt, ws,
+                                   TB_KEYS_MORTON, s)) != cudaSuccess)
+            return status_of(e);
+    } else {
+        const int passes = sort_plan(cfg).passes;
+        if ((e = launch_root(d_pos, n, ws, passes << cfg.radix_bits, s)) != cudaSuccess)
+            return status_of(e);
+        uint64_t *ka = (passes & 1) ? ws.keys_alt : d_pkey;
+        uint64_t *kb = (passes & 1) ? d_pkey : ws.keys_alt;
+        int32_t *pa = (passes & 1) ? ws.perm_alt : d_perm;
+        int32_t *pb = (passes & 1) ? d_perm : ws.perm_alt;
+        if ((e = launch_keys(d_pos, nullptr, n, ka, ws, cfg, TB_KEYS_MORTON, s)) != cudaSuccess)
+            return status_of(e);
+        uint64_t *kout = nullptr;
+        int32_t *pout = nullptr;
+        if ((e = launch_sort(ka, kb, pa, pb, n, ws, cfg, kout, pout, s)) != cudaSuccess)
+            return status_of(e);
+        if (kout != d_pkey || pout != d_perm) return TB_ECUDA;
+    }
 
     // the call ends by reading the device status (and the root cube)
     DevInfo h;

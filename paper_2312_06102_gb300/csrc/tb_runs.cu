@@ -28,16 +28,6 @@ namespace {
 
 constexpr int kRunThreads = 256;
 
-// Queue of long runs and the per-tile descent flags, laid out in one buffer.
-struct RunBuffers {
-    int32_t *queue;      // [n / kRunMax + 2] start positions of long runs
-    uint8_t *desc;       // [n / kRunTile + 1] tile holds a descent inside a run
-};
-__host__ __device__ inline int64_t run_queue_cap(int64_t n) { return n / kRunMax + 2; }
-__host__ __device__ inline RunBuffers run_buffers(int32_t *base, int64_t n) {
-    return {base, reinterpret_cast<uint8_t *>(base + run_queue_cap(n))};
-}
-
 __global__ void __launch_bounds__(kRunThreads)
     run_sort_kernel(uint64_t *__restrict__ keys, int32_t *__restrict__ vals, int64_t n, int shift0,
                     RunBuffers rb, DevInfo *info) {
@@ -55,56 +45,14 @@ __global__ void __launch_bounds__(kCtaThreads, 1)
     extern __shared__ __align__(16) unsigned char raw[];
     CtaSortShared &sm = *reinterpret_cast<CtaSortShared *>(raw);
     __shared__ uint32_t s_q;
-    __shared__ unsigned long long s_end;
-    __shared__ int s_desc;
     const uint32_t nq = *(volatile uint32_t *)&info->misc_ctr[5];
-    const int passes = (shift0 + kCtaRadixBits - 1) / kCtaRadixBits;
     for (;;) {
         if (threadIdx.x == 0) s_q = atomicAdd(&info->misc_ctr[6], 1u);
         __syncthreads();
         const uint32_t q = s_q;
         __syncthreads();
         if (q >= nq) return;
-        const int64_t a = rb.queue[q];
-        const uint64_t tp = keys[a] >> shift0;
-        // the run's end: the first later position with other upper bits;
-        // the first 4096 positions are scanned by the block, then binary search
-        if (threadIdx.x == 0) { s_end = (unsigned long long)n; s_desc = 0; }
-        __syncthreads();
-        int64_t base = a + 1;
-        for (int it = 0; it < 4 && base < n; ++it, base += kCtaThreads) {
-            const int64_t p = base + threadIdx.x;
-            if (p < n && (keys[p] >> shift0) != tp) atomicMin(&s_end, (unsigned long long)p);
-            __syncthreads();
-            const bool done = s_end < (unsigned long long)n;
-            __syncthreads();
-            if (done) break;
-        }
-        if (threadIdx.x == 0 && s_end == (unsigned long long)n && base < n) {
-            int64_t lo = base, hi = n;                  // first position with top > tp
-            while (lo < hi) {
-                const int64_t m = (lo + hi) >> 1;
-                if ((keys[m] >> shift0) <= tp) lo = m + 1; else hi = m;
-            }
-            s_end = (unsigned long long)lo;
-        }
-        __syncthreads();
-        const int64_t len = (int64_t)s_end - a;
-        // only a run with a descent needs sorting: look at the tile flags
-        const int64_t t0 = (a + 1) / kRunTile, t1 = (a + len - 1) / kRunTile;
-        for (int64_t t = t0 + threadIdx.x; t <= t1; t += kCtaThreads)
-            if (rb.desc[t]) s_desc = 1;
-        __syncthreads();
-        if (s_desc) {
-            cta_histograms(keys, a, len, 0, passes, sm);
-            const int np = cta_lsd_sort(keys, vals, alt_k, alt_v, a, len, 0, passes, false, sm);
-            if (np & 1)
-                for (int64_t p = a + threadIdx.x; p < a + len; p += kCtaThreads) {
-                    keys[p] = alt_k[p];
-                    vals[p] = alt_v[p];
-                }
-        }
-        __syncthreads();
+        sort_long_run<kCtaThreads>(keys, vals, alt_k, alt_v, n, shift0, rb.queue[q], rb.desc, sm);
     }
 }
 
@@ -129,6 +77,11 @@ cudaError_t launch_runs(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t 
                                                                    rb, ws.info);
     ++g_launches;
     return cudaGetLastError();
+}
+
+cudaError_t load_run_kernels() {
+    cudaError_t e = load_kernel(run_sort_kernel);
+    return e == cudaSuccess ? load_kernel(long_run_kernel) : e;
 }
 
 // int32 words for the queue and the tile flags of n keys

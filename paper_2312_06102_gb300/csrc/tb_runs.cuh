@@ -143,5 +143,65 @@ __device__ bool run_tile(uint64_t *__restrict__ keys, int32_t *__restrict__ vals
     return desc;
 }
 
+// Queue of long runs and the per-tile descent flags, laid out in one buffer.
+struct RunBuffers {
+    int32_t *queue;      // [n / kRunMax + 2] start positions of long runs
+    uint8_t *desc;       // [n / kRunTile + 1] tile holds a descent inside a run
+};
+__host__ __device__ inline int64_t run_queue_cap(int64_t n) { return n / kRunMax + 2; }
+__host__ __device__ inline RunBuffers run_buffers(int32_t *base, int64_t n) {
+    return {base, reinterpret_cast<uint8_t *>(base + run_queue_cap(n))};
+}
+
+// Sorts by its low shift0 bits the run of equal key >> shift0 that starts at
+// a, when one of its tiles holds a descent (`desc`, one flag per tile of the
+// n keys); a block of T threads.
+template <int T>
+__device__ void sort_long_run(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t *alt_v, int64_t n,
+                              int shift0, int64_t a, const uint8_t *desc, CtaSortSharedT<T> &sm) {
+    __shared__ unsigned long long s_end;
+    __shared__ int s_desc;
+    const int passes = (shift0 + kCtaRadixBits - 1) / kCtaRadixBits;
+    const uint64_t tp = keys[a] >> shift0;
+    // the run's end: the first later position with other upper bits;
+    // the first 4096 positions are scanned by the block, then binary search
+    if (threadIdx.x == 0) { s_end = (unsigned long long)n; s_desc = 0; }
+    __syncthreads();
+    int64_t base = a + 1;
+    for (int it = 0; it < 4 && base < n; ++it, base += T) {
+        const int64_t p = base + threadIdx.x;
+        if (p < n && (keys[p] >> shift0) != tp) atomicMin(&s_end, (unsigned long long)p);
+        __syncthreads();
+        const bool done = s_end < (unsigned long long)n;
+        __syncthreads();
+        if (done) break;
+    }
+    if (threadIdx.x == 0 && s_end == (unsigned long long)n && base < n) {
+        int64_t lo = base, hi = n;                  // first position with top > tp
+        while (lo < hi) {
+            const int64_t m = (lo + hi) >> 1;
+            if ((keys[m] >> shift0) <= tp) lo = m + 1; else hi = m;
+        }
+        s_end = (unsigned long long)lo;
+    }
+    __syncthreads();
+    const int64_t len = (int64_t)s_end - a;
+    // only a run with a descent needs sorting: look at the tile flags
+    const int64_t t0 = (a + 1) / kRunTile, t1 = (a + len - 1) / kRunTile;
+    for (int64_t t = t0 + threadIdx.x; t <= t1; t += T)
+        if (desc[t]) s_desc = 1;
+    __syncthreads();
+    if (s_desc) {
+        cta_histograms(keys, a, len, 0, passes, sm);
+        const int np = cta_lsd_sort(keys, vals, alt_k, alt_v, a, len, 0, passes, false, sm);
+        if (np & 1)
+            for (int64_t p = a + threadIdx.x; p < a + len; p += T) {
+                keys[p] = alt_k[p];
+                vals[p] = alt_v[p];
+            }
+    }
+    __syncthreads();
+}
+
 }  // namespace
 }  // namespace tb

@@ -345,7 +345,18 @@ static const int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
 const SortCfg *sort_variant(int i) { return (i >= 0 && i < kNumVariants) ? &kVariants[i] : nullptr; }
 
-SortCfg default_sort_cfg(int radix_bits) {
+// 8-bit digits: 256 x 8 up to 2^19 keys, where a pass is latency and smaller
+// tiles spread over more SMs (300,000 keys: build 109 us against 117 for
+// 512 x 8 and 119 for 256 x 16), 512 x 8 above (10^6: 160 against 181 and 160;
+// 2^22: 367 against 405 and 381; 2^27: 9.58 ms against 10.03 and 9.78).  Other
+// digits: their first variant.
+SortCfg default_sort_cfg(int radix_bits, int64_t n) {
+    if (radix_bits == 8) return n <= kSmallTileMax ? SortCfg{8, 256, 8} : SortCfg{8, 512, 8};
+    return first_sort_cfg(radix_bits);
+}
+
+// The first variant of a digit width: completes a named block or tile size.
+SortCfg first_sort_cfg(int radix_bits) {
     for (int i = 0; i < kNumVariants; ++i)
         if (kVariants[i].radix_bits == radix_bits) return kVariants[i];
     return kVariants[0];
@@ -360,6 +371,12 @@ bool sort_cfg_valid(const SortCfg &c) {
 }
 
 int64_t sort_tiles(const SortCfg &c, int64_t n) { return (n + c.tile() - 1) / c.tile(); }
+
+cudaError_t load_sort_kernels() {
+    // the default tile of every set tb_keys_sorted_noalloc takes
+    cudaError_t e = load_kernel(onesweep_kernel<8, 256, 8, true>);
+    return e == cudaSuccess ? load_kernel(onesweep_kernel<8, 256, 8, false>) : e;
+}
 
 SortPlan sort_plan(const SortCfg &c) {
     // global passes cover the upper ceil(40 / b) * b key bits; the runs of
