@@ -327,10 +327,15 @@ __device__ __forceinline__ void bulk_store_wait_read() {
     asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
 
-// Asynchronous 16-byte global -> shared copy (no registers held while it is
-// in flight); completion is awaited with cp_async_wait_all.
+// Asynchronous 16-byte (4-byte) global -> shared copy (no registers held while
+// it is in flight); completion is awaited with cp_async_wait_all.
 __device__ __forceinline__ void cp_async16(void *dst_smem, const void *src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst_smem)), "l"(src)
+                 : "memory");
+}
+
+__device__ __forceinline__ void cp_async4(void *dst_smem, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst_smem)), "l"(src)
                  : "memory");
 }
 

@@ -8,7 +8,7 @@
 //                        holds at most n_group), and every leaf holding more
 //                        (only depth-21 leaves of one key can);
 //   walk_kernel        : one warp per group (taken from an atomic ticket),
-//                        32 particles at a time (one per lane; a larger group
+//                        32 particles at a time (a larger group
 //                        is walked in chunks of 32, each with its own box).
 //                        The warp walks the tree from the root, up to 32 cells
 //                        at a time: a cell whose particle range meets the chunk's is
@@ -17,9 +17,9 @@
 //                        of mass to the group's bounding box (so l / d < theta
 //                        holds for every particle of the group); an opened leaf
 //                        contributes its particles one by one.  Accepted cells
-//                        and opened leaves go to lists in shared memory; when a
-//                        list is full, and at the end, every lane evaluates the
-//                        lists for its particles of the group.
+//                        and opened leaves' particles go to lists in shared
+//                        memory, which are evaluated, eight entries a step, as
+//                        they fill.
 // Forces (G = 1): a softened point mass m (r^2 + eps^2)^(-3/2) r for every
 // particle and cell; for a cell also the quadrupole term
 //   T r / |r|^5 - (5/2) (r.T r) r / |r|^7,  T = 3 Q - tr(Q) I,
@@ -36,14 +36,18 @@ namespace tb {
 namespace {
 
 constexpr int kWalkWarps = 4;
-constexpr int kWalkBlocks = 152 * 6;   // as many as fit (shared memory)
 constexpr int kWalkThreads = 32 * kWalkWarps;
-// cells waiting to be tested, per warp in global memory: a round takes at most
-// 32 cells and adds at most 7 per cell, and only cells above depth 21 have
+constexpr int kWalkPerSm = 4;          // blocks resident per SM (registers and shared memory)
+constexpr int kWalkBlocks = 152 * kWalkPerSm;
+// cells waiting to be tested, per warp: the first kStackNear in shared memory,
+// the rest in global memory.  A round takes at most 32 cells and adds at most
+// 7 per cell, and only cells above depth 21 have
 // children, so the stack stays below 21 * 256 + 1 entries
 constexpr int kStackCap = 6144;
-constexpr int kCellCap = 128;       // accepted cells
-constexpr int kRangeCap = 128;      // particle ranges of opened leaves
+constexpr int kStackNear = 768;
+constexpr int kCellCap = 40;           // accepted cells: under 8 left over and 32 of a round
+constexpr int kSrcLeaf = 16;           // leaves of at most this many go to the source list
+constexpr int kSrcCap = 640;           // sources: up to 128 waiting and 32 * kSrcLeaf of a round
 
 struct WalkTree {
     const int32_t *child_first, *child_end, *pfirst, *pend;
@@ -55,58 +59,174 @@ struct WalkTree {
     const float4 *rec;              // [C][4] per cell: com + m, com_lo, T xx xy xz yy, T yz zz
 };
 
-struct WarpLists {
-    float4 cell[kCellCap][4];       // the accepted cells' records, copied when accepted
-    int2 range[kRangeCap];
-};
-
-__device__ __forceinline__ float3 point_acc(float3 a, float rx, float ry, float rz, float m, float eps2) {
-    const float r2 = fmaf(rx, rx, fmaf(ry, ry, fmaf(rz, rz, eps2)));
-    const float inv = rsqrtf(r2);
-    const float f = m * inv * inv * inv;
-    a.x = fmaf(-f, rx, a.x);
-    a.y = fmaf(-f, ry, a.y);
-    a.z = fmaf(-f, rz, a.z);
-    return a;
+// Two FP32 values in one 64-bit register, and arithmetic on both at once
+// (each half rounded as the scalar operation).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(a), "f"(b));
+    return v;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &a, float &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t v;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t v;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(v) : "l"(a), "l"(b));
+    return v;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t v;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(v) : "l"(a), "l"(b), "l"(c));
+    return v;
+}
+__device__ __forceinline__ uint64_t dup2(float a) { return pack2(a, a); }
+// 1 / sqrt, the hardware's approximation (what rsqrtf rounds to) without its
+// steps for subnormal arguments: a distance below 1e-19 overflows the force
+// either way
+__device__ __forceinline__ uint64_t rsqrt2(uint64_t x) {
+    float a, b;
+    unpack2(x, a, b);
+    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(a));
+    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(b));
+    return pack2(a, b);
 }
 
-// the lists of one warp against its lane's particle k (when k < ke)
-__device__ float3 evaluate(const WalkTree &T, const WarpLists &W, int ncell, int nrange, int64_t k,
-                           int64_t ke, float eps2, bool use_quad, float3 a) {
-    const float4 x = k < ke ? T.xs[k] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-    for (int j = 0; j < ncell; ++j) {
-        const float4 c0 = W.cell[j][0], c1 = W.cell[j][1];
-        const float m = c0.w;
-        const float rx = (x.x - c0.x) - c1.x;
-        const float ry = (x.y - c0.y) - c1.y;
-        const float rz = (x.z - c0.z) - c1.z;
-        a = point_acc(a, rx, ry, rz, m, eps2);
-        if (use_quad) {
-            const float4 t0 = W.cell[j][2], t1 = W.cell[j][3];
-            const float txx = t0.x, txy = t0.y, txz = t0.z, tyy = t0.w, tyz = t1.x, tzz = t1.y;
-            const float trx = txx * rx + txy * ry + txz * rz;
-            const float try_ = txy * rx + tyy * ry + tyz * rz;
-            const float trz = txz * rx + tyz * ry + tzz * rz;
-            const float rtr = rx * trx + ry * try_ + rz * trz;
-            const float ir = rsqrtf(fmaf(rx, rx, fmaf(ry, ry, rz * rz)));
-            const float ir2 = ir * ir;
-            const float ir5 = ir2 * ir2 * ir;
-            const float s = 2.5f * rtr * ir5 * ir2;
-            a.x += trx * ir5 - s * rx;
-            a.y += try_ * ir5 - s * ry;
-            a.z += trz * ir5 - s * rz;
+// One warp's lists.  A cell's row is its record's first four float4 (centre
+// and mass, low centre, tensor) at a stride of five, which spreads eight rows
+// over all banks.
+struct WarpLists {
+    float4 cell[kCellCap][5];
+    int32_t src[kSrcCap];
+    int32_t stack[kStackNear];
+};
+
+// The chunk's targets and their accelerations.  Lane 8 g + i evaluates entry
+// i of each step's eight list entries for the targets t = 4 s + g, slots s =
+// 0 .. 7, two slots to a packed register: an entry read from shared memory
+// serves eight targets (one target per lane and entry after entry to all lanes
+// held the walk at 63% of the shared memory's bandwidth), and the steps run
+// over ceil(targets / 8) pairs only.
+constexpr int kPairs = 4;
+struct Chunk {
+    uint64_t x[kPairs], y[kPairs], z[kPairs];
+    uint64_t ax[kPairs], ay[kPairs], az[kPairs];
+    int pairs;
+};
+
+// Steps of eight accepted cells, rows [from, to) of the list; to - from is a
+// multiple of eight unless these are the last (missing rows are massless).
+template <bool QUAD>
+__device__ __forceinline__ void eval_cells(const WarpLists &W, int from, int to, float eps2, Chunk &C) {
+    const int i = threadIdx.x & 7;
+    const uint64_t E = dup2(eps2), K = dup2(-2.5f);
+    for (int j = from; j < to; j += 8) {
+        const bool in = j + i < to;
+        const float4 *row = W.cell[in ? j + i : from];
+        const float4 c0 = row[0], c1 = row[1];
+        const uint64_t cx = dup2(-c0.x), cy = dup2(-c0.y), cz = dup2(-c0.z);
+        const uint64_t lx = dup2(-c1.x), ly = dup2(-c1.y), lz = dup2(-c1.z);
+        const uint64_t nm = dup2(in ? -c0.w : 0.f);
+        uint64_t txx = 0, txy = 0, txz = 0, tyy = 0, tyz = 0, tzz = 0;
+        if constexpr (QUAD) {
+            const float4 t0 = row[2], t1 = row[3];
+            txx = dup2(in ? t0.x : 0.f); txy = dup2(in ? t0.y : 0.f); txz = dup2(in ? t0.z : 0.f);
+            tyy = dup2(in ? t0.w : 0.f); tyz = dup2(in ? t1.x : 0.f); tzz = dup2(in ? t1.y : 0.f);
+        }
+#pragma unroll
+        for (int p = 0; p < kPairs; ++p) {
+            if (p >= C.pairs) break;
+            const uint64_t rx = add2(add2(C.x[p], cx), lx);
+            const uint64_t ry = add2(add2(C.y[p], cy), ly);
+            const uint64_t rz = add2(add2(C.z[p], cz), lz);
+            const uint64_t r2 = fma2(rx, rx, fma2(ry, ry, mul2(rz, rz)));
+            const uint64_t inv = rsqrt2(add2(r2, E));
+            uint64_t f = mul2(mul2(mul2(nm, inv), inv), inv);
+            if constexpr (QUAD) {
+                const uint64_t tx = fma2(txx, rx, fma2(txy, ry, mul2(txz, rz)));
+                const uint64_t ty = fma2(txy, rx, fma2(tyy, ry, mul2(tyz, rz)));
+                const uint64_t tz = fma2(txz, rx, fma2(tyz, ry, mul2(tzz, rz)));
+                const uint64_t rtr = fma2(rx, tx, fma2(ry, ty, mul2(rz, tz)));
+                const uint64_t ir = rsqrt2(r2);
+                const uint64_t ir2 = mul2(ir, ir);
+                const uint64_t ir5 = mul2(mul2(ir2, ir2), ir);
+                f = fma2(mul2(mul2(rtr, K), ir5), ir2, f);
+                C.ax[p] = fma2(tx, ir5, C.ax[p]);
+                C.ay[p] = fma2(ty, ir5, C.ay[p]);
+                C.az[p] = fma2(tz, ir5, C.az[p]);
+            }
+            C.ax[p] = fma2(f, rx, C.ax[p]);
+            C.ay[p] = fma2(f, ry, C.ay[p]);
+            C.az[p] = fma2(f, rz, C.az[p]);
         }
     }
-    for (int j = 0; j < nrange; ++j) {
-        const int2 r = W.range[j];
-        for (int q = r.x; q < r.y; ++q) {
-            if (q == k) continue;                       // no self-force
-            const float4 y = T.xs[q];
-            a = point_acc(a, x.x - y.x, x.y - y.y, x.z - y.z, y.w, eps2);
+}
+
+// One step of eight source particles; y is this lane's (m = 0 when there is
+// none).  With SELF, `slot` is the slot of this lane's targets that is the
+// source itself, or -1, and takes no force from it.
+template <bool SELF>
+__device__ __forceinline__ void eval_sources(float4 y, int slot, float eps2, Chunk &C) {
+    const uint64_t E = dup2(eps2);
+    const uint64_t sx = dup2(-y.x), sy = dup2(-y.y), sz = dup2(-y.z), nm = dup2(-y.w);
+#pragma unroll
+    for (int p = 0; p < kPairs; ++p) {
+        if (p >= C.pairs) break;
+        const uint64_t rx = add2(C.x[p], sx), ry = add2(C.y[p], sy), rz = add2(C.z[p], sz);
+        const uint64_t inv = rsqrt2(fma2(rx, rx, fma2(ry, ry, fma2(rz, rz, E))));
+        uint64_t f = mul2(mul2(mul2(nm, inv), inv), inv);
+        if constexpr (SELF) {
+            float a, b;
+            unpack2(f, a, b);
+            f = pack2(slot == 2 * p ? 0.f : a, slot == 2 * p + 1 ? 0.f : b);
         }
+        C.ax[p] = fma2(f, rx, C.ax[p]);
+        C.ay[p] = fma2(f, ry, C.ay[p]);
+        C.az[p] = fma2(f, rz, C.az[p]);
     }
-    return a;
+}
+
+// The source at sorted position q (none when !in) against the chunk [kb, ke).
+__device__ __forceinline__ void eval_source(float4 y, int q, bool in, int kb, int ke, float eps2,
+                                            Chunk &C) {
+    // a missing source is massless and away from every target
+    if (!in) y = make_float4(1e15f, 1e15f, 1e15f, 0.f);
+    const int t = q - kb;
+    const bool mine = in && q >= kb && q < ke;
+    if (__any_sync(0xffffffffu, mine))
+        eval_sources<true>(y, mine && (t & 3) == (int)(threadIdx.x & 31) >> 3 ? t >> 2 : -1, eps2, C);
+    else
+        eval_sources<false>(y, -1, eps2, C);
+}
+
+// Steps of eight listed sources, entries [from, to); the next step's
+// particles are loaded before this step's are used.
+__device__ __forceinline__ void eval_list(const WarpLists &W, const float4 *__restrict__ xs, int from, int to,
+                                          int kb, int ke, float eps2, Chunk &C) {
+    const int i = threadIdx.x & 7;
+    int q = W.src[min(from + i, to - 1)];
+    float4 y = xs[q];
+    for (int j = from; j < to; j += 8) {
+        const int qn = W.src[min(j + 8 + i, to - 1)];
+        const float4 yn = xs[qn];
+        eval_source(y, q, j + i < to, kb, ke, eps2, C);
+        q = qn;
+        y = yn;
+    }
+}
+
+// The sources [q0, q1) of one long leaf.
+__device__ __forceinline__ void eval_range(const float4 *__restrict__ xs, int q0, int q1, int kb, int ke,
+                                           float eps2, Chunk &C) {
+    const int i = threadIdx.x & 7;
+    for (int j = q0; j < q1; j += 8) {
+        const int q = min(j + i, q1 - 1);
+        eval_source(xs[q], q, j + i < q1, kb, ke, eps2, C);
+    }
 }
 
 // Per cell, kRec float4: the four the list evaluation reads (centre and
@@ -149,34 +269,23 @@ __global__ void walk_groups_kernel(const int32_t *__restrict__ parent, const int
     }
 }
 
-template <bool COUNT>
-__global__ void __launch_bounds__(kWalkThreads)
+template <bool QUAD, bool COUNT>
+__global__ void __launch_bounds__(kWalkThreads, kWalkPerSm)
     walk_kernel(WalkTree T, const int32_t *__restrict__ groups, uint32_t *ctr, int32_t *stacks,
-                float theta, float eps2, int use_quad, float *__restrict__ acc_out, DevInfo *info) {
+                float theta, float eps2, float *__restrict__ acc_out, DevInfo *info) {
     if (info->status & (kErrOverflow | kErrNonFinite)) return;
     __shared__ WarpLists lists[kWalkWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     WarpLists &W = lists[warp];
-    int32_t *stack = stacks + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
+    int32_t *far = stacks + ((int64_t)blockIdx.x * kWalkWarps + warp) * kStackCap;
     const uint32_t ngroups = *(volatile const uint32_t *)&ctr[0];
     const unsigned lt = lanemask_lt();
-    const float side = (float)T.side;
+    const float side = (float)T.side, theta2 = theta * theta;
     // interactions evaluated by this warp (lane 0 counts): target x accepted
     // cell, and target x source particle (self excluded); added to the
     // walk's totals when the warp is done
     unsigned long long n_cell_int = 0, n_pp_int = 0;
     unsigned long long *totals = reinterpret_cast<unsigned long long *>(ctr + 2);
-    auto count = [&](int ncell, int nrange, int64_t nt) {
-        if (!COUNT) return;
-        long long srcs = 0;
-        for (int j = lane; j < nrange; j += 32) srcs += W.range[j].y - W.range[j].x;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) srcs += __shfl_xor_sync(0xffffffffu, srcs, off);
-        if (lane == 0) {
-            n_cell_int += (unsigned long long)(ncell * nt);
-            n_pp_int += (unsigned long long)(srcs * nt);
-        }
-    };
     for (;;) {
         uint32_t gi = 0;
         if (lane == 0) gi = atomicAdd(&ctr[1], 1u);
@@ -189,14 +298,14 @@ __global__ void __launch_bounds__(kWalkThreads)
             return;
         }
         const int32_t g = groups[gi];
-        const int64_t gpf = T.pfirst[g], gpe = T.pend[g];
-        for (int64_t kb = gpf; kb < gpe; kb += 32) {
-            const int64_t ke = min64(gpe, kb + 32);
-            const int64_t k = kb + lane;
+        const int gpf = T.pfirst[g], gpe = T.pend[g];
+        for (int kb = gpf; kb < gpe; kb += min(32, gpe - kb)) {
+            const int nt = min(32, gpe - kb), ke = kb + nt;
             // bounding box of the chunk
             float bmin[3], bmax[3];
+            Chunk C;
             {
-                const float4 x = T.xs[k < ke ? k : kb];
+                const float4 x = T.xs[lane < nt ? kb + lane : kb];
                 bmin[0] = bmax[0] = x.x;
                 bmin[1] = bmax[1] = x.y;
                 bmin[2] = bmax[2] = x.z;
@@ -205,92 +314,155 @@ __global__ void __launch_bounds__(kWalkThreads)
                         bmin[a] = fminf(bmin[a], __shfl_xor_sync(0xffffffffu, bmin[a], off));
                         bmax[a] = fmaxf(bmax[a], __shfl_xor_sync(0xffffffffu, bmax[a], off));
                     }
+                // slot s of this lane: target 4 s + lane / 8 (the first, when
+                // there is no such target)
+                C.pairs = (nt + 7) / 8;
+#pragma unroll
+                for (int p = 0; p < kPairs; ++p) {
+                    const int t0 = 8 * p + (lane >> 3), t1 = t0 + 4;
+                    C.x[p] = pack2(__shfl_sync(0xffffffffu, x.x, t0), __shfl_sync(0xffffffffu, x.x, t1));
+                    C.y[p] = pack2(__shfl_sync(0xffffffffu, x.y, t0), __shfl_sync(0xffffffffu, x.y, t1));
+                    C.z[p] = pack2(__shfl_sync(0xffffffffu, x.z, t0), __shfl_sync(0xffffffffu, x.z, t1));
+                    C.ax[p] = C.ay[p] = C.az[p] = 0;
+                }
             }
-            float3 acc = make_float3(0.f, 0.f, 0.f);
-            int sp = 1, ncell = 0, nrange = 0;
-            if (lane == 0) stack[0] = 0;
+            int sp = 1, ncell = 0, nsrc = 0;
+            if (lane == 0) W.stack[0] = 0;
             __syncwarp();
             bool overflow = false;
             while (sp > 0) {
-                // room for this round: 32 accepted cells or leaf ranges, and
-                // 7 more stack entries per cell taken
-                if (ncell + 32 > kCellCap || nrange + 32 > kRangeCap) {
-                    count(ncell, nrange, ke - kb);
-                    acc = evaluate(T, W, ncell, nrange, k, ke, eps2, use_quad != 0, acc);
-                    ncell = nrange = 0;
-                    __syncwarp();
-                }
+                // at most 32 cells, and room for 7 more stack entries per cell
                 const int take = min(min(sp, 32), (kStackCap - sp) / 7);
                 if (take == 0) {
                     overflow = true;
                     break;
                 }
                 int c = -1;
-                if (lane < take) c = stack[sp - 1 - lane];
+                if (lane < take) {
+                    const int at = sp - 1 - lane;
+                    c = at < kStackNear ? W.stack[at] : far[at];
+                }
                 sp -= take;
-                __syncwarp();
-                int kind = 0;                           // 1 accept, 2 leaf, 3 open
-                int nch = 0, c0 = 0;
                 float4 r0 = make_float4(0.f, 0.f, 0.f, 0.f), r1 = r0;
                 int4 lk = make_int4(0, 0, 0, 0);        // pfirst, pend, child_first, child_end
                 if (c >= 0) {
-                    lk = reinterpret_cast<const int4 *>(T.rec + kRec * (int64_t)c)[4];
-                    const bool meets = lk.x < ke && kb < lk.y;
-                    c0 = lk.z;
+                    const float4 *rec = T.rec + kRec * (int64_t)c;
+                    lk = reinterpret_cast<const int4 *>(rec)[4];
+                    r0 = rec[0];
+                    r1 = rec[1];
+                }
+                // what earlier rounds listed, while these loads are on their way:
+                // whole steps from the lists' ends
+                cp_async_wait_all();
+                __syncwarp();
+                if (ncell >= 8) {
+                    eval_cells<QUAD>(W, ncell & 7, ncell, eps2, C);
+                    ncell &= 7;
+                }
+                if (nsrc > kSrcCap - 32 * kSrcLeaf) {
+                    eval_list(W, T.xs, nsrc & 7, nsrc, kb, ke, eps2, C);
+                    nsrc &= 7;
+                }
+                __syncwarp();
+                int kind = 0;                           // 1 accept, 2 leaf, 3 open
+                int nch = 0;
+                const int c0 = lk.z;
+                if (c >= 0) {
                     bool accept = false;
-                    if (!meets) {
-                        r0 = T.rec[kRec * (int64_t)c];
-                        r1 = T.rec[kRec * (int64_t)c + 1];
-                        const float l = scalbnf(side, -__float_as_int(r1.w));
+                    if (!(lk.x < ke && kb < lk.y)) {
+                        const float l = side * __int_as_float((127 - __float_as_int(r1.w)) << 23);   // side 2^-level
                         const float cx[3] = {r0.x + r1.x, r0.y + r1.y, r0.z + r1.z};
                         float d2 = 0.f;
                         for (int a = 0; a < 3; ++a) {
                             const float u = fmaxf(fmaxf(bmin[a] - cx[a], cx[a] - bmax[a]), 0.f);
                             d2 = fmaf(u, u, d2);
                         }
-                        accept = l * l < theta * theta * d2;
+                        accept = l * l < theta2 * d2;
                     }
                     if (accept) kind = 1;
                     else if (c0 < 0) kind = 2;
                     else { kind = 3; nch = lk.w - c0; }
                 }
                 const unsigned ba = __ballot_sync(0xffffffffu, kind == 1);
-                const unsigned bl = __ballot_sync(0xffffffffu, kind == 2);
                 if (kind == 1) {
-                    float4 *dst = W.cell[ncell + __popc(ba & lt)];
-                    dst[0] = r0;
-                    dst[1] = r1;
-                    dst[2] = T.rec[kRec * (int64_t)c + 2];
-                    dst[3] = T.rec[kRec * (int64_t)c + 3];
+                    float4 *row = W.cell[ncell + __popc(ba & lt)];
+                    const float4 *rec = T.rec + kRec * (int64_t)c;
+                    row[0] = r0;
+                    row[1] = r1;
+                    if constexpr (QUAD) {
+                        cp_async16(row + 2, rec + 2);
+                        cp_async16(row + 3, rec + 3);
+                    }
                 }
-                if (kind == 2) W.range[nrange + __popc(bl & lt)] = make_int2(lk.x, lk.y);
                 ncell += __popc(ba);
-                nrange += __popc(bl);
-                // children onto the stack (exclusive scan of the counts)
-                int pos = nch;
+                // prefixes of the children (low half) and of the listed sources
+                const int cnt = kind == 2 ? lk.y - lk.x : 0;
+                const int few = cnt <= kSrcLeaf ? cnt : 0;
+                const int both = nch | (few << 16);
+                int pos = both;
+#pragma unroll
                 for (int off = 1; off < 32; off <<= 1) {
                     const int y = __shfl_up_sync(0xffffffffu, pos, off);
                     if (lane >= off) pos += y;
                 }
                 const int total = __shfl_sync(0xffffffffu, pos, 31);
-                pos -= nch;
-                for (int j = 0; j < nch; ++j) stack[sp + pos + j] = c0 + nch - 1 - j;
-                sp += total;
+                pos -= both;
+                for (int j = 0; j < nch; ++j) {
+                    const int at = sp + (pos & 0xffff) + j;
+                    if (at < kStackNear) W.stack[at] = c0 + nch - 1 - j;
+                    else far[at] = c0 + nch - 1 - j;
+                }
+                for (int j = 0; j < few; ++j) W.src[nsrc + (pos >> 16) + j] = lk.x + j;
+                sp += total & 0xffff;
+                nsrc += total >> 16;
+                if (COUNT) {
+                    long long srcs = cnt;
+#pragma unroll
+                    for (int off = 16; off > 0; off >>= 1) srcs += __shfl_xor_sync(0xffffffffu, srcs, off);
+                    n_cell_int += (unsigned long long)(__popc(ba) * nt);
+                    n_pp_int += (unsigned long long)(srcs * nt);
+                }
+                // longer leaves at once, one after another
+                for (unsigned bl = __ballot_sync(0xffffffffu, cnt > kSrcLeaf); bl; bl &= bl - 1) {
+                    const int w = __ffs(bl) - 1;
+                    eval_range(T.xs, __shfl_sync(0xffffffffu, lk.x, w), __shfl_sync(0xffffffffu, lk.y, w), kb,
+                               ke, eps2, C);
+                }
                 __syncwarp();
             }
             if (overflow) {
+                cp_async_wait_all();
                 if (lane == 0) atomicOr(&info->status, kErrWalk);
                 return;
             }
-            count(ncell, nrange, ke - kb);
-            if (COUNT && lane == 0) n_pp_int -= (unsigned long long)(ke - kb);   // own pairs
-            acc = evaluate(T, W, ncell, nrange, k, ke, eps2, use_quad != 0, acc);
+            if (COUNT) n_pp_int -= (unsigned long long)nt;   // own pairs
+            cp_async_wait_all();
             __syncwarp();
-            if (k < ke) {
-                const int64_t i = T.perm[k];
-                acc_out[3 * i] = acc.x;
-                acc_out[3 * i + 1] = acc.y;
-                acc_out[3 * i + 2] = acc.z;
+            if (ncell) eval_cells<QUAD>(W, 0, ncell, eps2, C);
+            if (nsrc) eval_list(W, T.xs, 0, nsrc, kb, ke, eps2, C);
+            __syncwarp();
+            // the eight lanes' sums of each target; lane i of a group writes slot i
+            float out[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int p = 0; p < kPairs; ++p) {
+                float v[6];
+                unpack2(C.ax[p], v[0], v[3]);
+                unpack2(C.ay[p], v[1], v[4]);
+                unpack2(C.az[p], v[2], v[5]);
+#pragma unroll
+                for (int off = 1; off < 8; off <<= 1)
+                    for (int a = 0; a < 6; ++a) v[a] += __shfl_xor_sync(0xffffffffu, v[a], off);
+                for (int a = 0; a < 3; ++a) {
+                    if ((lane & 7) == 2 * p) out[a] = v[a];
+                    if ((lane & 7) == 2 * p + 1) out[a] = v[3 + a];
+                }
+            }
+            const int t = 4 * (lane & 7) + (lane >> 3);
+            if (t < nt) {
+                const int64_t i = T.perm[kb + t];
+                acc_out[3 * i] = out[0];
+                acc_out[3 * i + 1] = out[1];
+                acc_out[3 * i + 2] = out[2];
             }
         }
     }
@@ -327,12 +499,9 @@ cudaError_t launch_walk(const tb_tree &t, Workspace &ws, float theta, float eps,
                t.quad, t.aabb, ws.xs, t.perm, t.side, rec};
     // the interaction counts cost about 15% of the walk: only profiled walks
     // take them
-    if (ws.profile)
-        walk_kernel<true><<<kWalkBlocks, kWalkThreads, 0, s>>>(T, groups, ctr, stacks, theta,
-                                                               eps * eps, use_quad, acc, ws.info);
-    else
-        walk_kernel<false><<<kWalkBlocks, kWalkThreads, 0, s>>>(T, groups, ctr, stacks, theta,
-                                                                eps * eps, use_quad, acc, ws.info);
+    auto kern = use_quad ? (ws.profile ? walk_kernel<true, true> : walk_kernel<true, false>)
+                         : (ws.profile ? walk_kernel<false, true> : walk_kernel<false, false>);
+    kern<<<kWalkBlocks, kWalkThreads, 0, s>>>(T, groups, ctr, stacks, theta, eps * eps, acc, ws.info);
     ++g_launches;
     return cudaGetLastError();
 }
