@@ -70,7 +70,8 @@ struct BatchArgs {
 
 template <int T>
 __host__ __device__ inline size_t batch_front_smem(int ncrit) {
-    size_t a = sizeof(CtaSortSharedT<T>), b = lv_smem_bytes<T>(ncrit);
+    const bool fast = ncrit >= kLcMinN && ncrit <= kLcMaxN;
+    const size_t a = sizeof(CtaSortSharedT<T>), b = fast ? lc_smem_bytes<T>(ncrit) : lv_smem_bytes<T>(ncrit);
     return (a > b ? a : b);
 }
 
@@ -185,6 +186,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
     __shared__ int s_nlong;
     __shared__ int64_t s_long[32];
     __shared__ unsigned long long s_end;
+    __shared__ StartCounts s_sc;
     for (;;) {
         const int q = take_set(&A.queue[0], A.n_sets, &s_q);
         if (q < 0) return;
@@ -216,19 +218,22 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
         for (int i = threadIdx.x; i < kBPasses * kBRadix; i += blockDim.x) (&sm.hist[0][0])[i] = 0;
         __syncthreads();
         // ---- keys, records and every pass's digit histogram
+        const bool staged = ns <= CtaSortSharedT<T>::TILE;
         {
             const float lx = s_lo[0], ly = s_lo[1], lz = s_lo[2], shi = s_shi, slo = s_slo;
             const double sc = s_scale;
             const bool ex = s_exact, f32 = s_f32;
             const float m_eq = (float)(1.0 / (double)ns);
             // unsorted keys go where pass 0 reads them: kBPasses is odd, so the
-            // passes run kalt -> pkey -> ... -> pkey
+            // passes run kalt -> pkey -> ... -> pkey (a set of one sort tile keeps
+            // them in shared memory)
             for (int64_t i = o + threadIdx.x; i < o + ns; i += blockDim.x) {
                 const float x = A.pos[3 * i], y = A.pos[3 * i + 1], z = A.pos[3 * i + 2];
                 const uint64_t k = morton_key(quantise(x, lx, shi, slo, sc, ex, f32),
                                               quantise(y, ly, shi, slo, sc, ex, f32),
                                               quantise(z, lz, shi, slo, sc, ex, f32));
-                A.kalt[i] = k;
+                if (staged) sm.keys[i - o] = k;
+                else A.kalt[i] = k;
                 A.xm[i] = make_float4(x, y, z, A.mass ? A.mass[i] : m_eq);
                 for (int p = 0; p < kBPasses; ++p)
                     atomicAdd(&sm.hist[p][(k >> (kBShift0 + p * kBRadixBits)) & (kBRadix - 1)], 1u);
@@ -237,7 +242,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
         __syncthreads();
         // ---- stable LSD sort of the set by its upper key bits (digit counts
         // taken above), then the runs of equal upper bits by the low bits
-        cta_lsd_sort(A.kalt, A.palt, A.pkey, A.perm, o, ns, kBShift0, kBPasses, true, sm);
+        cta_lsd_sort(A.kalt, A.palt, A.pkey, A.perm, o, ns, kBShift0, kBPasses, true, staged, sm);
         __syncthreads();
         for (int64_t t0 = o; t0 < o + ns; t0 += kRunTile) {
             if (threadIdx.x == 0) s_nlong = 0;
@@ -263,7 +268,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
                 const int64_t len = (int64_t)s_end - a;
                 constexpr int low_passes = (kBShift0 + kBRadixBits - 1) / kBRadixBits;
                 cta_histograms(A.pkey, a, len, 0, low_passes, sm);
-                const int np = cta_lsd_sort(A.pkey, A.perm, A.kalt, A.palt, a, len, 0, low_passes, false, sm);
+                const int np = cta_lsd_sort(A.pkey, A.perm, A.kalt, A.palt, a, len, 0, low_passes, false, false, sm);
                 if (np & 1)
                     for (int64_t p = a + threadIdx.x; p < a + len; p += blockDim.x) {
                         A.pkey[p] = A.kalt[p];
@@ -273,16 +278,26 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
             }
         }
         // ---- cells and leaves started per level (the set is its own tree)
-        if (threadIdx.x < kLevelFields) s_tot[threadIdx.x] = 0;
-        __syncthreads();
-        for (int64_t s = o; s < o + ns; s += T) {
-            const int64_t e = min64(o + ns, s + T);
-            const Front f = tile_front<T>(A.pkey, o, o + ns, A.ncrit, s, e, raw, ts);
-            if (f.k < e) A.ml[f.k] = (uint16_t)(f.m | (f.L << 8));
-            warp_field_prefix(ts, nullptr, s_tile);
+        if (A.ncrit >= kLcMinN && A.ncrit <= kLcMaxN) {
+            // tiles of 4 T particles from a multiple of four on
+            if (threadIdx.x <= kLevels) s_sc.m[threadIdx.x] = s_sc.l[threadIdx.x] = 0;
+            for (int64_t s = o & ~int64_t(3); s < o + ns; s += 4 * T) {
+                count_tile4<T>(A.pkey, o, o + ns, A.ncrit, s, min64(o + ns, s + 4 * T), raw, s_sc, A.ml);
+                __syncthreads();
+            }
+            if (threadIdx.x < kLevelFields) s_tot[threadIdx.x] = s_sc.cells(threadIdx.x);
+        } else {
+            if (threadIdx.x < kLevelFields) s_tot[threadIdx.x] = 0;
             __syncthreads();
-            if (threadIdx.x < kLevelFields) s_tot[threadIdx.x] += s_tile[threadIdx.x];
-            __syncthreads();
+            for (int64_t s = o; s < o + ns; s += T) {
+                const int64_t e = min64(o + ns, s + T);
+                const Front f = tile_front<T>(A.pkey, o, o + ns, A.ncrit, s, e, raw, ts);
+                if (f.k < e) A.ml[f.k] = (uint16_t)(f.m | (f.L << 8));
+                warp_field_prefix(ts, nullptr, s_tile);
+                __syncthreads();
+                if (threadIdx.x < kLevelFields) s_tot[threadIdx.x] += s_tile[threadIdx.x];
+                __syncthreads();
+            }
         }
         if (threadIdx.x < kLevelFields)
             A.set_cnt[(int64_t)set * kLevelFields + threadIdx.x] = s_tot[threadIdx.x];
@@ -300,36 +315,39 @@ __global__ void __launch_bounds__(T, 1024 / T) batch_front_kernel(BatchArgs A) {
 // Cell and leaf offsets of the sets (in set order), totals and depth.
 // One block of up to 1024 threads.
 __device__ void batch_scan_block(const BatchArgs &A, int64_t cell_cap) {
-    __shared__ int64_t s_c[1024], s_l[1024];
+    __shared__ int64_t s_c[32], s_l[32];
     __shared__ int s_dmax;
     const int S = A.n_sets;
     const int nt = blockDim.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per = (S + nt - 1) / nt;
     const int lo = threadIdx.x * per, hi = min(S, lo + per);
     int64_t c = 0, l = 0;
     int dmax = 0;
     for (int s = lo; s < hi; ++s) {
         const uint32_t *r = A.set_cnt + (int64_t)s * kLevelFields;
+#pragma unroll
         for (int d = 0; d < kLevels; ++d) {
-            c += r[d];
-            if (r[d]) dmax = max(dmax, d);
+            const uint32_t v = r[d];
+            c += v;
+            if (v) dmax = d;
         }
         l += r[kLevels];
     }
+    // prefixes over the threads: within warps, then over the warps
+    int64_t rc = c, rl = l;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, rc, off), z = __shfl_up_sync(0xffffffffu, rl, off);
+        if (lane >= off) { rc += y; rl += z; }
+    }
     if (threadIdx.x == 0) s_dmax = 0;
-    s_c[threadIdx.x] = c;
-    s_l[threadIdx.x] = l;
+    if (lane == 31) { s_c[warp] = rc; s_l[warp] = rl; }
     __syncthreads();
-    atomicMax(&s_dmax, dmax);
-    if (threadIdx.x == 0) {
-        int64_t rc = 0, rl = 0;
-        for (int t = 0; t < nt; ++t) {
-            const int64_t vc = s_c[t], vl = s_l[t];
-            s_c[t] = rc;
-            s_l[t] = rl;
-            rc += vc;
-            rl += vl;
-        }
+    dmax = __reduce_max_sync(0xffffffffu, dmax);
+    if (lane == 0) atomicMax(&s_dmax, dmax);
+    for (int w = 0; w < warp; ++w) { rc += s_c[w]; rl += s_l[w]; }
+    if (threadIdx.x == nt - 1) {
         A.set_cell_off[S] = rc;
         A.set_leaf_off[S] = rl;
         A.info->n_cells = rc;
@@ -339,7 +357,8 @@ __device__ void batch_scan_block(const BatchArgs &A, int64_t cell_cap) {
         if (cell_cap > 0 && rc > cell_cap) A.info->status |= kErrOverflow;
     }
     __syncthreads();
-    int64_t rc = s_c[threadIdx.x], rl = s_l[threadIdx.x];
+    rc -= c;
+    rl -= l;
     for (int s = lo; s < hi; ++s) {
         A.set_cell_off[s] = rc;
         A.set_leaf_off[s] = rl;

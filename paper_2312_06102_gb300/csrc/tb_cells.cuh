@@ -163,6 +163,157 @@ __device__ __forceinline__ void warp_field_prefix(const TileSharedT<T> &ts,
     }
 }
 
+// m_k and L_k of the particles [s, e) of a tile, and the leaf starts' counts,
+// four consecutive particles per thread of a block of T, for n_crit in
+// [kLcMinN, kLcMaxN]; s is a multiple of four, e - s at most 4 T, and particles
+// before seg_lo take no part (a segment may start inside the tile's first
+// four).  c is kept one byte per
+// position; the window maxima of four neighbours share all but their ends:
+// L_{k0+j} = max(suffix max from byte j of c[k0-n .. k0-n+3],
+//                max of c[k0-n+4 .. k0-1],
+//                prefix max to byte j of c[k0 .. k0+3]),
+// taken four bytes at a time (byte-wise SIMD maxima).
+constexpr int kLcMinN = 3, kLcMaxN = 60;
+
+// Histograms of m and of L + 1 over the leaf starts (m <= L):
+// #cells started at level d = #{m <= d} - #{L + 1 <= d}.
+struct StartCounts {
+    uint32_t m[kLevels + 1], l[kLevels + 1];
+    // cells started at level f, or (f = kLevels) leaves
+    __device__ uint32_t cells(int f) const {
+        uint32_t v = 0;
+        if (f == kLevels) {
+            for (int d = 0; d < kLevels; ++d) v += m[d];
+        } else {
+            for (int d = 0; d <= f; ++d) v += m[d] - l[d];
+        }
+        return v;
+    }
+};
+
+__host__ __device__ inline int lc_halo_words(int ncrit) { return (ncrit + 3) / 4 + 1; }
+template <int T>
+__host__ __device__ inline size_t lc_keys(int ncrit) {
+    return (size_t)4 * T + 4 * lc_halo_words(ncrit) + ncrit + 4;
+}
+template <int T>
+__host__ __device__ inline size_t lc_smem_bytes(int ncrit) {
+    return lc_keys<T>(ncrit) * 8 + ((size_t)T + lc_halo_words(ncrit) + 2) * 4;
+}
+
+template <int T>
+__device__ void count_tile4(const uint64_t *__restrict__ skeys, int64_t seg_lo, int64_t seg_hi, int ncrit,
+                            int64_t s, int64_t e, unsigned char *raw, StartCounts &sc,
+                            uint16_t *__restrict__ ml) {
+    const int H = lc_halo_words(ncrit);
+    const int64_t base = s - 4 * H;                     // position of key[0] and of c byte 0
+    const int nk = (int)(e + ncrit - base);
+    const int nw = (int)((e - base + 3) / 4);
+    uint64_t *key = reinterpret_cast<uint64_t *>(raw);
+    uint32_t *cw = reinterpret_cast<uint32_t *>(raw + lc_keys<T>(ncrit) * 8);
+    // a tile away from both ends of the segment needs no bounds checks: every
+    // window [i, i + n] of its span exists and the keys load as 16-byte pairs
+    // (base is even, so key + base is 16-byte aligned when skeys is)
+    const bool interior = base >= seg_lo && e == s + 4 * T && e + ncrit + 1 <= seg_hi &&
+                          (reinterpret_cast<uintptr_t>(skeys) & 15u) == 0;
+    if (interior) {
+        const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(skeys + base);
+        ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(key);
+        for (int x = threadIdx.x; 2 * x < nk; x += T) dst[x] = src[x];
+    } else {
+        for (int x = threadIdx.x; x < nk; x += T) {
+            const int64_t i = base + x;
+            key[x] = (i >= seg_lo && i < seg_hi) ? skeys[i] : 0ull;
+        }
+    }
+    __syncthreads();
+    // c of four positions per word: min(21, minDepth(i, i+n)) where the
+    // window exists, else 0
+    for (int w = threadIdx.x; w < nw; w += T) {
+        uint32_t v = 0;
+        if (interior) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int x = 4 * w + j;
+                v |= (uint32_t)min(kDepthMax, min_depth(key[x], key[x + ncrit])) << (8 * j);
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int x = 4 * w + j;
+                const int64_t i = base + x;
+                if (i >= seg_lo && i + ncrit < seg_hi && i < e)
+                    v |= (uint32_t)min(kDepthMax, min_depth(key[x], key[x + ncrit])) << (8 * j);
+            }
+        }
+        cw[w] = v;
+    }
+    __syncthreads();
+    const int64_t k0 = s + 4 * (int64_t)threadIdx.x;
+    uint32_t Lw = 0, mw = 0xffffffffu;                  // bytes: L and m of k0 .. k0 + 3
+    if (k0 < e) {
+        const int x0 = (int)(k0 - base);                // multiple of 4
+        const uint32_t Tw = cw[x0 >> 2];
+        auto bytes4 = [&](int b) {                      // c bytes b .. b + 3 (b >= 0)
+            const int w = b >> 2, sh = (b & 3) * 8;
+            return sh ? __funnelshift_r(cw[w], cw[w + 1], sh) : cw[w];
+        };
+        const uint32_t Hw = bytes4(x0 - ncrit);
+        uint32_t I = 0;
+        const int mlen = ncrit - 4;                     // middle bytes x0 - n + 4 .. x0 - 1
+        if (mlen >= 4) {
+            for (int b = x0 - ncrit + 4; b + 4 <= x0; b += 4) I = __vmaxu4(I, bytes4(b));
+            I = __vmaxu4(I, bytes4(x0 - 4));
+        } else if (mlen > 0) {
+            I = bytes4(x0 - ncrit + 4) & ((1u << (8 * mlen)) - 1u);
+        }
+        I = __vmaxu4(I, I >> 16);
+        I = __vmaxu4(I, I >> 8);
+        I = (I & 0xffu) * 0x01010101u;
+        uint32_t S = __vmaxu4(Hw, Hw >> 8);
+        S = __vmaxu4(S, S >> 16);
+        uint32_t P = __vmaxu4(Tw, Tw << 8);
+        P = __vmaxu4(P, P << 16);
+        Lw = __vmaxu4(__vmaxu4(S, P), I);
+        mw = 0;
+        if (interior) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                mw |= (uint32_t)min_depth(key[x0 + j - 1], key[x0 + j]) << (8 * j);
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t k = k0 + j;
+                uint32_t m = 255u;
+                if (k >= seg_lo && k < e)
+                    m = (k == seg_lo) ? 0u : (uint32_t)min_depth(key[x0 + j - 1], key[x0 + j]);
+                mw |= m << (8 * j);
+            }
+        }
+        // m and L of the four particles, for the emission
+        if (k0 >= seg_lo && k0 + 4 <= e) {
+            uint2 v;
+            v.x = (mw & 0xffu) | ((Lw & 0xffu) << 8) | (((mw >> 8) & 0xffu) << 16) | (((Lw >> 8) & 0xffu) << 24);
+            v.y = ((mw >> 16) & 0xffu) | (((Lw >> 16) & 0xffu) << 8) | ((mw >> 24) << 16) | ((Lw >> 24) << 24);
+            *reinterpret_cast<uint2 *>(ml + k0) = v;
+        } else {
+            for (int j = 0; j < 4; ++j)
+                if (k0 + j >= seg_lo && k0 + j < e)
+                    ml[k0 + j] = (uint16_t)(((mw >> (8 * j)) & 0xffu) | (((Lw >> (8 * j)) & 0xffu) << 8));
+        }
+    }
+    // histograms over the leaf starts: about one
+    // particle in seven is a start, so plain shared atomics rarely collide
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const int m = (mw >> (8 * j)) & 0xff, L = (Lw >> (8 * j)) & 0xff;
+        if (m <= L) {
+            atomicAdd(&sc.m[m], 1u);
+            atomicAdd(&sc.l[L + 1], 1u);
+        }
+    }
+}
+
 struct EmitOut {
     uint64_t *ckey;
     uint8_t *level;

@@ -24,42 +24,12 @@ struct CtaSortSharedT {
     int32_t vals[TILE];
     uint32_t warp_hist[WARPS][kCtaRadix + 1];
     uint32_t hist[kCtaMaxPasses][kCtaRadix];
-    uint32_t run[kCtaRadix];
-    uint32_t tile_off[kCtaRadix + 1];
-    uint32_t cnt[kCtaRadix];
-    uint32_t carry[kCtaRadix / 32];
+    uint32_t run[kCtaRadix];                     // next place of each digit in the range
+    uint32_t loc[kCtaRadix];                     // where the digit starts in the tile
+    uint32_t base[kCtaRadix];                    // place in the range, less place in the tile
+    uint32_t carry[WARPS];
 };
 using CtaSortShared = CtaSortSharedT<kCtaThreads>;
-
-// Exclusive prefix of the kCtaRadix counts in[] into out[] (out may alias
-// in), with the total in out[kCtaRadix] when out_total is set: eight warps,
-// 32 digits each, one shuffle scan per warp and a carry across warps.  All
-// threads of the block call it; it ends with a barrier.
-template <int T>
-__device__ __forceinline__ void cta_digit_scan(const uint32_t *in, uint32_t *out, bool out_total,
-                                               uint32_t *s_carry /* [kCtaRadix / 32] */) {
-    static_assert(kCtaRadix == 256 && T >= kCtaRadix, "digit scan shape");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t v = 0, x = 0;
-    if (threadIdx.x < kCtaRadix) {
-        v = in[threadIdx.x];
-        x = v;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
-            if (lane >= off) x += y;
-        }
-        if (lane == 31) s_carry[warp] = x;
-    }
-    __syncthreads();
-    if (threadIdx.x < kCtaRadix) {
-        uint32_t c = 0;
-        for (int w = 0; w < warp; ++w) c += s_carry[w];
-        out[threadIdx.x] = c + x - v;
-        if (out_total && threadIdx.x == kCtaRadix - 1) out[kCtaRadix] = c + x;
-    }
-    __syncthreads();
-}
 
 // Digit counts of every pass over [o, o + ns) into sm.hist.
 template <int T>
@@ -75,28 +45,58 @@ __device__ void cta_histograms(const uint64_t *keys, int64_t o, int64_t ns, int 
     __syncthreads();
 }
 
+// Inclusive prefix over the digits of v, the count of digit threadIdx.x / L,
+// the same in the L = T / 256 lanes of a digit; one block barrier.
+template <int T>
+__device__ __forceinline__ uint32_t cta_digit_scan(uint32_t v, uint32_t *carry) {
+    constexpr int L = T / kCtaRadix;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t y = v;
+#pragma unroll
+    for (int off = L; off < 32; off <<= 1) {
+        const uint32_t z = __shfl_up_sync(0xffffffffu, y, off);
+        if (lane >= off) y += z;
+    }
+    if (lane == 31) carry[warp] = y;
+    __syncthreads();
+    return y + __reduce_add_sync(0xffffffffu, lane < warp ? carry[lane] : 0u);
+}
+
 // Stable LSD sort of [o, o + ns) by the digits at shift0 + 8 p, p < passes,
 // with sm.hist holding each pass's digit counts.  Buffers alternate
 // (keys, vals) -> (alt_k, alt_v) -> ...; with index_vals the first pass takes
 // each element's own position as its value.  Returns the number of passes
-// (the result is in alt_k / alt_v when it is odd).
+// (the result is in alt_k / alt_v when it is odd).  A range of at most one tile
+// stays in shared memory from pass to pass, and with `staged` its keys are
+// there (sm.keys) to begin with.  Five barriers a tile: what bounds it is
+// issue and barriers, as in the single-tree passes.
 template <int T>
 __device__ int cta_lsd_sort(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t *alt_v,
-                            int64_t o, int64_t ns, int shift0, int passes, bool index_vals,
+                            int64_t o, int64_t ns, int shift0, int passes, bool index_vals, bool staged,
                             CtaSortSharedT<T> &sm) {
-    constexpr int kCtaWarps = CtaSortSharedT<T>::WARPS;
-    constexpr int kCtaTile = CtaSortSharedT<T>::TILE;
+    constexpr int W = CtaSortSharedT<T>::WARPS;
+    constexpr int TILE = CtaSortSharedT<T>::TILE;
+    constexpr int L = T / kCtaRadix;             // lanes per digit, W / L warps each
+    static_assert(L >= 1 && L <= 32 && W % L == 0, "whole lanes per digit");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint64_t *src = keys, *dst = alt_k;
-    int32_t *vsrc = vals, *vdst = alt_v;
+    const int dg = threadIdx.x / L, part = threadIdx.x % L;
+    const unsigned lt = lanemask_lt();
+    const int n = (int)ns, first = (int)o;       // positions are 31-bit
+    const bool one = n <= TILE;
+    uint64_t *src = keys + o, *dst = alt_k + o;
+    int32_t *vsrc = vals + o, *vdst = alt_v + o;
+    for (int i = threadIdx.x; i < W * (kCtaRadix + 1); i += T) (&sm.warp_hist[0][0])[i] = 0;
     for (int p = 0; p < passes; ++p) {
         const int shift = shift0 + p * kCtaRadixBits;
-        cta_digit_scan<T>(sm.hist[p], sm.run, false, sm.carry);
-        for (int64_t tb = 0; tb < ns; tb += kCtaTile) {
-            const int valid = (int)min64(kCtaTile, ns - tb);
-            for (int i = threadIdx.x; i < kCtaWarps * (kCtaRadix + 1); i += T)
-                (&sm.warp_hist[0][0])[i] = 0;
+        const bool in_smem = one && (p > 0 || staged), last = p == passes - 1;
+        {
+            const uint32_t v = sm.hist[p][dg];
+            const uint32_t y = cta_digit_scan<T>(v, sm.carry);
+            if (part == 0) sm.run[dg] = y - v;
             __syncthreads();
+        }
+        for (int tb = 0; tb < n; tb += min(TILE, n - tb)) {
+            const int valid = min(TILE, n - tb);
             uint64_t key[kCtaItems];
             int32_t val[kCtaItems];
             uint32_t rank[kCtaItems];
@@ -104,69 +104,86 @@ __device__ int cta_lsd_sort(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int3
 #pragma unroll
             for (int i = 0; i < kCtaItems; ++i) {
                 const int e = wbase + i * 32 + lane;
+                key[i] = 0;
+                val[i] = 0;
                 if (e < valid) {
-                    key[i] = src[o + tb + e];
-                    val[i] = (p == 0 && index_vals) ? (int32_t)(o + tb + e) : vsrc[o + tb + e];
-                } else {
-                    key[i] = 0;
-                    val[i] = 0;
+                    const bool index = p == 0 && index_vals;
+                    key[i] = in_smem ? sm.keys[e] : src[tb + e];
+                    val[i] = index ? first + tb + e : (in_smem ? sm.vals[e] : vsrc[tb + e]);
                 }
             }
             // stable warp ranking: ballot peer masks, leader-updated counters
-            const unsigned lt = lanemask_lt();
-            uint32_t oldc[kCtaItems], lr[kCtaItems];
 #pragma unroll
             for (int i = 0; i < kCtaItems; ++i) {
-                const int e = wbase + i * 32 + lane;
-                const uint32_t d = (e < valid) ? (uint32_t)((key[i] >> shift) & (kCtaRadix - 1))
-                                               : (uint32_t)kCtaRadix;
-                unsigned peers = 0xffffffffu;
+                const bool in = wbase + i * 32 + lane < valid;
+                const uint32_t d = (uint32_t)(key[i] >> shift) & (kCtaRadix - 1);
+                unsigned peers = __ballot_sync(0xffffffffu, in);
+                if (!in) peers = 0;
 #pragma unroll
-                for (int b = 0; b <= kCtaRadixBits; ++b) {
+                for (int b = 0; b < kCtaRadixBits; ++b) {
                     const bool bit = (d >> b) & 1u;
                     const unsigned v = __ballot_sync(0xffffffffu, bit);
                     peers &= bit ? v : ~v;
                 }
                 const int leader = __ffs(peers) - 1;
-                oldc[i] = (lane == leader) ? atomicAdd(&sm.warp_hist[warp][d], (uint32_t)__popc(peers)) : 0u;
-                lr[i] = (uint32_t)leader | ((uint32_t)__popc(peers & lt) << 8);
+                uint32_t old = 0;
+                if (in && lane == leader) old = atomicAdd(&sm.warp_hist[warp][d], (uint32_t)__popc(peers));
+                rank[i] = __shfl_sync(0xffffffffu, old, leader & 31) + (uint32_t)__popc(peers & lt);
             }
+            __syncthreads();
+            // each warp's offset within its digit and the tile's count of the
+            // digit, L lanes a digit
+            uint32_t c[W / L], sum = 0;
 #pragma unroll
-            for (int i = 0; i < kCtaItems; ++i)
-                rank[i] = __shfl_sync(0xffffffffu, oldc[i], lr[i] & 31u) + (lr[i] >> 8);
-            __syncthreads();
-            // warp offsets within each digit, tile digit counts
-            for (int d = threadIdx.x; d < kCtaRadix; d += T) {
-                uint32_t acc = 0;
-                for (int w = 0; w < kCtaWarps; ++w) {
-                    const uint32_t c = sm.warp_hist[w][d];
-                    sm.warp_hist[w][d] = acc;
-                    acc += c;
-                }
-                sm.cnt[d] = acc;
+            for (int j = 0; j < W / L; ++j) {
+                c[j] = sm.warp_hist[part * (W / L) + j][dg];
+                sum += c[j];
+            }
+            uint32_t y = sum;
+#pragma unroll
+            for (int off = 1; off < L; off <<= 1) {
+                const uint32_t z = __shfl_up_sync(0xffffffffu, y, off, L);
+                if (part >= off) y += z;
+            }
+            uint32_t at = y - sum;
+#pragma unroll
+            for (int j = 0; j < W / L; ++j) {
+                sm.warp_hist[part * (W / L) + j][dg] = at;
+                at += c[j];
+            }
+            const uint32_t cnt = __shfl_sync(0xffffffffu, y, L - 1, L);
+            y = cta_digit_scan<T>(cnt, sm.carry);
+            if (part == 0) {
+                const uint32_t r = sm.run[dg];
+                sm.loc[dg] = y - cnt;
+                sm.base[dg] = r - (y - cnt);
+                sm.run[dg] = r + cnt;
             }
             __syncthreads();
-            cta_digit_scan<T>(sm.cnt, sm.tile_off, true, sm.carry);
 #pragma unroll
             for (int i = 0; i < kCtaItems; ++i) {
-                const int e = wbase + i * 32 + lane;
-                if (e < valid) {
-                    const uint32_t d = (uint32_t)((key[i] >> shift) & (kCtaRadix - 1));
-                    const uint32_t ps = sm.tile_off[d] + sm.warp_hist[warp][d] + rank[i];
+                if (wbase + i * 32 + lane < valid) {
+                    const uint32_t d = (uint32_t)(key[i] >> shift) & (kCtaRadix - 1);
+                    const uint32_t ps = sm.loc[d] + sm.warp_hist[warp][d] + rank[i];
                     sm.keys[ps] = key[i];
                     sm.vals[ps] = val[i];
                 }
             }
             __syncthreads();
-            for (int j = threadIdx.x; j < valid; j += T) {
-                const uint64_t k = sm.keys[j];
-                const uint32_t d = (uint32_t)((k >> shift) & (kCtaRadix - 1));
-                const int64_t to = o + sm.run[d] + (j - sm.tile_off[d]);
-                dst[to] = k;
-                vdst[to] = sm.vals[j];
+            for (int i = threadIdx.x; i < W * (kCtaRadix + 1); i += T) (&sm.warp_hist[0][0])[i] = 0;
+            if (!one || last) {
+#pragma unroll
+                for (int i = 0; i < kCtaItems; ++i) {
+                    const int j = i * T + (int)threadIdx.x;
+                    if (j < valid) {
+                        const uint64_t k = sm.keys[j];
+                        const uint32_t d = (uint32_t)(k >> shift) & (kCtaRadix - 1);
+                        const uint32_t to = sm.base[d] + (uint32_t)j;
+                        dst[to] = k;
+                        vdst[to] = sm.vals[j];
+                    }
+                }
             }
-            __syncthreads();
-            for (int d = threadIdx.x; d < kCtaRadix; d += T) sm.run[d] += sm.cnt[d];
             __syncthreads();
         }
         uint64_t *t = src; src = dst; dst = t;

@@ -193,7 +193,7 @@ __device__ void sort_long_run(uint64_t *keys, int32_t *vals, uint64_t *alt_k, in
     __syncthreads();
     if (s_desc) {
         cta_histograms(keys, a, len, 0, passes, sm);
-        const int np = cta_lsd_sort(keys, vals, alt_k, alt_v, a, len, 0, passes, false, sm);
+        const int np = cta_lsd_sort(keys, vals, alt_k, alt_v, a, len, 0, passes, false, false, sm);
         if (np & 1)
             for (int64_t p = a + threadIdx.x; p < a + len; p += T) {
                 keys[p] = alt_k[p];
