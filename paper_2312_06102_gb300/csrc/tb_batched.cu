@@ -15,10 +15,12 @@
 //   batch_emit_kernel   : persistent, one block per set: every cell with its
 //                         links (the single-tree emission from the m_k and L_k
 //                         the count stored, tile after tile with running
-//                         counts), then the set's particles in key order;
-//   batch_moments_kernel: persistent, one block per set: every leaf in key order,
-//                         then the other cells level by level, deepest first,
-//                         with a block barrier between levels.
+//                         counts);
+//   leaf_tile_kernel    : every leaf, as in the single tree: tiles of the whole
+//                         key order, whatever sets they hold;
+//   batch_up_kernel     : persistent, one block per set: the other cells level
+//                         by level, deepest first, with a block barrier
+//                         between levels.
 // The paper builds disjoint subtrees on dynamically scheduled threads
 // (Sec. 2.3.3); here the unit of dynamic scheduling is a whole set.
 #include <cfloat>
@@ -374,9 +376,10 @@ __global__ void __launch_bounds__(1024) batch_scan_kernel(BatchArgs A, int64_t c
     batch_scan_block(A, cell_cap);
 }
 
-// Every cell of one set with its links, then the set's particles in key
-// order (tiles of T particles; all T threads of the block).
-template <int T>
+// Every cell of one set with its links and (GATHER, for moments_set) the
+// set's particles in key order (tiles of T particles; all T threads of the
+// block).
+template <int T, bool GATHER>
 __device__ void emit_set(const BatchArgs &A, const EmitOut &out, int set) {
     __shared__ TileSharedT<T> ts;
     __shared__ uint32_t woff[T / 32][kLevelFields];
@@ -418,8 +421,10 @@ __device__ void emit_set(const BatchArgs &A, const EmitOut &out, int set) {
             __syncthreads();
         }
         // the set's particles in key order, for its moments
-        for (int64_t k = o + threadIdx.x; k < o + ns; k += blockDim.x) A.xs[k] = A.xm[A.perm[k]];
-        __syncthreads();
+        if constexpr (GATHER) {
+            for (int64_t k = o + threadIdx.x; k < o + ns; k += blockDim.x) A.xs[k] = A.xm[A.perm[k]];
+            __syncthreads();
+        }
     }
 }
 
@@ -430,7 +435,7 @@ __global__ void __launch_bounds__(T, 2048 / T) batch_emit_kernel(BatchArgs A, Em
     for (;;) {
         const int q = take_set(&A.queue[1], A.n_sets, &s_q);
         if (q < 0) return;
-        emit_set<T>(A, out, A.order[q]);
+        emit_set<T, false>(A, out, A.order[q]);
     }
 }
 
@@ -456,11 +461,10 @@ __device__ __noinline__ void leaf_sum_f64_serial(const MomOut &o, const float4 *
     finish_d(o, c, D, ref, bb, has64);
 }
 
-// Moments of one set: every leaf in key order, then the other cells level by
-// level, deepest first (all threads of the block).
+// The cells of one set above its leaves, level by level, deepest first (all
+// threads of the block).
 template <int MODE>
-__device__ void moments_set(const BatchArgs &A, const TreeIn &T, const MomOut &o,
-                            const int32_t *__restrict__ leaf_cell, int set) {
+__device__ void parents_set(const BatchArgs &A, const TreeIn &T, const MomOut &o, int set) {
     __shared__ int64_t s_lvl[kLevels + 1];
     {
         const int64_t ns = A.off[set + 1] - A.off[set];
@@ -473,15 +477,6 @@ __device__ void moments_set(const BatchArgs &A, const TreeIn &T, const MomOut &o
             }
             s_lvl[kLevels] = r;
         }
-        // every leaf of the set first, in key order (neighbouring lanes read
-        // neighbouring records), then the other cells level by level
-        const int64_t l0 = A.set_leaf_off[set], l1 = A.set_leaf_off[set + 1];
-        for (int64_t j = l0 + threadIdx.x; j < l1; j += blockDim.x) {
-            const int64_t c = leaf_cell[j];
-            const int64_t pf = T.pfirst[c], pe = T.pend[c];
-            if (pe - pf > kBigLeafSerial) leaf_sum_f64_serial(o, A.xs, c, pf, pe, MODE == TB_MOM_FP64);
-            else leaf_sum<MODE>(o, A.xs, c, pf, pe);
-        }
         __syncthreads();
         for (int d = kDepthMax - 1; d >= 0; --d) {
             for (int64_t c = s_lvl[d] + threadIdx.x; c < s_lvl[d + 1]; c += blockDim.x)
@@ -491,15 +486,52 @@ __device__ void moments_set(const BatchArgs &A, const TreeIn &T, const MomOut &o
     }
 }
 
+// Moments of one set in the one-launch build: every leaf in key order, then
+// the other cells.  Leaves are summed as the leaf tiles of the separate
+// launches sum them -- short ones by a thread, the others (in the compensated
+// mode those of more than kSplitLeaf, else those that do not fit their tile's
+// span) by a warp -- so that both give the same bits up to leaves of 2048.
+template <int MODE>
+__device__ void moments_set(const BatchArgs &A, const TreeIn &T, const MomOut &o,
+                            const int32_t *__restrict__ leaf_cell, int set, int64_t n_total) {
+    const int lane = threadIdx.x & 31;
+    if (A.off[set + 1] <= A.off[set]) return;
+    const int64_t l0 = A.set_leaf_off[set], l1 = A.set_leaf_off[set + 1];
+    for (int64_t j0 = l0 + threadIdx.x - lane; j0 < l1; j0 += blockDim.x) {
+        int64_t c = 0, pf = 0, pe = 0;
+        bool by_warp = false;
+        if (j0 + lane < l1) {
+            c = leaf_cell[j0 + lane];
+            pf = T.pfirst[c];
+            pe = T.pend[c];
+            const int64_t k0 = pf & ~int64_t(kLtTile - 1);
+            const bool staged = pe < k0 + kLtSpan || (pe == n_total && n_total <= k0 + kLtSpan);
+            by_warp = pe - pf <= kBigLeafThread &&
+                      (!staged || (MODE == TB_MOM_FP32_COMP && pe - pf > kSplitLeaf));
+            if (pe - pf > kBigLeafSerial) leaf_sum_f64_serial(o, A.xs, c, pf, pe, MODE == TB_MOM_FP64);
+            else if (!by_warp) leaf_sum<MODE>(o, A.xs, c, pf, pe);
+        }
+        for (unsigned b = __ballot_sync(0xffffffffu, by_warp); b; b &= b - 1) {
+            const int w = __ffs(b) - 1;
+            warp_leaf_sum<MODE>(o, (const float4 *)A.xs, __shfl_sync(0xffffffffu, c, w),
+                                __shfl_sync(0xffffffffu, pf, w), __shfl_sync(0xffffffffu, pe, w));
+        }
+    }
+    __syncthreads();
+    parents_set<MODE>(A, T, o, set);
+}
+
+// The children's loads bound this: one block's levels follow one another, each
+// a few dependent reads long, and few threads have a parent.
 template <int MODE>
 __global__ void __launch_bounds__(kBMomThreads, 3)
-    batch_moments_kernel(BatchArgs A, TreeIn T, MomOut o, const int32_t *__restrict__ leaf_cell) {
+    batch_up_kernel(BatchArgs A, TreeIn T, MomOut o) {
     if (A.info->status & (kErrOverflow | kErrNonFinite | kErrInvalid)) return;
     __shared__ int s_q;
     for (;;) {
         const int q = take_set(&A.queue[2], A.n_sets, &s_q);
         if (q < 0) return;
-        moments_set<MODE>(A, T, o, leaf_cell, A.order[q]);
+        parents_set<MODE>(A, T, o, A.order[q]);
     }
 }
 
@@ -575,8 +607,8 @@ __global__ void __launch_bounds__(T, 1024 / T)
         const int q = take_set(&A.queue[1], A.n_sets, &s_q);
         if (q < 0) return;
         const int set = order[q];
-        emit_set<T>(A, out, set);
-        moments_set<MODE>(A, Tr, o, leaf_cell, set);
+        emit_set<T, true>(A, out, set);
+        moments_set<MODE>(A, Tr, o, leaf_cell, set, n_total);
     }
 }
 
@@ -626,8 +658,10 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
         mark(ws, "batch_scan", s);
         return cudaSuccess;
     }
+    // the keys' second buffer is free by now
+    int32_t *start_cell = reinterpret_cast<int32_t *>(ws.keys_alt);
     EmitOut out{t.ckey, t.level, t.parent, t.child_first, t.child_end, t.pfirst, t.pend,
-                t.leaf_cell};
+                t.leaf_cell, start_cell};
     // the emission keeps 1024-thread tiles whatever the front's block size
     // (two blocks per SM at 32 registers): measured faster than 512 (0.96
     // against 1.10 ms on the 4,096-set workload)
@@ -635,18 +669,19 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
     ++g_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     mark(ws, "batch_emit", s);
+    if ((e = launch_batched_leaves(t, ws, mode, start_cell, s)) != cudaSuccess) return e;
     TreeIn Tr{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
     MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
     const int grid_mom = fit(3);
     switch (mode) {
         case TB_MOM_FP32_COMP:
-            batch_moments_kernel<TB_MOM_FP32_COMP><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o, t.leaf_cell);
+            batch_up_kernel<TB_MOM_FP32_COMP><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o);
             break;
         case TB_MOM_FP32_PLAIN:
-            batch_moments_kernel<TB_MOM_FP32_PLAIN><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o, t.leaf_cell);
+            batch_up_kernel<TB_MOM_FP32_PLAIN><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o);
             break;
         default:
-            batch_moments_kernel<TB_MOM_FP64><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o, t.leaf_cell);
+            batch_up_kernel<TB_MOM_FP64><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o);
             break;
     }
     ++g_launches;
@@ -681,7 +716,7 @@ cudaError_t launch_batched_one_t(const BatchArgs &A, int32_t S, int ncrit, int64
     BatchArgs a = A;
     int32_t *order = ws.set_order;
     EmitOut out{t.ckey, t.level, t.parent, t.child_first, t.child_end, t.pfirst, t.pend,
-                t.leaf_cell};
+                t.leaf_cell, nullptr};
     TreeIn Tr{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
     MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
     const int32_t *leaf_cell = t.leaf_cell;

@@ -392,7 +392,7 @@ cudaError_t launch_emit(const uint64_t *skeys, int64_t n, int ncrit, Workspace &
     (void)ncrit;
     const int64_t tiles = (n + kLvTile - 1) / kLvTile;
     EmitOut o{t.ckey, t.level, t.parent, t.child_first, t.child_end, t.pfirst, t.pend,
-              t.leaf_cell};
+              t.leaf_cell, nullptr};
     const int64_t blocks = (n + kEfTile - 1) / kEfTile;
     emit_starts_kernel<<<(unsigned)blocks, kEfThreads, 0, s>>>(skeys, ws.ml, n, ws.level_cnt, tiles,
                                                                ws.info, o);

@@ -319,6 +319,7 @@ struct EmitOut {
     uint8_t *level;
     int32_t *parent, *child_first, *child_end, *pfirst, *pend;
     int32_t *leaf_cell;
+    int32_t *start_cell;     // batched: the leaf cell that starts at each position
 };
 
 // Cells opened and closed by one particle.  P(d) is the global index of the
@@ -346,7 +347,9 @@ __device__ __forceinline__ void emit_particle(const Front &f, const PF &P, int64
             out.parent[idx] = (d == 0) ? -1 : (int32_t)P(d - 1) - (d == m ? 1 : 0);
             out.child_first[idx] = (d < L) ? (int32_t)P(d + 1) : -1;
         }
-        out.leaf_cell[P(kLevels)] = (int32_t)P(L);
+        const int32_t leaf = (int32_t)P(L);
+        out.leaf_cell[P(kLevels)] = leaf;
+        if (out.start_cell) out.start_cell[k] = leaf;
     }
     if (k == seg_hi - 1) {
         // the tree's last particle closes every cell holding it

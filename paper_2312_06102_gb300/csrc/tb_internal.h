@@ -141,6 +141,8 @@ cudaError_t launch_levels(const uint64_t *skeys, int64_t n, int n_crit, Workspac
 cudaError_t launch_emit(const uint64_t *skeys, int64_t n, int n_crit, Workspace &ws,
                         tb_tree &t, cudaStream_t s);
 cudaError_t launch_moments(tb_tree &t, Workspace &ws, int mode, cudaStream_t s);
+cudaError_t launch_batched_leaves(tb_tree &t, Workspace &ws, int mode, const int32_t *start_cell,
+                                  cudaStream_t s);
 cudaError_t launch_gather_records(const int32_t *perm, const float4 *xm, float4 *xs, int64_t n,
                                   cudaStream_t s);
 cudaError_t launch_wait_selftest(int64_t limit, uint32_t *status, uint32_t *flag, cudaStream_t s);
@@ -148,6 +150,7 @@ cudaError_t launch_wait_selftest(int64_t limit, uint32_t *status, uint32_t *flag
 int level_tile_size();
 int64_t bbox_grid();
 constexpr int64_t kSmallTileMax = int64_t(1) << 19;   // keys that take the small tiles by default
+constexpr int64_t kMidTileMax = int64_t(1) << 24;     // keys that take 512-thread tiles by default
 SortCfg default_sort_cfg(int radix_bits, int64_t n);
 SortCfg first_sort_cfg(int radix_bits);
 const SortCfg *sort_variant(int i);

@@ -39,69 +39,6 @@ namespace {
 
 // ------------------------------------------------------------ kernels
 
-// Shuffle every field of an accumulator down the warp by `off` lanes.
-template <class Acc>
-__device__ __forceinline__ Acc shfl_down_acc(const Acc &a, int off) {
-    Acc b;
-    constexpr int W = sizeof(Acc) / 4;
-    static_assert(sizeof(Acc) % 4 == 0, "accumulators are made of 4-byte words");
-    const uint32_t *u = reinterpret_cast<const uint32_t *>(&a);
-    uint32_t *v = reinterpret_cast<uint32_t *>(&b);
-#pragma unroll
-    for (int i = 0; i < W; ++i) v[i] = __shfl_down_sync(0xffffffffu, u[i], off);
-    return b;
-}
-
-// One leaf [pf, pe) summed by a whole warp (all 32 lanes call it): each lane
-// sums a stride of the members about the leaf's first member, then the
-// lanes' sums merge in a fixed tree (compensated merges in the compensated
-// mode) and lane 0 writes the cell.  `src` is any source of key-ordered
-// records (shared memory, or a PermSrc).
-template <int MODE, class Src>
-__device__ __forceinline__ void warp_leaf_sum(const MomOut &o, Src src, int64_t c, int64_t pf,
-                                              int64_t pe) {
-    using Acc = typename std::conditional<
-        MODE == TB_MOM_FP64, AccD,
-        typename std::conditional<MODE == TB_MOM_FP32_COMP, AccC, AccP>::type>::type;
-    const int lane = threadIdx.x & 31;
-    const float4 r0 = src[pf];
-    const float ref[3] = {r0.x, r0.y, r0.z};
-    float bb[6] = {r0.x, r0.y, r0.z, r0.x, r0.y, r0.z};
-    Acc A;
-    A.init();
-    for (int64_t k = pf + lane; k < pe; k += 32) {
-        const float4 v = src[k];
-        const float x[3] = {v.x, v.y, v.z};
-        for (int a = 0; a < 3; ++a) {
-            bb[a] = fminf(bb[a], x[a]);
-            bb[3 + a] = fmaxf(bb[3 + a], x[a]);
-        }
-        if constexpr (MODE == TB_MOM_FP64) {
-            const double dx[3] = {(double)x[0] - (double)ref[0], (double)x[1] - (double)ref[1],
-                                  (double)x[2] - (double)ref[2]};
-            A.add((double)v.w, dx);
-        } else {
-            const float dx[3] = {__fsub_rn(x[0], ref[0]), __fsub_rn(x[1], ref[1]),
-                                 __fsub_rn(x[2], ref[2])};
-            A.add(v.w, dx);
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        const Acc B = shfl_down_acc(A, off);
-        A.merge(B);
-        for (int a = 0; a < 3; ++a) {
-            bb[a] = fminf(bb[a], __shfl_down_sync(0xffffffffu, bb[a], off));
-            bb[3 + a] = fmaxf(bb[3 + a], __shfl_down_sync(0xffffffffu, bb[3 + a], off));
-        }
-    }
-    if (lane == 0) {
-        if constexpr (MODE == TB_MOM_FP64) finish_d(o, c, A, ref, bb, true);
-        else if constexpr (MODE == TB_MOM_FP32_COMP) finish_c(o, c, A, ref, bb);
-        else finish_p(o, c, A, ref, bb);
-    }
-}
-
 // Leaves, one block per tile of kLtTile consecutive key-order positions.
 //   1. The permutation of the tile and of a halo of kLtHalo positions past
 //      it is bulk-copied (TMA) into shared memory, and m_k | L_k << 8 of the
@@ -115,15 +52,14 @@ __device__ __forceinline__ void warp_leaf_sum(const MomOut &o, Src src, int64_t 
 //   3. k starts a leaf iff m_k <= L_k (Alg. 1 as a closed form); leaves tile
 //      the key order, so a leaf ends where the next one starts.  The leaves
 //      starting in the tile are listed in order; their index among all
-//      leaves comes from the scanned per-tile leaf counts of the cell pass.
+//      leaves comes from the scanned per-tile leaf counts of the cell pass (a
+//      batched build, which counts per set, noted each leaf's cell by its
+//      first position instead).
 //   4. One thread per leaf sums its members from shared memory.  A leaf that
 //      runs past the staged span (only a depth-21 leaf of identical keys, or
 //      n_crit above the halo, can) and, in the compensated mode, a leaf of
 //      more than kSplitLeaf members go to the queues of upward_kernel.
 constexpr int kLtThreads = 256;
-constexpr int kLtTile = 2048;                  // two cell-pass tiles of 1024
-constexpr int kLtHalo = 64;
-constexpr int kLtSpan = kLtTile + kLtHalo;
 constexpr int kLtPer = kLtTile / kLtThreads;   // positions per thread when listing starts
 static_assert(kLtTile == 2 * 1024, "leaf tiles span two tiles of the cell pass");
 
@@ -151,11 +87,12 @@ size_t leaf_tile_smem() { return sizeof(LeafTileSmem); }
 template <int MODE>
 __global__ void __launch_bounds__(kLtThreads, MODE == TB_MOM_FP64 ? 3 : 4)
     leaf_tile_kernel(MomOut o, const int32_t *__restrict__ leaf_cell,
+                     const int32_t *__restrict__ start_cell,
                      const int32_t *__restrict__ perm, const float4 *__restrict__ xm,
                      const uint16_t *__restrict__ ml, const uint32_t *__restrict__ leaf_off,
                      const int32_t *__restrict__ pend, int64_t n, float4 *__restrict__ xs,
                      int32_t *long_queue, int32_t *big_queue, DevInfo *info, int64_t wait_limit) {
-    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout)) return;
+    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout | kErrInvalid)) return;
     extern __shared__ __align__(128) unsigned char lt_raw[];
     LeafTileSmem &S = *reinterpret_cast<LeafTileSmem *>(lt_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -280,7 +217,7 @@ __global__ void __launch_bounds__(kLtThreads, MODE == TB_MOM_FP64 ? 3 : 4)
         if (flags & (1u << j)) S.start[pos++] = (uint16_t)(threadIdx.x * kLtPer + j);
     __syncthreads();
     // 4. one thread per leaf
-    const uint32_t jbase = leaf_off[2 * blockIdx.x];
+    const uint32_t jbase = start_cell ? 0u : leaf_off[2 * blockIdx.x];
     const int32_t nxt = S.next_start;
     // FP64: the leaves in order of their member counts (a counting sort, in
     // the permutation's place), so that the lanes of a warp run equally long.
@@ -315,7 +252,7 @@ __global__ void __launch_bounds__(kLtThreads, MODE == TB_MOM_FP64 ? 3 : 4)
         const uint32_t r = MODE == TB_MOM_FP64 ? (uint32_t)order[i] : i;
         const int x = S.start[r];
         const int xe = (r + 1 < total) ? (int)S.start[r + 1] : nxt;
-        const int64_t c = leaf_cell[jbase + r];
+        const int64_t c = start_cell ? start_cell[k0 + x] : leaf_cell[jbase + r];
         const bool staged = xe >= 0;
         if (!staged) {
             // the end is past the span: leaves too long for one warp apart
@@ -380,6 +317,7 @@ static_assert(kLmTile == 4 * kLmThreads, "the listing takes four children per th
 
 // Children's FP32 moments staged in shared memory: cell c at slot c - base.
 struct CellsStaged {
+    static constexpr bool kAhead = false;
     const LevelSmem *S;
     int64_t base;
     __device__ __forceinline__ float m(int64_t c) const { return S->mass[c - base]; }
@@ -664,7 +602,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kLmThreads, 5)
     upward_kernel(TreeIn T, MomOut o, PermSrc src, const int32_t *long_queue, DevInfo *info, int d_hi,
                   int d_lo, bool leaves, int64_t wait_limit) {
-    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout)) return;
+    if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout | kErrInvalid)) return;
     extern __shared__ __align__(128) unsigned char lm_raw[];
     LevelSmem &S = *reinterpret_cast<LevelSmem *>(lm_raw);
     __shared__ int64_t s_off[kLevels + 1];
@@ -728,12 +666,16 @@ __global__ void wait_selftest_kernel(int64_t limit, uint32_t *status, const uint
     }
 }
 
+// The long-leaf queue (at most n / 2 leaves of two or more members past the
+// first) sits in the upper half of the big-leaf buffer (at most n / 2049
+// entries in the lower).
+int32_t *long_queue(Workspace &ws, int64_t n) { return ws.big_leaf + (n + 1) / 2; }
+
+// The leaves' moments (leaf_tile_kernel), long ones queued for upward_kernel.
 template <int MODE>
-cudaError_t moments_impl(tb_tree &t, Workspace &ws, cudaStream_t s) {
-    TreeIn T{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
+cudaError_t leaves_impl(tb_tree &t, Workspace &ws, const int32_t *start_cell, cudaStream_t s) {
     MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
     const int64_t n = t.n_particles;
-    cudaError_t e;
     static std::atomic<uint64_t> attr_done{0};
     if (first_on_device(attr_done)) {
         cudaFuncSetAttribute(leaf_tile_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -746,19 +688,24 @@ cudaError_t moments_impl(tb_tree &t, Workspace &ws, cudaStream_t s) {
                              cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
     }
-    // the long-leaf queue (at most n / 2 leaves of two or more members past
-    // the first) sits in the upper half of the big-leaf buffer (at most
-    // n / 2049 entries in the lower)
-    int32_t *longq = ws.big_leaf + (n + 1) / 2;
     const int64_t tiles = (n + kLtTile - 1) / kLtTile;
     const int64_t level_tiles = (n + level_tile_size() - 1) / level_tile_size();
     const uint32_t *leaf_off = ws.level_cnt + (int64_t)kLevels * level_tiles;
     leaf_tile_kernel<MODE><<<(unsigned)tiles, kLtThreads, leaf_tile_smem(), s>>>(
-        o, t.leaf_cell, t.perm, ws.xm, ws.ml, leaf_off, t.pend, n,
-        t.pos_sorted ? reinterpret_cast<float4 *>(t.pos_sorted) : nullptr, longq, ws.big_leaf, ws.info,
-        g_wait_limit);
+        o, t.leaf_cell, start_cell, t.perm, ws.xm, ws.ml, leaf_off, t.pend, n,
+        t.pos_sorted ? reinterpret_cast<float4 *>(t.pos_sorted) : nullptr, long_queue(ws, n), ws.big_leaf,
+        ws.info, g_wait_limit);
     ++g_launches;
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
+template <int MODE>
+cudaError_t moments_impl(tb_tree &t, Workspace &ws, cudaStream_t s) {
+    TreeIn T{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
+    MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
+    const int64_t n = t.n_particles;
+    cudaError_t e = leaves_impl<MODE>(t, ws, nullptr, s);
+    if (e != cudaSuccess) return e;
     mark(ws, "leaves", s);
     // every level in one cooperative launch of as many blocks as are resident
     // at once, never more than the tiles a level of at most n cells can have
@@ -772,7 +719,7 @@ cudaError_t moments_impl(tb_tree &t, Workspace &ws, cudaStream_t s) {
         return e;
     const int64_t most = (n + kLmTile / 4 - 1) / (kLmTile / 4);
     if (grid > most) grid = most;
-    const int32_t *lq = longq;
+    const int32_t *lq = long_queue(ws, n);
     int64_t lim = g_wait_limit;
     void *args[] = {&T, &o, &src, &lq, &ws.info, &d_hi, &d_lo, &leaves, &lim};
     e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(upward_kernel<MODE>),
@@ -825,6 +772,31 @@ cudaError_t launch_gather_records(const int32_t *perm, const float4 *xm, float4 
     gather_records_kernel<<<(unsigned)g, 256, 0, s>>>(perm, xm, xs, n);
     ++g_launches;
     return cudaGetLastError();
+}
+
+// The leaves of a batched build: the tiles of the whole key order, then the
+// queued long ones.
+template <int MODE>
+static cudaError_t batched_leaves_impl(tb_tree &t, Workspace &ws, const int32_t *start_cell,
+                                       cudaStream_t s) {
+    cudaError_t e = leaves_impl<MODE>(t, ws, start_cell, s);
+    if (e != cudaSuccess) return e;
+    TreeIn T{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
+    MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
+    upward_kernel<MODE><<<152, kLmThreads, sizeof(LevelSmem), s>>>(
+        T, o, PermSrc{ws.xm, t.perm}, long_queue(ws, t.n_particles), ws.info, -1, -1, true, g_wait_limit);
+    ++g_launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_batched_leaves(tb_tree &t, Workspace &ws, int mode, const int32_t *start_cell,
+                                  cudaStream_t s) {
+    switch (mode) {
+        case TB_MOM_FP32_COMP: return batched_leaves_impl<TB_MOM_FP32_COMP>(t, ws, start_cell, s);
+        case TB_MOM_FP32_PLAIN: return batched_leaves_impl<TB_MOM_FP32_PLAIN>(t, ws, start_cell, s);
+        case TB_MOM_FP64: return batched_leaves_impl<TB_MOM_FP64>(t, ws, start_cell, s);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 cudaError_t launch_moments(tb_tree &t, Workspace &ws, int mode, cudaStream_t s) {

@@ -30,6 +30,7 @@ struct TreeIn {
 // moment, bounding box) as a parent's combination reads its children's:
 // straight from the tree's arrays ...
 struct CellsGlobal {
+    static constexpr bool kAhead = true;   // the next child's loads are issued ahead
     const float *mass, *com, *com_lo, *quad, *aabb;
     __device__ __forceinline__ float m(int64_t c) const { return mass[c]; }
     __device__ __forceinline__ float x(int64_t c, int a) const { return com[3 * c + a]; }
@@ -444,6 +445,74 @@ __device__ void leaf_sum(const MomOut &o, Src xs, int64_t c, int64_t pf, int64_t
     else finish_p(o, c, A, ref, bb);
 }
 
+// Positions a leaf tile covers and holds: see leaf_tile_kernel.
+constexpr int kLtTile = 2048;                  // two cell-pass tiles of 1024
+constexpr int kLtHalo = 64;
+constexpr int kLtSpan = kLtTile + kLtHalo;
+
+// Shuffle every field of an accumulator down the warp by `off` lanes.
+template <class Acc>
+__device__ __forceinline__ Acc shfl_down_acc(const Acc &a, int off) {
+    Acc b;
+    constexpr int W = sizeof(Acc) / 4;
+    static_assert(sizeof(Acc) % 4 == 0, "accumulators are made of 4-byte words");
+    const uint32_t *u = reinterpret_cast<const uint32_t *>(&a);
+    uint32_t *v = reinterpret_cast<uint32_t *>(&b);
+#pragma unroll
+    for (int i = 0; i < W; ++i) v[i] = __shfl_down_sync(0xffffffffu, u[i], off);
+    return b;
+}
+
+// One leaf [pf, pe) summed by a whole warp (all 32 lanes call it): each lane
+// sums a stride of the members about the leaf's first member, then the
+// lanes' sums merge in a fixed tree (compensated merges in the compensated
+// mode) and lane 0 writes the cell.  `src` is any source of key-ordered
+// records (shared memory, or a PermSrc).
+template <int MODE, class Src>
+__device__ __forceinline__ void warp_leaf_sum(const MomOut &o, Src src, int64_t c, int64_t pf,
+                                              int64_t pe) {
+    using Acc = typename std::conditional<
+        MODE == TB_MOM_FP64, AccD,
+        typename std::conditional<MODE == TB_MOM_FP32_COMP, AccC, AccP>::type>::type;
+    const int lane = threadIdx.x & 31;
+    const float4 r0 = src[pf];
+    const float ref[3] = {r0.x, r0.y, r0.z};
+    float bb[6] = {r0.x, r0.y, r0.z, r0.x, r0.y, r0.z};
+    Acc A;
+    A.init();
+    for (int64_t k = pf + lane; k < pe; k += 32) {
+        const float4 v = src[k];
+        const float x[3] = {v.x, v.y, v.z};
+        for (int a = 0; a < 3; ++a) {
+            bb[a] = fminf(bb[a], x[a]);
+            bb[3 + a] = fmaxf(bb[3 + a], x[a]);
+        }
+        if constexpr (MODE == TB_MOM_FP64) {
+            const double dx[3] = {(double)x[0] - (double)ref[0], (double)x[1] - (double)ref[1],
+                                  (double)x[2] - (double)ref[2]};
+            A.add((double)v.w, dx);
+        } else {
+            const float dx[3] = {__fsub_rn(x[0], ref[0]), __fsub_rn(x[1], ref[1]),
+                                 __fsub_rn(x[2], ref[2])};
+            A.add(v.w, dx);
+        }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const Acc B = shfl_down_acc(A, off);
+        A.merge(B);
+        for (int a = 0; a < 3; ++a) {
+            bb[a] = fminf(bb[a], __shfl_down_sync(0xffffffffu, bb[a], off));
+            bb[3 + a] = fmaxf(bb[3 + a], __shfl_down_sync(0xffffffffu, bb[3 + a], off));
+        }
+    }
+    if (lane == 0) {
+        if constexpr (MODE == TB_MOM_FP64) finish_d(o, c, A, ref, bb, true);
+        else if constexpr (MODE == TB_MOM_FP32_COMP) finish_c(o, c, A, ref, bb);
+        else finish_p(o, c, A, ref, bb);
+    }
+}
+
 // ----------------------------------------------------------- parents
 
 // Offset of child c's centre from the reference point ref, as a
@@ -611,15 +680,46 @@ __device__ void combine_children(const TreeIn &T, const MomOut &o, int64_t p, co
             for (int a = 0; a < 3; ++a) ref[a] = src.x(c0, a);
             AccS A;
             A.init();
-            for (int32_t c = c0; c < c1; ++c) {
-                float h[3], l[3], q[6], cb[6];
-                for (int a = 0; a < 3; ++a) child_offset(src, c, a, ref[a], h[a], l[a]);
-                qrow(c, q);
-                if (c > c0) {
-                    brow(c, cb);
-                    grow(bb, cb);
+            if constexpr (Src::kAhead) {
+                // a child's moments come from global memory: the next child's
+                // loads are issued before this one is added
+                struct Child {
+                    float m, x[3], xl[3], q[6], b[6];
+                } k, nx;
+                auto load = [&](int32_t c, Child &v) {
+                    v.m = src.m(c);
+                    for (int a = 0; a < 3; ++a) {
+                        v.x[a] = src.x(c, a);
+                        v.xl[a] = src.xl(c, a);
+                    }
+                    qrow(c, v.q);
+                    brow(c, v.b);
+                };
+                load(c0, k);
+                for (int32_t c = c0; c < c1; ++c) {
+                    if (c + 1 < c1) load(c + 1, nx);
+                    float h[3], l[3];
+                    for (int a = 0; a < 3; ++a) {
+                        float u, w;
+                        two_sum(k.x[a], -ref[a], u, w);
+                        w = __fadd_rn(w, k.xl[a]);
+                        fast_two_sum(u, w, h[a], l[a]);
+                    }
+                    grow(bb, k.b);
+                    A.add_cell(k.m, h, l, k.q);
+                    k = nx;
                 }
-                A.add_cell(src.m(c), h, l, q);
+            } else {
+                for (int32_t c = c0; c < c1; ++c) {
+                    float h[3], l[3], q[6], cb[6];
+                    for (int a = 0; a < 3; ++a) child_offset(src, c, a, ref[a], h[a], l[a]);
+                    qrow(c, q);
+                    if (c > c0) {
+                        brow(c, cb);
+                        grow(bb, cb);
+                    }
+                    A.add_cell(src.m(c), h, l, q);
+                }
             }
             finish_s(o, p, A, ref, bb);
             return;
