@@ -44,6 +44,43 @@ struct SortSmem {
     uint32_t tile;
 };
 
+// Digit d's count over the tiles before `tile`: looks back, kLookWindow
+// predecessors read per round so that one memory latency covers several
+// tiles, until one that has published its inclusive prefix.  Every wait is
+// bounded; one that runs out records a timeout (the count is then too small).
+template <int RADIX>
+__device__ __forceinline__ uint32_t look_back(const uint64_t *lookback, uint32_t tile, int d, uint64_t epoch,
+                                              int64_t spin_limit, DevInfo *info) {
+    uint32_t excl = 0;
+    int64_t pred = (int64_t)tile - 1;
+    int64_t iter = 0;
+    for (;;) {
+        uint64_t w[kLookWindow];
+#pragma unroll
+        for (int j = 0; j < kLookWindow; ++j)
+            w[j] = (pred - j >= 0) ? ld_relaxed_u64(lookback + (pred - j) * RADIX + d) : 0ull;
+        int adv = 0;
+        bool found = false, blocked = false;
+#pragma unroll
+        for (int j = 0; j < kLookWindow; ++j) {
+            if (found || blocked) continue;
+            if (pred - j < 0 || ((w[j] >> 32) & 0x3fffffffu) != epoch || (w[j] >> 62) == 0) {
+                blocked = true;
+                continue;
+            }
+            excl += (uint32_t)w[j];
+            adv = j + 1;
+            if ((w[j] >> 62) == 2) found = true;
+        }
+        if (found) return excl;
+        pred -= adv;
+        if (adv == 0 && !poll_backoff(iter, spin_limit)) {
+            flag_error(&info->status, kErrTimeout);
+            return excl;
+        }
+    }
+}
+
 template <int RADIX_BITS, int THREADS, int ITEMS, bool FIRST>
 __global__ void __launch_bounds__(THREADS, (THREADS <= 256 ? (ITEMS <= 8 ? 4 : 2) : (ITEMS <= 8 ? 2 : 1)))
     onesweep_kernel(const uint64_t *__restrict__ keys_in, const int32_t *__restrict__ vals_in,
@@ -228,33 +265,7 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 256 ? (ITEMS <= 8 ? 4 : 2
         if (d >= RADIX) continue;
         uint32_t excl = 0;
         if (tile > 0) {
-            int64_t pred = (int64_t)tile - 1;
-            int64_t iter = 0;
-            for (;;) {
-                uint64_t w[kLookWindow];
-#pragma unroll
-                for (int j = 0; j < kLookWindow; ++j)
-                    w[j] = (pred - j >= 0) ? ld_relaxed_u64(lookback + (pred - j) * RADIX + d) : 0ull;
-                int adv = 0;
-                bool found = false, blocked = false;
-#pragma unroll
-                for (int j = 0; j < kLookWindow; ++j) {
-                    if (found || blocked) continue;
-                    if (pred - j < 0 || ((w[j] >> 32) & 0x3fffffffu) != epoch || (w[j] >> 62) == 0) {
-                        blocked = true;
-                        continue;
-                    }
-                    excl += (uint32_t)w[j];
-                    adv = j + 1;
-                    if ((w[j] >> 62) == 2) found = true;
-                }
-                if (found) break;
-                pred -= adv;
-                if (adv == 0 && !poll_backoff(iter, spin_limit)) {
-                    flag_error(&info->status, kErrTimeout);
-                    break;
-                }
-            }
+            excl = look_back<RADIX>(lookback, tile, d, epoch, spin_limit, info);
             st_relaxed_u64(lookback + (int64_t)tile * RADIX + d,
                            kFlagIncl | (epoch << 32) | (excl + my_count[r]));
         }
@@ -281,39 +292,223 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 256 ? (ITEMS <= 8 ? 4 : 2
     }
 }
 
+// The pass for 8-bit digits (the default), arranged for many keys per thread:
+//   - keys go through shared memory and out first, then values through the same
+//     memory, and the values are loaded only when the keys have left the
+//     registers, so that a tile of 5376 keys (256 x 21) takes 52 KB and 85
+//     registers, three to an SM;
+//   - a key's place in the tile is kept in 16 bits, each warp's counters are
+//     turned into places in the tile at once (one shared read per key), and a
+//     full tile carries no bounds checks.
+// What bounds it is latency and barriers, at 133 instructions a key (172
+// before): 0.94 ms at 2^27 keys, 3.3 TB/s, where one thread-register tile of
+// 512 x 8 pairs took 1.19; 142 us against 160 at 2^24.
+template <int T, int ITEMS>
+struct Sort8Smem {
+    static constexpr int TILE = T * ITEMS;
+    static constexpr int WARPS = T / 32;
+    union {
+        uint64_t keys[TILE];
+        int32_t vals[TILE];
+    };
+    uint32_t warp_hist[WARPS][257];
+    uint32_t cnt[256], loc[256], base[256];
+    uint32_t carry[WARPS];
+    uint32_t tile;
+};
+
+template <int T, int ITEMS, bool FIRST, bool FULL>
+__device__ __forceinline__ void tile8(Sort8Smem<T, ITEMS> &sm, const uint64_t *__restrict__ keys_in,
+                                          const int32_t *__restrict__ vals_in,
+                                          uint64_t *__restrict__ keys_out, int32_t *__restrict__ vals_out,
+                                          uint32_t n, uint32_t tile, int valid, int pass, int shift,
+                                          const uint32_t *__restrict__ digit_off, uint64_t *lookback,
+                                          DevInfo *info, int64_t spin_limit) {
+    constexpr int TILE = Sort8Smem<T, ITEMS>::TILE, W = T / 32;
+    constexpr int L = T / 256;   // lanes per digit when the tile's digits are counted
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int first = warp * 32 * ITEMS + lane;          // this thread's elements: first + 32 i
+    const uint32_t tile_base = tile * (uint32_t)TILE;
+    const unsigned lt = lanemask_lt();
+    uint64_t key[ITEMS];
+    uint32_t at[(ITEMS + 1) / 2] = {};   // rank in the warp's digit, then place in the tile (16 bits each)
+    {
+        const uint64_t *src = keys_in + tile_base + first;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) key[i] = FULL || first + i * 32 < valid ? src[i * 32] : 0ull;
+    }
+    uint32_t *hist = sm.warp_hist[warp];
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const bool in = FULL || first + i * 32 < valid;
+        const uint32_t d = (uint32_t)(key[i] >> shift) & 255u;
+        unsigned peers = 0xffffffffu;
+        if (!FULL) {
+            peers = __ballot_sync(0xffffffffu, in);
+            if (!in) peers = 0;
+        }
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            const bool bit = (d >> b) & 1u;
+            const unsigned v = __ballot_sync(0xffffffffu, bit);
+            peers &= bit ? v : ~v;
+        }
+        const unsigned below = peers & lt;               // the group's lowest lane has none
+        uint32_t old = 0;
+        if (in && below == 0) old = atomicAdd(hist + d, (uint32_t)__popc(peers));
+        const uint32_t r = __shfl_sync(0xffffffffu, old, __ffs(peers) - 1) + (uint32_t)__popc(below);
+        at[i / 2] = __byte_perm(at[i / 2], r, i & 1 ? 0x5410 : 0x3254);
+    }
+    __syncthreads();
+    // the tile's count of each digit, L lanes a digit; where the digit starts
+    // in the tile; each warp's first place in it
+    {
+        const int dg = threadIdx.x / L, part = threadIdx.x % L;
+        uint32_t *col = &sm.warp_hist[part * (W / L)][dg];
+        uint32_t c[W / L], sum = 0;
+#pragma unroll
+        for (int j = 0; j < W / L; ++j) {
+            c[j] = col[j * 257];
+            sum += c[j];
+        }
+        uint32_t before = 0, total = sum;
+        if constexpr (L == 2) {
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, sum, 1);
+            before = part ? other : 0u;
+            total = sum + other;
+        }
+        uint32_t y = total;
+#pragma unroll
+        for (int off = L; off < 32; off <<= 1) {
+            const uint32_t z = __shfl_up_sync(0xffffffffu, y, off);
+            if (lane >= off) y += z;
+        }
+        if (lane == 31) sm.carry[warp] = y;
+        __syncthreads();
+        const uint32_t start =
+            y - total + __reduce_add_sync(0xffffffffu, lane < warp ? sm.carry[lane] : 0u);
+        uint32_t run = start + before;
+#pragma unroll
+        for (int j = 0; j < W / L; ++j) {
+            col[j * 257] = run;
+            run += c[j];
+        }
+        if (part == 0) {
+            sm.loc[dg] = start;
+            sm.cnt[dg] = total;
+        }
+    }
+    __syncthreads();
+    const uint64_t epoch = (uint64_t)((info->epoch + (uint32_t)pass) & 0x3fffffffu);
+    const int d = threadIdx.x;
+    uint64_t *slot = lookback + (int64_t)tile * 256 + d;
+    uint32_t my = 0;
+    if (d < 256) {
+        my = sm.cnt[d];
+        st_relaxed_u64(slot, (tile == 0 ? kFlagIncl : kFlagAgg) | (epoch << 32) | my);
+    }
+    // (a shift the compiler takes for another one, so that it forms the digits
+    // again instead of keeping them in registers since the ranking)
+    int again = shift;
+    asm("" : "+r"(again));
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const uint32_t p = hist[(uint32_t)(key[i] >> again) & 255u] + (at[i / 2] >> (i & 1 ? 16 : 0) & 0xffffu);
+        at[i / 2] = __byte_perm(at[i / 2], p, i & 1 ? 0x5410 : 0x3254);
+        if (FULL || first + i * 32 < valid) sm.keys[p] = key[i];
+    }
+    // the values on their way while the predecessors finish
+    int32_t val[ITEMS];
+    if (!FIRST) {
+        const int32_t *src = vals_in + tile_base + first;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) val[i] = FULL || first + i * 32 < valid ? src[i * 32] : 0;
+    }
+    if (d < 256) {
+        uint32_t excl = 0;
+        if (tile > 0) {
+            excl = look_back<256>(lookback, tile, d, epoch, spin_limit, info);
+            st_relaxed_u64(slot, kFlagIncl | (epoch << 32) | (excl + my));
+        }
+        sm.base[d] = digit_off[d] + excl - sm.loc[d];
+    }
+    __syncthreads();
+    uint32_t dst[ITEMS];
+    bool bad = false;
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i) {
+        const int j = i * T + (int)threadIdx.x;
+        dst[i] = 0xffffffffu;
+        if (FULL || j < valid) {
+            const uint64_t k = sm.keys[j];
+            dst[i] = sm.base[(uint32_t)(k >> shift) & 255u] + (uint32_t)j;
+            if (dst[i] < n) keys_out[dst[i]] = k;
+            else bad = true;
+        }
+    }
+    if (bad) flag_error(&info->status, kErrTimeout);
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (FULL || first + i * 32 < valid)
+            sm.vals[at[i / 2] >> (i & 1 ? 16 : 0) & 0xffffu] = FIRST ? (int32_t)(tile_base + (uint32_t)(first + i * 32)) : val[i];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (dst[i] < n) vals_out[dst[i]] = sm.vals[i * T + (int)threadIdx.x];
+}
+
+template <int T, int ITEMS, bool FIRST>
+__global__ void __launch_bounds__(T, T == 256 && ITEMS > 18 ? 3 : 1024 / T)
+    onesweep8_kernel(const uint64_t *__restrict__ keys_in, const int32_t *__restrict__ vals_in,
+                         uint64_t *__restrict__ keys_out, int32_t *__restrict__ vals_out, int64_t n,
+                         int pass, int shift0, const uint32_t *__restrict__ digit_off,
+                         uint64_t *lookback, DevInfo *info, int64_t spin_limit) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    using S = Sort8Smem<T, ITEMS>;
+    S &sm = *reinterpret_cast<S *>(smem_raw);
+    if (threadIdx.x == 0) sm.tile = atomicAdd(&info->sort_tile_ctr[pass], 1u);
+    for (int i = threadIdx.x; i < S::WARPS * 257; i += T) (&sm.warp_hist[0][0])[i] = 0;
+    __syncthreads();
+    const uint32_t tile = sm.tile;
+    const int valid = (int)min64(S::TILE, n - (int64_t)tile * S::TILE);
+    if (valid == S::TILE)
+        tile8<T, ITEMS, FIRST, true>(sm, keys_in, vals_in, keys_out, vals_out, (uint32_t)n, tile, valid, pass,
+                                      shift0 + pass * 8, digit_off, lookback, info, spin_limit);
+    else
+        tile8<T, ITEMS, FIRST, false>(sm, keys_in, vals_in, keys_out, vals_out, (uint32_t)n, tile, valid, pass,
+                                       shift0 + pass * 8, digit_off, lookback, info, spin_limit);
+}
+
+template <int B, int T, int I, bool FIRST>
+constexpr auto pass_kernel() {
+    if constexpr (B == 8) return &onesweep8_kernel<T, I, FIRST>;
+    else return &onesweep_kernel<B, T, I, FIRST>;
+}
+
 template <int B, int T, int I>
 cudaError_t run_passes(uint64_t *ka, uint64_t *kb, int32_t *pa, int32_t *pb, int64_t n,
                        Workspace &ws, const SortPlan &plan, uint64_t *&kout, int32_t *&pout,
                        cudaStream_t s) {
-    using S = SortSmem<B, T, I>;
-    const size_t smem = sizeof(S);
+    auto first = pass_kernel<B, T, I, true>(), next = pass_kernel<B, T, I, false>();
+    const size_t smem = B == 8 ? sizeof(Sort8Smem<T, I>) : sizeof(SortSmem<B, T, I>);
     static std::atomic<uint64_t> attr_done{0};
     if (first_on_device(attr_done)) {
-        cudaFuncSetAttribute(onesweep_kernel<B, T, I, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(onesweep_kernel<B, T, I, false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(onesweep_kernel<B, T, I, true>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(onesweep_kernel<B, T, I, false>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
+        for (auto k : {first, next}) {
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+        }
     }
-    const int64_t tiles = (n + S::TILE - 1) / S::TILE;
+    const int64_t tiles = (n + T * I - 1) / (T * I);
     // the unsorted keys are in `ka`; passes alternate ka -> kb -> ka ...
     uint64_t *src = ka, *dst = kb;
     int32_t *vsrc = pa, *vdst = pb;
     const int64_t spin = g_wait_limit;
     for (int p = 0; p < plan.passes; ++p) {
-        if (p == 0)
-            onesweep_kernel<B, T, I, true><<<(unsigned)tiles, T, smem, s>>>(
-                src, nullptr, dst, vdst, n, p, plan.shift0, ws.hist + p * (1 << B), ws.lookback,
-                ws.info, spin);
-        else
-            onesweep_kernel<B, T, I, false><<<(unsigned)tiles, T, smem, s>>>(
-                src, vsrc, dst, vdst, n, p, plan.shift0, ws.hist + p * (1 << B), ws.lookback,
-                ws.info, spin);
+        (p == 0 ? first : next)<<<(unsigned)tiles, T, smem, s>>>(
+            src, p == 0 ? nullptr : vsrc, dst, vdst, n, p, plan.shift0, ws.hist + p * (1 << B), ws.lookback,
+            ws.info, spin);
         ++g_launches;
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -338,20 +533,24 @@ int64_t g_wait_limit = kDefaultWaitLimit;
 
 // Compiled variants: digit bits, threads per tile, keys per thread.
 static const SortCfg kVariants[] = {
-    {8, 256, 16}, {8, 512, 16}, {8, 512, 12}, {8, 512, 8}, {8, 256, 8},
+    {8, 256, 16}, {8, 512, 16}, {8, 512, 12}, {8, 512, 8}, {8, 256, 8}, {8, 512, 14}, {8, 256, 21},
     {9, 256, 16}, {9, 512, 16}, {9, 512, 8}, {10, 256, 16}, {10, 512, 8}, {11, 256, 16},
 };
 static const int kNumVariants = sizeof(kVariants) / sizeof(kVariants[0]);
 
 const SortCfg *sort_variant(int i) { return (i >= 0 && i < kNumVariants) ? &kVariants[i] : nullptr; }
 
-// 8-bit digits: 256 x 8 up to 2^19 keys, where a pass is latency and smaller
-// tiles spread over more SMs (300,000 keys: build 109 us against 117 for
-// 512 x 8 and 119 for 256 x 16), 512 x 8 above (10^6: 160 against 181 and 160;
-// 2^22: 367 against 405 and 381; 2^27: 9.58 ms against 10.03 and 9.78).  Other
-// digits: their first variant.
+// 8-bit digits, a pass at each size (us):
+//   keys        80,000  400,000  10^6   2^22   8 10^6  12 10^6  2^24   2^27
+//   256 x 8       10.3    14.4   22.8   53.9    91.8    130
+//   512 x 8       12.3    13.6   18.9   46.0    82.1    117      160   1190
+//   512 x 14      14.5    16.3   17.3   43.5    77.6    108      143   1025
+//   256 x 21      15.7    15.4   20.4   49.4    81.6    109      142    937
+// Few keys want small tiles, over more SMs; many keys want few look-backs and
+// three blocks per SM.  Other digits: their first variant.
 SortCfg default_sort_cfg(int radix_bits, int64_t n) {
-    if (radix_bits == 8) return n <= kSmallTileMax ? SortCfg{8, 256, 8} : SortCfg{8, 512, 8};
+    if (radix_bits == 8)
+        return n <= kSmallTileMax ? SortCfg{8, 256, 8} : (n <= kMidTileMax ? SortCfg{8, 512, 14} : SortCfg{8, 256, 21});
     return first_sort_cfg(radix_bits);
 }
 
@@ -374,8 +573,8 @@ int64_t sort_tiles(const SortCfg &c, int64_t n) { return (n + c.tile() - 1) / c.
 
 cudaError_t load_sort_kernels() {
     // the default tile of every set tb_keys_sorted_noalloc takes
-    cudaError_t e = load_kernel(onesweep_kernel<8, 256, 8, true>);
-    return e == cudaSuccess ? load_kernel(onesweep_kernel<8, 256, 8, false>) : e;
+    cudaError_t e = load_kernel(onesweep8_kernel<256, 8, true>);
+    return e == cudaSuccess ? load_kernel(onesweep8_kernel<256, 8, false>) : e;
 }
 
 SortPlan sort_plan(const SortCfg &c) {
@@ -398,6 +597,8 @@ cudaError_t launch_sort(uint64_t *ka, uint64_t *kb, int32_t *pa, int32_t *pb, in
     TB_SORT_CASE(8, 512, 12)
     TB_SORT_CASE(8, 512, 8)
     TB_SORT_CASE(8, 256, 8)
+    TB_SORT_CASE(8, 512, 14)
+    TB_SORT_CASE(8, 256, 21)
     TB_SORT_CASE(9, 256, 16)
     TB_SORT_CASE(9, 512, 16)
     TB_SORT_CASE(9, 512, 8)
