@@ -126,6 +126,7 @@ __device__ void set_order_block(const int64_t *off, int32_t S, int32_t *order) {
 
 __global__ void __launch_bounds__(1024) set_order_kernel(const int64_t *off, int32_t S,
                                                          int32_t *order, const DevInfo *info) {
+    after_previous();
     if (info->status & kErrInvalid) return;
     set_order_block(off, S, order);
 }
@@ -309,6 +310,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
 
 template <int T>
 __global__ void __launch_bounds__(T, 1024 / T) batch_front_kernel(BatchArgs A) {
+    after_previous();
     if (A.info->status & kErrInvalid) return;
     extern __shared__ __align__(16) unsigned char raw[];
     front_sets<T>(A, raw);
@@ -372,6 +374,7 @@ __device__ void batch_scan_block(const BatchArgs &A, int64_t cell_cap) {
 }
 
 __global__ void __launch_bounds__(1024) batch_scan_kernel(BatchArgs A, int64_t cell_cap) {
+    after_previous();
     if (A.info->status & kErrInvalid) return;
     batch_scan_block(A, cell_cap);
 }
@@ -430,6 +433,7 @@ __device__ void emit_set(const BatchArgs &A, const EmitOut &out, int set) {
 
 template <int T>
 __global__ void __launch_bounds__(T, 2048 / T) batch_emit_kernel(BatchArgs A, EmitOut out) {
+    after_previous();
     if (A.info->status & (kErrOverflow | kErrNonFinite | kErrInvalid)) return;
     __shared__ int s_q;
     for (;;) {
@@ -526,6 +530,7 @@ __device__ void moments_set(const BatchArgs &A, const TreeIn &T, const MomOut &o
 template <int MODE>
 __global__ void __launch_bounds__(kBMomThreads, 3)
     batch_up_kernel(BatchArgs A, TreeIn T, MomOut o) {
+    after_previous();
     if (A.info->status & (kErrOverflow | kErrNonFinite | kErrInvalid)) return;
     __shared__ int s_q;
     for (;;) {
@@ -547,6 +552,7 @@ __device__ void set_check_grid(const int64_t *off, int32_t S, int64_t n_total, D
 }
 
 __global__ void set_check_kernel(const int64_t *off, int32_t S, int64_t n_total, DevInfo *info) {
+    after_previous();
     set_check_grid(off, S, n_total, info);
 }
 
@@ -645,14 +651,14 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
     // per SM, two emission blocks), at most one per set
     auto fit = [&](int per_sm) { return S < per_sm * nsm ? (S > 0 ? S : 1) : per_sm * nsm; };
     if (phase == 0) {
-        set_order_kernel<<<1, 1024, 0, s>>>(A.off, S, ws.set_order, ws.info);
+        launch_after(set_order_kernel, dim3(1), dim3(1024), 0, s, A.off, S, ws.set_order, ws.info);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        batch_front_kernel<T><<<fit(1024 / T), T, batch_front_smem<T>(ncrit), s>>>(A);
+        launch_after(batch_front_kernel<T>, dim3(fit(1024 / T)), dim3(T), batch_front_smem<T>(ncrit), s, A);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         mark(ws, "batch_front", s);
-        batch_scan_kernel<<<1, 1024, 0, s>>>(A, cell_cap);
+        launch_after(batch_scan_kernel, dim3(1), dim3(1024), 0, s, A, cell_cap);
         ++g_launches;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         mark(ws, "batch_scan", s);
@@ -665,7 +671,7 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
     // the emission keeps 1024-thread tiles whatever the front's block size
     // (two blocks per SM at 32 registers): measured faster than 512 (0.96
     // against 1.10 ms on the 4,096-set workload)
-    batch_emit_kernel<1024><<<fit(2), 1024, 0, s>>>(A, out);
+    launch_after(batch_emit_kernel<1024>, dim3(fit(2)), dim3(1024), 0, s, A, out);
     ++g_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     mark(ws, "batch_emit", s);
@@ -675,13 +681,13 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
     const int grid_mom = fit(3);
     switch (mode) {
         case TB_MOM_FP32_COMP:
-            batch_up_kernel<TB_MOM_FP32_COMP><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o);
+            launch_after(batch_up_kernel<TB_MOM_FP32_COMP>, dim3(grid_mom), dim3(kBMomThreads), 0, s, A, Tr, o);
             break;
         case TB_MOM_FP32_PLAIN:
-            batch_up_kernel<TB_MOM_FP32_PLAIN><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o);
+            launch_after(batch_up_kernel<TB_MOM_FP32_PLAIN>, dim3(grid_mom), dim3(kBMomThreads), 0, s, A, Tr, o);
             break;
         default:
-            batch_up_kernel<TB_MOM_FP64><<<grid_mom, kBMomThreads, 0, s>>>(A, Tr, o);
+            launch_after(batch_up_kernel<TB_MOM_FP64>, dim3(grid_mom), dim3(kBMomThreads), 0, s, A, Tr, o);
             break;
     }
     ++g_launches;

@@ -47,6 +47,7 @@ namespace {
 __global__ void __launch_bounds__(kLvThreads, 2)
     level_count_kernel(const uint64_t *__restrict__ skeys, int64_t n, int ncrit,
                        uint32_t *__restrict__ tile_cnt, int64_t n_tiles, uint16_t *__restrict__ ml) {
+    after_previous();
     extern __shared__ __align__(16) unsigned char raw[];
     __shared__ TileShared ts;
     __shared__ uint32_t tot[kLevelFields];
@@ -68,6 +69,7 @@ __global__ void __launch_bounds__(kLcThreads, 6)
     level_count_fast_kernel(const uint64_t *__restrict__ skeys, int64_t n, int ncrit,
                             uint32_t *__restrict__ tile_cnt, int64_t n_tiles,
                             uint16_t *__restrict__ ml) {
+    after_previous();
     extern __shared__ __align__(16) unsigned char raw[];
     __shared__ StartCounts sc;
     for (int x = threadIdx.x; x <= kLevels; x += kLcThreads) sc.m[x] = sc.l[x] = 0;
@@ -88,6 +90,7 @@ static_assert(kScanPer == 8, "the scan moves each thread's eight counts as two u
 
 __global__ void __launch_bounds__(kScanThreads)
     level_scan_kernel(uint32_t *tile_cnt, int64_t n_tiles, DevInfo *info, int64_t cell_cap) {
+    after_previous();
     const int f = blockIdx.x;
     uint32_t *row = tile_cnt + (int64_t)f * n_tiles;
     __shared__ __align__(16) uint32_t s_v[kScanChunk];
@@ -191,6 +194,7 @@ __global__ void __launch_bounds__(kEfThreads, 4)
     emit_starts_kernel(const uint64_t *__restrict__ skeys, const uint16_t *__restrict__ ml, int64_t n,
                        const uint32_t *__restrict__ tile_off, int64_t n_tiles, DevInfo *info_w,
                        EmitOut out) {
+    after_previous();
     const DevInfo *info = info_w;
     if (info->status & (kErrOverflow | kErrNonFinite)) return;
     __shared__ uint32_t s_entry[kEfTile];               // k - s | m << 11 | L << 16 | Lprev << 21
@@ -372,16 +376,16 @@ cudaError_t launch_levels(const uint64_t *skeys, int64_t n, int ncrit, Workspace
                                  cudaFuncAttributePreferredSharedMemoryCarveout,
                                  cudaSharedmemCarveoutMaxShared);
         }
-        level_count_fast_kernel<<<(unsigned)tiles, kLcThreads, lc_smem_bytes<kLcThreads>(ncrit), s>>>(
+        launch_after(level_count_fast_kernel, dim3((unsigned)tiles), dim3(kLcThreads), lc_smem_bytes<kLcThreads>(ncrit), s, 
             skeys, n, ncrit, ws.level_cnt, tiles, ws.ml);
     } else {
-        level_count_kernel<<<(unsigned)tiles, kLvThreads, smem, s>>>(skeys, n, ncrit, ws.level_cnt,
+        launch_after(level_count_kernel, dim3((unsigned)tiles), dim3(kLvThreads), smem, s, skeys, n, ncrit, ws.level_cnt,
                                                                      tiles, ws.ml);
     }
     ++g_launches;
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
-    level_scan_kernel<<<kLevelFields, kScanThreads, 0, s>>>(ws.level_cnt, tiles, ws.info,
+    launch_after(level_scan_kernel, dim3(kLevelFields), dim3(kScanThreads), 0, s, ws.level_cnt, tiles, ws.info,
                                                             ws.cell_cap_request);
     ++g_launches;
     return cudaGetLastError();
@@ -394,7 +398,7 @@ cudaError_t launch_emit(const uint64_t *skeys, int64_t n, int ncrit, Workspace &
     EmitOut o{t.ckey, t.level, t.parent, t.child_first, t.child_end, t.pfirst, t.pend,
               t.leaf_cell, nullptr};
     const int64_t blocks = (n + kEfTile - 1) / kEfTile;
-    emit_starts_kernel<<<(unsigned)blocks, kEfThreads, 0, s>>>(skeys, ws.ml, n, ws.level_cnt, tiles,
+    launch_after(emit_starts_kernel, dim3((unsigned)blocks), dim3(kEfThreads), 0, s, skeys, ws.ml, n, ws.level_cnt, tiles,
                                                                ws.info, o);
     ++g_launches;
     return cudaGetLastError();

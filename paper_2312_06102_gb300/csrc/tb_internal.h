@@ -206,6 +206,28 @@ inline bool first_on_device(std::atomic<uint64_t> &done) {
     return true;
 }
 
+// Launches a kernel of a chain of this library's own launches in one call,
+// with programmatic stream serialisation: it is set up while the previous
+// kernel drains, and waits in after_previous(), the kernel's first statement,
+// until that kernel has completed.  The first kernel of a call is launched
+// plainly, whatever the caller enqueued before it.  Saves 1 to 2.5 us a
+// launch: 3,001 particles 76 -> 68 us, 10^6 303 -> 278, 300 sets 170 -> 150, the
+// allocation-free call of 300,007 121 -> 100.
+template <class... P, class... A>
+cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <class K>
 cudaError_t load_kernel(K kernel) {
     cudaFuncAttributes a;

@@ -44,6 +44,7 @@ __global__ void __launch_bounds__(kRootThreads) root_kernel(const float *__restr
                                                             bool vec, float *__restrict__ part,
                                                             DevInfo *info, uint32_t *hist,
                                                             int hist_len, bool pow2) {
+    after_previous();
     Box b;
     b.init();
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(kKeysThreads, 6) keys_kernel(const float *__re
                                                             float4 *__restrict__ xm,
                                                             uint32_t *hist, int passes, int shift0,
                                                             DevInfo *info) {
+    after_previous();
     constexpr int RADIX = 1 << RADIX_BITS;
     extern __shared__ uint32_t s_hist[];   // [passes][RADIX]
     for (int i = threadIdx.x; i < passes * RADIX; i += blockDim.x) s_hist[i] = 0;
@@ -285,7 +287,7 @@ static cudaError_t keys_impl(const float *pos, const float *mass, int64_t n, uin
     int64_t grid = 152 * 6;
     int64_t need = (n + 4 * kKeysThreads - 1) / (4 * kKeysThreads);
     if (need < grid) grid = need < 1 ? 1 : need;
-    keys_kernel<B, H><<<(unsigned)grid, kKeysThreads, smem, s>>>(pos, mass, m_eq, n, vec, keys, ws.xm,
+    launch_after(keys_kernel<B, H>, dim3((unsigned)grid), dim3(kKeysThreads), smem, s, pos, mass, m_eq, n, vec, keys, ws.xm,
                                                               ws.hist, passes, shift0, ws.info);
     ++g_launches;
     return cudaGetLastError();

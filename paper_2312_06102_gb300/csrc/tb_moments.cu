@@ -92,6 +92,7 @@ __global__ void __launch_bounds__(kLtThreads, MODE == TB_MOM_FP64 ? 3 : 4)
                      const uint16_t *__restrict__ ml, const uint32_t *__restrict__ leaf_off,
                      const int32_t *__restrict__ pend, int64_t n, float4 *__restrict__ xs,
                      int32_t *long_queue, int32_t *big_queue, DevInfo *info, int64_t wait_limit) {
+    after_previous();
     if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout | kErrInvalid)) return;
     extern __shared__ __align__(128) unsigned char lt_raw[];
     LeafTileSmem &S = *reinterpret_cast<LeafTileSmem *>(lt_raw);
@@ -602,6 +603,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kLmThreads, 5)
     upward_kernel(TreeIn T, MomOut o, PermSrc src, const int32_t *long_queue, DevInfo *info, int d_hi,
                   int d_lo, bool leaves, int64_t wait_limit) {
+    after_previous();
     if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout | kErrInvalid)) return;
     extern __shared__ __align__(128) unsigned char lm_raw[];
     LevelSmem &S = *reinterpret_cast<LevelSmem *>(lm_raw);
@@ -691,10 +693,15 @@ cudaError_t leaves_impl(tb_tree &t, Workspace &ws, const int32_t *start_cell, cu
     const int64_t tiles = (n + kLtTile - 1) / kLtTile;
     const int64_t level_tiles = (n + level_tile_size() - 1) / level_tile_size();
     const uint32_t *leaf_off = ws.level_cnt + (int64_t)kLevels * level_tiles;
-    leaf_tile_kernel<MODE><<<(unsigned)tiles, kLtThreads, leaf_tile_smem(), s>>>(
-        o, t.leaf_cell, start_cell, t.perm, ws.xm, ws.ml, leaf_off, t.pend, n,
-        t.pos_sorted ? reinterpret_cast<float4 *>(t.pos_sorted) : nullptr, long_queue(ws, n), ws.big_leaf,
-        ws.info, g_wait_limit);
+    float4 *xs = t.pos_sorted ? reinterpret_cast<float4 *>(t.pos_sorted) : nullptr;
+    if (start_cell)   // batched: one chain with the build
+        launch_after(leaf_tile_kernel<MODE>, dim3((unsigned)tiles), dim3(kLtThreads), leaf_tile_smem(), s, o,
+                     t.leaf_cell, start_cell, t.perm, ws.xm, ws.ml, leaf_off, t.pend, n, xs,
+                     long_queue(ws, n), ws.big_leaf, ws.info, g_wait_limit);
+    else
+        leaf_tile_kernel<MODE><<<(unsigned)tiles, kLtThreads, leaf_tile_smem(), s>>>(
+            o, t.leaf_cell, start_cell, t.perm, ws.xm, ws.ml, leaf_off, t.pend, n, xs, long_queue(ws, n),
+            ws.big_leaf, ws.info, g_wait_limit);
     ++g_launches;
     return cudaGetLastError();
 }
@@ -783,8 +790,7 @@ static cudaError_t batched_leaves_impl(tb_tree &t, Workspace &ws, const int32_t 
     if (e != cudaSuccess) return e;
     TreeIn T{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
     MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
-    upward_kernel<MODE><<<152, kLmThreads, sizeof(LevelSmem), s>>>(
-        T, o, PermSrc{ws.xm, t.perm}, long_queue(ws, t.n_particles), ws.info, -1, -1, true, g_wait_limit);
+    launch_after(upward_kernel<MODE>, dim3(152), dim3(kLmThreads), sizeof(LevelSmem), s, T, o, PermSrc{ws.xm, t.perm}, long_queue(ws, t.n_particles), ws.info, -1, -1, true, g_wait_limit);
     ++g_launches;
     return cudaGetLastError();
 }

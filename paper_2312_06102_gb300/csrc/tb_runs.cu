@@ -31,6 +31,7 @@ constexpr int kRunThreads = 256;
 __global__ void __launch_bounds__(kRunThreads)
     run_sort_kernel(uint64_t *__restrict__ keys, int32_t *__restrict__ vals, int64_t n, int shift0,
                     RunBuffers rb, DevInfo *info) {
+    after_previous();
     __shared__ RunSmem sm;
     const int64_t s = (int64_t)blockIdx.x * kRunTile;
     const bool desc = run_tile<kRunThreads>(keys, vals, 0, s, n, shift0, sm, [&](int64_t a) {
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(kRunThreads)
 __global__ void __launch_bounds__(kCtaThreads, 1)
     long_run_kernel(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t *alt_v, int64_t n,
                     int shift0, RunBuffers rb, DevInfo *info) {
+    after_previous();
     extern __shared__ __align__(16) unsigned char raw[];
     CtaSortShared &sm = *reinterpret_cast<CtaSortShared *>(raw);
     __shared__ uint32_t s_q;
@@ -69,11 +71,11 @@ cudaError_t launch_runs(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t 
                              (int)sizeof(CtaSortShared));
     }
     const int64_t tiles = (n + kRunTile - 1) / kRunTile;
-    run_sort_kernel<<<(unsigned)tiles, kRunThreads, 0, s>>>(keys, vals, n, shift0, rb, ws.info);
+    launch_after(run_sort_kernel, dim3((unsigned)tiles), dim3(kRunThreads), 0, s, keys, vals, n, shift0, rb, ws.info);
     ++g_launches;
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    long_run_kernel<<<152, kCtaThreads, sizeof(CtaSortShared), s>>>(keys, vals, alt_k, alt_v, n, shift0,
+    launch_after(long_run_kernel, dim3(152), dim3(kCtaThreads), sizeof(CtaSortShared), s, keys, vals, alt_k, alt_v, n, shift0,
                                                                    rb, ws.info);
     ++g_launches;
     return cudaGetLastError();

@@ -107,6 +107,7 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     small_sort_kernel(const float *__restrict__ pos, const float *__restrict__ mass, float m_eq, int n,
                       uint64_t *pkey, int32_t *perm, uint64_t *alt_k, int32_t *alt_v,
                       float4 *__restrict__ xm, RunBuffers rb, DevInfo *info, bool pow2) {
+    after_previous();
     using S = SmallSmem<ITEMS>;
     constexpr int P = S::P;
     extern __shared__ __align__(16) unsigned char sm_raw[];

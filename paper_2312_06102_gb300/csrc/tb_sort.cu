@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 256 ? (ITEMS <= 8 ? 4 : 2
                     uint64_t *__restrict__ keys_out, int32_t *__restrict__ vals_out, int64_t n,
                     int pass, int shift0, const uint32_t *__restrict__ digit_off, uint64_t *lookback,
                     DevInfo *info, int64_t spin_limit) {
+    after_previous();
     using S = SortSmem<RADIX_BITS, THREADS, ITEMS>;
     constexpr int RADIX = S::RADIX;
     constexpr int WARPS = S::WARPS;
@@ -464,6 +465,7 @@ __global__ void __launch_bounds__(T, T == 256 && ITEMS > 18 ? 3 : 1024 / T)
                          uint64_t *__restrict__ keys_out, int32_t *__restrict__ vals_out, int64_t n,
                          int pass, int shift0, const uint32_t *__restrict__ digit_off,
                          uint64_t *lookback, DevInfo *info, int64_t spin_limit) {
+    after_previous();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using S = Sort8Smem<T, ITEMS>;
     S &sm = *reinterpret_cast<S *>(smem_raw);
@@ -506,7 +508,7 @@ cudaError_t run_passes(uint64_t *ka, uint64_t *kb, int32_t *pa, int32_t *pb, int
     int32_t *vsrc = pa, *vdst = pb;
     const int64_t spin = g_wait_limit;
     for (int p = 0; p < plan.passes; ++p) {
-        (p == 0 ? first : next)<<<(unsigned)tiles, T, smem, s>>>(
+        launch_after(p == 0 ? first : next, dim3((unsigned)tiles), dim3(T), smem, s, 
             src, p == 0 ? nullptr : vsrc, dst, vdst, n, p, plan.shift0, ws.hist + p * (1 << B), ws.lookback,
             ws.info, spin);
         ++g_launches;

@@ -242,6 +242,7 @@ __global__ void walk_pack_kernel(const float *__restrict__ mass, const float *__
                                  const int32_t *__restrict__ pend, const int32_t *__restrict__ child_first,
                                  const int32_t *__restrict__ child_end, int64_t n_cells,
                                  float4 *__restrict__ rec) {
+    after_previous();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n_cells; c += stride) {
         const float *q = quad + 6 * c;
@@ -259,6 +260,7 @@ __global__ void walk_pack_kernel(const float *__restrict__ mass, const float *__
 __global__ void walk_groups_kernel(const int32_t *__restrict__ parent, const int32_t *__restrict__ child_first,
                                    const int32_t *__restrict__ pfirst, const int32_t *__restrict__ pend,
                                    int64_t n_cells, int n_group, int32_t *groups, uint32_t *ctr) {
+    after_previous();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n_cells; c += stride) {
         const int64_t cnt = (int64_t)pend[c] - pfirst[c];
@@ -273,6 +275,7 @@ template <bool QUAD, bool COUNT>
 __global__ void __launch_bounds__(kWalkThreads, kWalkPerSm)
     walk_kernel(WalkTree T, const int32_t *__restrict__ groups, uint32_t *ctr, int32_t *stacks,
                 float theta, float eps2, float *__restrict__ acc_out, DevInfo *info) {
+    after_previous();
     if (info->status & (kErrOverflow | kErrNonFinite)) return;
     __shared__ WarpLists lists[kWalkWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -490,7 +493,7 @@ cudaError_t launch_walk(const tb_tree &t, Workspace &ws, float theta, float eps,
                                                       t.n_cells, n_group, groups, ctr);
     ++g_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    walk_pack_kernel<<<(unsigned)grid, 256, 0, s>>>(t.mass, t.com, t.com_lo, t.quad, t.level, t.pfirst,
+    launch_after(walk_pack_kernel, dim3((unsigned)grid), dim3(256), 0, s, t.mass, t.com, t.com_lo, t.quad, t.level, t.pfirst,
                                                     t.pend, t.child_first, t.child_end, t.n_cells,
                                                     rec);
     ++g_launches;
@@ -501,7 +504,7 @@ cudaError_t launch_walk(const tb_tree &t, Workspace &ws, float theta, float eps,
     // take them
     auto kern = use_quad ? (ws.profile ? walk_kernel<true, true> : walk_kernel<true, false>)
                          : (ws.profile ? walk_kernel<false, true> : walk_kernel<false, false>);
-    kern<<<kWalkBlocks, kWalkThreads, 0, s>>>(T, groups, ctr, stacks, theta, eps * eps, acc, ws.info);
+    launch_after(kern, dim3(kWalkBlocks), dim3(kWalkThreads), 0, s, T, groups, ctr, stacks, theta, eps * eps, acc, ws.info);
     ++g_launches;
     return cudaGetLastError();
 }
