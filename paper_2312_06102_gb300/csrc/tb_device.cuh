@@ -88,6 +88,68 @@ __device__ __forceinline__ uint64_t hilbert_key(uint32_t x, uint32_t y, uint32_t
     return morton_key(x ^ t, y ^ t, z ^ t);
 }
 
+// The same key from the Morton key by a table of two levels a step.  Going
+// down, the transform so far is a permutation of the axes and an inversion of
+// each (48 states: which axis feeds x, y and z, and three flips; the parity
+// correction of hilbert_key inverts a digit's three bits where the number of
+// flips is odd).  hilbert_level is one level, its definition.
+constexpr int kHilbertStates = 48;
+constexpr int kHilbertTab = kHilbertStates * 64;   // entries: digits (6 bits) | next state << 6
+
+__device__ __forceinline__ uint32_t hilbert_level(uint32_t &state, uint32_t digit) {
+    const uint32_t perm = state >> 3;
+    uint32_t a[3], f[3] = {state & 1u, (state >> 1) & 1u, (state >> 2) & 1u};
+    a[0] = perm >> 1;                                  // the axis that feeds x, ...
+    const uint32_t lo = a[0] == 0 ? 1u : 0u, hi = a[0] == 2 ? 1u : 2u;
+    a[1] = perm & 1u ? hi : lo;
+    a[2] = perm & 1u ? lo : hi;
+    uint32_t v[3];
+    for (int i = 0; i < 3; ++i) v[i] = ((digit >> (2 - a[i])) & 1u) ^ f[i];
+    const uint32_t odd = f[0] ^ f[1] ^ f[2];
+    const uint32_t g0 = v[0], g1 = v[1] ^ v[0], g2 = v[2] ^ v[1] ^ v[0];
+    const uint32_t out = ((g0 ^ odd) << 2) | ((g1 ^ odd) << 1) | (g2 ^ odd);
+    f[0] ^= v[0];
+    for (int i = 1; i < 3; ++i) {
+        if (v[i]) {
+            f[0] ^= 1u;
+        } else {
+            const uint32_t t = a[0], u = f[0];
+            a[0] = a[i];
+            a[i] = t;
+            f[0] = f[i];
+            f[i] = u;
+        }
+    }
+    state = ((2 * a[0] + (a[1] > a[2] ? 1u : 0u)) << 3) | f[0] | (f[1] << 1) | (f[2] << 2);
+    return out;
+}
+
+__device__ __forceinline__ void hilbert_table(uint16_t *tab) {
+    for (int e = threadIdx.x; e < kHilbertTab; e += blockDim.x) {
+        uint32_t st = e >> 6;
+        const uint32_t hi = hilbert_level(st, (e >> 3) & 7), lo = hilbert_level(st, e & 7);
+        tab[e] = (uint16_t)((hi << 3) | lo | (st << 6));
+    }
+}
+
+// 11 table steps in place of 20 dependent levels of a dozen operations.
+__device__ __forceinline__ uint64_t hilbert_of_morton(uint64_t m, const uint16_t *tab) {
+    uint32_t base = 0;                                 // state * 64
+    uint32_t out[3] = {0, 0, 0};                       // levels 20 .. 11, 10 .. 1, 0
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t in = (uint32_t)(m >> (33 - 30 * h)) & 0x3fffffffu;
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            const uint32_t v = tab[base + ((in >> (24 - 6 * i)) & 63u)];
+            out[h] = (out[h] << 6) | (v & 63u);
+            base = v & ~63u;
+        }
+    }
+    out[2] = (tab[base + (((uint32_t)m & 7u) << 3)] >> 3) & 7u;
+    return (1ull << 63) | ((uint64_t)out[0] << 33) | ((uint64_t)out[1] << 3) | out[2];
+}
+
 // Exact error-free sum a + b = s + e (Knuth's TwoSum, no branch).
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = __fadd_rn(a, b);

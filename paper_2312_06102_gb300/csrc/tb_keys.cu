@@ -154,7 +154,9 @@ __global__ void __launch_bounds__(kKeysThreads, 6) keys_kernel(const float *__re
                                                             DevInfo *info) {
     after_previous();
     constexpr int RADIX = 1 << RADIX_BITS;
-    extern __shared__ uint32_t s_hist[];   // [passes][RADIX]
+    extern __shared__ uint32_t s_hist[];   // [passes][RADIX], then the Hilbert table
+    uint16_t *tab = reinterpret_cast<uint16_t *>(s_hist + passes * RADIX);
+    if constexpr (HILBERT) hilbert_table(tab);
     for (int i = threadIdx.x; i < passes * RADIX; i += blockDim.x) s_hist[i] = 0;
     __shared__ float s_lo[3];
     __shared__ float s_shi, s_slo;
@@ -182,7 +184,8 @@ __global__ void __launch_bounds__(kKeysThreads, 6) keys_kernel(const float *__re
         const uint32_t qx = quantise(x, lx, shi, slo, sc, exact, f32),
                        qy = quantise(y, ly, shi, slo, sc, exact, f32),
                        qz = quantise(z, lz, shi, slo, sc, exact, f32);
-        return HILBERT ? hilbert_key(qx, qy, qz) : morton_key(qx, qy, qz);
+        const uint64_t m = morton_key(qx, qy, qz);
+        return HILBERT ? hilbert_of_morton(m, tab) : m;
     };
 
     const int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -278,7 +281,7 @@ static cudaError_t keys_impl(const float *pos, const float *mass, int64_t n, uin
                      (reinterpret_cast<uintptr_t>(mass) & 15u) == 0 &&
                      (reinterpret_cast<uintptr_t>(keys) & 15u) == 0;
     const float m_eq = (float)(1.0 / (double)(n > 0 ? n : 1));
-    size_t smem = sizeof(uint32_t) * passes * (1 << B);
+    size_t smem = sizeof(uint32_t) * passes * (1 << B) + (H ? sizeof(uint16_t) * kHilbertTab : 0);
     static std::atomic<uint64_t> attr_done{0};
     if (first_on_device(attr_done)) {
         cudaFuncSetAttribute(keys_kernel<B, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
