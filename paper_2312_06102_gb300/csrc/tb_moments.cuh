@@ -218,6 +218,18 @@ __device__ void write_cell_f32(const MomOut &o, int64_t c, float M, const float 
     }
 }
 
+// A cell written to the tree and to a copy of its level (cells from `base` on)
+// that the next level is combined from.
+struct MomBoth {
+    MomOut tree, copy;
+    int64_t base;
+};
+__device__ void write_cell_f32(const MomBoth &o, int64_t c, float M, const float ch[3],
+                               const float cl[3], const float Q[6], const float bb[6]) {
+    write_cell_f32(o.tree, c, M, ch, cl, Q, bb);
+    write_cell_f32(o.copy, c - o.base, M, ch, cl, Q, bb);
+}
+
 __device__ void write_cell_f64(const MomOut &o, int64_t c, double M, const double com[3],
                                const double Q[6], const float bb[6], bool has64) {
     float ch[3], cl[3], q[6];
@@ -271,7 +283,8 @@ __device__ void finish_c(const MomOut &o, int64_t c, const AccC &A, const float 
     write_cell_f32(o, c, Mh + Ml, ch, cl, Q, bb);
 }
 
-__device__ void finish_s(const MomOut &o, int64_t c, const AccS &A, const float ref[3],
+template <class Out>
+__device__ void finish_s(const Out &o, int64_t c, const AccS &A, const float ref[3],
                          const float bb[6]) {
     float Mh, Ml;
     fast_two_sum(A.M, A.Mc, Mh, Ml);
@@ -570,7 +583,7 @@ __device__ __noinline__ void combine_f64(MomOut o, int64_t p, int32_t c0, int32_
         write_cell_f64(o, p, M, com, Q, bb, MODE == TB_MOM_FP64);
 }
 
-// FP64 mode: parent p (none when p < 0) from its children by four lanes,
+// FP64 mode: parent p (none when p < 0) from its children [c0, c1) by four lanes,
 // lane j taking children j and j + 4; the lanes' sums meet in two shuffle
 // rounds.  The same two passes as combine_f64 -- mass and first moment about
 // the first child's centre, then second moments about the centre of mass --
@@ -578,15 +591,10 @@ __device__ __noinline__ void combine_f64(MomOut o, int64_t p, int32_t c0, int32_
 // what a level of few cells costs (20 us a level with one lane per parent).
 // All lanes of the warp call it.
 template <class Src>
-__device__ __forceinline__ void combine_f64_quad(const TreeIn &T, const MomOut &o, int64_t p,
+__device__ __forceinline__ void combine_f64_quad(const MomOut &o, int64_t p, int32_t c0, int32_t c1,
                                                  const Src &src) {
     constexpr unsigned kAll = 0xffffffffu;
     const int j = threadIdx.x & 3;
-    int32_t c0 = 0, c1 = 0;
-    if (p >= 0) {
-        c0 = T.child_first[p];
-        c1 = T.child_end[p];
-    }
     double ref[3] = {0.0, 0.0, 0.0}, m[2] = {0.0, 0.0}, d[2][3];
     if (p >= 0)
         for (int a = 0; a < 3; ++a) ref[a] = o.com64[3 * (int64_t)c0 + a];
@@ -650,9 +658,9 @@ __device__ __forceinline__ void combine_f64_quad(const TreeIn &T, const MomOut &
 // Parent p from its children, whose FP32 moments come from `src` (the tree's
 // arrays, or a copy staged in shared memory); the FP64 route reads the tree's
 // arrays.
-template <int MODE, class Src>
-__device__ void combine_children(const TreeIn &T, const MomOut &o, int64_t p, const Src &src) {
-    const int32_t c0 = T.child_first[p], c1 = T.child_end[p];
+template <int MODE, class Src, class Out>
+__device__ __forceinline__ void combine_range(const TreeIn &T, const Out &o, int64_t p, int32_t c0,
+                                              int32_t c1, const Src &src) {
     auto qrow = [&](int64_t c, float v[6]) {
         const float2 x = src.q2(c, 0), y = src.q2(c, 1), z = src.q2(c, 2);
         v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y; v[4] = z.x; v[5] = z.y;
@@ -722,9 +730,8 @@ __device__ void combine_children(const TreeIn &T, const MomOut &o, int64_t p, co
                 }
             }
             finish_s(o, p, A, ref, bb);
-            return;
         }
-    }
+    } else {
     for (int32_t c = c0 + 1; c < c1; ++c) {
         float cb[6];
         brow(c, cb);
@@ -757,6 +764,12 @@ __device__ void combine_children(const TreeIn &T, const MomOut &o, int64_t p, co
         for (int a = 0; a < 3; ++a) { ch[a] = ref[a] + r[a]; cl[a] = 0.f; }
         write_cell_f32(o, p, M, ch, cl, Q, bb);
     }
+    }
+}
+
+template <int MODE, class Src>
+__device__ void combine_children(const TreeIn &T, const MomOut &o, int64_t p, const Src &src) {
+    combine_range<MODE>(T, o, p, T.child_first[p], T.child_end[p], src);
 }
 
 
