@@ -34,9 +34,15 @@ namespace tb {
 
 namespace {
 
-// front / emit blocks: T threads, one particle per thread per cell tile;
-// T = 512 (two sets per SM at a time) or 1024
+// front blocks: T threads per set, 1024 / T sets per SM at a time.  T = 512
+// unless the sets are few and large, where a set's own time counts (300 sets
+// of 4,000 to 65,536 particles: 1.28 ms with 1024 threads, 1.69 with 512; 600 of
+// 1,000 to 30,000: 771 and 890 us; 4,096 of 256 to 65,536: 5.85 and 5.16 ms), or many
+// and small, where the number of sets at a time does (1,000 sets of 32 to 700: 121
+// us with 256 threads, 163 with 512).
 constexpr int kBDefaultThreads = 512;
+inline bool batch_few_large(int32_t S, int64_t n) { return S <= 608 && n >= int64_t(S) * 4096; }
+inline bool batch_many_small(int32_t S, int64_t n) { return S > 304 && n <= int64_t(S) * 512; }
 constexpr int kBRadixBits = kCtaRadixBits;
 constexpr int kBRadix = kCtaRadix;
 // the block sort orders the upper 40 key bits in five passes; the runs of
@@ -670,24 +676,30 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
                 t.leaf_cell, start_cell};
     // the emission keeps 1024-thread tiles whatever the front's block size
     // (two blocks per SM at 32 registers): measured faster than 512 (0.96
-    // against 1.10 ms on the 4,096-set workload)
-    launch_after(batch_emit_kernel<1024>, dim3(fit(2)), dim3(1024), 0, s, A, out);
+    // against 1.10 ms on the 4,096-set workload); many small sets take small
+    // blocks, and so do their parents
+    const bool small = batch_many_small(S, t.n_particles);
+    if (small) launch_after(batch_emit_kernel<256>, dim3(fit(8)), dim3(256), 0, s, A, out);
+    else launch_after(batch_emit_kernel<1024>, dim3(fit(2)), dim3(1024), 0, s, A, out);
     ++g_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     mark(ws, "batch_emit", s);
     if ((e = launch_batched_leaves(t, ws, mode, start_cell, s)) != cudaSuccess) return e;
     TreeIn Tr{t.child_first, t.child_end, t.pfirst, t.pend, ws.big_leaf, t.parent};
     MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
-    const int grid_mom = fit(3);
+    // (4,096 sets: 5.06 ms with 128 threads, 5.19 with 256; 1,000 sets of 1,000 to
+    // 65,536: 2.14 and 2.00)
+    const int up_threads = small ? 64 : (S > 1824 ? kBMomThreads / 2 : kBMomThreads);
+    const int grid_mom = fit(3 * kBMomThreads / up_threads);
     switch (mode) {
         case TB_MOM_FP32_COMP:
-            launch_after(batch_up_kernel<TB_MOM_FP32_COMP>, dim3(grid_mom), dim3(kBMomThreads), 0, s, A, Tr, o);
+            launch_after(batch_up_kernel<TB_MOM_FP32_COMP>, dim3(grid_mom), dim3(up_threads), 0, s, A, Tr, o);
             break;
         case TB_MOM_FP32_PLAIN:
-            launch_after(batch_up_kernel<TB_MOM_FP32_PLAIN>, dim3(grid_mom), dim3(kBMomThreads), 0, s, A, Tr, o);
+            launch_after(batch_up_kernel<TB_MOM_FP32_PLAIN>, dim3(grid_mom), dim3(up_threads), 0, s, A, Tr, o);
             break;
         default:
-            launch_after(batch_up_kernel<TB_MOM_FP64>, dim3(grid_mom), dim3(kBMomThreads), 0, s, A, Tr, o);
+            launch_after(batch_up_kernel<TB_MOM_FP64>, dim3(grid_mom), dim3(up_threads), 0, s, A, Tr, o);
             break;
     }
     ++g_launches;
@@ -763,7 +775,10 @@ cudaError_t launch_batched(const float *pos, const float *mass, const int64_t *o
     BatchArgs A{pos, mass, off, ws.set_order, S, ncrit, t.pkey, t.perm, ws.keys_alt,
                 ws.perm_alt, ws.xm, ws.xs, ws.ml, ws.set_cnt, t.set_cell_offset, ws.set_leaf_off,
                 t.set_root, ws.set_ctr, ws.info, ws.root_pow2 ? 1 : 0};
-    switch (threads ? threads : kBDefaultThreads) {
+    const int64_t n = t.n_particles;
+    switch (threads ? threads
+                    : (batch_few_large(S, n) ? 1024 : (batch_many_small(S, n) ? 256 : kBDefaultThreads))) {
+        case 256: return launch_batched_t<256>(A, S, ncrit, t, ws, cell_cap, phase, mode, s);
         case 512: return launch_batched_t<512>(A, S, ncrit, t, ws, cell_cap, phase, mode, s);
         case 1024: return launch_batched_t<1024>(A, S, ncrit, t, ws, cell_cap, phase, mode, s);
         default: return cudaErrorInvalidValue;

@@ -195,3 +195,20 @@ def test_batched_empty():
     t = m.build_batched(torch.zeros((0, 3), dtype=torch.float32, device="cuda"), None,
                         torch.zeros(4, dtype=torch.int64, device="cuda"))
     assert t.n_cells == 0
+
+
+@pytest.mark.parametrize("sizes", ["many small", "few large"])
+def test_batched_default_block_sizes(sizes):
+    """The default block size follows the sets: 256 threads for more than 304
+    sets of at most 512 particles on average, 1024 for at most 608 of at least
+    4096.  Structure and moments as with a named size, and the oracle's."""
+    rng = np.random.default_rng(8)
+    n = rng.integers(0, 900, 400) if sizes == "many small" else rng.integers(3000, 9000, 6)
+    assert (n.mean() <= 512) if sizes == "many small" else (n.mean() >= 4096)
+    pos, mass, offsets = _sets([int(v) for v in n], 21)
+    a, *_ = _run(pos, mass, offsets)
+    b, *_ = _run(pos, mass, offsets, threads=512)
+    for k in ("pkey", "perm", "ckey", "level", "parent", "child_first", "child_end", "pfirst",
+              "pend", "mass", "com", "com_lo", "quad", "aabb"):
+        assert np.array_equal(to_np(getattr(a, k)), to_np(getattr(b, k))), k
+    _check_sets(a, pos, mass, offsets, 16, sets=range(0, len(n), 37 if len(n) > 50 else 1))
