@@ -96,7 +96,7 @@ typedef struct {
                                 order, Sec. 2.3 step 3) */
     int32_t radix_bits;      /* 0 = tuned default; else 8..11 (sort digit width);
                                 tb_build only.  With all three sort fields 0 a
-                                set of up to 65,536 particles takes one launch for
+                                set of up to 32,768 particles takes one launch for
                                 root, keys and sort (unless tb_profile is on) */
     int32_t sort_threads;    /* 0 = tuned default; else threads per sort tile; tb_build only */
     int32_t sort_items;      /* 0 = tuned default; else keys per thread of a sort tile

@@ -253,7 +253,7 @@ def _check(code, what):
 KEYS_MORTON, KEYS_HILBERT = 0, 1
 # sets up to this size are sorted in one launch when no variant is named: a
 # tuned variant of the radix passes would only slow them down
-ONE_LAUNCH_SORT_MAX = 65536
+ONE_LAUNCH_SORT_MAX = 32768
 
 
 def build(pos: torch.Tensor, mass: torch.Tensor | None = None, n_crit: int = 16,

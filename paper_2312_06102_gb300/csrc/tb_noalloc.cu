@@ -82,7 +82,7 @@ cudaError_t scratch_address(unsigned char **out) {
 }
 
 // Every kernel a call can reach, loaded by the first call that sorts, whatever
-// its size: sets of up to 65,536 particles and larger ones take different
+// its size: sets of up to 32,768 particles and larger ones take different
 // kernels, and a later call of the other kind must not load (allocate).
 cudaError_t load_kernels_once() {
     static std::atomic<uint64_t> done{0};

@@ -2,9 +2,10 @@
 // in one launch (Sec. 2.2; Sec. 2.3 steps 1 and 2).
 //
 // The launches of the general path (root, keys, five radix passes, two run
-// steps) cost a small set 4 to 12 us each, nearly all of it latency: 87 us at
-// 3,001 particles, 24 here, and 94 against 58 at 65,536; from 80,000 on the
-// many SMs of the general passes win.  Here one cluster of up to 16
+// steps) cost a small set 4 to 8 us each, nearly all of it latency.  tb_build
+// with those and with this launch, us: 59 and 37 at 3,001 particles, 64 and 51 at
+// 20,000, 63 and 57 at 32,768; from 50,000 on (64 and 70, with 4096 positions a
+// block) the many SMs of the general passes win.  Here one cluster of up to 16
 // blocks takes the whole set.  Block r owns positions [r P, (r + 1) P) of the
 // current order, in registers while a pass ranks them:
 //   1. particles to registers (records written out), bounding box by shuffles
@@ -17,9 +18,7 @@
 //      memory and stores them, runs of consecutive addresses, to the places'
 //      owners' shared memory (the last pass: to global memory); a cluster
 //      barrier.  A pass reads its pairs into registers before its first
-//      barrier and stores after it, so the owners need one buffer.  Blocks of
-//      4096 positions go through global buffers, which L2 holds, instead:
-//      65,536 particles 58 us against 61, 3,001 26 against 24;
+//      barrier and stores after it, so the owners need one buffer;
 //   3. runs of equal upper bits ordered in place by the low bits
 //      (tb_runs.cuh), tiles shared out over the blocks, long runs after.
 // Barriers are the cluster's own (barrier.cluster); nothing spins.
@@ -37,18 +36,15 @@ constexpr int kSmBits = 8;
 constexpr int kSmRadix = 1 << kSmBits;
 constexpr int kSmPasses = 5;
 constexpr int kSmShift0 = 63 - kSmPasses * kSmBits;
-static_assert(kSmPasses & 1, "an odd number of passes ends in pkey");
-constexpr int kSmMaxItems = 4;
-constexpr int kSmLong = 128;      // long runs a block can queue (16 a tile, at most 4 tiles)
+constexpr int kSmMaxItems = 2;
+constexpr int kSmLong = 64;       // long runs a block can queue (16 a tile, at most 2 tiles)
 
 template <int ITEMS>
 struct SmallSmem {
     static constexpr int P = kSmThreads * ITEMS;   // positions per block
-    static constexpr bool kRemote = ITEMS < 4;     // passes store to the owners' shared memory
-    static constexpr int Q = kRemote ? P : 1;
-    uint64_t key[Q];                               // this block's part of the current order
+    uint64_t key[P];                               // this block's part of the current order
     uint64_t skey[P];                              // its pairs ordered by the pass's digit
-    int32_t val[Q];
+    int32_t val[P];
     int32_t sval[P];
     uint32_t hist[kSmWarps][kSmRadix + 1];
     uint32_t cnt[2][kSmRadix];                     // this block's digit counts, by pass parity
@@ -195,22 +191,12 @@ __global__ void __launch_bounds__(kSmThreads, 1)
     const unsigned lt = lanemask_lt();
     for (int p = 0; p < kSmPasses; ++p) {
         const int shift = kSmShift0 + p * kSmBits;
-        // buffers alternate; the last pass (even) writes to pkey and perm
-        uint64_t *out_k = (p & 1) ? alt_k : pkey;
-        int32_t *out_v = (p & 1) ? alt_v : perm;
         if (p > 0) {
-            const uint64_t *in_k = (p & 1) ? pkey : alt_k;
-            const int32_t *in_v = (p & 1) ? perm : alt_v;
 #pragma unroll
             for (int i = 0; i < ITEMS; ++i) {
                 const int e = wbase + i * 32 + lane;
-                if constexpr (S::kRemote) {
-                    key[i] = sm.key[e];
-                    val[i] = sm.val[e];
-                } else if (e < mine) {
-                    key[i] = __ldcg(reinterpret_cast<const unsigned long long *>(in_k) + first + e);
-                    val[i] = __ldcg(in_v + first + e);
-                }
+                key[i] = sm.key[e];
+                val[i] = sm.val[e];
             }
         }
         for (int i = threadIdx.x; i < kSmWarps * (kSmRadix + 1); i += kSmThreads) (&sm.hist[0][0])[i] = 0;
@@ -273,8 +259,8 @@ __global__ void __launch_bounds__(kSmThreads, 1)
                 tot += __shfl_xor_sync(0xffffffffu, tot, off);
                 pre += __shfl_xor_sync(0xffffffffu, pre, off);
             }
-            // prefixes over the digits of all blocks' counts (at most 2^16, low
-            // 18 bits) and of this block's (at most 2^12, high 14 bits) at once
+            // prefixes over the digits of all blocks' counts (at most 2^15, low
+            // 18 bits) and of this block's (at most 2^11, high 14 bits) at once
             const uint32_t own = sm.cnt[p & 1][dg], both = tot | (own << 18);
             uint32_t y = both;   // inclusive over the warp's eight digits
 #pragma unroll
@@ -307,13 +293,13 @@ __global__ void __launch_bounds__(kSmThreads, 1)
             const uint64_t k = sm.skey[j];
             const uint32_t d = (uint32_t)(k >> shift) & (kSmRadix - 1);
             const uint32_t to = sm.base[d] + (uint32_t)j;
-            if (S::kRemote && p + 1 < kSmPasses) {
+            if (p + 1 < kSmPasses) {
                 const uint32_t q = to / P, e = to % P;
-                st_remote(remote(&sm.key[e % S::Q], q), k);
-                st_remote(remote(&sm.val[e % S::Q], q), sm.sval[j]);
+                st_remote(remote(&sm.key[e], q), k);
+                st_remote(remote(&sm.val[e], q), sm.sval[j]);
             } else {
-                out_k[to] = k;
-                out_v[to] = sm.sval[j];
+                pkey[to] = k;
+                perm[to] = sm.sval[j];
             }
         }
         cluster_sync();
@@ -385,7 +371,6 @@ cudaError_t dispatch_small(const float *pos, const float *mass, int64_t n, int m
                  : launch_small_t<I, false>(pos, mass, (int)n, pkey, perm, alt_k, alt_v, ws, ask, clusters, s);
     TB_SMALL(1)
     TB_SMALL(2)
-    TB_SMALL(4)
 #undef TB_SMALL
     return cudaErrorInvalidValue;
 }
@@ -417,8 +402,7 @@ int64_t small_sort_max() { return (int64_t)small_blocks() * kSmThreads * kSmMaxI
 
 cudaError_t load_small_kernels() {
     cudaError_t e = load_kernel(small_sort_kernel<1, false>);
-    if (e == cudaSuccess) e = load_kernel(small_sort_kernel<2, false>);
-    return e == cudaSuccess ? load_kernel(small_sort_kernel<4, false>) : e;
+    return e == cudaSuccess ? load_kernel(small_sort_kernel<2, false>) : e;
 }
 
 // Root cube (with the build record's start), records, sorted keys and
