@@ -61,22 +61,89 @@ __global__ void __launch_bounds__(kLvThreads, 2)
     if (threadIdx.x < kLevelFields) tile_cnt[(int64_t)threadIdx.x * n_tiles + t] = tot[threadIdx.x];
 }
 
+// One thread: the level offsets, counts and depth from the field totals; the
+// record's counters cleared for what follows.
+__device__ __forceinline__ void finish_levels(DevInfo *info, const uint32_t *tot, int64_t cell_cap) {
+    int64_t off = 0;
+    int dmax = 0;
+    for (int d = 0; d < kLevels; ++d) {
+        uint32_t c = tot[d];
+        info->level_offset[d] = off;
+        off += c;
+        if (c) dmax = d;
+    }
+    info->level_offset[kLevels] = off;
+    info->n_cells = off;
+    info->n_leaves = tot[kLevels];
+    info->max_depth = dmax;
+    if (cell_cap > 0 && off > cell_cap) info->status |= kErrOverflow;
+    info->misc_ctr[1] = 0;
+    // the moments' leaf queues, and the barrier count of their upward pass
+    for (int i : {2, 5, 7}) info->misc_ctr[i] = 0;
+}
+
 // The same counts, four consecutive particles per thread, for n_crit in
 // [kLcMinN, kLcMaxN] (count_tile4); a block of 256 threads takes one count tile.
+// With at most kLcScanTiles tiles the last block to finish also forms the
+// prefixes over the tiles, a warp per field, and saves the scan's launch (5 of
+// 65 us at 3,001 particles).
 constexpr int kLcThreads = kLvTile / 4;
+constexpr int kLcScanTiles = 256;
+
+__device__ __forceinline__ void scan_few_tiles(uint32_t *tile_cnt, int n_tiles, DevInfo *info,
+                                               int64_t cell_cap) {
+    constexpr int PER = kLcScanTiles / 32;
+    __shared__ uint32_t s_tot[kLevelFields];
+    const int lane = threadIdx.x & 31;
+    for (int f = threadIdx.x >> 5; f < kLevelFields; f += kLcThreads / 32) {
+        uint32_t *row = tile_cnt + (int64_t)f * n_tiles;
+        uint32_t v[PER], sum = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int t = lane * PER + j;
+            v[j] = t < n_tiles ? __ldcg(row + t) : 0u;
+            sum += v[j];
+        }
+        uint32_t x = sum;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
+        }
+        if (lane == 31) s_tot[f] = x;
+        x -= sum;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            const int t = lane * PER + j;
+            if (t < n_tiles) row[t] = x;
+            x += v[j];
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) finish_levels(info, s_tot, cell_cap);
+}
 
 __global__ void __launch_bounds__(kLcThreads, 6)
     level_count_fast_kernel(const uint64_t *__restrict__ skeys, int64_t n, int ncrit,
-                            uint32_t *__restrict__ tile_cnt, int64_t n_tiles,
-                            uint16_t *__restrict__ ml) {
+                            uint32_t *tile_cnt, int64_t n_tiles, uint16_t *__restrict__ ml, DevInfo *info,
+                            int64_t cell_cap) {
     after_previous();
     extern __shared__ __align__(16) unsigned char raw[];
     __shared__ StartCounts sc;
+    __shared__ bool s_last;
     for (int x = threadIdx.x; x <= kLevels; x += kLcThreads) sc.m[x] = sc.l[x] = 0;
     const int64_t t = blockIdx.x, s = t * kLvTile;
     count_tile4<kLcThreads>(skeys, 0, n, ncrit, s, min64(n, s + kLvTile), raw, sc, ml);
     __syncthreads();
     if (threadIdx.x < kLevelFields) tile_cnt[(int64_t)threadIdx.x * n_tiles + t] = sc.cells(threadIdx.x);
+    if (n_tiles > kLcScanTiles) return;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&info->misc_ctr[1], 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    scan_few_tiles(tile_cnt, (int)n_tiles, info, cell_cap);
 }
 
 // One block per field: exclusive prefix over tiles (in place); the last block
@@ -155,22 +222,7 @@ __global__ void __launch_bounds__(kScanThreads)
     if (!s_last || threadIdx.x != 0) return;
     __threadfence();
     const uint32_t *tot = tile_cnt + (int64_t)kLevelFields * n_tiles;
-    int64_t off = 0;
-    int dmax = 0;
-    for (int d = 0; d < kLevels; ++d) {
-        uint32_t c = __ldcg(&tot[d]);
-        info->level_offset[d] = off;
-        off += c;
-        if (c) dmax = d;
-    }
-    info->level_offset[kLevels] = off;
-    info->n_cells = off;
-    info->n_leaves = __ldcg(&tot[kLevels]);
-    info->max_depth = dmax;
-    if (cell_cap > 0 && off > cell_cap) info->status |= kErrOverflow;
-    info->misc_ctr[1] = 0;
-    // the moments' leaf queues, and the barrier count of their upward pass
-    for (int i : {2, 5, 7}) info->misc_ctr[i] = 0;
+    finish_levels(info, tot, cell_cap);
 }
 
 // Emission over the leaf starts only, one count tile (1024 particles) per
@@ -377,7 +429,11 @@ cudaError_t launch_levels(const uint64_t *skeys, int64_t n, int ncrit, Workspace
                                  cudaSharedmemCarveoutMaxShared);
         }
         launch_after(level_count_fast_kernel, dim3((unsigned)tiles), dim3(kLcThreads), lc_smem_bytes<kLcThreads>(ncrit), s, 
-            skeys, n, ncrit, ws.level_cnt, tiles, ws.ml);
+            skeys, n, ncrit, ws.level_cnt, tiles, ws.ml, ws.info, ws.cell_cap_request);
+        if (tiles <= kLcScanTiles) {
+            ++g_launches;
+            return cudaGetLastError();
+        }
     } else {
         launch_after(level_count_kernel, dim3((unsigned)tiles), dim3(kLvThreads), smem, s, skeys, n, ncrit, ws.level_cnt,
                                                                      tiles, ws.ml);

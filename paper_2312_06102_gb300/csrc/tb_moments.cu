@@ -519,8 +519,7 @@ __device__ __forceinline__ bool grid_meet(uint32_t *ctr, uint32_t target, bool w
     fence_proxy_async();
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(ctr, 1u);
+        red_release_u32(ctr, 1u);
         if (wait) {
             int64_t it = 0;
             while (ld_acquire_u32(ctr) < target)
@@ -529,7 +528,6 @@ __device__ __forceinline__ bool grid_meet(uint32_t *ctr, uint32_t target, bool w
                     ok = false;
                     break;
                 }
-            __threadfence();
             fence_proxy_async();
         }
     }
@@ -724,11 +722,22 @@ __global__ void __launch_bounds__(kLmThreads, 5)
     }
     __syncthreads();
     const int solo = s_solo;
+    int deepest = d_hi;
+    while (deepest > d_lo && s_off[deepest + 1] == s_off[deepest + 2]) --deepest;
+    bool tail = d_hi > d_lo;   // the deepest levels, while one tile each: block 0 alone as well
     for (int d = d_hi; d >= d_lo; --d) {
         const int64_t off1 = s_off[d + 1], off2 = s_off[d + 2];
         if (off1 == off2) continue;
         const uint32_t act = s_act[d];
         if (blockIdx.x >= act) return;
+        const bool was = tail && d < deepest;
+        tail = tail && d > solo && off2 - off1 <= kLmTile;
+        if (was && !tail && d > solo) {
+            // the first level for all: what block 0 combined is its children
+            met += act;
+            if (!grid_meet(meet, met, true, wait_limit, info)) return;
+        }
+        if (tail && blockIdx.x != 0) continue;
         if (MODE == TB_MOM_FP32_COMP && two && d <= solo && d_lo == 0) {
             solo_levels(T, o, info, &S, s_off, d, phase, wait_limit);
             break;
@@ -736,7 +745,7 @@ __global__ void __launch_bounds__(kLmThreads, 5)
         // smaller tiles where the level would leave blocks idle or give a few
         // of them one tile more
         int tile = kLmTile;
-        if (d > solo)
+        if (d > solo && !tail)
             while (tile > kLmMinTile && off2 - off1 <= (int64_t)act * tile * 2) tile /= 2;
         const int64_t tiles = (off2 - off1 + tile - 1) / tile;
         for (int64_t t = blockIdx.x; t < tiles; t += act) {
@@ -746,7 +755,7 @@ __global__ void __launch_bounds__(kLmThreads, 5)
             __syncthreads();
         }
         if (d == d_lo) break;
-        if (d > solo) {
+        if (d > solo && !tail) {
             met += act;
             if (!grid_meet(meet, met, blockIdx.x < s_act[d - 1], wait_limit, info)) return;
         } else {
