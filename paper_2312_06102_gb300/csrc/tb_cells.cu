@@ -226,60 +226,63 @@ __global__ void __launch_bounds__(kScanThreads)
 }
 
 // Emission over the leaf starts only, one count tile (1024 particles) per
-// block of 256 threads, four blocks per SM.  Only a leaf start (m_k <= L_k)
-// opens or closes cells, one particle in four to seven on the tree
-// workloads, so the block first lists them in order in shared memory
-// (four particles per thread, a block-wide prefix of the counts) and then
-// runs the per-level prefix and the writes over that list, 32 starts per
-// warp: every lane holds a start, and the level masks are built for the
-// list, not for every particle.  The tree's last particle, which closes every
+// block of 256 threads.  Only a leaf start (m_k <= L_k) opens or closes cells,
+// one particle in four to seven on the tree workloads, so each warp first
+// lists the starts of its 128 particles in order and then works on that list,
+// 32 starts at a time: every lane holds a start, and the level masks (a 32 x
+// 32 bit transpose) are built for the list, not for every particle.  The
+// warps meet once, to exchange how many cells of each level they start; what
+// bound the kernel before, with the starts of the whole block in one list,
+// were its seven barriers (2^27 clustered 0.97 ms, now 0.71; 2^24 120 and 88 us).
+// The tree's last particle, which closes every
 // cell that holds it, is handled by its own thread: those are the last cells
 // of their levels.
 constexpr int kEfThreads = 256;
 constexpr int kEfWarps = kEfThreads / 32;
-static_assert(kEfWarps <= 32, "one warp scans the warps' counts");
 constexpr int kEfTile = 4 * kEfThreads;                // four particles per thread
-static_assert(kEfTile % kLvTile == 0 && kEfTile <= 2048, "whole count tiles; offsets fit 11 bits");
-constexpr int kEfChunks = kEfTile / 32;
+constexpr int kEfSpan = kEfTile / kEfWarps;            // particles of a warp
+static_assert(kEfTile == kLvTile && kEfSpan == 128, "a count tile per block, four particles per lane");
 
-__global__ void __launch_bounds__(kEfThreads, 4)
+struct EmitWarp {
+    uint32_t entry[kEfSpan];                            // k - the warp's first | m << 8 | L << 16 | Lprev << 24
+    uint32_t mask[kEfSpan / 32][kLevels];               // level masks of each chunk of 32 starts
+    uint32_t base[kLevels + 2];                         // next cell of each level before the chunk
+};
+
+__global__ void __launch_bounds__(kEfThreads, 6)
     emit_starts_kernel(const uint64_t *__restrict__ skeys, const uint16_t *__restrict__ ml, int64_t n,
                        const uint32_t *__restrict__ tile_off, int64_t n_tiles, DevInfo *info_w,
                        EmitOut out) {
     after_previous();
     const DevInfo *info = info_w;
     if (info->status & (kErrOverflow | kErrNonFinite)) return;
-    __shared__ uint32_t s_entry[kEfTile];               // k - s | m << 11 | L << 16 | Lprev << 21
-    __shared__ uint32_t s_mask[kEfChunks][kLevels];     // level masks of each chunk of 32 starts
-    __shared__ uint32_t s_cpre[kEfChunks][kLevels];     // starts of each level in earlier chunks
-    __shared__ uint32_t s_base[kLevelFields];           // first level-d cell (leaf) of the block
-    __shared__ uint32_t s_wcnt[kEfWarps];
-    __shared__ uint8_t s_Llast[kEfThreads];
-    __shared__ uint32_t s_total;
+    __shared__ EmitWarp s_warp[kEfWarps];
+    __shared__ uint32_t s_cnt[kEfWarps][kLevelFields];  // cells (leaves) each warp starts per level
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t t0 = (int64_t)blockIdx.x * (kEfTile / kLvTile);   // first count tile of the block
-    const int64_t s = (int64_t)blockIdx.x * kEfTile, e = min64(n, s + kEfTile);
-    if (threadIdx.x < kLevelFields)
-        s_base[threadIdx.x] = ((threadIdx.x < kLevels) ? (uint32_t)info->level_offset[threadIdx.x] : 0u) +
-                              tile_off[(int64_t)threadIdx.x * n_tiles + t0];
-    // m and L of four particles per thread
-    const int64_t k0 = s + 4 * (int64_t)threadIdx.x;
+    EmitWarp &W = s_warp[warp];
+    const int64_t s = (int64_t)blockIdx.x * kEfTile + warp * kEfSpan;
+    // where the block's cells of level `lane` (its leaves) start
+    uint32_t base = 0;
+    if (lane < kLevelFields)
+        base = (lane < kLevels ? (uint32_t)info->level_offset[lane] : 0u) +
+               tile_off[(int64_t)lane * n_tiles + blockIdx.x];
+    // m and L of four particles per lane
+    const int64_t k0 = s + 4 * lane;
     uint32_t m[4], L[4];
-    if (k0 + 4 <= e) {
+    if (k0 + 4 <= n) {
         const uint2 v = *reinterpret_cast<const uint2 *>(ml + k0);
         m[0] = v.x & 0xffu; L[0] = (v.x >> 8) & 0xffu; m[1] = (v.x >> 16) & 0xffu; L[1] = v.x >> 24;
         m[2] = v.y & 0xffu; L[2] = (v.y >> 8) & 0xffu; m[3] = (v.y >> 16) & 0xffu; L[3] = v.y >> 24;
     } else {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const uint32_t v = (k0 + j < e) ? (uint32_t)ml[k0 + j] : 255u;
+            const uint32_t v = (k0 + j < n) ? (uint32_t)ml[k0 + j] : 255u;
             m[j] = v & 0xffu;
-            L[j] = (k0 + j < e) ? (v >> 8) : 0u;
+            L[j] = v >> 8;
         }
     }
-    s_Llast[threadIdx.x] = (uint8_t)L[3];
-    uint32_t Lbefore = 0;
-    if (threadIdx.x == 0 && s > 0) Lbefore = (uint32_t)(ml[s - 1] >> 8);
+    uint32_t Lp = __shfl_up_sync(0xffffffffu, L[3], 1);
+    if (lane == 0) Lp = s > 0 && s < n ? (uint32_t)(ml[s - 1] >> 8) : 0u;
     // the tree's last particle closes the cells holding it: the last cell of
     // each level 0 .. L, whose children end where the next level ends
     if (k0 <= n - 1 && n - 1 < k0 + 4) {
@@ -290,54 +293,35 @@ __global__ void __launch_bounds__(kEfThreads, 4)
             out.child_end[idx] = (d < (int)Ll) ? (int32_t)info->level_offset[d + 2] : -1;
         }
     }
-    __syncthreads();
-    const uint32_t Lp0 = threadIdx.x > 0 ? (uint32_t)s_Llast[threadIdx.x - 1] : Lbefore;
+    // the warp's starts in order
     uint32_t cnt = 0;
 #pragma unroll
     for (int j = 0; j < 4; ++j) cnt += (m[j] <= L[j]) ? 1u : 0u;
     uint32_t x = cnt;
+#pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
         if (lane >= off) x += y;
     }
-    if (lane == 31) s_wcnt[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        // exclusive prefix of the warps' counts, by shuffles
-        const uint32_t c = lane < kEfWarps ? s_wcnt[lane] : 0u;
-        uint32_t r = c;
+    const int total = (int)__shfl_sync(0xffffffffu, x, 31);
+    uint32_t pos = x - cnt;
 #pragma unroll
-        for (int off = 1; off < kEfWarps; off <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, r, off);
-            if (lane >= off) r += y;
-        }
-        if (lane < kEfWarps) s_wcnt[lane] = r - c;
-        if (lane == kEfWarps - 1) s_total = r;
-    }
-    __syncthreads();
-    uint32_t pos = s_wcnt[warp] + x - cnt;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if (m[j] <= L[j]) {
-            const uint32_t lp = j ? L[j - 1] : Lp0;
-            s_entry[pos++] = (uint32_t)(4 * threadIdx.x + j) | (m[j] << 11) | (L[j] << 16) | (lp << 21);
-        }
-    }
-    __syncthreads();
-    const int total = (int)s_total;
-    const int nchunks = (total + 31) / 32;
-    // the keys of the warp's first chunk of starts, loaded now so that the
-    // mask and prefix phases below cover their latency
+    for (int j = 0; j < 4; ++j)
+        if (m[j] <= L[j])
+            W.entry[pos++] = (uint32_t)(4 * lane + j) | (m[j] << 8) | (L[j] << 16) | ((j ? L[j - 1] : Lp) << 24);
+    __syncwarp();
+    // the keys of the first chunk of starts, loaded now so that the masks and
+    // the barrier cover their latency
     uint64_t Kfirst = 0;
-    if (warp * 32 + lane < total) Kfirst = skeys[s + (s_entry[warp * 32 + lane] & 2047u)];
-    // level masks of every chunk of 32 starts (a 32 x 32 bit transpose)
-    for (int c = warp; c < nchunks; c += kEfWarps) {
+    if (lane < total) Kfirst = skeys[s + (W.entry[lane] & 255u)];
+    // level masks of every chunk of 32 starts; lane d counts level d
+    uint32_t mine = 0;
+    for (int c = 0; 32 * c < total; ++c) {
         const int i = c * 32 + lane;
         uint32_t v = 0;
         if (i < total) {
-            const uint32_t en = s_entry[i];
-            const uint32_t mm = (en >> 11) & 31u, LL = (en >> 16) & 31u;
-            v = (2u << LL) - (1u << mm);
+            const uint32_t en = W.entry[i];
+            v = (2u << ((en >> 16) & 31u)) - (1u << ((en >> 8) & 31u));
         }
         uint32_t msk = 0x0000ffffu;
 #pragma unroll
@@ -346,61 +330,59 @@ __global__ void __launch_bounds__(kEfThreads, 4)
             if (lane & j) v ^= ((y >> j) ^ v) & msk;
             else v ^= (((v >> j) ^ y) & msk) << j;
         }
-        if (lane < kLevels) s_mask[c][lane] = v;
+        if (lane < kLevels) W.mask[c][lane] = v;
+        mine += __popc(v);
     }
+    if (lane == kLevels) mine = (uint32_t)total;
+    if (lane < kLevelFields) s_cnt[warp][lane] = mine;
     __syncthreads();
-    // per level, the starts in earlier chunks: a warp per level, a lane per
-    // chunk, 32 chunks at a time
-    for (int d = warp; d < kLevels; d += kEfWarps) {
-        uint32_t carry = 0;
-        for (int g = 0; g < nchunks; g += 32) {
-            const int c = g + lane;
-            const uint32_t v = c < nchunks ? (uint32_t)__popc(s_mask[c][d]) : 0u;
-            uint32_t r = v;
+    if (lane < kLevelFields) {
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, r, off);
-                if (lane >= off) r += y;
-            }
-            if (c < nchunks) s_cpre[c][d] = carry + r - v;
-            carry += __shfl_sync(0xffffffffu, r, 31);
-        }
+        for (int w = 0; w < kEfWarps; ++w)
+            if (w < warp) base += s_cnt[w][lane];
+        W.base[lane] = base;
     }
-    __syncthreads();
+    __syncwarp();
     const unsigned lt = lanemask_lt();
-    for (int c = warp; c < nchunks; c += kEfWarps) {
+    for (int c = 0; 32 * c < total; ++c) {
         const int i = c * 32 + lane;
-        if (i >= total) continue;
-        const uint32_t en = s_entry[i];
-        const int64_t k = s + (en & 2047u);
-        const int mm = (int)((en >> 11) & 31u), LL = (int)((en >> 16) & 31u), Lp = (int)((en >> 21) & 31u);
-        auto P = [&](int d) { return s_base[d] + s_cpre[c][d] + (uint32_t)__popc(s_mask[c][d] & lt); };
-        const uint64_t K = c == warp ? Kfirst : skeys[k];
-        // P(d) of consecutive levels: each loop computes one new level per step
-        const uint32_t pm = P(mm);
-        if (k > 0) {
-            // close the cells holding k-1 but not k
-            uint32_t pd = pm;
-            for (int d = mm; d <= Lp; ++d) {
-                const uint32_t pn = d < Lp ? P(d + 1) : 0u;
-                out.pend[pd - 1] = (int32_t)k;
-                out.child_end[pd - 1] = (d < Lp) ? (int32_t)pn : -1;
+        if (i < total) {
+            const uint32_t en = W.entry[i];
+            const int64_t k = s + (en & 255u);
+            const int mm = (int)((en >> 8) & 31u), LL = (int)((en >> 16) & 31u), Lq = (int)(en >> 24);
+            auto P = [&](int d) { return W.base[d] + (uint32_t)__popc(W.mask[c][d] & lt); };
+            const uint64_t K = c == 0 ? Kfirst : skeys[k];
+            // P(d) of consecutive levels: each loop computes one new level per step
+            const uint32_t pm = P(mm);
+            if (k > 0) {
+                // close the cells holding k-1 but not k
+                uint32_t pd = pm;
+                for (int d = mm; d <= Lq; ++d) {
+                    const uint32_t pn = d < Lq ? P(d + 1) : 0u;
+                    out.pend[pd - 1] = (int32_t)k;
+                    out.child_end[pd - 1] = (d < Lq) ? (int32_t)pn : -1;
+                    pd = pn;
+                }
+            }
+            uint32_t pprev = mm > 0 ? P(mm - 1) : 0u, pd = pm;
+            for (int d = mm;; ++d) {
+                const uint32_t pn = d < LL ? P(d + 1) : 0u;
+                out.ckey[pd] = cell_key(K, d);
+                out.level[pd] = (uint8_t)d;
+                out.pfirst[pd] = (int32_t)k;
+                out.parent[pd] = (d == 0) ? -1 : (int32_t)pprev - (d == mm ? 1 : 0);
+                out.child_first[pd] = (d < LL) ? (int32_t)pn : -1;
+                if (d == LL) break;
+                pprev = pd;
                 pd = pn;
             }
+            out.leaf_cell[W.base[kLevels] + (uint32_t)i] = (int32_t)pd;
         }
-        uint32_t pprev = mm > 0 ? P(mm - 1) : 0u, pd = pm;
-        for (int d = mm;; ++d) {
-            const uint32_t pn = d < LL ? P(d + 1) : 0u;
-            out.ckey[pd] = cell_key(K, d);
-            out.level[pd] = (uint8_t)d;
-            out.pfirst[pd] = (int32_t)k;
-            out.parent[pd] = (d == 0) ? -1 : (int32_t)pprev - (d == mm ? 1 : 0);
-            out.child_first[pd] = (d < LL) ? (int32_t)pn : -1;
-            if (d == LL) break;
-            pprev = pd;
-            pd = pn;
+        if (32 * (c + 1) < total) {
+            __syncwarp();
+            if (lane < kLevels) W.base[lane] += (uint32_t)__popc(W.mask[c][lane]);
+            __syncwarp();
         }
-        out.leaf_cell[s_base[kLevels] + (uint32_t)i] = (int32_t)pd;
     }
 }
 
