@@ -331,8 +331,7 @@ tb_status tb_build(const float *d_pos, const float *d_mass, int64_t n, const tb_
     // a sort variant or times the stages
     const bool named = params->radix_bits || params->sort_threads || params->sort_items;
     if (!named && !ws.profile && n <= small_sort_max()) {
-        e = launch_small_sort(d_pos, d_mass, n, t.pkey, t.perm, ws.keys_alt, ws.perm_alt, ws,
-                              params->key_order, s);
+        e = launch_small_sort(d_pos, d_mass, n, t.pkey, t.perm, ws, params->key_order, s);
         if (e != cudaSuccess) return from_cuda(e);
     } else {
         const int passes = sort_plan(cfg).passes;

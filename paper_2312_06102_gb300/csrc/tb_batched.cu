@@ -45,10 +45,13 @@ inline bool batch_few_large(int32_t S, int64_t n) { return S <= 608 && n >= int6
 inline bool batch_many_small(int32_t S, int64_t n) { return S > 304 && n <= int64_t(S) * 512; }
 constexpr int kBRadixBits = kCtaRadixBits;
 constexpr int kBRadix = kCtaRadix;
-// the block sort orders the upper 40 key bits in five passes; the runs of
-// equal upper bits are then ordered in place (tb_runs.cuh)
-constexpr int kBPasses = 5;
-constexpr int kBShift0 = 63 - kBPasses * kBRadixBits;
+// the block sort orders the upper 40 key bits in five passes, or the upper 32
+// in four for sets of up to 2^17 particles; the runs of equal upper bits are
+// then ordered in place (tb_runs.cuh), the long ones by the same block sort of
+// their low bits.  So a set of tight clumps, all of it in long runs, takes
+// eight passes either way, and any other small set one less.
+constexpr int kBMaxPasses = 5;
+__device__ __forceinline__ int batch_passes(int64_t ns) { return ns <= (int64_t(1) << 17) ? 4 : kBMaxPasses; }
 constexpr int kBMomThreads = 256;
 constexpr int kBigLeafSerial = 1 << 20;       // leaves above this are summed in FP64
 
@@ -224,7 +227,8 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
             A.set_root[4 * (int64_t)set + 3] = r.side;
             if (s_bad) atomicOr(&A.info->status, kErrNonFinite);
         }
-        for (int i = threadIdx.x; i < kBPasses * kBRadix; i += blockDim.x) (&sm.hist[0][0])[i] = 0;
+        const int passes = batch_passes(ns), shift0 = 63 - passes * kBRadixBits;
+        for (int i = threadIdx.x; i < kBMaxPasses * kBRadix; i += blockDim.x) (&sm.hist[0][0])[i] = 0;
         __syncthreads();
         // ---- keys, records and every pass's digit histogram
         const bool staged = ns <= CtaSortSharedT<T>::TILE;
@@ -233,49 +237,50 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
             const double sc = s_scale;
             const bool ex = s_exact, f32 = s_f32;
             const float m_eq = (float)(1.0 / (double)ns);
-            // unsorted keys go where pass 0 reads them: kBPasses is odd, so the
-            // passes run kalt -> pkey -> ... -> pkey (a set of one sort tile keeps
-            // them in shared memory)
+            // unsorted keys go where pass 0 reads them, so that the last pass
+            // ends in pkey (a set of one sort tile keeps them in shared memory)
+            uint64_t *unsorted = passes & 1 ? A.kalt : A.pkey;
             for (int64_t i = o + threadIdx.x; i < o + ns; i += blockDim.x) {
                 const float x = A.pos[3 * i], y = A.pos[3 * i + 1], z = A.pos[3 * i + 2];
                 const uint64_t k = morton_key(quantise(x, lx, shi, slo, sc, ex, f32),
                                               quantise(y, ly, shi, slo, sc, ex, f32),
                                               quantise(z, lz, shi, slo, sc, ex, f32));
                 if (staged) sm.keys[i - o] = k;
-                else A.kalt[i] = k;
+                else unsorted[i] = k;
                 A.xm[i] = make_float4(x, y, z, A.mass ? A.mass[i] : m_eq);
-                for (int p = 0; p < kBPasses; ++p)
-                    atomicAdd(&sm.hist[p][(k >> (kBShift0 + p * kBRadixBits)) & (kBRadix - 1)], 1u);
+                for (int p = 0; p < passes; ++p)
+                    atomicAdd(&sm.hist[p][(k >> (shift0 + p * kBRadixBits)) & (kBRadix - 1)], 1u);
             }
         }
         __syncthreads();
         // ---- stable LSD sort of the set by its upper key bits (digit counts
         // taken above), then the runs of equal upper bits by the low bits
-        cta_lsd_sort(A.kalt, A.palt, A.pkey, A.perm, o, ns, kBShift0, kBPasses, true, staged, sm);
+        if (passes & 1) cta_lsd_sort(A.kalt, A.palt, A.pkey, A.perm, o, ns, shift0, passes, true, staged, sm);
+        else cta_lsd_sort(A.pkey, A.perm, A.kalt, A.palt, o, ns, shift0, passes, true, staged, sm);
         __syncthreads();
         for (int64_t t0 = o; t0 < o + ns; t0 += kRunTile) {
             if (threadIdx.x == 0) s_nlong = 0;
             __syncthreads();
-            run_tile<T>(A.pkey, A.perm, o, t0, o + ns, kBShift0, *reinterpret_cast<RunSmem *>(raw),
+            run_tile<T>(A.pkey, A.perm, o, t0, o + ns, shift0, *reinterpret_cast<RunSmem *>(raw),
                                 [&](int64_t a) { s_long[atomicAdd(&s_nlong, 1)] = a; });
             const int nl = s_nlong;
             for (int j = 0; j < nl; ++j) {
                 // a run of more than kRunMax keys (at most 16 start in a tile):
                 // its end, then the block sort of its low bits
                 const int64_t a = s_long[j];
-                const uint64_t tp = A.pkey[a] >> kBShift0;
+                const uint64_t tp = A.pkey[a] >> shift0;
                 if (threadIdx.x == 0) s_end = (unsigned long long)(o + ns);
                 __syncthreads();
                 for (int64_t base = a + 1; base < o + ns; base += blockDim.x) {
                     const int64_t p = base + threadIdx.x;
-                    if (p < o + ns && (A.pkey[p] >> kBShift0) != tp) atomicMin(&s_end, (unsigned long long)p);
+                    if (p < o + ns && (A.pkey[p] >> shift0) != tp) atomicMin(&s_end, (unsigned long long)p);
                     __syncthreads();
                     const bool done = s_end < (unsigned long long)(o + ns);
                     __syncthreads();
                     if (done) break;
                 }
                 const int64_t len = (int64_t)s_end - a;
-                constexpr int low_passes = (kBShift0 + kBRadixBits - 1) / kBRadixBits;
+                const int low_passes = (shift0 + kBRadixBits - 1) / kBRadixBits;
                 cta_histograms(A.pkey, a, len, 0, low_passes, sm);
                 const int np = cta_lsd_sort(A.pkey, A.perm, A.kalt, A.palt, a, len, 0, low_passes, false, false, sm);
                 if (np & 1)

@@ -183,8 +183,7 @@ cudaError_t load_small_kernels();
 // root, keys and sort of a small set in one launch
 int64_t small_sort_max();
 cudaError_t launch_small_sort(const float *pos, const float *mass, int64_t n, uint64_t *pkey, int32_t *perm,
-                              uint64_t *alt_k, int32_t *alt_v, Workspace &ws, int key_order,
-                              cudaStream_t s);
+                              Workspace &ws, int key_order, cudaStream_t s);
 
 // tree walk: int32 words of its scratch (counters, groups, per-warp stacks)
 int64_t walk_buffer_words(int64_t n_cells);

@@ -148,8 +148,7 @@ extern "C" tb_status tb_keys_sorted_noalloc(const float *d_pos, int64_t n, uint6
     }
     if (n >= 2 && (e = load_kernels_once()) != cudaSuccess) return status_of(e);
     if (n <= small_sort_max()) {
-        if ((e = launch_small_sort(d_pos, nullptr, n, d_pkey, d_perm, ws.keys_alt, ws.perm_alt, ws,
-                                   TB_KEYS_MORTON, s)) != cudaSuccess)
+        if ((e = launch_small_sort(d_pos, nullptr, n, d_pkey, d_perm, ws, TB_KEYS_MORTON, s)) != cudaSuccess)
             return status_of(e);
     } else {
         const int passes = sort_plan(cfg).passes;

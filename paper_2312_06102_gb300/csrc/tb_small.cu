@@ -11,7 +11,7 @@
 //   1. particles to registers (records written out), bounding box by shuffles
 //      and, across the blocks, distributed shared memory; every block forms
 //      the same root cube; keys;
-//   2. five stable 8-bit passes over the upper 40 key bits, as in the general
+//   2. four stable 8-bit passes over the upper 32 key bits, as in the general
 //      sort: ballot ranking within warps, digit counts of the block; a cluster
 //      barrier; every block reads all blocks' counts and so knows where each
 //      of its digits goes; the block orders its pairs by digit in shared
@@ -20,7 +20,9 @@
 //      barrier.  A pass reads its pairs into registers before its first
 //      barrier and stores after it, so the owners need one buffer;
 //   3. runs of equal upper bits ordered in place by the low bits
-//      (tb_runs.cuh), tiles shared out over the blocks, long runs after.
+//      (tb_runs.cuh), tiles shared out over the blocks.  A set with runs too
+//      long for that and out of order (tight clumps) takes eight passes over
+//      the whole key instead, over the order reached.
 // Barriers are the cluster's own (barrier.cluster); nothing spins.
 #include <cfloat>
 
@@ -34,10 +36,10 @@ constexpr int kSmThreads = 1024;
 constexpr int kSmWarps = kSmThreads / 32;
 constexpr int kSmBits = 8;
 constexpr int kSmRadix = 1 << kSmBits;
-constexpr int kSmPasses = 5;
+constexpr int kSmPasses = 4;
 constexpr int kSmShift0 = 63 - kSmPasses * kSmBits;
+constexpr int kSmAllPasses = 8;   // of the whole key
 constexpr int kSmMaxItems = 2;
-constexpr int kSmLong = 64;       // long runs a block can queue (16 a tile, at most 2 tiles)
 
 template <int ITEMS>
 struct SmallSmem {
@@ -101,16 +103,15 @@ __device__ __forceinline__ void warp_box(float mn[3], float mx[3], uint32_t &bad
 template <int ITEMS, bool HILBERT>
 __global__ void __launch_bounds__(kSmThreads, 1)
     small_sort_kernel(const float *__restrict__ pos, const float *__restrict__ mass, float m_eq, int n,
-                      uint64_t *pkey, int32_t *perm, uint64_t *alt_k, int32_t *alt_v,
-                      float4 *__restrict__ xm, RunBuffers rb, DevInfo *info, bool pow2) {
+                      uint64_t *pkey, int32_t *perm, float4 *__restrict__ xm, DevInfo *info,
+                      bool pow2) {
     after_previous();
     using S = SmallSmem<ITEMS>;
     constexpr int P = S::P;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     S &sm = *reinterpret_cast<S *>(sm_raw);
     __shared__ RootCube s_cube;
-    __shared__ int32_t s_long[kSmLong];
-    __shared__ uint32_t s_nlong;
+    __shared__ uint32_t s_long, s_desc, s_again;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t rank = cluster_rank(), blocks = gridDim.x;   // one cluster
     const int first = (int)rank * P;
@@ -164,7 +165,7 @@ __global__ void __launch_bounds__(kSmThreads, 1)
             warp_box(mn, mx, bad);
             if (lane == 0) {
                 s_cube = root_cube(mn, mx, pow2);
-                s_nlong = 0;
+                s_long = s_desc = 0;
                 if (rank == 0) begin_build(info, s_cube, mx, bad != 0u);
             }
         }
@@ -189,149 +190,162 @@ __global__ void __launch_bounds__(kSmThreads, 1)
 
     // 2. passes
     const unsigned lt = lanemask_lt();
-    for (int p = 0; p < kSmPasses; ++p) {
-        const int shift = kSmShift0 + p * kSmBits;
-        if (p > 0) {
+    const int tiles = (n + kRunTile - 1) / kRunTile;
+    for (int passes = kSmPasses, shift0 = kSmShift0;; passes = kSmAllPasses, shift0 = 0) {
+        for (int p = 0; p < passes; ++p) {
+            const int shift = shift0 + p * kSmBits;
+            if (p > 0) {
+#pragma unroll
+                for (int i = 0; i < ITEMS; ++i) {
+                    const int e = wbase + i * 32 + lane;
+                    key[i] = sm.key[e];
+                    val[i] = sm.val[e];
+                }
+            }
+            for (int i = threadIdx.x; i < kSmWarps * (kSmRadix + 1); i += kSmThreads) (&sm.hist[0][0])[i] = 0;
+            __syncthreads();
+            // stable ranks within the warp; positions past the set take no part
+            uint32_t at[ITEMS];
 #pragma unroll
             for (int i = 0; i < ITEMS; ++i) {
-                const int e = wbase + i * 32 + lane;
-                key[i] = sm.key[e];
-                val[i] = sm.val[e];
-            }
-        }
-        for (int i = threadIdx.x; i < kSmWarps * (kSmRadix + 1); i += kSmThreads) (&sm.hist[0][0])[i] = 0;
-        __syncthreads();
-        // stable ranks within the warp; positions past the set take no part
-        uint32_t at[ITEMS];
+                const bool in = wbase + i * 32 + lane < mine;
+                const uint32_t d = (uint32_t)(key[i] >> shift) & (kSmRadix - 1);
+                unsigned peers = __ballot_sync(0xffffffffu, in);
+                if (!in) peers = 0;
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const bool in = wbase + i * 32 + lane < mine;
-            const uint32_t d = (uint32_t)(key[i] >> shift) & (kSmRadix - 1);
-            unsigned peers = __ballot_sync(0xffffffffu, in);
-            if (!in) peers = 0;
-#pragma unroll
-            for (int b = 0; b < kSmBits; ++b) {
-                const bool bit = (d >> b) & 1u;
-                const unsigned v = __ballot_sync(0xffffffffu, bit);
-                peers &= bit ? v : ~v;
+                for (int b = 0; b < kSmBits; ++b) {
+                    const bool bit = (d >> b) & 1u;
+                    const unsigned v = __ballot_sync(0xffffffffu, bit);
+                    peers &= bit ? v : ~v;
+                }
+                const int leader = __ffs(peers) - 1;
+                uint32_t old = 0;
+                if (in && lane == leader) old = atomicAdd(&sm.hist[warp][d], (uint32_t)__popc(peers));
+                at[i] = __shfl_sync(0xffffffffu, old, leader & 31) + (uint32_t)__popc(peers & lt);
             }
-            const int leader = __ffs(peers) - 1;
-            uint32_t old = 0;
-            if (in && lane == leader) old = atomicAdd(&sm.hist[warp][d], (uint32_t)__popc(peers));
-            at[i] = __shfl_sync(0xffffffffu, old, leader & 31) + (uint32_t)__popc(peers & lt);
-        }
-        __syncthreads();
-        // each warp's offset within its digit, the block's count of the digit:
-        // four lanes a digit, eight warps each
-        const int dg = threadIdx.x >> 2, part = threadIdx.x & 3;
-        {
-            uint32_t c[kSmWarps / 4], sum = 0;
-#pragma unroll
-            for (int j = 0; j < kSmWarps / 4; ++j) {
-                c[j] = sm.hist[part * (kSmWarps / 4) + j][dg];
-                sum += c[j];
-            }
-            uint32_t y = sum;
-#pragma unroll
-            for (int off = 1; off < 4; off <<= 1) {
-                const uint32_t z = __shfl_up_sync(0xffffffffu, y, off, 4);
-                if (part >= off) y += z;
-            }
-            uint32_t run = y - sum;
-#pragma unroll
-            for (int j = 0; j < kSmWarps / 4; ++j) {
-                sm.hist[part * (kSmWarps / 4) + j][dg] = run;
-                run += c[j];
-            }
-            if (part == 3) sm.cnt[p & 1][dg] = y;
-        }
-        cluster_sync();
-        // every block's count of the digit: those before this one's, and all
-        {
-            uint32_t tot = 0, pre = 0;
-            for (uint32_t q = part; q < blocks; q += 4) {
-                const uint32_t v = ld_remote(remote(&sm.cnt[p & 1][dg], q));
-                tot += v;
-                if (q < rank) pre += v;
-            }
-#pragma unroll
-            for (int off = 1; off < 4; off <<= 1) {
-                tot += __shfl_xor_sync(0xffffffffu, tot, off);
-                pre += __shfl_xor_sync(0xffffffffu, pre, off);
-            }
-            // prefixes over the digits of all blocks' counts (at most 2^15, low
-            // 18 bits) and of this block's (at most 2^11, high 14 bits) at once
-            const uint32_t own = sm.cnt[p & 1][dg], both = tot | (own << 18);
-            uint32_t y = both;   // inclusive over the warp's eight digits
-#pragma unroll
-            for (int off = 4; off < 32; off <<= 1) {
-                const uint32_t z = __shfl_up_sync(0xffffffffu, y, off);
-                if (lane >= off) y += z;
-            }
-            if (lane == 31) sm.carry[warp] = y;
             __syncthreads();
-            y += __reduce_add_sync(0xffffffffu, lane < warp ? sm.carry[lane] : 0u) - both;
-            if (part == 0) {
-                sm.loc[dg] = y >> 18;
-                sm.base[dg] = (y & 0x3ffffu) + pre - (y >> 18);
-            }
-        }
-        __syncthreads();
+            // each warp's offset within its digit, the block's count of the digit:
+            // four lanes a digit, eight warps each
+            const int dg = threadIdx.x >> 2, part = threadIdx.x & 3;
+            {
+                uint32_t c[kSmWarps / 4], sum = 0;
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            if (wbase + i * 32 + lane >= mine) continue;
-            const uint32_t d = (uint32_t)(key[i] >> shift) & (kSmRadix - 1);
-            const uint32_t e = sm.loc[d] + sm.hist[warp][d] + at[i];
-            sm.skey[e] = key[i];
-            sm.sval[e] = val[i];
-        }
-        __syncthreads();
+                for (int j = 0; j < kSmWarps / 4; ++j) {
+                    c[j] = sm.hist[part * (kSmWarps / 4) + j][dg];
+                    sum += c[j];
+                }
+                uint32_t y = sum;
 #pragma unroll
-        for (int i = 0; i < ITEMS; ++i) {
-            const int j = i * kSmThreads + (int)threadIdx.x;
-            if (j >= mine) continue;
-            const uint64_t k = sm.skey[j];
-            const uint32_t d = (uint32_t)(k >> shift) & (kSmRadix - 1);
-            const uint32_t to = sm.base[d] + (uint32_t)j;
-            if (p + 1 < kSmPasses) {
-                const uint32_t q = to / P, e = to % P;
-                st_remote(remote(&sm.key[e], q), k);
-                st_remote(remote(&sm.val[e], q), sm.sval[j]);
-            } else {
-                pkey[to] = k;
-                perm[to] = sm.sval[j];
+                for (int off = 1; off < 4; off <<= 1) {
+                    const uint32_t z = __shfl_up_sync(0xffffffffu, y, off, 4);
+                    if (part >= off) y += z;
+                }
+                uint32_t run = y - sum;
+#pragma unroll
+                for (int j = 0; j < kSmWarps / 4; ++j) {
+                    sm.hist[part * (kSmWarps / 4) + j][dg] = run;
+                    run += c[j];
+                }
+                if (part == 3) sm.cnt[p & 1][dg] = y;
             }
+            cluster_sync();
+            // every block's count of the digit: those before this one's, and all
+            {
+                uint32_t tot = 0, pre = 0;
+                for (uint32_t q = part; q < blocks; q += 4) {
+                    const uint32_t v = ld_remote(remote(&sm.cnt[p & 1][dg], q));
+                    tot += v;
+                    if (q < rank) pre += v;
+                }
+#pragma unroll
+                for (int off = 1; off < 4; off <<= 1) {
+                    tot += __shfl_xor_sync(0xffffffffu, tot, off);
+                    pre += __shfl_xor_sync(0xffffffffu, pre, off);
+                }
+                // prefixes over the digits of all blocks' counts (at most 2^15, low
+                // 18 bits) and of this block's (at most 2^11, high 14 bits) at once
+                const uint32_t own = sm.cnt[p & 1][dg], both = tot | (own << 18);
+                uint32_t y = both;   // inclusive over the warp's eight digits
+#pragma unroll
+                for (int off = 4; off < 32; off <<= 1) {
+                    const uint32_t z = __shfl_up_sync(0xffffffffu, y, off);
+                    if (lane >= off) y += z;
+                }
+                if (lane == 31) sm.carry[warp] = y;
+                __syncthreads();
+                y += __reduce_add_sync(0xffffffffu, lane < warp ? sm.carry[lane] : 0u) - both;
+                if (part == 0) {
+                    sm.loc[dg] = y >> 18;
+                    sm.base[dg] = (y & 0x3ffffu) + pre - (y >> 18);
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) {
+                if (wbase + i * 32 + lane >= mine) continue;
+                const uint32_t d = (uint32_t)(key[i] >> shift) & (kSmRadix - 1);
+                const uint32_t e = sm.loc[d] + sm.hist[warp][d] + at[i];
+                sm.skey[e] = key[i];
+                sm.sval[e] = val[i];
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) {
+                const int j = i * kSmThreads + (int)threadIdx.x;
+                if (j >= mine) continue;
+                const uint64_t k = sm.skey[j];
+                const uint32_t d = (uint32_t)(k >> shift) & (kSmRadix - 1);
+                const uint32_t to = sm.base[d] + (uint32_t)j;
+                if (p + 1 < passes) {
+                    const uint32_t q = to / P, e = to % P;
+                    st_remote(remote(&sm.key[e], q), k);
+                    st_remote(remote(&sm.val[e], q), sm.sval[j]);
+                } else {
+                    pkey[to] = k;
+                    perm[to] = sm.sval[j];
+                }
+            }
+            cluster_sync();
+        }
+
+        if (passes == kSmAllPasses) return;
+
+        // 3. runs of equal upper bits
+        for (int t = rank; t < tiles; t += blocks) {
+            const bool desc = run_tile<kSmThreads>(pkey, perm, 0, (int64_t)t * kRunTile, n, kSmShift0,
+                                                   *reinterpret_cast<RunSmem *>(sm_raw),
+                                                   [&](int64_t) { s_long = 1; });
+            if (threadIdx.x == 0 && desc) s_desc = 1;
         }
         cluster_sync();
+        // any block with a long run, and any descent: again, over the whole key
+        if (warp == 0) {
+            const uint32_t q = lane < blocks ? lane : rank;
+            const uint32_t l = ld_remote(remote(&s_long, q)), d = ld_remote(remote(&s_desc, q));
+            const bool again = __any_sync(0xffffffffu, l != 0) && __any_sync(0xffffffffu, d != 0);
+            if (lane == 0) s_again = again ? 1u : 0u;
+        }
+        cluster_sync();   // no block leaves while another reads its flags
+        if (!s_again) return;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const int e = wbase + i * 32 + lane;
+            if (e < mine) {
+                key[i] = __ldcg(reinterpret_cast<const unsigned long long *>(pkey) + first + e);
+                val[i] = __ldcg(perm + first + e);
+            }
+        }
     }
-
-    // 3. runs of equal upper bits
-    const int tiles = (n + kRunTile - 1) / kRunTile;
-    for (int t = rank; t < tiles; t += blocks) {
-        const bool desc = run_tile<kSmThreads>(pkey, perm, 0, (int64_t)t * kRunTile, n, kSmShift0,
-                                               *reinterpret_cast<RunSmem *>(sm_raw), [&](int64_t a) {
-                                                   s_long[atomicAdd(&s_nlong, 1u)] = (int32_t)a;
-                                               });
-        if (threadIdx.x == 0) rb.desc[t] = desc ? 1 : 0;
-    }
-    cluster_sync();
-    const uint32_t nl = s_nlong;
-    for (uint32_t j = 0; j < nl; ++j)
-        sort_long_run<kSmThreads>(pkey, perm, alt_k, alt_v, n, kSmShift0, s_long[j], rb.desc,
-                                  *reinterpret_cast<CtaSortSharedT<kSmThreads> *>(sm_raw));
 }
 
 template <int ITEMS>
 constexpr size_t small_smem() {
-    const size_t a = sizeof(SmallSmem<ITEMS>), b = sizeof(CtaSortSharedT<kSmThreads>);
-    const size_t c = sizeof(RunSmem);
-    return a > b ? (a > c ? a : c) : (b > c ? b : c);
+    return sizeof(SmallSmem<ITEMS>) > sizeof(RunSmem) ? sizeof(SmallSmem<ITEMS>) : sizeof(RunSmem);
 }
 
 template <int ITEMS, bool H>
 cudaError_t launch_small_t(const float *pos, const float *mass, int n, uint64_t *pkey, int32_t *perm,
-                           uint64_t *alt_k, int32_t *alt_v, Workspace &ws, bool ask, int *clusters,
-                           cudaStream_t s) {
+                           Workspace &ws, bool ask, int *clusters, cudaStream_t s) {
     auto kern = small_sort_kernel<ITEMS, H>;
     const int blocks = (n + SmallSmem<ITEMS>::P - 1) / SmallSmem<ITEMS>::P;
     static std::atomic<uint64_t> attr_done{0};
@@ -355,20 +369,20 @@ cudaError_t launch_small_t(const float *pos, const float *mass, int n, uint64_t 
     cfg.numAttrs = 1;
     if (ask) return cudaOccupancyMaxActiveClusters(clusters, kern, &cfg);
     const float m_eq = (float)(1.0 / (double)n);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, pos, mass, m_eq, n, pkey, perm, alt_k, alt_v, ws.xm,
-                                       run_buffers(ws.long_runs, n), ws.info, ws.root_pow2);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, pos, mass, m_eq, n, pkey, perm, ws.xm, ws.info,
+                                       ws.root_pow2);
     if (e == cudaSuccess) ++g_launches;
     return e;
 }
 
 cudaError_t dispatch_small(const float *pos, const float *mass, int64_t n, int max_blocks, uint64_t *pkey,
-                           int32_t *perm, uint64_t *alt_k, int32_t *alt_v, Workspace &ws, int key_order,
-                           bool ask, int *clusters, cudaStream_t s) {
+                           int32_t *perm, Workspace &ws, int key_order, bool ask, int *clusters,
+                           cudaStream_t s) {
     const bool h = key_order == TB_KEYS_HILBERT;
 #define TB_SMALL(I)                                                                                     \
     if (n <= (int64_t)I * kSmThreads * max_blocks)                                                      \
-        return h ? launch_small_t<I, true>(pos, mass, (int)n, pkey, perm, alt_k, alt_v, ws, ask, clusters, s) \
-                 : launch_small_t<I, false>(pos, mass, (int)n, pkey, perm, alt_k, alt_v, ws, ask, clusters, s);
+        return h ? launch_small_t<I, true>(pos, mass, (int)n, pkey, perm, ws, ask, clusters, s) \
+                 : launch_small_t<I, false>(pos, mass, (int)n, pkey, perm, ws, ask, clusters, s);
     TB_SMALL(1)
     TB_SMALL(2)
 #undef TB_SMALL
@@ -387,7 +401,7 @@ int small_blocks() {
         int clusters = 0;
         const cudaError_t e =
             dispatch_small(nullptr, nullptr, (int64_t)16 * kSmThreads * kSmMaxItems, 16, nullptr, nullptr,
-                           nullptr, nullptr, none, TB_KEYS_MORTON, true, &clusters, nullptr);
+                           none, TB_KEYS_MORTON, true, &clusters, nullptr);
         if (e != cudaSuccess) cudaGetLastError();
         v = e == cudaSuccess && clusters > 0 ? 16 : 8;
         known[dev].store(v, std::memory_order_relaxed);
@@ -406,12 +420,10 @@ cudaError_t load_small_kernels() {
 }
 
 // Root cube (with the build record's start), records, sorted keys and
-// permutation of 1 <= n <= small_sort_max() particles; alt_k and alt_v hold n.
+// permutation of 1 <= n <= small_sort_max() particles.
 cudaError_t launch_small_sort(const float *pos, const float *mass, int64_t n, uint64_t *pkey, int32_t *perm,
-                              uint64_t *alt_k, int32_t *alt_v, Workspace &ws, int key_order,
-                              cudaStream_t s) {
-    return dispatch_small(pos, mass, n, small_blocks(), pkey, perm, alt_k, alt_v, ws, key_order, false,
-                          nullptr, s);
+                              Workspace &ws, int key_order, cudaStream_t s) {
+    return dispatch_small(pos, mass, n, small_blocks(), pkey, perm, ws, key_order, false, nullptr, s);
 }
 
 }  // namespace tb
