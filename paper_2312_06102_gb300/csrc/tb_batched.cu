@@ -187,6 +187,7 @@ __device__ void set_root_cube(const float *__restrict__ pos, int64_t o, int64_t 
 // block's dynamic shared memory (batch_front_smem<T> bytes).
 template <int T>
 __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
+    static_assert(sizeof(RunSmem) <= sizeof(CtaSortSharedT<T>), "a run tile lies in the sort's shared memory");
     CtaSortSharedT<T> &sm = *reinterpret_cast<CtaSortSharedT<T> *>(raw);
     __shared__ TileSharedT<T> ts;
     __shared__ float s_red[(T / 32) * 6];

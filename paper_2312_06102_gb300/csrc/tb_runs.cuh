@@ -15,10 +15,12 @@ constexpr int kRunSpan = kRunTile + kRunMax;                 // positions a tile
 constexpr int kRunChunks = kRunSpan / 32 + 1;                // 32-position start masks (+ one past)
 
 struct RunSmem {
-    // sk[x + 2] = keys[s + x] for x in [-1, nw); sk[nw + 2] is a sentinel
-    // whose upper bits differ from every key's (keys leave bit 63 clear)
-    __align__(16) uint64_t sk[kRunSpan + 4];
+    // sk[x + 2] = keys[s + x] for x in [-1, nw); before the range's first key,
+    // that key's complement, whose upper bits differ from it
+    __align__(16) uint64_t sk[kRunSpan + 2];
     uint32_t smask[kRunChunks];   // bit l of chunk c: position 32 c + l starts a run
+    uint32_t count;               // positions in list
+    uint16_t list[kRunSpan];      // the positions in runs of two keys and more
 };
 
 // Orders in place, by (low shift0 bits, position), every run of equal
@@ -27,6 +29,10 @@ struct RunSmem {
 // starting at a in the tile.  All THREADS threads of the block take part.
 // Returns, the same in every thread, whether a key of the tile is smaller
 // than its predecessor in the same run (a descent).
+//
+// Bound by instruction issue.  In the tree workloads 2% to 8% of the keys lie
+// in runs of two and more, yet a quarter to a half of all warps hold one, so
+// the members are listed first and ranked by full warps.
 template <int THREADS, class QueueLong>
 __device__ bool run_tile(uint64_t *__restrict__ keys, int32_t *__restrict__ vals, int64_t lo, int64_t s,
                          int64_t hi, int shift0, RunSmem &S, QueueLong queue_long) {
@@ -45,38 +51,49 @@ __device__ bool run_tile(uint64_t *__restrict__ keys, int32_t *__restrict__ vals
         for (int x = threadIdx.x; x < nw; x += THREADS) sk[x + 2] = keys[s + x];
     }
     if (threadIdx.x == 0) {
-        sk[1] = s > lo ? keys[s - 1] : ~0ull;
-        sk[nw + 2] = ~0ull;
+        S.count = 0;
+        sk[1] = s > lo ? keys[s - 1] : ~keys[s];
     }
     __syncthreads();
     const uint64_t lim = uint64_t(1) << shift0;   // equal upper bits <=> xor below lim
     const uint64_t lowm = lim - 1;
-    // start masks; positions past the loaded ones count as starts
+    // a run crossing the tile's end: its members past the end move too
+    const bool crossing = te == kRunTile && nw > te && (sk[te + 2] ^ sk[te + 1]) < lim;
+    const int tm = crossing ? nw : te;
+    // start masks (positions past the loaded ones count as starts), and the
+    // list of the members of longer runs, in any order
     bool multi = false;
     for (int c = warp; c < kRunChunks; c += THREADS / 32) {
         const int x = c * 32 + lane;
         const bool st = x >= nw || ((sk[x + 2] ^ sk[x + 1]) >= lim);
         const uint32_t m = __ballot_sync(0xffffffffu, st);
         if (lane == 0) smask[c] = m;
-        multi |= (m != 0xffffffffu) && c * 32 <= te;   // includes position te (a run from te - 1)
+        bool next = (m >> ((lane + 1) & 31)) & 1u;
+        if (lane == 31) next = x + 1 >= nw || ((sk[x + 3] ^ sk[x + 2]) >= lim);
+        const bool mem = x < tm && !(st && next);
+        const uint32_t mm = __ballot_sync(0xffffffffu, mem);
+        if (mm == 0u) continue;
+        multi = true;
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(&S.count, (uint32_t)__popc(mm));
+        at = __shfl_sync(0xffffffffu, at, 0);
+        if (mem) S.list[at + __popc(mm & ((1u << lane) - 1u))] = (uint16_t)x;
     }
     // a tile of single-key runs is done (the barrier also publishes the masks)
     if (!__syncthreads_or(multi)) return false;
-    // a run crossing the tile's end: its members past the end move too
-    const bool crossing = te == kRunTile && nw > te && !((smask[te >> 5] >> (te & 31)) & 1u);
-    int32_t dst[PER + 1];   // new position - s of the key at position x, or -1
+    const uint32_t members = S.count;
+    int32_t dst[PER + 1];   // new position - s of the key at the list's i-th place, or -1
     int32_t val[PER + 1];
     bool desc = false;
 #pragma unroll
     for (int i = 0; i <= PER; ++i) {
         dst[i] = -1;
-        const int x = i < PER ? (int)threadIdx.x + i * THREADS : te + (int)threadIdx.x;
-        if (i < PER ? x >= te : (!crossing || x >= nw)) continue;
+        const uint32_t e = threadIdx.x + (uint32_t)(i * THREADS);
+        if (e >= members) continue;
+        const int x = S.list[e];
         const int c = x >> 5, l = x & 31;
         const uint32_t m = smask[c];
         const bool st_here = (m >> l) & 1u;
-        const bool st_next = l < 31 ? ((m >> (l + 1)) & 1u) : (smask[c + 1] & 1u);
-        if (st_here && st_next) continue;               // a run of one key
         const uint64_t kx = sk[x + 2];
         if (!st_here) desc |= (kx & lowm) < (sk[x + 1] & lowm);
         // the run [a, b) from the start masks, looking at most kScan chunks
@@ -135,7 +152,7 @@ __device__ bool run_tile(uint64_t *__restrict__ keys, int32_t *__restrict__ vals
 #pragma unroll
     for (int i = 0; i <= PER; ++i) {
         if (dst[i] < 0) continue;
-        const int x = i < PER ? (int)threadIdx.x + i * THREADS : te + (int)threadIdx.x;
+        const int x = S.list[threadIdx.x + i * THREADS];
         keys[s + dst[i]] = sk[x + 2];
         vals[s + dst[i]] = val[i];
     }

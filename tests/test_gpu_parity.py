@@ -164,6 +164,25 @@ def test_sort_runs_from_tile_end(order):
     _check(pos, None, 4)
 
 
+@pytest.mark.parametrize("length", [2, 3, 31, 127, 128, 129])
+def test_sort_every_key_in_a_run(length):
+    """Every key shares its upper bits with length - 1 others, so a run-step
+    tile lists all of its 2048 positions and up to 128 beyond; runs of 128
+    and fewer are ranked there, longer ones by the block sort."""
+    rng = np.random.default_rng(length)
+    n = -(-40_000 // length)
+    cell = np.unique(rng.integers(0, 2 ** 36, n))
+    corner = np.stack([cell >> 24, (cell >> 12) & 4095, cell & 4095], 1) * 2.0 + 1.0
+    inside = rng.random((len(cell) * length, 3)) * [0.4, 0.9, 0.9]
+    pts = (np.repeat(corner, length, 0) + inside) * 2.0 ** -13
+    pts = np.concatenate([pts, [[0.0, 0.0, 0.0], [1.0, 1.0, 1.0]]]).astype(np.float32)
+    pos = pts[rng.permutation(len(pts))]
+    top = np.sort(oracle.keys(pos)[0]) >> np.uint64(23)
+    _, counts = np.unique(top, return_counts=True)
+    assert sorted(set(counts.tolist())) == [1, length]
+    _check(pos, None, 16)
+
+
 def test_lattice_complete_octree():
     pos, mass = lattice(5)
     t, o = _check(pos, mass, 1)
