@@ -12,7 +12,16 @@ namespace {
 constexpr int kRunTile = 2048;
 constexpr int kRunMax = 128;                                 // longest run ordered in place
 constexpr int kRunSpan = kRunTile + kRunMax;                 // positions a tile loads
-constexpr int kRunChunks = kRunSpan / 32 + 1;                // 32-position start masks (+ one past)
+constexpr int kRunChunks = kRunSpan / 32 + 2;                // 32-position start masks (+ one past), even
+
+// Bits 0..15 of v to the even bits.
+__device__ __forceinline__ uint32_t spread16(uint32_t v) {
+    v &= 0xffffu;
+    v = (v | (v << 8)) & 0x00ff00ffu;
+    v = (v | (v << 4)) & 0x0f0f0f0fu;
+    v = (v | (v << 2)) & 0x33333333u;
+    return (v | (v << 1)) & 0x55555555u;
+}
 
 struct RunSmem {
     // sk[x + 2] = keys[s + x] for x in [-1, nw); before the range's first key,
@@ -30,9 +39,12 @@ struct RunSmem {
 // Returns, the same in every thread, whether a key of the tile is smaller
 // than its predecessor in the same run (a descent).
 //
-// Bound by instruction issue.  In the tree workloads 2% to 8% of the keys lie
-// in runs of two and more, yet a quarter to a half of all warps hold one, so
-// the members are listed first and ranked by full warps.
+// Bound by instruction issue and by the latency of one tile's loads.  In the
+// tree workloads 2% to 8% of the keys lie in runs of two and more, yet a
+// quarter to a half of all warps hold one, so the members are listed first and
+// ranked by full warps (2^24 particles 66 to 61 us); and the start masks come
+// from the keys as they are loaded, 64 a warp step, all loads first (56 us;
+// each step loading its own keys 70).
 template <int THREADS, class QueueLong>
 __device__ bool run_tile(uint64_t *__restrict__ keys, int32_t *__restrict__ vals, int64_t lo, int64_t s,
                          int64_t hi, int shift0, RunSmem &S, QueueLong queue_long) {
@@ -42,42 +54,64 @@ __device__ bool run_tile(uint64_t *__restrict__ keys, int32_t *__restrict__ vals
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int te = (int)min64(kRunTile, hi - s);
     const int nw = (int)min64(kRunSpan, hi - s);
-    if ((reinterpret_cast<uintptr_t>(keys + s) & 15u) == 0) {
-        const ulonglong2 *src2 = reinterpret_cast<const ulonglong2 *>(keys + s);
-        ulonglong2 *dst2 = reinterpret_cast<ulonglong2 *>(sk + 2);
-        for (int x = threadIdx.x; x < nw / 2; x += THREADS) dst2[x] = src2[x];
-        if (threadIdx.x == 0 && (nw & 1)) sk[nw + 1] = keys[s + nw - 1];
-    } else {
-        for (int x = threadIdx.x; x < nw; x += THREADS) sk[x + 2] = keys[s + x];
-    }
-    if (threadIdx.x == 0) {
-        S.count = 0;
-        sk[1] = s > lo ? keys[s - 1] : ~keys[s];
-    }
-    __syncthreads();
     const uint64_t lim = uint64_t(1) << shift0;   // equal upper bits <=> xor below lim
     const uint64_t lowm = lim - 1;
     // a run crossing the tile's end: its members past the end move too
-    const bool crossing = te == kRunTile && nw > te && (sk[te + 2] ^ sk[te + 1]) < lim;
+    const bool crossing = te == kRunTile && nw > te && (keys[s + te] ^ keys[s + te - 1]) < lim;
     const int tm = crossing ? nw : te;
-    // start masks (positions past the loaded ones count as starts), and the
-    // list of the members of longer runs, in any order
+    const bool vec = (reinterpret_cast<uintptr_t>(keys + s) & 15u) == 0;
+    if (threadIdx.x == 0) S.count = 0;
+    __syncthreads();
+    // keys, start masks (positions past the loaded ones count as starts) and
+    // the list of the members of longer runs, in any order: two neighbouring
+    // positions a thread, 64 a warp
     bool multi = false;
-    for (int c = warp; c < kRunChunks; c += THREADS / 32) {
-        const int x = c * 32 + lane;
-        const bool st = x >= nw || ((sk[x + 2] ^ sk[x + 1]) >= lim);
-        const uint32_t m = __ballot_sync(0xffffffffu, st);
-        if (lane == 0) smask[c] = m;
-        bool next = (m >> ((lane + 1) & 31)) & 1u;
-        if (lane == 31) next = x + 1 >= nw || ((sk[x + 3] ^ sk[x + 2]) >= lim);
-        const bool mem = x < tm && !(st && next);
-        const uint32_t mm = __ballot_sync(0xffffffffu, mem);
-        if (mm == 0u) continue;
+    constexpr int ROUNDS = (kRunChunks * 32 + 2 * THREADS - 1) / (2 * THREADS);
+    uint64_t r0[ROUNDS], r1[ROUNDS], re[ROUNDS];
+#pragma unroll
+    for (int i = 0; i < ROUNDS; ++i) {
+        const int x = warp * 64 + i * 2 * THREADS + 2 * lane;
+        r0[i] = r1[i] = re[i] = 0;
+        if (vec && x + 1 < nw) {
+            const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(keys + s + x);
+            r0[i] = v.x;
+            r1[i] = v.y;
+        } else if (x < nw) {
+            r0[i] = keys[s + x];
+            if (x + 1 < nw) r1[i] = keys[s + x + 1];
+        }
+        // lane 0: the key before the warp's first; lane 31: the key after its last
+        const int y = lane == 0 ? x - 1 : x + 2;
+        if ((lane == 0 || lane == 31) && y < nw && x < nw && s + y >= lo) re[i] = keys[s + y];
+    }
+#pragma unroll
+    for (int i = 0; i < ROUNDS; ++i) {
+        const int w0 = warp * 64 + i * 2 * THREADS;
+        if (w0 >= kRunChunks * 32) break;
+        const int x = w0 + 2 * lane;
+        const uint64_t k0 = r0[i], k1 = r1[i];
+        const uint64_t edge = x == 0 && s == lo ? ~k0 : re[i];
+        if (x + 1 < nw) *reinterpret_cast<ulonglong2 *>(sk + x + 2) = make_ulonglong2(k0, k1);
+        else if (x < nw) sk[x + 2] = k0;
+        if (x == 0) sk[1] = edge;
+        uint64_t before = __shfl_up_sync(0xffffffffu, k1, 1);
+        if (lane == 0) before = edge;
+        const bool st0 = x >= nw || (k0 ^ before) >= lim;
+        const bool st1 = x + 1 >= nw || (k1 ^ k0) >= lim;
+        const uint32_t b0 = __ballot_sync(0xffffffffu, st0), b1 = __ballot_sync(0xffffffffu, st1);
+        bool st2 = (b0 >> ((lane + 1) & 31)) & 1u;
+        if (lane == 31) st2 = x + 2 >= nw || (edge ^ k1) >= lim;
+        const bool in0 = x < tm && !(st0 && st1), in1 = x + 1 < tm && !(st1 && st2);
+        if (lane < 2) smask[(w0 >> 5) + lane] = spread16(b0 >> (16 * lane)) | (spread16(b1 >> (16 * lane)) << 1);
+        const uint32_t m0 = __ballot_sync(0xffffffffu, in0), m1 = __ballot_sync(0xffffffffu, in1);
+        if ((m0 | m1) == 0u) continue;
         multi = true;
         uint32_t at = 0;
-        if (lane == 0) at = atomicAdd(&S.count, (uint32_t)__popc(mm));
+        if (lane == 0) at = atomicAdd(&S.count, (uint32_t)(__popc(m0) + __popc(m1)));
         at = __shfl_sync(0xffffffffu, at, 0);
-        if (mem) S.list[at + __popc(mm & ((1u << lane) - 1u))] = (uint16_t)x;
+        const uint32_t below = (1u << lane) - 1u;
+        if (in0) S.list[at + __popc(m0 & below)] = (uint16_t)x;
+        if (in1) S.list[at + __popc(m0) + __popc(m1 & below)] = (uint16_t)(x + 1);
     }
     // a tile of single-key runs is done (the barrier also publishes the masks)
     if (!__syncthreads_or(multi)) return false;
