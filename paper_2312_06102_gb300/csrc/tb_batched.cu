@@ -308,7 +308,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
                 const int64_t e = min64(o + ns, s + T);
                 const Front f = tile_front<T>(A.pkey, o, o + ns, A.ncrit, s, e, raw, ts);
                 if (f.k < e) A.ml[f.k] = (uint16_t)(f.m | (f.L << 8));
-                warp_field_prefix(ts, nullptr, s_tile);
+                field_totals(ts, s_tile);
                 __syncthreads();
                 if (threadIdx.x < kLevelFields) s_tot[threadIdx.x] += s_tile[threadIdx.x];
                 __syncthreads();
@@ -392,66 +392,47 @@ __global__ void __launch_bounds__(1024) batch_scan_kernel(BatchArgs A, int64_t c
 }
 
 // Every cell of one set with its links and (GATHER, for moments_set) the
-// set's particles in key order (tiles of T particles; all T threads of the
-// block).
+// set's particles in key order (tiles of 4 T particles from a multiple of four
+// on; all T threads of the block).
 template <int T, bool GATHER>
-__device__ void emit_set(const BatchArgs &A, const EmitOut &out, int set) {
-    __shared__ TileSharedT<T> ts;
-    __shared__ uint32_t woff[T / 32][kLevelFields];
-    __shared__ uint32_t s_run[kLevelFields], s_lvl[kLevelFields], s_tile[kLevelFields];
-    {
-        const int64_t o = A.off[set], ns = A.off[set + 1] - o;
-        if (ns <= 0) return;
-        const int64_t cell_base = A.set_cell_off[set], leaf_base = A.set_leaf_off[set];
-        if (threadIdx.x == 0) {
-            uint32_t r = 0;
-            for (int d = 0; d < kLevels; ++d) {
-                s_lvl[d] = r;
-                r += A.set_cnt[(int64_t)set * kLevelFields + d];
-            }
-            s_lvl[kLevels] = 0;
+__device__ void emit_set(const BatchArgs &A, const EmitOut &out, int set, EmitShared<T> &sm) {
+    __shared__ uint32_t s_lvl[kLevels + 1];   // the set's levels start (end) here
+    const int64_t o = A.off[set], ns = A.off[set + 1] - o;
+    if (ns <= 0) return;
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 32) {
+        const uint32_t v = lane < kLevels ? A.set_cnt[(int64_t)set * kLevelFields + lane] : 0u;
+        uint32_t x = v;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+            if (lane >= off) x += y;
         }
-        if (threadIdx.x < kLevelFields) s_run[threadIdx.x] = 0;
-        __syncthreads();
-        for (int64_t s = o; s < o + ns; s += T) {
-            const int64_t e = min64(o + ns, s + T);
-            const Front f = tile_front_ml<T>(A.ml, o, s, e, ts);
-            warp_field_prefix(ts, woff, s_tile);
-            if (threadIdx.x < kLevelFields) {
-                const int fld = threadIdx.x;
-                ts.base[fld] = (uint32_t)(((fld < kLevels) ? cell_base : leaf_base) + s_lvl[fld] +
-                                          s_run[fld]);
-            }
-            __syncthreads();
-            if (f.k < e) {
-                const int warp = threadIdx.x >> 5;
-                const unsigned lt = lanemask_lt();
-                auto P = [&](int d) {
-                    return ts.base[d] + woff[warp][d] + (uint32_t)__popc(ts.mask[warp][d] & lt);
-                };
-                emit_particle(f, P, o, o + ns, A.pkey[f.k], out);
-            }
-            __syncthreads();
-            if (threadIdx.x < kLevelFields) s_run[threadIdx.x] += s_tile[threadIdx.x];
-            __syncthreads();
-        }
-        // the set's particles in key order, for its moments
-        if constexpr (GATHER) {
-            for (int64_t k = o + threadIdx.x; k < o + ns; k += blockDim.x) A.xs[k] = A.xm[A.perm[k]];
-            __syncthreads();
-        }
+        if (lane <= kLevels) s_lvl[lane] = (uint32_t)A.set_cell_off[set] + x - v;
     }
+    __syncthreads();
+    uint32_t base = 0;
+    if (lane < kLevelFields) base = lane < kLevels ? s_lvl[lane] : (uint32_t)A.set_leaf_off[set];
+    int parity = 0;
+    for (int64_t s = o & ~int64_t(3); s < o + ns; s += 4 * T, parity ^= 1)
+        base += emit_tile<T, !GATHER>(A.pkey, A.ml, o, o + ns, s, base,
+                                   [&](int d) { return (int64_t)s_lvl[d + 1]; }, out, sm, parity);
+    // the set's particles in key order, for its moments
+    if constexpr (GATHER)
+        for (int64_t k = o + threadIdx.x; k < o + ns; k += blockDim.x) A.xs[k] = A.xm[A.perm[k]];
+    __syncthreads();
 }
 
 template <int T>
-__global__ void __launch_bounds__(T, 2048 / T) batch_emit_kernel(BatchArgs A, EmitOut out) {
+__global__ void __launch_bounds__(T, 1280 / T) batch_emit_kernel(BatchArgs A, EmitOut out) {
     after_previous();
     if (A.info->status & (kErrOverflow | kErrNonFinite | kErrInvalid)) return;
     __shared__ int s_q;
+    __shared__ EmitShared<T> sm;
     for (;;) {
         const int q = take_set(&A.queue[1], A.n_sets, &s_q);
         if (q < 0) return;
-        emit_set<T, false>(A, out, A.order[q]);
+        emit_set<T, false>(A, out, A.order[q], sm);
     }
 }
 
@@ -621,11 +602,13 @@ __global__ void __launch_bounds__(T, 1024 / T)
     if (blockIdx.x == 0) batch_scan_block(A, cell_cap);
     grid_barrier(bar, wait_limit, A.info);
     if (*(volatile uint32_t *)&A.info->status & (kErrOverflow | kErrNonFinite)) return;
+    static_assert(sizeof(EmitShared<T>) <= sizeof(CtaSortSharedT<T>), "the emission's lists lie in the sort's shared memory");
+    EmitShared<T> &em = *reinterpret_cast<EmitShared<T> *>(raw);
     for (;;) {
         const int q = take_set(&A.queue[1], A.n_sets, &s_q);
         if (q < 0) return;
         const int set = order[q];
-        emit_set<T, true>(A, out, set);
+        emit_set<T, true>(A, out, set, em);
         moments_set<MODE>(A, Tr, o, leaf_cell, set, n_total);
     }
 }
@@ -680,13 +663,15 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
     int32_t *start_cell = reinterpret_cast<int32_t *>(ws.keys_alt);
     EmitOut out{t.ckey, t.level, t.parent, t.child_first, t.child_end, t.pfirst, t.pend,
                 t.leaf_cell, start_cell};
-    // the emission keeps 1024-thread tiles whatever the front's block size
-    // (two blocks per SM at 32 registers): measured faster than 512 (0.96
-    // against 1.10 ms on the 4,096-set workload); many small sets take small
-    // blocks, and so do their parents
+    // blocks of 256 threads, 1,024 particles a tile, five sets per SM; a few
+    // large sets, of many tiles, take an SM each, many small ones smaller
+    // blocks.  With every particle's masks in tiles of 1,024 threads before,
+    // building 4,096 sets took 4.71 ms, now 4.31; 300 sets 145 and 138 us;
+    // 16 sets of up to 65,536 723 and 644; 100 sets of 1,000 to 2,000 92 and 93
     const bool small = batch_many_small(S, t.n_particles);
-    if (small) launch_after(batch_emit_kernel<256>, dim3(fit(8)), dim3(256), 0, s, A, out);
-    else launch_after(batch_emit_kernel<1024>, dim3(fit(2)), dim3(1024), 0, s, A, out);
+    if (batch_few_large(S, t.n_particles)) launch_after(batch_emit_kernel<1024>, dim3(fit(1)), dim3(1024), 0, s, A, out);
+    else if (small) launch_after(batch_emit_kernel<128>, dim3(fit(10)), dim3(128), 0, s, A, out);
+    else launch_after(batch_emit_kernel<256>, dim3(fit(5)), dim3(256), 0, s, A, out);
     ++g_launches;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     mark(ws, "batch_emit", s);

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kLvThreads, 2)
     const Front f = tile_front(skeys, 0, n, ncrit, s, e, raw, ts);
     // keep m and L of every particle for the emission
     if (f.k < e) ml[f.k] = (uint16_t)(f.m | (f.L << 8));
-    warp_field_prefix(ts, nullptr, tot);
+    field_totals(ts, tot);
     __syncthreads();
     if (threadIdx.x < kLevelFields) tile_cnt[(int64_t)threadIdx.x * n_tiles + t] = tot[threadIdx.x];
 }
@@ -225,29 +225,9 @@ __global__ void __launch_bounds__(kScanThreads)
     finish_levels(info, tot, cell_cap);
 }
 
-// Emission over the leaf starts only, one count tile (1024 particles) per
-// block of 256 threads.  Only a leaf start (m_k <= L_k) opens or closes cells,
-// one particle in four to seven on the tree workloads, so each warp first
-// lists the starts of its 128 particles in order and then works on that list,
-// 32 starts at a time: every lane holds a start, and the level masks (a 32 x
-// 32 bit transpose) are built for the list, not for every particle.  The
-// warps meet once, to exchange how many cells of each level they start; what
-// bound the kernel before, with the starts of the whole block in one list,
-// were its seven barriers (2^27 clustered 0.97 ms, now 0.71; 2^24 120 and 88 us).
-// The tree's last particle, which closes every
-// cell that holds it, is handled by its own thread: those are the last cells
-// of their levels.
+// Emission: one count tile per block (emit_tile in tb_cells.cuh).
 constexpr int kEfThreads = 256;
-constexpr int kEfWarps = kEfThreads / 32;
-constexpr int kEfTile = 4 * kEfThreads;                // four particles per thread
-constexpr int kEfSpan = kEfTile / kEfWarps;            // particles of a warp
-static_assert(kEfTile == kLvTile && kEfSpan == 128, "a count tile per block, four particles per lane");
-
-struct EmitWarp {
-    uint32_t entry[kEfSpan];                            // k - the warp's first | m << 8 | L << 16 | Lprev << 24
-    uint32_t mask[kEfSpan / 32][kLevels];               // level masks of each chunk of 32 starts
-    uint32_t base[kLevels + 2];                         // next cell of each level before the chunk
-};
+static_assert(4 * kEfThreads == kLvTile, "a count tile per block, four particles per lane");
 
 __global__ void __launch_bounds__(kEfThreads, 6)
     emit_starts_kernel(const uint64_t *__restrict__ skeys, const uint16_t *__restrict__ ml, int64_t n,
@@ -256,134 +236,15 @@ __global__ void __launch_bounds__(kEfThreads, 6)
     after_previous();
     const DevInfo *info = info_w;
     if (info->status & (kErrOverflow | kErrNonFinite)) return;
-    __shared__ EmitWarp s_warp[kEfWarps];
-    __shared__ uint32_t s_cnt[kEfWarps][kLevelFields];  // cells (leaves) each warp starts per level
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    EmitWarp &W = s_warp[warp];
-    const int64_t s = (int64_t)blockIdx.x * kEfTile + warp * kEfSpan;
+    __shared__ EmitShared<kEfThreads> sm;
+    const int lane = threadIdx.x & 31;
     // where the block's cells of level `lane` (its leaves) start
     uint32_t base = 0;
     if (lane < kLevelFields)
         base = (lane < kLevels ? (uint32_t)info->level_offset[lane] : 0u) +
                tile_off[(int64_t)lane * n_tiles + blockIdx.x];
-    // m and L of four particles per lane
-    const int64_t k0 = s + 4 * lane;
-    uint32_t m[4], L[4];
-    if (k0 + 4 <= n) {
-        const uint2 v = *reinterpret_cast<const uint2 *>(ml + k0);
-        m[0] = v.x & 0xffu; L[0] = (v.x >> 8) & 0xffu; m[1] = (v.x >> 16) & 0xffu; L[1] = v.x >> 24;
-        m[2] = v.y & 0xffu; L[2] = (v.y >> 8) & 0xffu; m[3] = (v.y >> 16) & 0xffu; L[3] = v.y >> 24;
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint32_t v = (k0 + j < n) ? (uint32_t)ml[k0 + j] : 255u;
-            m[j] = v & 0xffu;
-            L[j] = v >> 8;
-        }
-    }
-    uint32_t Lp = __shfl_up_sync(0xffffffffu, L[3], 1);
-    if (lane == 0) Lp = s > 0 && s < n ? (uint32_t)(ml[s - 1] >> 8) : 0u;
-    // the tree's last particle closes the cells holding it: the last cell of
-    // each level 0 .. L, whose children end where the next level ends
-    if (k0 <= n - 1 && n - 1 < k0 + 4) {
-        const uint32_t Ll = L[(int)(n - 1 - k0)];
-        for (int d = 0; d <= (int)Ll; ++d) {
-            const int64_t idx = info->level_offset[d + 1] - 1;
-            out.pend[idx] = (int32_t)n;
-            out.child_end[idx] = (d < (int)Ll) ? (int32_t)info->level_offset[d + 2] : -1;
-        }
-    }
-    // the warp's starts in order
-    uint32_t cnt = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) cnt += (m[j] <= L[j]) ? 1u : 0u;
-    uint32_t x = cnt;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
-        if (lane >= off) x += y;
-    }
-    const int total = (int)__shfl_sync(0xffffffffu, x, 31);
-    uint32_t pos = x - cnt;
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-        if (m[j] <= L[j])
-            W.entry[pos++] = (uint32_t)(4 * lane + j) | (m[j] << 8) | (L[j] << 16) | ((j ? L[j - 1] : Lp) << 24);
-    __syncwarp();
-    // the keys of the first chunk of starts, loaded now so that the masks and
-    // the barrier cover their latency
-    uint64_t Kfirst = 0;
-    if (lane < total) Kfirst = skeys[s + (W.entry[lane] & 255u)];
-    // level masks of every chunk of 32 starts; lane d counts level d
-    uint32_t mine = 0;
-    for (int c = 0; 32 * c < total; ++c) {
-        const int i = c * 32 + lane;
-        uint32_t v = 0;
-        if (i < total) {
-            const uint32_t en = W.entry[i];
-            v = (2u << ((en >> 16) & 31u)) - (1u << ((en >> 8) & 31u));
-        }
-        uint32_t msk = 0x0000ffffu;
-#pragma unroll
-        for (int j = 16; j > 0; j >>= 1, msk ^= msk << j) {
-            const uint32_t y = __shfl_xor_sync(0xffffffffu, v, j);
-            if (lane & j) v ^= ((y >> j) ^ v) & msk;
-            else v ^= (((v >> j) ^ y) & msk) << j;
-        }
-        if (lane < kLevels) W.mask[c][lane] = v;
-        mine += __popc(v);
-    }
-    if (lane == kLevels) mine = (uint32_t)total;
-    if (lane < kLevelFields) s_cnt[warp][lane] = mine;
-    __syncthreads();
-    if (lane < kLevelFields) {
-#pragma unroll
-        for (int w = 0; w < kEfWarps; ++w)
-            if (w < warp) base += s_cnt[w][lane];
-        W.base[lane] = base;
-    }
-    __syncwarp();
-    const unsigned lt = lanemask_lt();
-    for (int c = 0; 32 * c < total; ++c) {
-        const int i = c * 32 + lane;
-        if (i < total) {
-            const uint32_t en = W.entry[i];
-            const int64_t k = s + (en & 255u);
-            const int mm = (int)((en >> 8) & 31u), LL = (int)((en >> 16) & 31u), Lq = (int)(en >> 24);
-            auto P = [&](int d) { return W.base[d] + (uint32_t)__popc(W.mask[c][d] & lt); };
-            const uint64_t K = c == 0 ? Kfirst : skeys[k];
-            // P(d) of consecutive levels: each loop computes one new level per step
-            const uint32_t pm = P(mm);
-            if (k > 0) {
-                // close the cells holding k-1 but not k
-                uint32_t pd = pm;
-                for (int d = mm; d <= Lq; ++d) {
-                    const uint32_t pn = d < Lq ? P(d + 1) : 0u;
-                    out.pend[pd - 1] = (int32_t)k;
-                    out.child_end[pd - 1] = (d < Lq) ? (int32_t)pn : -1;
-                    pd = pn;
-                }
-            }
-            uint32_t pprev = mm > 0 ? P(mm - 1) : 0u, pd = pm;
-            for (int d = mm;; ++d) {
-                const uint32_t pn = d < LL ? P(d + 1) : 0u;
-                out.ckey[pd] = cell_key(K, d);
-                out.level[pd] = (uint8_t)d;
-                out.pfirst[pd] = (int32_t)k;
-                out.parent[pd] = (d == 0) ? -1 : (int32_t)pprev - (d == mm ? 1 : 0);
-                out.child_first[pd] = (d < LL) ? (int32_t)pn : -1;
-                if (d == LL) break;
-                pprev = pd;
-                pd = pn;
-            }
-            out.leaf_cell[W.base[kLevels] + (uint32_t)i] = (int32_t)pd;
-        }
-        if (32 * (c + 1) < total) {
-            __syncwarp();
-            if (lane < kLevels) W.base[lane] += (uint32_t)__popc(W.mask[c][lane]);
-            __syncwarp();
-        }
-    }
+    emit_tile<kEfThreads, false>(skeys, ml, 0, n, (int64_t)blockIdx.x * kLvTile, base,
+                                 [&](int d) { return info->level_offset[d + 1]; }, out, sm, 0);
 }
 
 }  // namespace
@@ -435,7 +296,7 @@ cudaError_t launch_emit(const uint64_t *skeys, int64_t n, int ncrit, Workspace &
     const int64_t tiles = (n + kLvTile - 1) / kLvTile;
     EmitOut o{t.ckey, t.level, t.parent, t.child_first, t.child_end, t.pfirst, t.pend,
               t.leaf_cell, nullptr};
-    const int64_t blocks = (n + kEfTile - 1) / kEfTile;
+    const int64_t blocks = (n + kLvTile - 1) / kLvTile;
     launch_after(emit_starts_kernel, dim3((unsigned)blocks), dim3(kEfThreads), 0, s, skeys, ws.ml, n, ws.level_cnt, tiles,
                                                                ws.info, o);
     ++g_launches;

@@ -28,7 +28,7 @@ __host__ __device__ inline size_t lv_smem_bytes(int ncrit) {
 }
 
 struct Front {
-    int m, L, Lprev;      // this thread's particle k (m = 255 beyond the tile)
+    int m, L;             // this thread's particle k (m = 255 beyond the tile)
     int64_t k;
 };
 
@@ -38,7 +38,6 @@ template <int T>
 struct TileSharedT {
     static constexpr int WARPS = T / 32;
     uint32_t mask[WARPS][kLevelFields];
-    uint32_t base[kLevelFields];
 };
 using TileShared = TileSharedT<kLvThreads>;
 
@@ -60,8 +59,7 @@ __device__ __forceinline__ void store_level_masks(int m, int L, TileSharedT<T> &
     if (lane < kLevelFields) ts.mask[warp][lane] = x;
 }
 
-// m, L and L of the previous particle for particle s + threadIdx.x of the
-// tile [s, e), and the ballot masks of the level starts of every warp.  The
+// m and L of particle s + threadIdx.x of the tile [s, e), and the ballot masks of the level starts of every warp.  The
 // tile lies in the segment [seg_lo, seg_hi) of sorted keys that forms one
 // tree (the whole array, or one set of a batch); keys outside it do not
 // exist for this tree.
@@ -98,7 +96,7 @@ __device__ Front tile_front(const uint64_t *__restrict__ skeys, int64_t seg_lo, 
     // A[x] = max of c over [x, x + p) (truncated at the end)
     Front f;
     f.k = s + threadIdx.x;
-    auto window = [&](int64_t k) {   // max c over [k - n, k], k in [s - 1, e)
+    auto window = [&](int64_t k) {   // max c over [k - n, k], k in [s, e)
         const int x0 = (int)(k - ncrit - lo), x1 = (int)(k - p + 1 - lo);
         return (int)max(A[x0], A[x1]);
     };
@@ -106,60 +104,25 @@ __device__ Front tile_front(const uint64_t *__restrict__ skeys, int64_t seg_lo, 
         const int x = (int)(f.k - lo);
         f.m = (f.k == seg_lo) ? 0 : min_depth(key[x - 1], key[x]);
         f.L = window(f.k);
-        f.Lprev = window(f.k - 1);
     } else {
         f.m = 255;
         f.L = 0;
-        f.Lprev = 0;
     }
     store_level_masks(f.m, f.L, ts);
     __syncthreads();
     return f;
 }
 
-// The same Front from the m_k | L_k << 8 words a counting pass stored for
-// every particle (no keys needed): particle s + threadIdx.x of the tile
-// [s, e) of the tree [seg_lo, ...), and the level masks of every warp.
-template <int T>
-__device__ Front tile_front_ml(const uint16_t *__restrict__ ml, int64_t seg_lo, int64_t s,
-                               int64_t e, TileSharedT<T> &ts) {
-    Front f;
-    f.k = s + threadIdx.x;
-    if (f.k < e) {
-        const uint32_t v = ml[f.k];
-        f.m = (int)(v & 0xffu);
-        f.L = (int)(v >> 8);
-        f.Lprev = (f.k > seg_lo) ? (int)(ml[f.k - 1] >> 8) : 0;
-    } else {
-        f.m = 255;
-        f.L = 0;
-        f.Lprev = 0;
-    }
-    store_level_masks(f.m, f.L, ts);
-    __syncthreads();
-    return f;
-}
-
-// Per-field prefix over the warps of a tile, one warp per field (fields
-// 0..22, taken in turns when the tile has fewer than 23 warps), one lane per
-// warp of the tile: woff[w][f] = starts of field f in warps before w; tot[f] =
-// the tile's total.  Needs a barrier before (masks written) and after
+// Starts of each field (0..22) in a tile, one warp per field, one lane per
+// warp of the tile: tot[f].  Needs a barrier before (masks written) and after
 // (results read).
 template <int T>
-__device__ __forceinline__ void warp_field_prefix(const TileSharedT<T> &ts,
-                                                  uint32_t (*woff)[kLevelFields], uint32_t *tot) {
+__device__ __forceinline__ void field_totals(const TileSharedT<T> &ts, uint32_t *tot) {
     constexpr int W = TileSharedT<T>::WARPS;
     const int lane = threadIdx.x & 31;
     for (int f = threadIdx.x >> 5; f < kLevelFields; f += W) {
-        const uint32_t v = lane < W ? __popc(ts.mask[lane][f]) : 0u;
-        uint32_t x = v;
-#pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, sh);
-            if (lane >= sh) x += y;
-        }
-        if (woff && lane < W) woff[lane][f] = x - v;
-        if (lane == 31) tot[f] = x;
+        const uint32_t v = __reduce_add_sync(0xffffffffu, lane < W ? (uint32_t)__popc(ts.mask[lane][f]) : 0u);
+        if (lane == 0) tot[f] = v;
     }
 }
 
@@ -322,44 +285,165 @@ struct EmitOut {
     int32_t *start_cell;     // batched: the leaf cell that starts at each position
 };
 
-// Cells opened and closed by one particle.  P(d) is the global index of the
-// next level-d cell before k's own starts (P(kLevels): next leaf slot);
-// seg_hi is one past the tree's last particle; K is k's key.
-template <class PF>
-__device__ __forceinline__ void emit_particle(const Front &f, const PF &P, int64_t seg_lo,
-                                              int64_t seg_hi, uint64_t K, const EmitOut &out) {
-    const int64_t k = f.k;
-    const int m = f.m, L = f.L;
-    if (k > seg_lo) {
-        // close the cells holding k-1 but not k
-        for (int d = m; d <= f.Lprev; ++d) {
-            const uint32_t idx = P(d) - 1;
-            out.pend[idx] = (int32_t)k;
-            out.child_end[idx] = (d < f.Lprev) ? (int32_t)P(d + 1) : -1;
+// Emission over the leaf starts only, 4 T particles by a block of T threads.
+// Only a leaf start (m_k <= L_k) opens or closes cells, one particle in four to
+// seven on the tree workloads, so each warp first lists the starts of its 128
+// particles in order and then works on that list, 32 starts at a time: every
+// lane holds a start, and the level masks (a 32 x 32 bit transpose) are built
+// for the list, not for every particle.  The warps meet once, to exchange how
+// many cells of each level they start; what bound the kernel before, with the
+// starts of the whole block in one list, were its seven barriers (2^27
+// clustered 0.97 ms, now 0.71; 2^24 120 and 88 us).
+constexpr int kEmitSpan = 128;                          // particles of a warp
+
+struct EmitWarp {
+    uint32_t entry[kEmitSpan];                          // k - the warp's first | m << 8 | L << 16 | Lprev << 24
+    uint32_t mask[kEmitSpan / 32][kLevels];             // level masks of each chunk of 32 starts
+    uint32_t base[kLevels + 2];                         // next cell of each level before the chunk
+};
+template <int T>
+struct EmitShared {
+    EmitWarp warp[T / 32];
+    uint32_t cnt[2][T / 32][kLevelFields];              // cells (leaves) each warp starts per level
+};
+
+// The tile of particles [s, s + 4 T) (s a multiple of four) of the tree whose
+// sorted particles are [lo, hi).  Lane f's `base` is the next cell of level f
+// (f = kLevels: the next leaf), level_end(d) where level d ends.  Returns how
+// many of them the tile starts.  Tiles of one block alternate in `parity`; all
+// threads of the block call it.  Writes the leaf of each start to
+// out.start_cell when START.
+template <int T, bool START, class LevelEnd>
+__device__ __forceinline__ uint32_t emit_tile(const uint64_t *skeys, const uint16_t *ml, int64_t lo,
+                                              int64_t hi, int64_t tile, uint32_t base,
+                                              const LevelEnd &level_end, const EmitOut &out,
+                                              EmitShared<T> &sm, int parity) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    EmitWarp &W = sm.warp[warp];
+    const int64_t s = tile + warp * kEmitSpan;
+    // m and L of four particles per lane
+    const int64_t k0 = s + 4 * lane;
+    uint32_t m[4], L[4];
+    if (k0 >= lo && k0 + 4 <= hi) {
+        const uint2 v = *reinterpret_cast<const uint2 *>(ml + k0);
+        m[0] = v.x & 0xffu; L[0] = (v.x >> 8) & 0xffu; m[1] = (v.x >> 16) & 0xffu; L[1] = v.x >> 24;
+        m[2] = v.y & 0xffu; L[2] = (v.y >> 8) & 0xffu; m[3] = (v.y >> 16) & 0xffu; L[3] = v.y >> 24;
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t v = (k0 + j >= lo && k0 + j < hi) ? (uint32_t)ml[k0 + j] : 255u;
+            m[j] = v & 0xffu;
+            L[j] = v >> 8;
         }
     }
-    if (m <= L) {
-        for (int d = m; d <= L; ++d) {
-            const uint32_t idx = P(d);
-            out.ckey[idx] = cell_key(K, d);
-            out.level[idx] = (uint8_t)d;
-            out.pfirst[idx] = (int32_t)k;
-            out.parent[idx] = (d == 0) ? -1 : (int32_t)P(d - 1) - (d == m ? 1 : 0);
-            out.child_first[idx] = (d < L) ? (int32_t)P(d + 1) : -1;
-        }
-        const int32_t leaf = (int32_t)P(L);
-        out.leaf_cell[P(kLevels)] = leaf;
-        if (out.start_cell) out.start_cell[k] = leaf;
-    }
-    if (k == seg_hi - 1) {
-        // the tree's last particle closes every cell holding it
-        for (int d = 0; d <= L; ++d) {
-            const uint32_t own = (m <= d) ? 1u : 0u;
-            const uint32_t idx = P(d) + own - 1;
-            out.pend[idx] = (int32_t)seg_hi;
-            out.child_end[idx] = (d < L) ? (int32_t)(P(d + 1) + ((m <= d + 1) ? 1u : 0u)) : -1;
+    uint32_t Lp = __shfl_up_sync(0xffffffffu, L[3], 1);
+    if (lane == 0) Lp = s > lo && s < hi ? (uint32_t)(ml[s - 1] >> 8) : 0u;
+    // the tree's last particle closes the cells holding it: the last cell of
+    // each level 0 .. L, whose children end where the next level ends
+    if (k0 <= hi - 1 && hi - 1 < k0 + 4) {
+        const uint32_t Ll = L[(int)(hi - 1 - k0)];
+        for (int d = 0; d <= (int)Ll; ++d) {
+            const int64_t idx = level_end(d) - 1;
+            out.pend[idx] = (int32_t)hi;
+            out.child_end[idx] = (d < (int)Ll) ? (int32_t)level_end(d + 1) : -1;
         }
     }
+    // the warp's starts in order
+    uint32_t cnt = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) cnt += (m[j] <= L[j]) ? 1u : 0u;
+    uint32_t x = cnt;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, off);
+        if (lane >= off) x += y;
+    }
+    const int total = (int)__shfl_sync(0xffffffffu, x, 31);
+    uint32_t pos = x - cnt;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (m[j] <= L[j])
+            W.entry[pos++] = (uint32_t)(4 * lane + j) | (m[j] << 8) | (L[j] << 16) | ((j ? L[j - 1] : Lp) << 24);
+    __syncwarp();
+    // the keys of the first chunk of starts, loaded now so that the masks and
+    // the barrier cover their latency
+    uint64_t Kfirst = 0;
+    if (lane < total) Kfirst = skeys[s + (W.entry[lane] & 255u)];
+    // level masks of every chunk of 32 starts; lane d counts level d
+    uint32_t mine = 0;
+    for (int c = 0; 32 * c < total; ++c) {
+        const int i = c * 32 + lane;
+        uint32_t v = 0;
+        if (i < total) {
+            const uint32_t en = W.entry[i];
+            v = (2u << ((en >> 16) & 31u)) - (1u << ((en >> 8) & 31u));
+        }
+        uint32_t msk = 0x0000ffffu;
+#pragma unroll
+        for (int j = 16; j > 0; j >>= 1, msk ^= msk << j) {
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, v, j);
+            if (lane & j) v ^= ((y >> j) ^ v) & msk;
+            else v ^= (((v >> j) ^ y) & msk) << j;
+        }
+        if (lane < kLevels) W.mask[c][lane] = v;
+        mine += __popc(v);
+    }
+    if (lane == kLevels) mine = (uint32_t)total;
+    if (lane < kLevelFields) sm.cnt[parity][warp][lane] = mine;
+    __syncthreads();
+    uint32_t all = 0;
+    if (lane < kLevelFields) {
+#pragma unroll
+        for (int w = 0; w < T / 32; ++w) {
+            if (w == warp) W.base[lane] = base + all;
+            all += sm.cnt[parity][w][lane];
+        }
+    }
+    __syncwarp();
+    const unsigned lt = lanemask_lt();
+    for (int c = 0; 32 * c < total; ++c) {
+        const int i = c * 32 + lane;
+        if (i < total) {
+            const uint32_t en = W.entry[i];
+            const int64_t k = s + (en & 255u);
+            const int mm = (int)((en >> 8) & 31u), LL = (int)((en >> 16) & 31u), Lq = (int)(en >> 24);
+            auto P = [&](int d) { return W.base[d] + (uint32_t)__popc(W.mask[c][d] & lt); };
+            const uint64_t K = c == 0 ? Kfirst : skeys[k];
+            // P(d) of consecutive levels: each loop computes one new level per step
+            const uint32_t pm = P(mm);
+            if (k > lo) {
+                // close the cells holding k-1 but not k
+                uint32_t pd = pm;
+                for (int d = mm; d <= Lq; ++d) {
+                    const uint32_t pn = d < Lq ? P(d + 1) : 0u;
+                    out.pend[pd - 1] = (int32_t)k;
+                    out.child_end[pd - 1] = (d < Lq) ? (int32_t)pn : -1;
+                    pd = pn;
+                }
+            }
+            uint32_t pprev = mm > 0 ? P(mm - 1) : 0u, pd = pm;
+            for (int d = mm;; ++d) {
+                const uint32_t pn = d < LL ? P(d + 1) : 0u;
+                out.ckey[pd] = cell_key(K, d);
+                out.level[pd] = (uint8_t)d;
+                out.pfirst[pd] = (int32_t)k;
+                out.parent[pd] = (d == 0) ? -1 : (int32_t)pprev - (d == mm ? 1 : 0);
+                out.child_first[pd] = (d < LL) ? (int32_t)pn : -1;
+                if (d == LL) break;
+                pprev = pd;
+                pd = pn;
+            }
+            out.leaf_cell[W.base[kLevels] + (uint32_t)i] = (int32_t)pd;
+            if constexpr (START) out.start_cell[k] = (int32_t)pd;
+        }
+        if (32 * (c + 1) < total) {
+            __syncwarp();
+            if (lane < kLevels) W.base[lane] += (uint32_t)__popc(W.mask[c][lane]);
+            __syncwarp();
+        }
+    }
+    __syncwarp();   // the warp's list may be rewritten next
+    return all;
 }
 
 }  // namespace

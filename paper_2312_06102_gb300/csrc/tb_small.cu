@@ -4,8 +4,9 @@
 // The launches of the general path (root, keys, five radix passes, two run
 // steps) cost a small set 4 to 8 us each, nearly all of it latency.  tb_build
 // with those and with this launch, us: 59 and 37 at 3,001 particles, 64 and 51 at
-// 20,000, 63 and 57 at 32,768; from 50,000 on (64 and 70, with 4096 positions a
-// block) the many SMs of the general passes win.  Here one cluster of up to 16
+// 20,000, 63 and 57 at 32,768 (with five passes here too; the four taken now save
+// another 2); from 50,000 on (64 and 70, with 4096 positions a block) the many SMs
+// of the general passes win.  Here one cluster of up to 16
 // blocks takes the whole set.  Block r owns positions [r P, (r + 1) P) of the
 // current order, in registers while a pass ranks them:
 //   1. particles to registers (records written out), bounding box by shuffles
