@@ -43,9 +43,9 @@ from synth import WORKLOADS, batched_plummer, workload  # noqa: E402
 # the digest of the kernel source it was taken on; reported only while the
 # source is unchanged (see profiles/).
 NCU_TRAFFIC = {
-    # onesweep pass <8, 512, 8>, N = 2^25 clustered, passes 2, 3 and 4 of a
+    # radix passes of 256 x 21 pairs, N = 2^25 clustered, the five passes of a
     # timed build: dram__bytes_read.sum + dram__bytes_write.sum, their mean
-    "639068564be370b2": {"bytes": 770.47e6, "n": 1 << 25, "variant": (8, 512, 8)},
+    "df6d162fd8b545dd": {"bytes": 746.24e6, "n": 1 << 25, "variant": (8, 256, 21)},
 }
 
 METRIC = "tree-build Mparticles/s + HBM roofline %; batched vs plain on same GB300"
