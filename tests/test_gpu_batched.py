@@ -212,3 +212,16 @@ def test_batched_default_block_sizes(sizes):
               "pend", "mass", "com", "com_lo", "quad", "aabb"):
         assert np.array_equal(to_np(getattr(a, k)), to_np(getattr(b, k))), k
     _check_sets(a, pos, mass, offsets, 16, sets=range(0, len(n), 37 if len(n) > 50 else 1))
+
+
+@pytest.mark.parametrize("sizes", ["many small", "few large", "between"])
+def test_batched_emission_tile_ends(sizes):
+    """The emission takes a set in tiles of 512, 4096 or 1024 particles (by the
+    number and size of the sets) from a multiple of four on: sets that end one
+    particle around a tile's end, starting at every remainder."""
+    n = {"many small": [1, 510, 511, 512, 513, 514, 515, 3] * 40,
+         "few large": [4093, 4094, 4095, 4096, 4097, 4098, 8191, 8195],
+         "between": [1, 1021, 1022, 1023, 1024, 1025, 2047, 2049, 0, 3]}[sizes]
+    pos, mass, offsets = _sets(n, 33)
+    t, *_ = _run(pos, mass, offsets)
+    _check_sets(t, pos, mass, offsets, 16, sets=range(0, len(n), 1 if len(n) < 50 else 9))
