@@ -78,8 +78,7 @@ __device__ __forceinline__ void finish_levels(DevInfo *info, const uint32_t *tot
     info->max_depth = dmax;
     if (cell_cap > 0 && off > cell_cap) info->status |= kErrOverflow;
     info->misc_ctr[1] = 0;
-    // the moments' leaf queues, and the barrier count of their upward pass
-    for (int i : {2, 5, 7}) info->misc_ctr[i] = 0;
+    info->misc_ctr[2] = info->misc_ctr[5] = 0;   // the moments' leaf queues
 }
 
 // The same counts, four consecutive particles per thread, for n_crit in

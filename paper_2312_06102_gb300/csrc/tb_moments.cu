@@ -94,6 +94,8 @@ __global__ void __launch_bounds__(kLtThreads, MODE == TB_MOM_FP64 ? 3 : 4)
                      int32_t *long_queue, int32_t *big_queue, DevInfo *info, int64_t wait_limit) {
     after_previous();
     if (info->status & (kErrOverflow | kErrNonFinite | kErrTimeout | kErrInvalid)) return;
+    // the barrier count of the upward pass that follows starts from zero
+    if (blockIdx.x == 0 && threadIdx.x == 0) info->misc_ctr[7] = 0;
     extern __shared__ __align__(128) unsigned char lt_raw[];
     LeafTileSmem &S = *reinterpret_cast<LeafTileSmem *>(lt_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -765,9 +767,11 @@ __global__ void __launch_bounds__(kLmThreads, 5)
             __syncthreads();
         }
     }
-    // block 0 leaves the counters clear for the next call on this build
-    if (blockIdx.x == 0 && threadIdx.x == 0 && d_lo == 0)
-        for (int i : {2, 5, 7}) info->misc_ctr[i] = 0;
+    // block 0 leaves the queues clear for the next call on this build: every
+    // block read their lengths before the first meeting, if they were not zero.
+    // (The barrier count is not cleared here, where a block may still be on its
+    // way out of that meeting: the next leaf launch does it.)
+    if (blockIdx.x == 0 && threadIdx.x == 0 && d_lo == 0) info->misc_ctr[2] = info->misc_ctr[5] = 0;
 }
 
 __global__ void wait_selftest_kernel(int64_t limit, uint32_t *status, const uint32_t *flag) {

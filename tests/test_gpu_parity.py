@@ -391,6 +391,29 @@ def test_moments_repeat_on_one_build(mode):
             assert np.array_equal(to_np(getattr(t, k)), v), k
 
 
+@pytest.mark.parametrize("n,n_crit", [(30_000, 1000), (300_000, 100)])
+def test_moments_with_queued_leaves_many_times(n, n_crit):
+    """Leaves past the leaf tiles' halo are queued, and every block of the
+    upward pass meets after them.  30,000 particles in leaves of about 470:
+    one block goes on alone from there; 300,000 in leaves of about 75: further
+    meetings of fewer blocks follow.  The count of arrivals starts from zero in
+    every call, so that 200 calls in a row give the same bits and no timeout."""
+    pos, mass = uniform_cube(n, 61)
+    t, o = _check(pos, mass, n_crit)
+    m = tb()
+    p, w = torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda()
+    m.moments(t, p, w)
+    keys = ("mass", "com", "com_lo", "quad", "aabb")
+    a = {k: getattr(t, k).clone() for k in keys}
+    for i in range(200):
+        if i % 50 == 25:
+            m.build(p, w, n_crit=n_crit, tree=t)
+        m.moments(t, p, w)
+        for k, v in a.items():
+            assert torch.equal(getattr(t, k), v), (i, k)
+    assert t.sync() == 0
+
+
 @pytest.mark.parametrize("gen,n_crit", [("plummer", 16), ("clustered", 8), ("stress", 16),
                                          ("uniform", 1)])
 def test_root_pow2(gen, n_crit):
