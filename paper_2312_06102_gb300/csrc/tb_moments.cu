@@ -37,6 +37,14 @@ namespace tb {
 
 namespace {
 
+// A wait for bulk copies gave up: one thread waits for them again before the
+// block leaves, so that none of them lands in shared memory that has gone to
+// another block.  The caller's limit, which may be a poll or two
+// (tb_set_wait_limit), does not count here: copies depend on no other block.
+__device__ __forceinline__ void drain(uint64_t *bar, uint32_t parity) {
+    mbar_wait_bounded(bar, parity, kDefaultWaitLimit);
+}
+
 // ------------------------------------------------------------ kernels
 
 // Leaves, one block per tile of kLtTile consecutive key-order positions.
@@ -122,11 +130,11 @@ __global__ void __launch_bounds__(kLtThreads, MODE == TB_MOM_FP64 ? 3 : 4)
         ok = mbar_wait_bounded(&S.bar, phase, wait_limit);
         phase ^= 1u;
     }
-    // a copy that did not complete: record it and leave once it has
+    // a copy that did not complete in time: record it and leave once it has
     if (!__syncthreads_and(ok)) {
         if (threadIdx.x == 0) {
             flag_error(&info->status, kErrTimeout);
-            mbar_wait_bounded(&S.bar, 0, wait_limit);
+            drain(&S.bar, 0);
         }
         return;
     }
@@ -150,7 +158,7 @@ __global__ void __launch_bounds__(kLtThreads, MODE == TB_MOM_FP64 ? 3 : 4)
         if (!__syncthreads_and(ok)) {
             if (threadIdx.x == 0) {
                 flag_error(&info->status, kErrTimeout);
-                mbar_wait_bounded(&S.bar, phase, wait_limit);
+                drain(&S.bar, phase);
             }
             return;
         }
@@ -371,7 +379,7 @@ __device__ __forceinline__ bool staged_wait(LevelSmem &S, uint32_t &phase, DevIn
     if (__syncthreads_and(ok)) return true;
     if (threadIdx.x == 0) {
         flag_error(&info->status, kErrTimeout);
-        mbar_wait_bounded(&S.bar, phase ^ 1u, wait_limit);
+        drain(&S.bar, phase ^ 1u);
     }
     return false;
 }
@@ -493,7 +501,10 @@ __device__ __noinline__ void solo_levels(TreeIn T, MomOut o, DevInfo *info, Leve
         const Staged g(off[d + 1], off[d + 2], off[d + 1], off[d + 2]);
         const Staged h(off[d], off[d + 1], off[d], off[d + 1]);
         if (threadIdx.x == 0 && d > 0) stage<TB_MOM_FP32_COMP>(T, o, B, h);
-        if (!staged_wait(A, phase[cur], info, wait_limit)) return;
+        if (!staged_wait(A, phase[cur], info, wait_limit)) {
+            if (threadIdx.x == 0 && d > 0) drain(&B.bar, phase[cur ^ 1]);   // its copies too
+            return;
+        }
         const uint32_t total = list_parents(A, g);
         if (d > 0 && !staged_wait(B, phase[cur ^ 1], info, wait_limit)) return;
         if (d > 0) phase[cur ^ 1] ^= 1u;   // waited for here, not in the next step

@@ -4,6 +4,7 @@
   that a look-back which finds a predecessor tile not yet published gives up
   at once; the build reports TB_ETIMEOUT, every access stays in bounds, and
   the next build of the same tree with the default limit is exact.
+- A wait of the moments' upward pass that runs out, in the same way.
 - A device allocation that fails: the library's TB_FAULT_ALLOC=k hook makes
   its k-th cudaMalloc fail in a child process; the build reports TB_ENOMEM
   and releasing the half-made tree succeeds.
@@ -51,6 +52,34 @@ def test_lookback_wait_runs_out_then_next_build_is_exact():
     torch.cuda.synchronize()
     assert t.sync() == 0
     assert_structure_equal(t, oracle.build_tree(pos, 16))
+
+
+@pytest.mark.parametrize("n,mode", [(20_000, 0), (400_000, 0), (400_000, 2)])
+def test_moment_waits_run_out_then_next_build_is_exact(n, mode):
+    """The moments under a limit of one poll: whichever of their waits give up
+    (for staged copies, which are then waited for before the block leaves, or
+    for other blocks), the call ends, reports TB_ETIMEOUT if any did, and the
+    next build and moments are exact."""
+    m = tb()
+    pos, mass = uniform_cube(n, 29)
+    p, w = torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda()
+    t = m.moments(m.build(p, w, mom_mode=mode), p, w)
+    assert t.sync() == 0
+    keys = ("mass", "com", "com_lo", "quad", "aabb")
+    want = {k: getattr(t, k).clone() for k in keys}
+    for _ in range(20):
+        m.build(p, w, mom_mode=mode, tree=t)
+        m.set_wait_limit(1)
+        try:
+            m.moments(t, p, w)
+            st = t.sync()
+        finally:
+            m.set_wait_limit(0)
+        assert m.STATUS[st] in ("TB_OK", "TB_ETIMEOUT")
+    m.moments(m.build(p, w, mom_mode=mode, tree=t), p, w)
+    assert t.sync() == 0
+    for k in keys:
+        assert torch.equal(getattr(t, k), want[k]), k
 
 
 _CHILD = r"""
