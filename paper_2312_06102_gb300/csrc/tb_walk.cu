@@ -166,8 +166,8 @@ __device__ __forceinline__ void eval_cells(const WarpLists &W, int from, int to,
     }
 }
 
-// One step of eight source particles; y is this lane's (m = 0 when there is
-// none).  With SELF, `slot` is the slot of this lane's targets that is the
+// One step of eight source particles; y is this lane's, eps2 its softening (a
+// missing source has no mass and a softening of 1).  With SELF, `slot` is the slot of this lane's targets that is the
 // source itself, or -1, and takes no force from it.
 template <bool SELF>
 __device__ __forceinline__ void eval_sources(float4 y, int slot, float eps2, Chunk &C) {
@@ -190,11 +190,15 @@ __device__ __forceinline__ void eval_sources(float4 y, int slot, float eps2, Chu
     }
 }
 
-// The source at sorted position q (none when !in) against the chunk [kb, ke).
+// The source at sorted position q against the chunk [kb, ke).  When !in there is
+// none: y is then some other source, and counts with no mass and a softening of
+// 1, so that the distance is not 0 even if it is a target itself.
 __device__ __forceinline__ void eval_source(float4 y, int q, bool in, int kb, int ke, float eps2,
                                             Chunk &C) {
-    // a missing source is massless and away from every target
-    if (!in) y = make_float4(1e15f, 1e15f, 1e15f, 0.f);
+    if (!in) {
+        y.w = 0.f;
+        eps2 = 1.f;
+    }
     const int t = q - kb;
     const bool mine = in && q >= kb && q < ke;
     if (__any_sync(0xffffffffu, mine))

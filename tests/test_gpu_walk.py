@@ -110,6 +110,28 @@ def test_no_worse_than_the_per_particle_walk_and_quadrupole_helps():
         assert np.median(g) < np.median(gm)
 
 
+@pytest.mark.parametrize("theta", [0.0, 0.5])
+def test_unsoftened_with_a_particle_at_any_place(theta):
+    """eps = 0 in a box of side 1e15 with a particle at each of its corners and
+    at its centre, the number of particles no multiple of the eight that a step
+    of the walk takes: the sources a step lacks must not meet a target."""
+    rng = np.random.default_rng(45)
+    pos = rng.random((1001, 3))
+    pos[:8] = [[i & 1, i >> 1 & 1, i >> 2] for i in range(8)]
+    pos[8] = 0.5
+    pos = (pos * 1e15).astype(np.float32)
+    mass = np.full(len(pos), 1e12, np.float32)         # forces of about 1e-15
+    m, t = _setup(pos, mass)
+    acc = to_np(m.walk(t, theta, 0.0, use_quad=False)).astype(np.float64)
+    assert np.isfinite(acc).all()
+    e = _rel(acc, oracle.direct_acc(pos, mass, np.arange(len(pos)), 0.0))
+    if theta == 0.0:
+        # as in the direct sum above, without a softening
+        assert np.median(e) <= 1e-5 and e.max() <= 1e-3, (np.median(e), e.max())
+    else:
+        assert np.median(e) <= 1e-1
+
+
 def test_walk_arguments():
     m = tb()
     pos, mass = plummer(3000, 44)
