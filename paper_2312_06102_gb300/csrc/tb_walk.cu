@@ -29,6 +29,8 @@
 // particle order.  A walk on a tree with profiling enabled also counts the
 // interactions it evaluated (target-cell and target-particle pairs), read
 // back by tb_walk_counts.
+#include <cfloat>
+
 #include "tb_device.cuh"
 
 namespace tb {
@@ -85,14 +87,21 @@ __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
     return v;
 }
 __device__ __forceinline__ uint64_t dup2(float a) { return pack2(a, a); }
-// 1 / sqrt, the hardware's approximation (what rsqrtf rounds to) without its
-// steps for subnormal arguments: a distance below 1e-19 overflows the force
-// either way
+// 1 / sqrt.  With FULL for every argument; without it, the hardware's
+// approximation alone (what rsqrtf rounds to), which takes a subnormal argument
+// for 0.  launch_walk knows when no argument can be one; the steps that scale
+// those cost a tenth of the walk (2^20 particles 1.98 and 2.19 ms).
+template <bool FULL>
 __device__ __forceinline__ uint64_t rsqrt2(uint64_t x) {
     float a, b;
     unpack2(x, a, b);
-    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(a));
-    asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(b));
+    if constexpr (FULL) {
+        a = rsqrtf(a);
+        b = rsqrtf(b);
+    } else {
+        asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(a));
+        asm("rsqrt.approx.ftz.f32 %0, %0;" : "+f"(b));
+    }
     return pack2(a, b);
 }
 
@@ -120,7 +129,7 @@ struct Chunk {
 
 // Steps of eight accepted cells, rows [from, to) of the list; to - from is a
 // multiple of eight unless these are the last (missing rows are massless).
-template <bool QUAD>
+template <bool QUAD, bool FULL>
 __device__ __forceinline__ void eval_cells(const WarpLists &W, int from, int to, float eps2, Chunk &C) {
     const int i = threadIdx.x & 7;
     const uint64_t E = dup2(eps2), K = dup2(-2.5f);
@@ -144,14 +153,14 @@ __device__ __forceinline__ void eval_cells(const WarpLists &W, int from, int to,
             const uint64_t ry = add2(add2(C.y[p], cy), ly);
             const uint64_t rz = add2(add2(C.z[p], cz), lz);
             const uint64_t r2 = fma2(rx, rx, fma2(ry, ry, mul2(rz, rz)));
-            const uint64_t inv = rsqrt2(add2(r2, E));
+            const uint64_t inv = rsqrt2<FULL>(add2(r2, E));
             uint64_t f = mul2(mul2(mul2(nm, inv), inv), inv);
             if constexpr (QUAD) {
                 const uint64_t tx = fma2(txx, rx, fma2(txy, ry, mul2(txz, rz)));
                 const uint64_t ty = fma2(txy, rx, fma2(tyy, ry, mul2(tyz, rz)));
                 const uint64_t tz = fma2(txz, rx, fma2(tyz, ry, mul2(tzz, rz)));
                 const uint64_t rtr = fma2(rx, tx, fma2(ry, ty, mul2(rz, tz)));
-                const uint64_t ir = rsqrt2(r2);
+                const uint64_t ir = rsqrt2<FULL>(r2);
                 const uint64_t ir2 = mul2(ir, ir);
                 const uint64_t ir5 = mul2(mul2(ir2, ir2), ir);
                 f = fma2(mul2(mul2(rtr, K), ir5), ir2, f);
@@ -167,9 +176,10 @@ __device__ __forceinline__ void eval_cells(const WarpLists &W, int from, int to,
 }
 
 // One step of eight source particles; y is this lane's, eps2 its softening (a
-// missing source has no mass and a softening of 1).  With SELF, `slot` is the slot of this lane's targets that is the
-// source itself, or -1, and takes no force from it.
-template <bool SELF>
+// missing source has no mass and a softening of 1).  With SELF, `slot` is the
+// slot of this lane's targets that is the source itself, or -1, and takes no
+// force from it.
+template <bool SELF, bool FULL>
 __device__ __forceinline__ void eval_sources(float4 y, int slot, float eps2, Chunk &C) {
     const uint64_t E = dup2(eps2);
     const uint64_t sx = dup2(-y.x), sy = dup2(-y.y), sz = dup2(-y.z), nm = dup2(-y.w);
@@ -177,7 +187,7 @@ __device__ __forceinline__ void eval_sources(float4 y, int slot, float eps2, Chu
     for (int p = 0; p < kPairs; ++p) {
         if (p >= C.pairs) break;
         const uint64_t rx = add2(C.x[p], sx), ry = add2(C.y[p], sy), rz = add2(C.z[p], sz);
-        const uint64_t inv = rsqrt2(fma2(rx, rx, fma2(ry, ry, fma2(rz, rz, E))));
+        const uint64_t inv = rsqrt2<FULL>(fma2(rx, rx, fma2(ry, ry, fma2(rz, rz, E))));
         uint64_t f = mul2(mul2(mul2(nm, inv), inv), inv);
         if constexpr (SELF) {
             float a, b;
@@ -193,6 +203,7 @@ __device__ __forceinline__ void eval_sources(float4 y, int slot, float eps2, Chu
 // The source at sorted position q against the chunk [kb, ke).  When !in there is
 // none: y is then some other source, and counts with no mass and a softening of
 // 1, so that the distance is not 0 even if it is a target itself.
+template <bool FULL>
 __device__ __forceinline__ void eval_source(float4 y, int q, bool in, int kb, int ke, float eps2,
                                             Chunk &C) {
     if (!in) {
@@ -202,13 +213,14 @@ __device__ __forceinline__ void eval_source(float4 y, int q, bool in, int kb, in
     const int t = q - kb;
     const bool mine = in && q >= kb && q < ke;
     if (__any_sync(0xffffffffu, mine))
-        eval_sources<true>(y, mine && (t & 3) == (int)(threadIdx.x & 31) >> 3 ? t >> 2 : -1, eps2, C);
+        eval_sources<true, FULL>(y, mine && (t & 3) == (int)(threadIdx.x & 31) >> 3 ? t >> 2 : -1, eps2, C);
     else
-        eval_sources<false>(y, -1, eps2, C);
+        eval_sources<false, FULL>(y, -1, eps2, C);
 }
 
 // Steps of eight listed sources, entries [from, to); the next step's
 // particles are loaded before this step's are used.
+template <bool FULL>
 __device__ __forceinline__ void eval_list(const WarpLists &W, const float4 *__restrict__ xs, int from, int to,
                                           int kb, int ke, float eps2, Chunk &C) {
     const int i = threadIdx.x & 7;
@@ -217,19 +229,20 @@ __device__ __forceinline__ void eval_list(const WarpLists &W, const float4 *__re
     for (int j = from; j < to; j += 8) {
         const int qn = W.src[min(j + 8 + i, to - 1)];
         const float4 yn = xs[qn];
-        eval_source(y, q, j + i < to, kb, ke, eps2, C);
+        eval_source<FULL>(y, q, j + i < to, kb, ke, eps2, C);
         q = qn;
         y = yn;
     }
 }
 
 // The sources [q0, q1) of one long leaf.
+template <bool FULL>
 __device__ __forceinline__ void eval_range(const float4 *__restrict__ xs, int q0, int q1, int kb, int ke,
                                            float eps2, Chunk &C) {
     const int i = threadIdx.x & 7;
     for (int j = q0; j < q1; j += 8) {
         const int q = min(j + i, q1 - 1);
-        eval_source(xs[q], q, j + i < q1, kb, ke, eps2, C);
+        eval_source<FULL>(xs[q], q, j + i < q1, kb, ke, eps2, C);
     }
 }
 
@@ -275,7 +288,7 @@ __global__ void walk_groups_kernel(const int32_t *__restrict__ parent, const int
     }
 }
 
-template <bool QUAD, bool COUNT>
+template <bool QUAD, bool COUNT, bool FULL>
 __global__ void __launch_bounds__(kWalkThreads, kWalkPerSm)
     walk_kernel(WalkTree T, const int32_t *__restrict__ groups, uint32_t *ctr, int32_t *stacks,
                 float theta, float eps2, float *__restrict__ acc_out, DevInfo *info) {
@@ -363,11 +376,11 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkPerSm)
                 cp_async_wait_all();
                 __syncwarp();
                 if (ncell >= 8) {
-                    eval_cells<QUAD>(W, ncell & 7, ncell, eps2, C);
+                    eval_cells<QUAD, FULL>(W, ncell & 7, ncell, eps2, C);
                     ncell &= 7;
                 }
                 if (nsrc > kSrcCap - 32 * kSrcLeaf) {
-                    eval_list(W, T.xs, nsrc & 7, nsrc, kb, ke, eps2, C);
+                    eval_list<FULL>(W, T.xs, nsrc & 7, nsrc, kb, ke, eps2, C);
                     nsrc &= 7;
                 }
                 __syncwarp();
@@ -432,7 +445,7 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkPerSm)
                 // longer leaves at once, one after another
                 for (unsigned bl = __ballot_sync(0xffffffffu, cnt > kSrcLeaf); bl; bl &= bl - 1) {
                     const int w = __ffs(bl) - 1;
-                    eval_range(T.xs, __shfl_sync(0xffffffffu, lk.x, w), __shfl_sync(0xffffffffu, lk.y, w), kb,
+                    eval_range<FULL>(T.xs, __shfl_sync(0xffffffffu, lk.x, w), __shfl_sync(0xffffffffu, lk.y, w), kb,
                                ke, eps2, C);
                 }
                 __syncwarp();
@@ -445,8 +458,8 @@ __global__ void __launch_bounds__(kWalkThreads, kWalkPerSm)
             if (COUNT) n_pp_int -= (unsigned long long)nt;   // own pairs
             cp_async_wait_all();
             __syncwarp();
-            if (ncell) eval_cells<QUAD>(W, 0, ncell, eps2, C);
-            if (nsrc) eval_list(W, T.xs, 0, nsrc, kb, ke, eps2, C);
+            if (ncell) eval_cells<QUAD, FULL>(W, 0, ncell, eps2, C);
+            if (nsrc) eval_list<FULL>(W, T.xs, 0, nsrc, kb, ke, eps2, C);
             __syncwarp();
             // the eight lanes' sums of each target; lane i of a group writes slot i
             float out[3] = {0.f, 0.f, 0.f};
@@ -504,11 +517,22 @@ cudaError_t launch_walk(const tb_tree &t, Workspace &ws, float theta, float eps,
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     WalkTree T{t.child_first, t.child_end, t.pfirst, t.pend, t.level, t.mass, t.com, t.com_lo,
                t.quad, t.aabb, ws.xs, t.perm, t.side, rec};
+    // No argument of rsqrt2 is subnormal when eps^2 is not, for a softened
+    // distance, and for the plain distance r of an accepted cell when the side
+    // is at least theta 2^-39.  The cell has l < theta d and l >= side 2^-21; d
+    // along its longest axis is at least d / sqrt(3); the centre's low part,
+    // half a unit in the last place of the high part at most, takes at most half of
+    // that away; so r^2 > l^2 / (12 theta^2) >= 2^-124 where 2^-126 is normal.
+    const float eps2 = eps * eps;
+    const bool full = !(eps2 >= FLT_MIN && t.side >= (double)theta * 0x1p-39);
     // the interaction counts cost about 15% of the walk: only profiled walks
     // take them
-    auto kern = use_quad ? (ws.profile ? walk_kernel<true, true> : walk_kernel<true, false>)
-                         : (ws.profile ? walk_kernel<false, true> : walk_kernel<false, false>);
-    launch_after(kern, dim3(kWalkBlocks), dim3(kWalkThreads), 0, s, T, groups, ctr, stacks, theta, eps * eps, acc, ws.info);
+    auto pick = [&](auto plain, auto counting) { return ws.profile ? counting : plain; };
+    auto kern = use_quad ? (full ? pick(walk_kernel<true, false, true>, walk_kernel<true, true, true>)
+                                 : pick(walk_kernel<true, false, false>, walk_kernel<true, true, false>))
+                         : (full ? pick(walk_kernel<false, false, true>, walk_kernel<false, true, true>)
+                                 : pick(walk_kernel<false, false, false>, walk_kernel<false, true, false>));
+    launch_after(kern, dim3(kWalkBlocks), dim3(kWalkThreads), 0, s, T, groups, ctr, stacks, theta, eps2, acc, ws.info);
     ++g_launches;
     return cudaGetLastError();
 }

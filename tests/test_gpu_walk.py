@@ -132,6 +132,27 @@ def test_unsoftened_with_a_particle_at_any_place(theta):
         assert np.median(e) <= 1e-1
 
 
+@pytest.mark.parametrize("theta,eps", [(0.0, 0.0), (0.0, 2e-20), (0.5, 0.0), (0.5, 2e-20)])
+def test_distances_below_the_square_root_of_the_normal_range(theta, eps):
+    """1,000 particles on a jittered lattice of spacing h = 1e-20, masses 1e-30:
+    squared distances are subnormal (from 3.6e-41, in steps of 1.4e-45) and the
+    forces, about 1e10, are not.  A squared distance is off by three half steps
+    at most, 6e-5 of the least, so a pair's force by 9e-5, and the 26 pairs nearest
+    by less than 26 * 9e-5 / 0.36 = 7e-3 of m / h^2; the others count less.  (The
+    cells' first moments, m h, underflow, so that their centres are only within
+    the cell: with cells accepted the forces are finite, no more.)"""
+    h, rng = 1e-20, np.random.default_rng(46)
+    grid = np.stack(np.meshgrid(*[np.arange(10.0)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    pos = ((grid + 0.2 * (2 * rng.random(grid.shape) - 1)) * h).astype(np.float32)
+    mass = np.full(len(pos), 1e-30, np.float32)
+    m, t = _setup(pos, mass)
+    acc = to_np(m.walk(t, theta, eps, use_quad=False)).astype(np.float64)
+    assert np.isfinite(acc).all()
+    if theta == 0.0:
+        err = np.linalg.norm(acc - oracle.direct_acc(pos, mass, np.arange(len(pos)), eps), axis=1)
+        assert err.max() <= 7e-3 * 1e-30 / h ** 2, err.max()
+
+
 def test_walk_arguments():
     m = tb()
     pos, mass = plummer(3000, 44)
