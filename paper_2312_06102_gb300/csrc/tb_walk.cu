@@ -235,14 +235,15 @@ __device__ __forceinline__ void eval_list(const WarpLists &W, const float4 *__re
     }
 }
 
-// The sources [q0, q1) of one long leaf.
+// The sources [q0, q1) of one long leaf (unsigned: the last step may pass the
+// largest position, 2^31 - 1).
 template <bool FULL>
 __device__ __forceinline__ void eval_range(const float4 *__restrict__ xs, int q0, int q1, int kb, int ke,
                                            float eps2, Chunk &C) {
-    const int i = threadIdx.x & 7;
-    for (int j = q0; j < q1; j += 8) {
-        const int q = min(j + i, q1 - 1);
-        eval_source<FULL>(xs[q], q, j + i < q1, kb, ke, eps2, C);
+    const uint32_t i = threadIdx.x & 7, end = (uint32_t)q1;
+    for (uint32_t j = (uint32_t)q0; j < end; j += 8) {
+        const int q = (int)min(j + i, end - 1);
+        eval_source<FULL>(xs[q], q, j + i < end, kb, ke, eps2, C);
     }
 }
 
