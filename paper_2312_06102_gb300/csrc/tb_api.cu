@@ -112,7 +112,9 @@ tb_status ensure_fixed(TreeState &S) {
     return TB_OK;
 }
 
-// need_xs: the key-ordered records are scratch of the one-launch batched build
+// need_xs: the key-ordered records are scratch of the one-launch batched build;
+// every batched tree has them, since a later call with that option may be
+// captured and must not allocate
 tb_status ensure_particles(TreeState &S, int64_t n, const SortCfg &cfg, bool reorder,
                            bool need_xs) {
     Workspace &ws = S.ws;
@@ -465,8 +467,7 @@ tb_status tb_build_batched(const float *d_pos, const float *d_mass, const int64_
     t.n_particles = n_total;
     t.n_crit = params->n_crit;
     t.n_sets = n_sets;
-    st = ensure_particles(*S, n_total, default_sort_cfg(8, n_total), false,
-                          params->cell_capacity > 0 && params->batch_one_launch);
+    st = ensure_particles(*S, n_total, default_sort_cfg(8, n_total), false, true);
     if (st != TB_OK) return st;
     if (n_sets > ws.set_cap || !t.set_cell_offset) {
         cudaDeviceSynchronize();

@@ -171,6 +171,30 @@ def test_batched_graph_replay_with_jitter(one_launch):
         _check_sets(t, pj, b.mass, b.offsets, 16, sets=[0, 1, 17, 40, 63])
 
 
+@pytest.mark.parametrize("cap", [0, 9000])
+def test_batched_one_launch_captured_on_a_tree_of_separate_launches(cap):
+    """A tree from an earlier call with the same sets, whatever its options,
+    takes a captured one-launch build without allocating."""
+    m = tb()
+    pos, mass, offsets = _sets([3000, 0, 700, 5000], 35)
+    t, p, w, off = _run(pos, mass, offsets, cap=cap)
+    cap = max(cap, t.n_cells)
+    want = {k: getattr(t, k)[:t.n_cells].clone() for k in ("ckey", "mass", "com", "quad", "aabb")}
+    # (another tree, so that the kernel itself is loaded)
+    m.build_batched(p, w, off, cell_capacity=cap, batch_threads=512, one_launch=True)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        m.build_batched(p, w, off, cell_capacity=cap, batch_threads=512, one_launch=True, tree=t)
+    for k in want:
+        getattr(t, k).zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert t.sync() == 0
+    for k, v in want.items():
+        assert torch.equal(getattr(t, k)[:t.n_cells], v), k
+
+
 def test_batched_root_pow2():
     """Every set's root cube with its side forced to a power of two (Sec. 2.2)
     equals the oracle's tree of that set under the same root."""
