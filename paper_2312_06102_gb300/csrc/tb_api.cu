@@ -120,10 +120,12 @@ tb_status ensure_particles(TreeState &S, int64_t n, const SortCfg &cfg, bool reo
     Workspace &ws = S.ws;
     tb_tree &t = S.pub;
     const int64_t tiles = (n + cfg.tile() - 1) / cfg.tile();
-    // look-back words for this set and for any smaller one rebuilt in its
-    // place, which may take smaller tiles (2048 keys up to kSmallTileMax)
+    // look-back words for this set, for any smaller one rebuilt in its place,
+    // which may take smaller tiles (2048 keys up to kSmallTileMax), and for a
+    // rebuild that names a variant of 8-bit digits and 4096 keys a tile or more
     const int64_t small = (min64(n, kSmallTileMax) + 2047) / 2048 * 256;
-    const int64_t need_lb = max64(tiles * (int64_t(1) << cfg.radix_bits), small);
+    const int64_t named = (n + 4095) / 4096 * 256;
+    const int64_t need_lb = max64(tiles * (int64_t(1) << cfg.radix_bits), max64(small, named));
     const int64_t ltiles = (n + level_tile_size() - 1) / level_tile_size();
     if (n > ws.n_cap || need_lb > ws.tiles_cap || ltiles > ws.level_tiles_cap) {
         cudaDeviceSynchronize();

@@ -241,6 +241,29 @@ def test_graph_captured_build_and_moments():
         assert em.max() <= TOL_MASS and ec.max() <= TOL_COM and eq.max() <= TOL_QUAD
 
 
+@pytest.mark.parametrize("cfg", [(8, 256, 16), (8, 512, 8), (8, 512, 16)])
+def test_named_variant_captured_on_a_tree_built_by_default(cfg):
+    """A tree built with the default tiles holds enough look-back words for a
+    named variant of 8-bit digits and at least 4096 keys a tile, so that a captured rebuild with
+    one does not allocate."""
+    m = tb()
+    p = torch.from_numpy(uniform_cube(2_000_000, 19)[0]).cuda()
+    t = m.build(p, None)
+    assert t.sync() == 0
+    cap = t.n_cells
+    want = t.perm.clone()
+    m.build(p, None, cell_capacity=cap, sort_cfg=cfg)     # loads the kernels
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        m.build(p, None, cell_capacity=cap, sort_cfg=cfg, tree=t)
+    t.perm.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert t.sync() == 0 and t.n_cells == cap
+    assert torch.equal(t.perm, want)
+
+
 def test_capacity_overflow_reported():
     m = tb()
     pos, mass = uniform_cube(40_000, 9)
