@@ -12,6 +12,13 @@ namespace tb {
 
 int64_t g_launches = 0;
 
+// Test hook: TB_FAULT_LOAD=k makes the process's first k loads of a kernel
+// ahead of its launch fail.
+bool fault_load() {
+    static int64_t left = std::getenv("TB_FAULT_LOAD") ? std::atoll(std::getenv("TB_FAULT_LOAD")) : 0;
+    return left > 0 && left-- > 0;
+}
+
 namespace {
 
 // Test hook: TB_FAULT_ALLOC=k makes the k-th device allocation of the

@@ -632,13 +632,10 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
                              int64_t cell_cap, int phase, int mode, cudaStream_t s) {
     cudaError_t e;
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        const int sm_front = (int)batch_front_smem<T>(kMaxNcrit);
-        cudaFuncSetAttribute(batch_front_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             sm_front);
-        cudaFuncSetAttribute(batch_front_kernel<T>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-    }
+    if ((e = once_on_device(attr_done, [] {
+             return allow_smem(batch_front_kernel<T>, batch_front_smem<T>(kMaxNcrit), true);
+         })) != cudaSuccess)
+        return e;
     int dev = 0, nsm = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -707,16 +704,12 @@ cudaError_t launch_batched_one_t(const BatchArgs &A, int32_t S, int ncrit, int64
     auto kern = batch_all_kernel<T, MODE>;
     const size_t smem = batch_front_smem<T>(ncrit);
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)batch_front_smem<T>(kMaxNcrit));
-        cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-    }
+    cudaError_t e = once_on_device(attr_done, [&] { return allow_smem(kern, batch_front_smem<T>(kMaxNcrit), true); });
+    if (e != cudaSuccess) return e;
     int dev = 0, nsm = 152, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) return cudaErrorCooperativeLaunchTooLarge;
     // every block resident at once (the grid barriers need it), at most one

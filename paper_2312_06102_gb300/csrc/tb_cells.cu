@@ -255,21 +255,12 @@ cudaError_t launch_levels(const uint64_t *skeys, int64_t n, int ncrit, Workspace
     const int64_t tiles = (n + kLvTile - 1) / kLvTile;
     const size_t smem = lv_smem_bytes(ncrit);
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        cudaFuncSetAttribute(level_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)lv_smem_bytes(kMaxNcrit));
-        cudaFuncSetAttribute(level_count_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-    }
+    cudaError_t err = once_on_device(attr_done, [] {
+        const cudaError_t e = allow_smem(level_count_kernel, lv_smem_bytes(kMaxNcrit), true);
+        return e == cudaSuccess ? allow_smem(level_count_fast_kernel, lc_smem_bytes<kLcThreads>(kLcMaxN), true) : e;
+    });
+    if (err != cudaSuccess) return err;
     if (ncrit >= kLcMinN && ncrit <= kLcMaxN) {
-        static std::atomic<uint64_t> fast_attr_done{0};
-        if (first_on_device(fast_attr_done)) {
-            cudaFuncSetAttribute(level_count_fast_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)lc_smem_bytes<kLcThreads>(kLcMaxN));
-            cudaFuncSetAttribute(level_count_fast_kernel,
-                                 cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
-        }
         launch_after(level_count_fast_kernel, dim3((unsigned)tiles), dim3(kLcThreads), lc_smem_bytes<kLcThreads>(ncrit), s, 
             skeys, n, ncrit, ws.level_cnt, tiles, ws.ml, ws.info, ws.cell_cap_request);
         if (tiles <= kLcScanTiles) {
@@ -281,7 +272,7 @@ cudaError_t launch_levels(const uint64_t *skeys, int64_t n, int ncrit, Workspace
                                                                      tiles, ws.ml);
     }
     ++g_launches;
-    cudaError_t err = cudaGetLastError();
+    err = cudaGetLastError();
     if (err != cudaSuccess) return err;
     launch_after(level_scan_kernel, dim3(kLevelFields), dim3(kScanThreads), 0, s, ws.level_cnt, tiles, ws.info,
                                                             ws.cell_cap_request);

@@ -192,17 +192,33 @@ cudaError_t launch_walk(const tb_tree &t, Workspace &ws, float theta, float eps,
 
 void mark(Workspace &ws, const char *name, cudaStream_t s);
 
-// Kernel attributes (dynamic shared memory above 48 KB, carve-out) belong to
-// a device.  A launcher keeps one bit per device in `done` and sets its
-// attributes the first time it runs on each device; two host threads that
-// race here both set the same values, which is harmless.
-inline bool first_on_device(std::atomic<uint64_t> &done) {
+// Runs `set` (attributes of kernels, their loading) the first time a launcher
+// runs on each device: those belong to a device.  `done` keeps one bit per
+// device, set when it succeeded: a call that fails, for lack of memory say,
+// leaves it to the next one.  Two host threads that race here both set the
+// same values, which is harmless.
+template <class F>
+cudaError_t once_on_device(std::atomic<uint64_t> &done, F set) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return true;
-    const uint64_t bit = uint64_t(1) << dev;
-    if (done.load(std::memory_order_acquire) & bit) return false;
-    done.fetch_or(bit, std::memory_order_acq_rel);
-    return true;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev >= 0 && dev < 64 ? uint64_t(1) << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = set();
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_acq_rel);
+    else cudaGetLastError();   // reported here, not by a later launch
+    return e;
+}
+
+// Dynamic shared memory a kernel may be launched with; `most` asks for the
+// largest shared-memory division of L1.
+template <class K>
+cudaError_t allow_smem(K kernel, size_t bytes, bool most) {
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess && most)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 cudaSharedmemCarveoutMaxShared);
+    return e;
 }
 
 // Launches a kernel of a chain of this library's own launches in one call,
@@ -227,8 +243,11 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+bool fault_load();   // test hook (TB_FAULT_LOAD): this load fails
+
 template <class K>
 cudaError_t load_kernel(K kernel) {
+    if (fault_load()) return cudaErrorMemoryAllocation;
     cudaFuncAttributes a;
     return cudaFuncGetAttributes(&a, kernel);
 }

@@ -283,9 +283,8 @@ static cudaError_t keys_impl(const float *pos, const float *mass, int64_t n, uin
     const float m_eq = (float)(1.0 / (double)(n > 0 ? n : 1));
     size_t smem = sizeof(uint32_t) * passes * (1 << B) + (H ? sizeof(uint16_t) * kHilbertTab : 0);
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        cudaFuncSetAttribute(keys_kernel<B, H>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 1024);
-    }
+    const cudaError_t e = once_on_device(attr_done, [] { return allow_smem(keys_kernel<B, H>, 64 * 1024, false); });
+    if (e != cudaSuccess) return e;
     // six resident blocks per SM (42 registers), one wave
     int64_t grid = 152 * 6;
     int64_t need = (n + 4 * kKeysThreads - 1) / (4 * kKeysThreads);

@@ -808,17 +808,11 @@ cudaError_t leaves_impl(tb_tree &t, Workspace &ws, const int32_t *start_cell, cu
     MomOut o{t.mass, t.com, t.com_lo, t.quad, t.aabb, t.mass64, t.com64, t.quad64};
     const int64_t n = t.n_particles;
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        cudaFuncSetAttribute(leaf_tile_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)leaf_tile_smem());
-        cudaFuncSetAttribute(leaf_tile_kernel<MODE>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute(upward_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(2 * sizeof(LevelSmem)));
-        cudaFuncSetAttribute(upward_kernel<MODE>,
-                             cudaFuncAttributePreferredSharedMemoryCarveout,
-                             cudaSharedmemCarveoutMaxShared);
-    }
+    const cudaError_t set = once_on_device(attr_done, [] {
+        const cudaError_t e = allow_smem(leaf_tile_kernel<MODE>, leaf_tile_smem(), true);
+        return e == cudaSuccess ? allow_smem(upward_kernel<MODE>, 2 * sizeof(LevelSmem), true) : e;
+    });
+    if (set != cudaSuccess) return set;
     const int64_t tiles = (n + kLtTile - 1) / kLtTile;
     const int64_t level_tiles = (n + level_tile_size() - 1) / level_tile_size();
     const uint32_t *leaf_off = ws.level_cnt + (int64_t)kLevels * level_tiles;

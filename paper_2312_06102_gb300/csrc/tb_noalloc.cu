@@ -74,7 +74,10 @@ cudaError_t scratch_address(unsigned char **out) {
     if (!g_scratch_addr[dev]) {
         void *p = nullptr;
         e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
-        if (e != cudaSuccess) return e;
+        if (e != cudaSuccess) {
+            cudaGetLastError();   // reported here, not by the next call's launches
+            return e;
+        }
         g_scratch_addr[dev] = static_cast<unsigned char *>(p);
     }
     *out = g_scratch_addr[dev];
@@ -82,15 +85,16 @@ cudaError_t scratch_address(unsigned char **out) {
 }
 
 // Every kernel a call can reach, loaded by the first call that sorts, whatever
-// its size: sets of up to 32,768 particles and larger ones take different
+// its size (by the next one when that fails): sets of up to 32,768 particles and larger ones take different
 // kernels, and a later call of the other kind must not load (allocate).
 cudaError_t load_kernels_once() {
     static std::atomic<uint64_t> done{0};
-    if (!first_on_device(done)) return cudaSuccess;
-    cudaError_t e = load_key_kernels();
-    if (e == cudaSuccess) e = load_sort_kernels();
-    if (e == cudaSuccess) e = load_run_kernels();
-    return e == cudaSuccess ? load_small_kernels() : e;
+    return once_on_device(done, [] {
+        cudaError_t e = load_key_kernels();
+        if (e == cudaSuccess) e = load_sort_kernels();
+        if (e == cudaSuccess) e = load_run_kernels();
+        return e == cudaSuccess ? load_small_kernels() : e;
+    });
 }
 
 tb_status status_of(cudaError_t e) {

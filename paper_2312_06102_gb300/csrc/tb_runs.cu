@@ -66,14 +66,12 @@ cudaError_t launch_runs(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t 
     if (shift0 <= 0 || n <= 1) return cudaSuccess;
     if (shift0 > 32) return cudaErrorInvalidValue;   // the run step ranks the low bits as 32-bit words
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        cudaFuncSetAttribute(long_run_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(CtaSortShared));
-    }
+    cudaError_t e = once_on_device(attr_done, [] { return allow_smem(long_run_kernel, sizeof(CtaSortShared), false); });
+    if (e != cudaSuccess) return e;
     const int64_t tiles = (n + kRunTile - 1) / kRunTile;
     launch_after(run_sort_kernel, dim3((unsigned)tiles), dim3(kRunThreads), 0, s, keys, vals, n, shift0, rb, ws.info);
     ++g_launches;
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     launch_after(long_run_kernel, dim3(152), dim3(kCtaThreads), sizeof(CtaSortShared), s, keys, vals, alt_k, alt_v, n, shift0,
                                                                    rb, ws.info);

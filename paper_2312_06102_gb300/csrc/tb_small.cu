@@ -350,13 +350,11 @@ cudaError_t launch_small_t(const float *pos, const float *mass, int n, uint64_t 
     auto kern = small_sort_kernel<ITEMS, H>;
     const int blocks = (n + SmallSmem<ITEMS>::P - 1) / SmallSmem<ITEMS>::P;
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)small_smem<ITEMS>());
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e = once_on_device(attr_done, [&] {
+        const cudaError_t a = allow_smem(kern, small_smem<ITEMS>(), false);
+        return a == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : a;
+    });
+    if (e != cudaSuccess) return e;
     cudaLaunchAttribute attr{};
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = blocks;
@@ -370,7 +368,7 @@ cudaError_t launch_small_t(const float *pos, const float *mass, int n, uint64_t 
     cfg.numAttrs = 1;
     if (ask) return cudaOccupancyMaxActiveClusters(clusters, kern, &cfg);
     const float m_eq = (float)(1.0 / (double)n);
-    cudaError_t e = cudaLaunchKernelEx(&cfg, kern, pos, mass, m_eq, n, pkey, perm, ws.xm, ws.info,
+    e = cudaLaunchKernelEx(&cfg, kern, pos, mass, m_eq, n, pkey, perm, ws.xm, ws.info,
                                        ws.root_pow2);
     if (e == cudaSuccess) ++g_launches;
     return e;
@@ -404,6 +402,7 @@ int small_blocks() {
             dispatch_small(nullptr, nullptr, (int64_t)16 * kSmThreads * kSmMaxItems, 16, nullptr, nullptr,
                            none, TB_KEYS_MORTON, true, &clusters, nullptr);
         if (e != cudaSuccess) cudaGetLastError();
+        if (e == cudaErrorMemoryAllocation) return 8;   // asked again by the next call
         v = e == cudaSuccess && clusters > 0 ? 16 : 8;
         known[dev].store(v, std::memory_order_relaxed);
     }

@@ -495,13 +495,11 @@ cudaError_t run_passes(uint64_t *ka, uint64_t *kb, int32_t *pa, int32_t *pb, int
     auto first = pass_kernel<B, T, I, true>(), next = pass_kernel<B, T, I, false>();
     const size_t smem = B == 8 ? sizeof(Sort8Smem<T, I>) : sizeof(SortSmem<B, T, I>);
     static std::atomic<uint64_t> attr_done{0};
-    if (first_on_device(attr_done)) {
-        for (auto k : {first, next}) {
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 cudaSharedmemCarveoutMaxShared);
-        }
-    }
+    cudaError_t e = once_on_device(attr_done, [&] {
+        const cudaError_t a = allow_smem(first, smem, true);
+        return a == cudaSuccess ? allow_smem(next, smem, true) : a;
+    });
+    if (e != cudaSuccess) return e;
     const int64_t tiles = (n + T * I - 1) / (T * I);
     // the unsorted keys are in `ka`; passes alternate ka -> kb -> ka ...
     uint64_t *src = ka, *dst = kb;
@@ -512,7 +510,7 @@ cudaError_t run_passes(uint64_t *ka, uint64_t *kb, int32_t *pa, int32_t *pb, int
             src, p == 0 ? nullptr : vsrc, dst, vdst, n, p, plan.shift0, ws.hist + p * (1 << B), ws.lookback,
             ws.info, spin);
         ++g_launches;
-        cudaError_t e = cudaGetLastError();
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         mark(ws, "sort_pass", s);
         uint64_t *t = src; src = dst; dst = t;
@@ -521,7 +519,7 @@ cudaError_t run_passes(uint64_t *ka, uint64_t *kb, int32_t *pa, int32_t *pb, int
     kout = src;
     pout = vsrc;
     // finish the runs of equal upper bits; the other buffers are free scratch
-    cudaError_t e = launch_runs(src, vsrc, dst, vdst, n, plan.shift0, ws.long_runs, ws, s);
+    e = launch_runs(src, vsrc, dst, vdst, n, plan.shift0, ws.long_runs, ws, s);
     if (e != cudaSuccess) return e;
     if (plan.shift0 > 0) mark(ws, "sort_runs", s);
     return cudaSuccess;

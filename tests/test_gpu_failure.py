@@ -8,6 +8,9 @@
 - A device allocation that fails: the library's TB_FAULT_ALLOC=k hook makes
   its k-th cudaMalloc fail in a child process; the build reports TB_ENOMEM
   and releasing the half-made tree succeeds.
+- A kernel of the allocation-free sort that cannot be loaded: TB_FAULT_LOAD=k
+  makes the first k loads fail in a child process; each call that meets one
+  reports TB_ENOMEM, and the next call tries again.
 """
 import os
 import subprocess
@@ -107,3 +110,31 @@ def test_allocation_failure_reports_enomem(k):
     assert r.returncode == 0, r.stderr[-2000:]
     assert "RESULT TB_ENOMEM" in r.stdout, r.stdout
     assert "FREED" in r.stdout
+
+
+_LOADS = r"""
+import sys, torch
+sys.path.insert(0, sys.argv[1])
+import paper_2312_06102_gb300 as tb
+p = torch.rand(100000, 3, device="cuda")
+k = torch.empty(100000, dtype=torch.uint64, device="cuda")
+q = torch.empty(100000, dtype=torch.int32, device="cuda")
+for n in (2, 2, 2, 100000):
+    st, _ = tb.keys_sorted_noalloc(p[:n], k[:n], q[:n])
+    print("RESULT", tb.STATUS[st])
+t = tb.build(p, None)
+print("EQUAL", torch.equal(q, t.perm), torch.equal(k.view(torch.int64), t.pkey.view(torch.int64)))
+"""
+
+
+def test_noalloc_loads_again_after_a_failed_load():
+    """Small sets launch one kernel and larger ones others, and all are loaded by
+    the first call that can: after two calls in which a load failed, whatever
+    their size, the third loads them all."""
+    env = dict(os.environ, TB_FAULT_LOAD="2")
+    r = subprocess.run([sys.executable, "-c", _LOADS, ROOT], env=env, capture_output=True,
+                       text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert [v.split()[1] for v in r.stdout.splitlines() if v.startswith("RESULT")] == \
+        ["TB_ENOMEM", "TB_ENOMEM", "TB_OK", "TB_OK"], r.stdout
+    assert "EQUAL True True" in r.stdout
