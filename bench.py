@@ -675,7 +675,8 @@ def run_batched(a, tb, torch):
     w = torch.from_numpy(b.mass).cuda()
     off = torch.from_numpy(b.offsets).cuda()
     jit = Jitter(torch, b, spec["seed"])
-    # the block size per set (512 or 1024 threads), tuned untimed unless named
+    # the block size per set (512 or 1024 threads, or 0, the library's rule), tuned
+    # untimed unless named
     bt, bt_ms = 0, None
     if a.batch_threads:
         bt = a.batch_threads
@@ -783,7 +784,7 @@ def run_batched(a, tb, torch):
             "plain_loop_mparticles_s": round(n / plain_ms / 1e3, 2),
             "speedup_vs_plain": round(plain_ms / batched_ms, 1),
             "kernels_per_batched_build": int(per_build),
-            "batch_threads": int(bt) if bt else 512,
+            "batch_threads": int(bt),
             "one_launch_ms_per_build": round(one_ms, 4),
             "batch_threads_autotune_ms": ({str(k): round(v, 3) for k, v in bt_ms.items()}
                                           if bt_ms else None),

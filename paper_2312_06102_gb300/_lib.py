@@ -294,11 +294,19 @@ def build_batched(pos: torch.Tensor, mass: torch.Tensor | None, set_offsets: tor
     one_launch (with cell_capacity > 0) runs it as one cooperative launch."""
     if set_offsets.dtype != torch.int64 or not set_offsets.is_cuda:
         raise ValueError("set_offsets must be an int64 CUDA tensor")
-    t = tree if tree is not None else Tree()
     if not batch_threads:
         from . import autotune
         batch_threads = autotune.cached_batched(set_offsets.shape[0] - 1,
                                                 pos.shape[0] if n_total is None else n_total) or 0
+    return _build_batched(pos, mass, set_offsets, n_crit, mom_mode, cell_capacity, radix_bits,
+                          batch_threads, tree, n_total, stream, key_order, one_launch, root_pow2)
+
+
+def _build_batched(pos, mass, set_offsets, n_crit=16, mom_mode=MOM_FP32_COMP, cell_capacity=0,
+                   radix_bits=0, batch_threads=0, tree=None, n_total=None, stream=None,
+                   key_order=KEYS_MORTON, one_launch=False, root_pow2=False) -> Tree:
+    """build_batched with the block size as given: 0 is the library's own rule."""
+    t = tree if tree is not None else Tree()
     p = _params(n_crit, mom_mode, cell_capacity, 0, radix_bits, batch_threads)
     p.key_order = int(key_order)
     p.batch_one_launch = int(bool(one_launch))

@@ -8,9 +8,10 @@ and size class (log2 of the particle count) in _build/autotune.json.
 variant.
 
 tune_batched() does the same for the batched build's block size (512 or
-1024 threads per set: two sets per SM at a time, or one), keyed by GPU name,
-the number of sets and the size class of the mean set;
-`build_batched()` uses the cached choice when the caller names none.
+1024 threads per set: two sets per SM at a time, or one; or 0, the library's
+own rule, which takes smaller blocks for many small sets), keyed by GPU name,
+the number of sets and the size class of the mean set; `build_batched()` uses
+the cached choice when the caller names none.
 """
 from __future__ import annotations
 
@@ -84,7 +85,7 @@ def tune(pos: torch.Tensor, mass: torch.Tensor | None = None, n_crit: int = 16, 
     return best, times
 
 
-BATCH_THREADS = (512, 1024)
+BATCH_THREADS = (0, 512, 1024)
 
 
 def _bkey(n_sets: int, n_total: int) -> str:
@@ -93,9 +94,10 @@ def _bkey(n_sets: int, n_total: int) -> str:
 
 
 def cached_batched(n_sets: int, n_total: int):
-    """Cached batch_threads for this many sets and particles on this GPU, or None."""
+    """Cached batch_threads for this many sets and particles on this GPU, or None.
+    A choice made without timing the library's rule (0) does not count."""
     v = _load().get(_bkey(n_sets, n_total))
-    return int(v["threads"]) if v else None
+    return int(v["threads"]) if v and "0" in v["ms"] else None
 
 
 def tune_batched(pos: torch.Tensor, mass: torch.Tensor | None, set_offsets: torch.Tensor,
@@ -104,15 +106,15 @@ def tune_batched(pos: torch.Tensor, mass: torch.Tensor | None, set_offsets: torc
     times = {}
     tree = None
     for th in BATCH_THREADS:
-        tree = _lib.build_batched(pos, mass, set_offsets, n_crit=n_crit, batch_threads=th,
-                                  tree=tree)
+        tree = _lib._build_batched(pos, mass, set_offsets, n_crit=n_crit, batch_threads=th,
+                                   tree=tree)
         cap = tree.n_cells
         torch.cuda.synchronize()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record()
         for _ in range(reps):
-            _lib.build_batched(pos, mass, set_offsets, n_crit=n_crit, batch_threads=th,
-                               cell_capacity=cap, tree=tree)
+            _lib._build_batched(pos, mass, set_offsets, n_crit=n_crit, batch_threads=th,
+                                cell_capacity=cap, tree=tree)
         e1.record()
         torch.cuda.synchronize()
         if tree.sync() != 0:

@@ -221,6 +221,15 @@ def test_batched_empty():
     assert t.n_cells == 0
 
 
+def test_tuning_times_the_default_rule():
+    """The autotuner's choice is never slower than the rule it replaces."""
+    from paper_2312_06102_gb300 import autotune
+    pos, mass, offsets = _sets([100] * 400, 5)
+    best, ms = autotune.tune_batched(torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda(),
+                                     torch.from_numpy(offsets).cuda(), save=False)
+    assert set(ms) == {0, 512, 1024} and ms[best] == min(ms.values())
+
+
 @pytest.mark.parametrize("sizes", ["many small", "few large"])
 def test_batched_default_block_sizes(sizes):
     """The default block size follows the sets: 256 threads for more than 304
