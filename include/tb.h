@@ -311,14 +311,17 @@ const char *tb_stage_name(tb_tree *tree, int32_t i);
  * TB_ETIMEOUT when the wait ran out and the context is still usable. */
 tb_status tb_selftest_wait(int64_t spin_limit, tb_stream stream);
 
-/* Test hook for the bounded waits of the radix sort (Sec. 2.3 step 2): each
- * pass's look-back on earlier tiles gives up after `polls` polls of a
- * predecessor that has not published yet (the default, 2^26 polls with a
- * back-off, is about 17 s) and the build then reports TB_ETIMEOUT.  A small
- * limit makes a multi-tile sort run out on purpose; its keys and cells are
- * then not valid, but every access stays in bounds and the next build with
- * the default limit is correct.  polls = 0 restores the default.  The
- * setting is process-wide and applies to sorts enqueued after the call.
+/* Test hook for the bounded waits: of each radix pass's look-back on earlier
+ * tiles (Sec. 2.3 step 2) for a predecessor that has not published yet; of
+ * tb_moments for the copies a block has staged, and of the upward pass's
+ * barriers between levels for the other blocks; of the one-launch batched
+ * build's barriers.  Each gives up after `polls` polls (the default, 2^26 polls
+ * with a back-off, is about 17 s), and the build or moments then report
+ * TB_ETIMEOUT.  With a small limit a multi-tile sort, and tb_moments on a tree
+ * of several hundred thousand particles, run out on purpose; their results are
+ * then not valid, but every access stays in bounds, and the next build (and
+ * moments) with the default limit is correct.  polls = 0 restores the default.
+ * The setting is process-wide and applies to work enqueued after the call.
  * Returns TB_OK, or TB_EINVAL for polls < 0. */
 tb_status tb_set_wait_limit(int64_t polls);
 

@@ -365,8 +365,8 @@ def selftest_wait(spin_limit: int, stream=None) -> int:
 
 
 def set_wait_limit(polls: int) -> int:
-    """tb_set_wait_limit: polls after which a radix-pass look-back wait gives
-    up (0 restores the default)."""
+    """tb_set_wait_limit: polls after which a bounded wait of a sort, of the
+    moments or of a one-launch batched build gives up (0 restores the default)."""
     return int(lib().tb_set_wait_limit(int(polls)))
 
 

@@ -70,6 +70,7 @@ def test_moment_waits_run_out_then_next_build_is_exact(n, mode):
     assert t.sync() == 0
     keys = ("mass", "com", "com_lo", "quad", "aabb")
     want = {k: getattr(t, k).clone() for k in keys}
+    ran_out = 0
     for _ in range(20):
         m.build(p, w, mom_mode=mode, tree=t)
         m.set_wait_limit(1)
@@ -79,6 +80,10 @@ def test_moment_waits_run_out_then_next_build_is_exact(n, mode):
         finally:
             m.set_wait_limit(0)
         assert m.STATUS[st] in ("TB_OK", "TB_ETIMEOUT")
+        ran_out += m.STATUS[st] == "TB_ETIMEOUT"
+    # hundreds of blocks do not all reach a barrier within one poll of each other
+    # (20,000 particles have one level of several blocks only)
+    assert ran_out > 0 or n == 20_000
     m.moments(m.build(p, w, mom_mode=mode, tree=t), p, w)
     assert t.sync() == 0
     for k in keys:
