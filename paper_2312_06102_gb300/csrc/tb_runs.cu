@@ -44,6 +44,10 @@ __global__ void __launch_bounds__(kCtaThreads, 1)
     long_run_kernel(uint64_t *keys, int32_t *vals, uint64_t *alt_k, int32_t *alt_v, int64_t n,
                     int shift0, RunBuffers rb, DevInfo *info) {
     after_previous();
+    // after a look-back that gave up the keys are not in order: the search for a
+    // run's end could then take in another queued run, and two blocks would sort
+    // the same keys, each with digit counts that no longer hold
+    if (info->status & kErrTimeout) return;
     extern __shared__ __align__(16) unsigned char raw[];
     CtaSortShared &sm = *reinterpret_cast<CtaSortShared *>(raw);
     __shared__ uint32_t s_q;

@@ -29,11 +29,17 @@ from gpu_util import assert_structure_equal, tb, torch  # noqa: E402
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-def test_lookback_wait_runs_out_then_next_build_is_exact():
+@pytest.mark.parametrize("gen", ["uniform", "clumps"])
+def test_lookback_wait_runs_out_then_next_build_is_exact(gen):
+    """(Clumps: runs of some thousand keys with equal upper bits, which are left
+    alone when the passes before did not order them.)"""
     m = tb()
     # 2^21 particles: 512 tiles of 4096 keys in each of the five passes, with
     # hundreds of tiles in flight at once
     pos, mass = uniform_cube(1 << 21, 23)
+    if gen == "clumps":
+        rng = np.random.default_rng(24)
+        pos = (rng.random((512, 3))[rng.integers(0, 512, len(pos))] + 5e-5 * (pos - 0.5)).astype(np.float32)
     p = torch.from_numpy(pos).cuda()
     w = torch.from_numpy(mass).cuda()
     t = m.Tree()
