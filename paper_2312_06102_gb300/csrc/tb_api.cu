@@ -12,6 +12,13 @@ namespace tb {
 
 int64_t g_launches = 0;
 
+// Test hook: TB_FAULT_COOPERATIVE=1 stands for a device that takes no cooperative
+// launch, to exercise the launches per level and per phase.
+bool fault_cooperative() {
+    static const bool v = std::getenv("TB_FAULT_COOPERATIVE") != nullptr;
+    return v;
+}
+
 // Test hook: TB_FAULT_LOAD=k makes the process's first k loads of a kernel
 // ahead of its launch fail.
 bool fault_load() {

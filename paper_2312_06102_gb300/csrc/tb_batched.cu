@@ -724,8 +724,9 @@ cudaError_t launch_batched_one_t(const BatchArgs &A, int32_t S, int ncrit, int64
     const int32_t *leaf_cell = t.leaf_cell;
     int64_t nt = n_total, cap = cell_cap, lim = g_wait_limit;
     void *args[] = {&a, &order, &out, &Tr, &o, &leaf_cell, &nt, &cap, &lim};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), dim3(grid), dim3(T), args,
-                                    smem, s);
+    e = fault_cooperative() ? cudaErrorCooperativeLaunchTooLarge
+                            : cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(kern), dim3(grid),
+                                                          dim3(T), args, smem, s);
     if (e != cudaSuccess) return e;
     ++g_launches;
     mark(ws, "batch_all", s);

@@ -244,6 +244,7 @@ cudaError_t launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t sme
 }
 
 bool fault_load();   // test hook (TB_FAULT_LOAD): this load fails
+bool fault_cooperative();   // test hook (TB_FAULT_COOPERATIVE): the device takes no cooperative launch
 
 template <class K>
 cudaError_t load_kernel(K kernel) {

@@ -856,8 +856,10 @@ cudaError_t moments_impl(tb_tree &t, Workspace &ws, cudaStream_t s) {
     const int32_t *lq = long_queue(ws, n);
     int64_t lim = g_wait_limit;
     void *args[] = {&T, &o, &src, &lq, &ws.info, &d_hi, &d_lo, &leaves, &two, &lim};
-    e = cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(upward_kernel<MODE>),
-                                    dim3((unsigned)grid), dim3(kLmThreads), args, smem, s);
+    e = fault_cooperative()
+            ? cudaErrorCooperativeLaunchTooLarge
+            : cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(upward_kernel<MODE>),
+                                          dim3((unsigned)grid), dim3(kLmThreads), args, smem, s);
     if (e == cudaSuccess) {
         ++g_launches;
     } else {

@@ -11,6 +11,8 @@
 - A kernel of the allocation-free sort that cannot be loaded: TB_FAULT_LOAD=k
   makes the first k loads fail in a child process; each call that meets one
   reports TB_ENOMEM, and the next call tries again.
+- A device that takes no cooperative launch: TB_FAULT_COOPERATIVE=1 in a child
+  process; the same results come from one launch per level or phase.
 """
 import os
 import subprocess
@@ -149,3 +151,51 @@ def test_noalloc_loads_again_after_a_failed_load():
     assert [v.split()[1] for v in r.stdout.splitlines() if v.startswith("RESULT")] == \
         ["TB_ENOMEM", "TB_ENOMEM", "TB_OK", "TB_OK"], r.stdout
     assert "EQUAL True True" in r.stdout
+
+
+_SEPARATE = r"""
+import sys
+import numpy as np, torch
+sys.path.insert(0, sys.argv[1])
+import paper_2312_06102_gb300 as tb
+from synth import clustered_halos
+pos, mass = clustered_halos(50_000, 27, n_halo=40)
+# a leaf of 3,000 (summed by a block) and one of 300 (by a warp) among the queued
+pos = np.concatenate([pos, np.full((3000, 3), pos[5], np.float32), np.full((300, 3), pos[7], np.float32)])
+mass = np.concatenate([mass, np.full(3300, mass[3], np.float32)])
+p, w = torch.from_numpy(pos).cuda(), torch.from_numpy(mass).cuda()
+off = torch.tensor([0, 20_000, 20_000, 53_300], device="cuda")
+out = {}
+for mode in (0, 1, 2):
+    t = tb.moments(tb.build(p, w, n_crit=8, mom_mode=mode), p, w)
+    tb.moments(t, p, w)
+    n0 = tb.kernel_launches()
+    tb.moments(t, p, w)
+    out[f"launches{mode}"] = tb.kernel_launches() - n0
+    b = tb.build_batched(p, w, off, mom_mode=mode, cell_capacity=30_000, one_launch=True)
+    for name, v in (("single", t), ("batched", b)):
+        assert v.sync() == 0
+        for k in ("mass", "com", "com_lo", "quad", "aabb") + (("mass64", "com64", "quad64") if mode == 2 else ()):
+            out[f"{name}{mode}{k}"] = getattr(v, k)[:v.n_cells].cpu().numpy()
+np.savez(sys.argv[2], **out)
+"""
+
+
+def test_without_cooperative_launches(tmp_path):
+    got = []
+    for i, extra in enumerate(({}, {"TB_FAULT_COOPERATIVE": "1"})):
+        path = str(tmp_path / f"{i}.npz")
+        r = subprocess.run([sys.executable, "-c", _SEPARATE, ROOT, path], env=dict(os.environ, **extra),
+                           capture_output=True, text=True, timeout=600)
+        assert r.returncode == 0, r.stderr[-2000:]
+        got.append(dict(np.load(path)))
+    a, b = got
+    for mode in (0, 1, 2):
+        # leaves and one upward launch; leaves, queued leaves and 21 levels
+        assert (a.pop(f"launches{mode}"), b.pop(f"launches{mode}")) == (2, 23)
+    for k in a:
+        if k.startswith("batched"):
+            # (leaves of more than 2048 are summed in another order)
+            assert a[k].shape == b[k].shape and np.isfinite(b[k]).all()
+        else:
+            assert np.array_equal(a[k], b[k]), k
