@@ -29,8 +29,9 @@ struct TreeIn {
 // The FP32 moments of cells (mass, centre of mass and its low part, second
 // moment, bounding box) as a parent's combination reads its children's:
 // straight from the tree's arrays ...
+template <bool AHEAD>
 struct CellsGlobal {
-    static constexpr bool kAhead = true;   // the next child's loads are issued ahead
+    static constexpr bool kAhead = AHEAD;   // the next child's loads are issued ahead
     const float *mass, *com, *com_lo, *quad, *aabb;
     __device__ __forceinline__ float m(int64_t c) const { return mass[c]; }
     __device__ __forceinline__ float x(int64_t c, int a) const { return com[3 * c + a]; }
@@ -43,7 +44,8 @@ struct CellsGlobal {
         return reinterpret_cast<const float2 *>(aabb + 6 * c)[i];
     }
 };
-__device__ __forceinline__ CellsGlobal cells_of(const MomOut &o) {
+template <bool AHEAD>
+__device__ __forceinline__ CellsGlobal<AHEAD> cells_of(const MomOut &o) {
     return {o.mass, o.com, o.com_lo, o.quad, o.aabb};
 }
 
