@@ -196,7 +196,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
     __shared__ double s_scale;
     __shared__ bool s_exact, s_f32;
     __shared__ int s_q;
-    __shared__ int s_nlong;
+    __shared__ int s_nlong, s_desc;
     __shared__ int64_t s_long[32];
     __shared__ unsigned long long s_end;
     __shared__ StartCounts s_sc;
@@ -267,28 +267,38 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
             const int nl = s_nlong;
             for (int j = 0; j < nl; ++j) {
                 // a run of more than kRunMax keys (at most 16 start in a tile):
-                // its end, then the block sort of its low bits
+                // its end, then the block sort of its low bits, unless they are
+                // in order (identical keys, as of particles on a lattice)
                 const int64_t a = s_long[j];
                 const uint64_t tp = A.pkey[a] >> shift0;
-                if (threadIdx.x == 0) s_end = (unsigned long long)(o + ns);
+                if (threadIdx.x == 0) {
+                    s_end = (unsigned long long)(o + ns);
+                    s_desc = 0;
+                }
                 __syncthreads();
                 for (int64_t base = a + 1; base < o + ns; base += blockDim.x) {
                     const int64_t p = base + threadIdx.x;
-                    if (p < o + ns && (A.pkey[p] >> shift0) != tp) atomicMin(&s_end, (unsigned long long)p);
+                    if (p < o + ns) {
+                        const uint64_t k = A.pkey[p];
+                        if ((k >> shift0) != tp) atomicMin(&s_end, (unsigned long long)p);
+                        else if (k < A.pkey[p - 1]) s_desc = 1;
+                    }
                     __syncthreads();
                     const bool done = s_end < (unsigned long long)(o + ns);
                     __syncthreads();
                     if (done) break;
                 }
-                const int64_t len = (int64_t)s_end - a;
-                const int low_passes = (shift0 + kBRadixBits - 1) / kBRadixBits;
-                cta_histograms(A.pkey, a, len, 0, low_passes, sm);
-                const int np = cta_lsd_sort(A.pkey, A.perm, A.kalt, A.palt, a, len, 0, low_passes, false, false, sm);
-                if (np & 1)
-                    for (int64_t p = a + threadIdx.x; p < a + len; p += blockDim.x) {
-                        A.pkey[p] = A.kalt[p];
-                        A.perm[p] = A.palt[p];
-                    }
+                if (s_desc) {
+                    const int64_t len = (int64_t)s_end - a;
+                    const int low_passes = (shift0 + kBRadixBits - 1) / kBRadixBits;
+                    cta_histograms(A.pkey, a, len, 0, low_passes, sm);
+                    const int np = cta_lsd_sort(A.pkey, A.perm, A.kalt, A.palt, a, len, 0, low_passes, false, false, sm);
+                    if (np & 1)
+                        for (int64_t p = a + threadIdx.x; p < a + len; p += blockDim.x) {
+                            A.pkey[p] = A.kalt[p];
+                            A.perm[p] = A.palt[p];
+                        }
+                }
                 __syncthreads();
             }
         }

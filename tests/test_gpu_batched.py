@@ -17,8 +17,10 @@ def _run(pos, mass, offsets, n_crit=16, cap=0, mode=0, tree=None, threads=512, r
     p = torch.from_numpy(np.ascontiguousarray(pos, np.float32)).cuda()
     w = None if mass is None else torch.from_numpy(np.ascontiguousarray(mass, np.float32)).cuda()
     off = torch.from_numpy(np.asarray(offsets, np.int64)).cuda()
-    t = m.build_batched(p, w, off, n_crit=n_crit, cell_capacity=cap, mom_mode=mode, tree=tree,
-                        batch_threads=threads, root_pow2=root_pow2)
+    # threads = 0: the library's rule, whatever choice a tuner has cached
+    build = m._lib._build_batched if threads == 0 else m.build_batched
+    t = build(p, w, off, n_crit=n_crit, cell_capacity=cap, mom_mode=mode, tree=tree,
+              batch_threads=threads, root_pow2=root_pow2)
     torch.cuda.synchronize()
     assert t.sync() == 0
     return t, p, w, off
@@ -219,6 +221,55 @@ def test_batched_empty():
     t = m.build_batched(torch.zeros((0, 3), dtype=torch.float32, device="cuda"), None,
                         torch.zeros(4, dtype=torch.int64, device="cuda"))
     assert t.n_cells == 0
+
+
+def _clumped_set(n, width, rng):
+    """The unit cube's corners and, in random order, n - 2 particles in two cubes
+    of the given width, each from a corner of a depth-13 cell on."""
+    pos = (rng.integers(0, 2, (n, 1)) * 0.5 + 0.125) + width * rng.random((n, 3))
+    pos[0], pos[1] = 0.0, 1.0
+    return pos[rng.permutation(n)].astype(np.float32)
+
+
+def _long_runs(pos, shift):
+    """(longest run of keys equal above `shift`, runs of more than 128 that a
+    stable sort by those upper bits leaves out of order)"""
+    k = oracle.keys(pos)[0]
+    k = k[np.argsort(k >> np.uint64(shift), kind="stable")]
+    start = np.flatnonzero(np.r_[True, np.diff(k >> np.uint64(shift)) != 0])
+    end = np.r_[start[1:], len(k)]
+    descent = np.r_[0, np.cumsum(np.r_[False, k[1:] < k[:-1]])]
+    out = (end - start > 128) & (descent[end] - descent[start + 1] > 0)
+    return (end - start).max(), int(out.sum())
+
+
+@pytest.mark.parametrize("threads", [0, 512, 1024])
+@pytest.mark.parametrize("width", [2.0 ** -13, 2.0 ** -10.5, 2.0 ** -8])
+def test_batched_long_runs(threads, width):
+    """Sets with runs of more than 128 keys of equal upper bits that hold several
+    hundred distinct keys out of order, or (the last set) identical keys only.
+    Cubes of width 2^-13 are one run each above bit 31 and above bit 23; of
+    2^-10.5, a few runs above bit 31 and none above bit 23; of 2^-8, some seventy
+    runs above bit 31 in the largest set.  threads = 0 takes blocks of 256 here."""
+    rng = np.random.default_rng(int(-np.log2(width)))
+    sizes = [1500, 5, 2100, 20_000, 0, 60_000, 3]
+    parts = [_clumped_set(n, width, rng) if n > 100 else uniform_cube(max(n, 1), 70 + i)[0][:n]
+             for i, n in enumerate(sizes)]
+    if width < 2.0 ** -8:
+        for part in (parts[0], parts[2], parts[3], parts[5]):
+            assert _long_runs(part, 31)[1] > 0
+            assert (_long_runs(part, 23)[1] > 0) == (width == 2.0 ** -13)
+    else:
+        assert _long_runs(parts[5], 31)[1] > 50 and _long_runs(parts[5], 23)[0] <= 128
+    parts.append(rng.integers(0, 2, (3000, 3)).astype(np.float32))
+    assert _long_runs(parts[-1], 31) == (_long_runs(parts[-1], 23)[0], 0)
+    if threads == 0:
+        parts += [uniform_cube(6, 80 + i)[0] for i in range(300)]
+    n = [len(v) for v in parts]
+    assert threads or (len(n) > 304 and np.mean(n) <= 512)
+    pos, offsets = np.concatenate(parts), np.r_[0, np.cumsum(n)]
+    t, *_ = _run(pos, None, offsets, threads=threads)
+    _check_sets(t, pos, None, offsets, 16, sets=range(8))
 
 
 def test_tuning_times_the_default_rule():
