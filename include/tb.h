@@ -213,9 +213,9 @@ tb_status tb_moments(tb_tree *tree, const float *d_pos, const float *d_mass, tb_
  * from work queues, phases separated by grid barriers with bounded waits);
  * otherwise, and always with cell_capacity 0, it takes separate launches.
  * Of params it reads n_crit, mom_mode, cell_capacity and batch_threads;
- * key_order must be TB_KEYS_MORTON.  Each set is sorted by one block (five
- * 8-bit passes over the upper 40 key bits, then its runs of equal upper
- * bits), so radix_bits, sort_threads, sort_items and reorder are not used. */
+ * key_order must be TB_KEYS_MORTON.  Each set is sorted by one block (8-bit
+ * passes over its upper 32 or 40 key bits, then its runs of equal upper bits),
+ * so radix_bits, sort_threads, sort_items and reorder are not used. */
 tb_status tb_build_batched(const float *d_pos, const float *d_mass, const int64_t *d_set_offsets,
                            int32_t n_sets, int64_t n_total, const tb_params *params,
                            tb_stream stream, tb_tree **tree);

@@ -46,12 +46,13 @@ inline bool batch_many_small(int32_t S, int64_t n) { return S > 304 && n <= int6
 constexpr int kBRadixBits = kCtaRadixBits;
 constexpr int kBRadix = kCtaRadix;
 // the block sort orders the upper 40 key bits in five passes, or the upper 32
-// in four for sets of up to 2^17 particles; the runs of equal upper bits are
-// then ordered in place (tb_runs.cuh), the long ones by the same block sort of
-// their low bits.  So a set of tight clumps, all of it in long runs, takes
-// eight passes either way, and any other small set one less.
+// in four; the runs of equal upper bits are then ordered in place
+// (tb_runs.cuh), the long ones by the same block sort of their low bits, one
+// after another.  Four passes for sets of up to 2^17 particles, unless many of
+// their runs would be long (clumps), which fifth_pass tells.
 constexpr int kBMaxPasses = 5;
-__device__ __forceinline__ int batch_passes(int64_t ns) { return ns <= (int64_t(1) << 17) ? 4 : kBMaxPasses; }
+constexpr int kBTopShift = 63 - 4 * kBRadixBits;   // above this the upper 32 bits
+constexpr int64_t kBFourMax = int64_t(1) << 17;
 constexpr int kBMomThreads = 256;
 constexpr int kBigLeafSerial = 1 << 20;       // leaves above this are summed in FP64
 
@@ -183,6 +184,53 @@ __device__ void set_root_cube(const float *__restrict__ pos, int64_t o, int64_t 
     __syncthreads();
 }
 
+// Whether many of a set's runs of equal upper 32 bits will be long: of more
+// than kRunMax keys, each of which costs a block sort of its low bits (about 8 us,
+// as much as a pass over four tiles of the sort).  If so, prepares a fifth pass
+// before the four: its digit counts before theirs, and the keys where it starts
+// from.  A long run brings one digit of every pass to kRunMax, which rules it out
+// for most sets of up to 2^14 particles by the counts at hand.  Otherwise every
+// step-th group of 32 keys, one key per counter at most, is counted by a hash of
+// the upper 32 bits, in the place of the values: a long run brings its counter to
+// kRunMax / step on average, and one other key beside it.  (Two more than that
+// are asked for where keys are left out: at 2^17 keys 0.4% of the counters have
+// them by chance, a fifth of those of the shortest long runs do.)  200 sets of 2^17
+// particles in two cubes of 0.3% of the side each: 13.3 ms with four passes, 4.4
+// with five; 4,096 sets without clumps pay 0.8% for the question.  All threads of
+// the block, after a barrier; ends with one.
+template <int T>
+__device__ bool fifth_pass(CtaSortSharedT<T> &sm, uint64_t *keys, uint64_t *alt, int ns, bool staged) {
+    constexpr int E = CtaSortSharedT<T>::TILE;
+    uint32_t *count = reinterpret_cast<uint32_t *>(sm.vals);
+    const int d = threadIdx.x;
+    if (!__syncthreads_or(d < kBRadix && sm.hist[0][d] > kRunMax)) return false;
+    const int step = ns <= E ? 1 : 1 << (32 - __clz((ns - 1) / E));
+    for (int i = threadIdx.x; i < E; i += T) count[i] = 0;
+    __syncthreads();
+    for (int i = (d & ~31) * step + (d & 31); i < ns; i += T * step) {
+        const uint64_t k = staged ? sm.keys[i] : keys[i];
+        atomicAdd(count + (((uint32_t)(k >> kBTopShift) * 0x9e3779b1u) >> (__clz(E) + 1)), 1u);
+    }
+    __syncthreads();
+    const uint32_t many = kRunMax / step + (step > 1 ? 4 : 2);
+    bool run = false;
+    for (int i = threadIdx.x; i < E; i += T) run |= count[i] >= many;
+    // counted by the threads that find one, which are others for nearly each
+    if (__syncthreads_count(run) <= ns / E / 4) return false;
+    if (d < kBRadix) {
+        for (int p = 4; p > 0; --p) sm.hist[p][d] = sm.hist[p - 1][d];
+        sm.hist[0][d] = 0;
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < ns; i += T) {
+        const uint64_t k = staged ? sm.keys[i] : keys[i];
+        if (!staged) alt[i] = k;
+        atomicAdd(&sm.hist[0][(k >> (kBTopShift - kBRadixBits)) & (kBRadix - 1)], 1u);
+    }
+    __syncthreads();
+    return true;
+}
+
 // Every set from work queue 0: root cube, keys, sort, counts.  `raw` is the
 // block's dynamic shared memory (batch_front_smem<T> bytes).
 template <int T>
@@ -196,7 +244,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
     __shared__ double s_scale;
     __shared__ bool s_exact, s_f32;
     __shared__ int s_q;
-    __shared__ int s_nlong, s_desc;
+    __shared__ int s_nlong, s_desc, s_passes;
     __shared__ int64_t s_long[32];
     __shared__ unsigned long long s_end;
     __shared__ StartCounts s_sc;
@@ -228,7 +276,8 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
             A.set_root[4 * (int64_t)set + 3] = r.side;
             if (s_bad) atomicOr(&A.info->status, kErrNonFinite);
         }
-        const int passes = batch_passes(ns), shift0 = 63 - passes * kBRadixBits;
+        const int passes0 = ns <= kBFourMax ? 4 : kBMaxPasses, shift00 = 63 - passes0 * kBRadixBits;
+        if (threadIdx.x == 0) s_passes = passes0;
         for (int i = threadIdx.x; i < kBMaxPasses * kBRadix; i += blockDim.x) (&sm.hist[0][0])[i] = 0;
         __syncthreads();
         // ---- keys, records and every pass's digit histogram
@@ -240,7 +289,7 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
             const float m_eq = (float)(1.0 / (double)ns);
             // unsorted keys go where pass 0 reads them, so that the last pass
             // ends in pkey (a set of one sort tile keeps them in shared memory)
-            uint64_t *unsorted = passes & 1 ? A.kalt : A.pkey;
+            uint64_t *unsorted = passes0 & 1 ? A.kalt : A.pkey;
             for (int64_t i = o + threadIdx.x; i < o + ns; i += blockDim.x) {
                 const float x = A.pos[3 * i], y = A.pos[3 * i + 1], z = A.pos[3 * i + 2];
                 const uint64_t k = morton_key(quantise(x, lx, shi, slo, sc, ex, f32),
@@ -249,11 +298,14 @@ __device__ void front_sets(const BatchArgs &A, unsigned char *raw) {
                 if (staged) sm.keys[i - o] = k;
                 else unsorted[i] = k;
                 A.xm[i] = make_float4(x, y, z, A.mass ? A.mass[i] : m_eq);
-                for (int p = 0; p < passes; ++p)
-                    atomicAdd(&sm.hist[p][(k >> (shift0 + p * kBRadixBits)) & (kBRadix - 1)], 1u);
+                for (int p = 0; p < passes0; ++p)
+                    atomicAdd(&sm.hist[p][(k >> (shift00 + p * kBRadixBits)) & (kBRadix - 1)], 1u);
             }
         }
         __syncthreads();
+        if (passes0 == 4 && ns > kRunMax && fifth_pass<T>(sm, A.pkey + o, A.kalt + o, (int)ns, staged) && threadIdx.x == 0) s_passes = kBMaxPasses;
+        __syncthreads();
+        const int passes = s_passes, shift0 = 63 - passes * kBRadixBits;
         // ---- stable LSD sort of the set by its upper key bits (digit counts
         // taken above), then the runs of equal upper bits by the low bits
         if (passes & 1) cta_lsd_sort(A.kalt, A.palt, A.pkey, A.perm, o, ns, shift0, passes, true, staged, sm);

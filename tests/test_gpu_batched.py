@@ -272,6 +272,26 @@ def test_batched_long_runs(threads, width):
     _check_sets(t, pos, None, offsets, 16, sets=range(8))
 
 
+@pytest.mark.parametrize("threads", [0, 512, 1024])
+def test_batched_sets_around_the_four_pass_limit(threads):
+    """Sets of up to 2^17 particles take four passes, or five when many runs of
+    equal upper 32 bits are long, and larger ones five: sets of one size on each
+    side, spread out and in cubes of width 2^-8 (512 long runs above bit 31, none
+    above bit 23).  threads = 0 takes blocks of 256 here."""
+    rng = np.random.default_rng(17)
+    n = 1 << 17
+    parts = [uniform_cube(n, 91)[0], uniform_cube(n + 1, 92)[0], _clumped_set(n, 2.0 ** -8, rng),
+             _clumped_set(n + 1, 2.0 ** -8, rng)]
+    assert _long_runs(parts[2], 31)[1] > 256 and _long_runs(parts[2], 23)[0] <= 128
+    if threads == 0:
+        parts += [uniform_cube(6, 80 + i)[0] for i in range(1100)]
+    sizes = [len(v) for v in parts]
+    assert threads or (len(sizes) > 304 and np.mean(sizes) <= 512)
+    pos, offsets = np.concatenate(parts), np.r_[0, np.cumsum(sizes)]
+    t, *_ = _run(pos, None, offsets, threads=threads)
+    _check_sets(t, pos, None, offsets, 16, sets=range(5 if threads == 0 else 4))
+
+
 def test_tuning_times_the_default_rule():
     """The autotuner's choice is never slower than the rule it replaces."""
     from paper_2312_06102_gb300 import autotune
