@@ -301,21 +301,26 @@ def test_tuning_times_the_default_rule():
     assert set(ms) == {0, 512, 1024} and ms[best] == min(ms.values())
 
 
+@pytest.mark.parametrize("n_crit", [2, 16, 100])
 @pytest.mark.parametrize("sizes", ["many small", "few large"])
-def test_batched_default_block_sizes(sizes):
+def test_batched_default_block_sizes(sizes, n_crit):
     """The default block size follows the sets: 256 threads for more than 304
     sets of at most 512 particles on average, 1024 for at most 608 of at least
-    4096.  Structure and moments as with a named size, and the oracle's."""
+    4096.  Structure and moments as with a named size, and the oracle's; sets
+    around the sort tile of 256 threads (1,024 keys), and n_crit in and out of the
+    range of the four-particle counts."""
     rng = np.random.default_rng(8)
     n = rng.integers(0, 900, 400) if sizes == "many small" else rng.integers(3000, 9000, 6)
+    if sizes == "many small":
+        n[:185:37] = [1023, 1024, 1025, 2048, 2049]
     assert (n.mean() <= 512) if sizes == "many small" else (n.mean() >= 4096)
     pos, mass, offsets = _sets([int(v) for v in n], 21)
-    a, *_ = _run(pos, mass, offsets)
-    b, *_ = _run(pos, mass, offsets, threads=512)
+    a, *_ = _run(pos, mass, offsets, n_crit=n_crit, threads=0)
+    b, *_ = _run(pos, mass, offsets, n_crit=n_crit, threads=512)
     for k in ("pkey", "perm", "ckey", "level", "parent", "child_first", "child_end", "pfirst",
               "pend", "mass", "com", "com_lo", "quad", "aabb"):
         assert np.array_equal(to_np(getattr(a, k)), to_np(getattr(b, k))), k
-    _check_sets(a, pos, mass, offsets, 16, sets=range(0, len(n), 37 if len(n) > 50 else 1))
+    _check_sets(a, pos, mass, offsets, n_crit, sets=range(0, len(n), 37 if len(n) > 50 else 1))
 
 
 @pytest.mark.parametrize("sizes", ["many small", "few large", "between"])

@@ -156,12 +156,14 @@ def _runs_at_tile_ends():
     return pos
 
 
+@pytest.mark.parametrize("radix_bits", [0, 8])
 @pytest.mark.parametrize("order", [0, 1])
-def test_sort_runs_from_tile_end(order):
+def test_sort_runs_from_tile_end(order, radix_bits):
+    """By the one-launch sort, and (8 named) by the general passes and run step."""
     pos = _runs_at_tile_ends()
     if order:
         pos = pos[::-1].copy()
-    _check(pos, None, 4)
+    _check(pos, None, 4, radix_bits=radix_bits)
 
 
 @pytest.mark.parametrize("length", [2, 3, 31, 127, 128, 129])

@@ -22,8 +22,8 @@ def _positions(n, kind):
         return plummer(n, 70 + n % 97)[0]
     rng = np.random.default_rng(n)
     if kind == "clumps":
-        # two tight clumps and a far point: nearly all upper key bits equal,
-        # runs longer than a tile of the run step, in input order and not
+        # two tight clumps and a far point: few distinct keys, in runs longer
+        # than a tile of the run step
         pos = (rng.integers(0, 2, (n, 1)) * 0.25 + 1e-7 * rng.random((n, 3))).astype(np.float32)
         pos[0] = 1.0
         return pos
@@ -53,6 +53,32 @@ def test_keys_and_order_equal_the_oracle(n, kind):
         st, root = m.keys_sorted_noalloc(p, k, q)
         assert st == 0 and root[3] == side
         assert np.array_equal(to_np(k), okeys) and np.array_equal(to_np(q), operm)
+
+
+@pytest.mark.parametrize("hilbert", [False, True])
+@pytest.mark.parametrize("n", [1500, 16_385, 32_768])
+def test_long_runs_out_of_order_take_the_whole_key(n, hilbert):
+    """Two cubes of width 2^-13, each within one depth-10 cell and of hundreds of
+    distinct keys in random order: runs of more than 128 keys of equal upper 32
+    bits that hold a descent, which the sort takes eight more passes for."""
+    m = tb()
+    rng = np.random.default_rng(n)
+    pos = rng.integers(0, 2, (n, 1)) * 0.5 + 0.12515 + 2.0 ** -13 * rng.random((n, 3))
+    pos[0], pos[1] = 0.0, 1.0
+    pos = pos[rng.permutation(n)].astype(np.float32)
+    keys = oracle.keys(pos, "hilbert" if hilbert else "morton")[0]
+    assert len(np.unique(keys)) > n // 2
+    k = keys[np.argsort(keys >> np.uint64(31), kind="stable")]
+    same = (k[1:] >> np.uint64(31)) == (k[:-1] >> np.uint64(31))
+    start = np.flatnonzero(np.r_[True, ~same])
+    length = np.diff(np.r_[start, n])
+    descents = np.add.reduceat(np.r_[0, (same & (k[1:] < k[:-1])).astype(int)], start)
+    assert ((length > 128) & (descents > 0)).any()
+    okeys, operm = oracle.sort(keys)
+    t = m.build(torch.from_numpy(pos).cuda(), None, key_order=m.KEYS_HILBERT if hilbert else m.KEYS_MORTON)
+    assert t.sync() == 0
+    assert np.array_equal(to_np(t.pkey), okeys)
+    assert np.array_equal(to_np(t.perm), operm)
 
 
 @pytest.mark.parametrize("n", [1, 1500, 16_385, 32_768])
