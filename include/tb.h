@@ -102,8 +102,9 @@ typedef struct {
     int32_t sort_items;      /* 0 = tuned default; else keys per thread of a sort tile
                                 (compiled variants: see tb_sort_variant); tb_build only */
     int32_t batch_threads;   /* tb_build_batched only: threads of the block that builds
-                                one set, 512 (two sets per SM at a time; the default
-                                for 0) or 1024 (one) */
+                                one set, 512 (two sets per SM at a time) or 1024
+                                (one); 0: by the number and mean size of the sets
+                                (256, 512 or 1024; 512 with batch_one_launch) */
     int32_t key_order;       /* tb_key_order: TB_KEYS_MORTON (default) or TB_KEYS_HILBERT
                                 (tb_build only; tb_build_batched takes Morton keys) */
     int32_t batch_one_launch; /* tb_build_batched with cell_capacity > 0 only: 1 runs the

@@ -5,8 +5,8 @@
 // would give for the set alone), with a fixed number of launches whatever the
 // number of sets:
 //   set_order_kernel    : sets ordered largest first (work-queue order);
-//   batch_front_kernel  : persistent, one 1024-thread block per set taken from
-//                         an atomic work queue: root cube, keys, (x, y, z, m)
+//   batch_front_kernel  : persistent, one block of 256, 512 or 1024 threads per set
+//                         taken from an atomic work queue: root cube, keys, (x, y, z, m)
 //                         records and the digit histograms of every pass, then a
 //                         stable LSD radix sort of the set inside the block (its
 //                         tiles in order, so no look-back is needed), then the
@@ -705,7 +705,7 @@ cudaError_t launch_batched_t(const BatchArgs &A, int32_t S, int ncrit, tb_tree &
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     // persistent grids: as many blocks as fit at once (1024 / T front blocks
-    // per SM, two emission blocks), at most one per set
+    // per SM), at most one per set
     auto fit = [&](int per_sm) { return S < per_sm * nsm ? (S > 0 ? S : 1) : per_sm * nsm; };
     if (phase == 0) {
         launch_after(set_order_kernel, dim3(1), dim3(1024), 0, s, A.off, S, ws.set_order, ws.info);

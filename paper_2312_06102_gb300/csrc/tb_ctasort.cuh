@@ -1,8 +1,8 @@
 // tb_ctasort.cuh -- a stable LSD radix sort of one contiguous range of
-// (64-bit key, 32-bit value) pairs by a single block of T threads (T = 512 or
-// 1024): every pass takes the range's tiles in order with running per-digit
-// offsets, so it needs no coordination with other blocks.  Used for the sets
-// of a batched build and for the rare long runs left by the single-tree sort.
+// (64-bit key, 32-bit value) pairs by a single block of T threads (T = 256, 512
+// or 1024): every pass takes the range's tiles in order with running per-digit
+// offsets, so it needs no coordination with other blocks.  Used for the sets of
+// a batched build and for the rare long runs left by the single-tree sort.
 #pragma once
 
 #include "tb_device.cuh"

@@ -90,7 +90,8 @@ struct Workspace {
     float *bbox_part = nullptr;      // [blocks][8]
     uint32_t *level_cnt = nullptr;   // [level tiles][kLevelFields]
     uint16_t *ml = nullptr;          // [n] m_k | L_k << 8 of each sorted particle
-    int32_t *long_runs = nullptr;    // [n / 1024 + 2] sort runs too long for the run step
+    int32_t *long_runs = nullptr;    // long_run_capacity(n) words: sort runs too long for the run
+                                     // step, and the tiles' descent flags
     int32_t *big_leaf = nullptr;     // [n] queue of depth-21 leaves too long for one thread
     DevInfo *info = nullptr;
     DevInfo *h_info = nullptr;       // pinned host mirror

@@ -2,9 +2,9 @@
 // (Sec. 2.3 step 2).
 //
 // The paper sorts on the CPU with parallel sorting by regular sampling; on
-// the GPU the keys are sorted by ceil(63 / b) stable least-significant-digit
-// passes of b bits (bit 63 is always 1).  Each pass is one "onesweep" launch
-// (Adinets & Merrill 2022):
+// the GPU the keys are sorted by ceil(40 / b) stable least-significant-digit
+// passes of b bits, over their upper bits (bit 63 is always 1).  Each pass is one
+// "onesweep" launch (Adinets & Merrill 2022):
 //   - every block takes the next tile id from an atomic counter, so a block
 //     only ever waits on tiles that blocks already running own;
 //   - it ranks its tile's digits stably, warp by warp (ballot peer masks,
@@ -296,13 +296,15 @@ __global__ void __launch_bounds__(THREADS, (THREADS <= 256 ? (ITEMS <= 8 ? 4 : 2
 // The pass for 8-bit digits (the default), arranged for many keys per thread:
 //   - keys go through shared memory and out first, then values through the same
 //     memory, and the values are loaded only when the keys have left the
-//     registers, so that a tile of 5376 keys (256 x 21) takes 52 KB and 85
-//     registers, three to an SM;
+//     registers, so that a tile of 5376 keys (256 x 21) takes 52 KB, three to an
+//     SM, at 80 registers (of which 112 to 124 bytes a thread spill; 512 x 14, two
+//     to an SM at 64, spills 120 to 128);
 //   - a key's place in the tile is kept in 16 bits, each warp's counters are
 //     turned into places in the tile at once (one shared read per key), and a
 //     full tile carries no bounds checks.
-// What bounds it is latency and barriers, at 133 instructions a key (172
-// before): 0.94 ms at 2^27 keys, 3.3 TB/s, where one thread-register tile of
+// What bounds it is latency: the warps wait on the tile's barriers and on shared
+// memory, with 40% of the issue slots and a third of DRAM busy.  133
+// instructions a key (172 before), 0.94 ms at 2^27 keys, 3.3 TB/s, where one thread-register tile of
 // 512 x 8 pairs took 1.19; 142 us against 160 at 2^24.
 template <int T, int ITEMS>
 struct Sort8Smem {

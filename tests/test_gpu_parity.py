@@ -381,12 +381,11 @@ def test_deterministic_repeat():
 
 @pytest.mark.parametrize("mode", [0, 1, 2])
 def test_moments_repeat_on_one_build(mode):
-    """Parents are combined by the last of their children to finish, which
-    counts arrivals per cell and clears the count as it combines: calling
+    """Every call clears the leaf queues and the barrier count it used: calling
     tb_moments again on the same build gives the same moments bit for bit.
     Identical particles add a leaf of 3,000 (block-summed) and one of 300
     (past the leaf tile's halo, summed from the queue), whose ancestors are
-    combined from those launches."""
+    combined after those."""
     pos, mass = clustered_halos(1 << 16, 21, n_halo=40)
     pos = np.concatenate([pos, np.full((3000, 3), pos[5], np.float32),
                           np.full((300, 3), pos[7], np.float32)])
